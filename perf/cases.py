@@ -221,3 +221,99 @@ def tolerance(case):
     # the tensor-core path against the fp32 kernels on the same bits: 3.5e-3 .. 5e-3 per tensor, single values up to 0.24
     # (rows of a few tokens that cancel); the fp32 kernels with chunks of 16 against chunks of 64: 6e-7, values to 7e-6
     return {"rel": 1.5e-2, "max": 0.6} if case["dtype"] == "bf16" else {"rel": 1e-5, "max": 2e-4}
+
+
+# ---------------------------------------------------------------------------------------------------------------
+# the same results in 64 bits, from the equations of the layer alone (chunks of 64 tokens, reverse pass by autograd)
+
+def _exact_sequence(variant, q, k, v, g, beta, state):
+    """One batch of equally long sequences, [B, H, T, d]: q and k (GDN: q and v) already carry their gates."""
+    outs = []
+    n = q.shape[2]
+    parts = [x.split(64, 2) if x is not None else None for x in (q, k, v, g, beta)]
+    for i in range((n + 63) // 64):
+        qc, kc, vc, gc = (p[i] for p in parts[:4])
+        b = gc.cumsum(2)                                     # [B, H, C, d_k or 1]
+        last = b[:, :, -1:]
+        if variant == "gdn":
+            ratio = torch.exp((b - b.transpose(2, 3)).tril())            # e^{b_i - b_j} for j <= i
+            low = (parts[4][i] * (kc @ kc.transpose(2, 3)) * ratio).tril(-1)
+            rhs = parts[4][i] * (vc - torch.exp(b) * (kc @ state))
+            u = torch.linalg.solve_triangular(low, rhs, upper=False, unitriangular=True)
+            outs.append((qc * torch.exp(b)) @ state + ((qc @ kc.transpose(2, 3)) * ratio).tril() @ u)
+            state = torch.exp(last) * state + (torch.exp(last - b) * kc).transpose(2, 3) @ u
+        else:
+            qh, kh = qc * torch.exp(b), kc * torch.exp(-b)
+            outs.append((qh @ kh.transpose(2, 3)).tril() @ vc + qh @ state)
+            state = torch.exp(last).transpose(2, 3) * (state + kh.transpose(2, 3) @ vc)
+    return torch.cat(outs, 2), state
+
+
+def _exact_layer(case, q, k, v, decay, lq, lk, beta, h0):
+    variant, (B, T, H) = case["variant"], q.shape[:3]
+    gq, gk = torch.softmax(lq, -1).unsqueeze(-1), torch.softmax(lk, -1).unsqueeze(-1)
+    q = gq * q
+    if variant == "gdn":
+        v = gk * v
+    else:
+        k = gk * k
+    g = decay if variant == "gla" else (decay.view(1, 1, H, 1).expand(B, T, H, 1) if variant == "retnet" else decay.unsqueeze(-1))
+    beta = beta.unsqueeze(-1) if variant == "gdn" else None
+    cuts = _lengths(case) if case["kind"] == "packed" else [0, T]
+    lens = [b - a for a, b in zip(cuts, cuts[1:])]
+    parts = [x.transpose(1, 2).split(lens, 2) if x is not None else [None] * len(lens) for x in (q, k, v, g, beta)]
+    outs, states = [], []
+    for i in range(len(lens)):
+        start = h0 if h0 is not None else q.new_zeros(B, H, case["dk"], case["dv"])
+        o, st = _exact_sequence(variant, *(p[i] for p in parts), start)
+        outs.append(o)
+        states.append(st)
+    return torch.cat(outs, 2).transpose(1, 2), torch.cat(states)
+
+
+def _exact_feature_map(x, taps, normalize):
+    B, T, H, d = x.shape
+    padded = torch.nn.functional.pad(x.reshape(B, T, H * d), (0, 0, 3, 0))
+    y = sum(taps[:, j] * padded[:, j:j + T] for j in range(4)).view(B, T, H, d)
+    z = y * torch.sigmoid(y)
+    return z / torch.sqrt((z * z).sum(-1, keepdim=True) + 1e-6) if normalize else z
+
+
+def exact(case, seed):
+    s = prepare(case, seed)
+    kind, variant = case["kind"], case["variant"]
+    x = {n: t.double() for n, t in s.items() if isinstance(t, torch.Tensor) and n not in ("ht", "ws")}
+    del s
+    if kind in ("decode", "prefill"):
+        if x["q"].dim() == 3:                                # one token a call: no token axis
+            t = {n: x[n].unsqueeze(1) for n in ("q", "k", "v", "lq", "lk") + (("beta",) if variant == "gdn" else ())}
+            t["decay"] = x["decay"] if variant == "retnet" else x["decay"].unsqueeze(1)
+        else:
+            t = x
+        with torch.no_grad():
+            o, st = _exact_layer(case, t["q"], t["k"], t["v"], t["decay"], t["lq"], t["lk"], t.get("beta"),
+                                 x.get("state", x.get("h0")))
+        return dict(o=o, ht=st) if kind == "prefill" else dict(o=o.reshape(x["q"].shape[:-1] + (case["dv"],)), state=st)
+    grads = {n: t.requires_grad_() for n, t in x.items() if n not in ("dO", "dy", "h0")}
+    if kind != "layer":
+        o, st = _exact_layer(case, x["q"], x["k"], x["v"], x["decay"], x["lq"], x["lk"], x.get("beta"), x.get("h0"))
+        o.backward(x["dO"])
+        return dict(o=o.detach(), ht=st.detach(), dq=grads["q"].grad, dk=grads["k"].grad, dv=grads["v"].grad,
+                    dlog_decay=None if variant == "retnet" else grads["decay"].grad,
+                    dbeta=grads["beta"].grad if variant == "gdn" else None,
+                    dgq_logits=grads["lq"].grad, dgk_logits=grads["lk"].grad, dh0=None)
+    q, k, v = x["x_q"], x["x_k"], x["x_v"]
+    if variant == "gdn":
+        q, k, v = (_exact_feature_map(x["x_" + n], x["taps_" + n], n != "v") for n in "qkv")
+    lq, lk = (torch.einsum("bthc,ch->bth", t, x[w]) for t, w in ((q, "w_gq"), (k, "w_gk")))
+    o, _ = _exact_layer(case, q, k, v, x["decay"], lq, lk, x.get("beta"), None)
+    y = o.flatten(2) @ x["w_o"]
+    y.backward(x["dy"])
+    out = dict(y=y.detach(), dw_o=x["w_o"].grad, dw_gq=x["w_gq"].grad, dw_gk=x["w_gk"].grad,
+               dlog_decay=None if variant == "retnet" else x["decay"].grad,
+               dbeta=x["beta"].grad if variant == "gdn" else None)
+    for n in "qkv":
+        out["dx_" + n] = x["x_" + n].grad
+        if variant == "gdn":
+            out["dtaps_" + n] = x["taps_" + n].grad
+    return out
