@@ -110,7 +110,8 @@ sla_status sla_plan_destroy(sla_plan *plan);
 sla_status sla_plan_set_sequences(sla_plan *plan, const int32_t *cu_seqlens, int32_t n_seq);
 
 /* Bytes of caller-provided scratch that sla_forward / sla_backward need for this plan (it depends on the kernels the
- * plan selects; 0 means none is needed and the workspace pointer may then be NULL). */
+ * plan selects; 0 means none is needed and the workspace pointer may then be NULL).  sla_forward on a bf16 Softmax-GatedDeltaNet
+ * plan without SLA_FLAG_SAVE_FOR_BACKWARD also accepts less, or none: it then runs on slower kernels that need no scratch. */
 sla_status sla_plan_workspace_bytes(const sla_plan *plan, size_t *forward_bytes, size_t *backward_bytes);
 
 /* Synchronises with nothing; copies the plan's device status word back (on the legacy default

@@ -77,7 +77,7 @@ static void plan_workspace_sizes(sla_plan *p) {
                                                            : sla::gla_tc_backward_workspace_bytes(d, &p->varlen);
     }
     if (sla::gdn_tc_supported(d) && !generic) {
-        p->fwd_bytes = 0;
+        p->fwd_bytes = sla::gdn_tc_forward_workspace_bytes(d, &p->varlen);
         p->bwd_bytes = sla::gdn_tc_backward_workspace_bytes(d, &p->varlen);
     }
     if ((p->flags & SLA_FLAG_SAVE_FOR_BACKWARD) && forward_can_save(*p) && p->bwd_bytes > p->fwd_bytes)
@@ -313,7 +313,12 @@ sla_status sla_forward(sla_plan *plan, const void *q, const void *k, const void 
     const void *ptrs[] = {q, k, v, log_decay, beta, gq_logits, gk_logits, h0, o, ht, workspace};
     for (const void *p : ptrs)
         if (!aligned16(p)) return SLA_ERR_INVALID_ARG;
-    if (plan->fwd_bytes > 0 && (!workspace || workspace_bytes < plan->fwd_bytes)) return SLA_ERR_WORKSPACE;
+    if (plan->fwd_bytes > 0 && (!workspace || workspace_bytes < plan->fwd_bytes)) {
+        // Softmax-GatedDeltaNet has a kernel that needs none: a caller without scratch gets that one
+        const bool scratch_free = sla::gdn_tc_supported(d) && !(plan->flags & (SLA_FLAG_FORCE_GENERIC | SLA_FLAG_SAVE_FOR_BACKWARD));
+        if (!scratch_free) return SLA_ERR_WORKSPACE;
+        workspace = nullptr;
+    }
     sla::FwdArgs a{q, k, v, log_decay, beta, gq_logits, gk_logits, h0, o, ht, (float *)workspace, plan->d_status,
                    plan->varlen.n_seq ? &plan->varlen : nullptr};
     plan->tracer.start((cudaStream_t)cuda_stream);

@@ -572,14 +572,19 @@ bool gdn_tc_supported(const Dims &d) {
 
 int gdn_tc_configure() {
     if (!encode_fn()) return -1;
+    if (gdn_chunk_configure() != 0) return -1;
     return cudaFuncSetAttribute(k_gdn_fwd_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gd::SMEM_BYTES) ==
                    cudaSuccess ? 0 : -1;
 }
 
+size_t gdn_tc_forward_workspace_bytes(const Dims &d, const Varlen *vl) {
+    return gdn_chunk_selected(d, vl) ? gdn_chunk_forward_workspace_bytes(d, vl) : 0;
+}
+
 // per-sequence tensor maps of a packed batch (q, k, v and, when given, o) into region `r`
 static const CUtensorMap *gdn_varlen_maps(const Dims &d, const FwdArgs &a, int r, cudaStream_t st) {
-    const void *key[] = {a.q, a.k, a.v, a.o};
-    return varlen_maps(*a.vl, r, key, 4, st, [&](const SeqInfo &si, CUtensorMap *m) {
+    const void *key[] = {a.q, a.k, a.v, a.o, nullptr};      // (the chunk-parallel kernels keep other maps of these tensors here)
+    return varlen_maps(*a.vl, r, key, 5, st, [&](const SeqInfo &si, CUtensorMap *m) {
         const size_t tok = (size_t)si.t0 * d.H;      // (q, k are d_k wide, v, o and their gradients d_v)
         if (!make_tile_map(m + 0, (const __nv_bfloat16 *)a.q + tok * d.dk, 1, si.T, d.H, d.dk) ||
             !make_tile_map(m + 1, (const __nv_bfloat16 *)a.k + tok * d.dk, 1, si.T, d.H, d.dk) ||
@@ -607,7 +612,10 @@ int gdn_tc_forward_save(const Dims &d, const FwdArgs &a, uint8_t *save, int *sta
 }
 
 // Forward; with `save` not null it also leaves the per-chunk records for a later gradient sweep over the same inputs.
+// Without a workspace (a.ws null) every shape runs on the one-CTA-per-sequence kernel.
 int gdn_tc_forward(const Dims &d, const FwdArgs &a, uint8_t *save, int *status, cudaStream_t st, Tracer &tr) {
+    if ((save || a.ws) && gdn_chunk_selected(d, a.vl))
+        return gdn_chunk_forward(d, a, save ? save : reinterpret_cast<uint8_t *>(a.ws), save != nullptr, status, st, tr);
     CUtensorMap mq, mk, mv, mo;
     if (!make_tile_map(&mq, a.q, d.B, d.T, d.H, d.dk) || !make_tile_map(&mk, a.k, d.B, d.T, d.H, d.dk) ||
         !make_tile_map(&mv, a.v, d.B, d.T, d.H, d.dv) || !make_tile_map(&mo, a.o, d.B, d.T, d.H, d.dv))

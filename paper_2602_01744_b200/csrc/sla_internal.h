@@ -155,9 +155,10 @@ void gla_tc_backward_segment_table(const Dims &d, int P, int L, Varlen &segs);
 size_t gla_tc_backward_segmented_workspace_bytes(const Dims &d, const Varlen &segs);
 int gla_tc_backward_segmented(const Dims &d, const BwdArgs &a, Varlen &segs, int *status, cudaStream_t st, Tracer &tr);
 
-// ---- tensor-core Softmax-GatedDeltaNet forward (WY form): sla_gdn_tc.cu.  Needs no workspace. ----
+// ---- tensor-core Softmax-GatedDeltaNet forward (WY form): sla_gdn_tc.cu.  One CTA per sequence, needs no workspace. ----
 bool gdn_tc_supported(const Dims &d);
 int gdn_tc_configure();
+size_t gdn_tc_forward_workspace_bytes(const Dims &d, const Varlen *vl = nullptr);
 int gdn_tc_forward(const Dims &d, const FwdArgs &a, uint8_t *save, int *status, cudaStream_t st, Tracer &tr);
 uint8_t *gdn_tc_records(float *ws);        // where in the backward workspace the per-chunk records sit
 int gdn_tc_forward_save(const Dims &d, const FwdArgs &a, uint8_t *save, int *status, cudaStream_t st, Tracer &tr);
@@ -165,6 +166,14 @@ int gdn_tc_forward_save(const Dims &d, const FwdArgs &a, uint8_t *save, int *sta
 int gdn_tc_bwd_configure();
 size_t gdn_tc_backward_workspace_bytes(const Dims &d, const Varlen *vl = nullptr);
 int gdn_tc_backward(const Dims &d, const BwdArgs &a, bool have_records, int *status, cudaStream_t st, Tracer &tr);
+// Chunk-parallel form of the same (sla_gdn_chunk.cu): per-chunk records prepared and consumed in parallel, two products a
+// chunk on the serial chain.  gdn_tc_forward / gdn_tc_backward take it where gdn_chunk_selected says so.
+bool gdn_chunk_selected(const Dims &d, const Varlen *vl);
+int gdn_chunk_configure();
+size_t gdn_chunk_forward_workspace_bytes(const Dims &d, const Varlen *vl);     // records of a forward that saves nothing
+size_t gdn_chunk_record_bytes(const Dims &d, const Varlen *vl);                // records of a training step
+int gdn_chunk_forward(const Dims &d, const FwdArgs &a, uint8_t *rec, bool save, int *status, cudaStream_t st, Tracer &tr);
+int gdn_chunk_backward(const Dims &d, const BwdArgs &a, bool have_records, int *status, cudaStream_t st, Tracer &tr);
 int gate_bwd_prod(const float *lq, const float *lk, const float *pq, const float *pk, float *dlq, float *dlk, long n_tok,
                   int H, cudaStream_t st);
 

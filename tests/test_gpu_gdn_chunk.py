@@ -1,0 +1,71 @@
+"""GPU parity of the chunk-parallel Softmax-GatedDeltaNet kernels (taken from more than 16 chunks per sequence or 256 chunks in
+all on) against the fp64 oracle, at the edges of their ranges."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2602_01744_b200 import api
+from paper_2602_01744_b200.inputs import CONFIGS, make_inputs, small
+from tests import gpu_util as gu
+
+pytestmark = pytest.mark.gpu
+
+
+# 17 chunks, the last of 1 and of 63 tokens; one head; more (sequence, head, slice) items than SMs, one and two chunks each;
+# head widths; the batch that just passes 256 chunks
+@pytest.mark.parametrize("B,T,H,dk,dv,with_h0", [(1, 1025, 1, 128, 128, True), (1, 1151, 3, 128, 128, False), (20, 64, 16, 128, 128, True),
+                                                 (10, 65, 16, 128, 128, True), (2, 1090, 2, 64, 64, True), (1, 1100, 5, 64, 128, True),
+                                                 (1, 1100, 5, 128, 64, False), (1, 1280, 16, 64, 64, True)])
+def test_chunk_parallel_step_matches_the_oracle(B, T, H, dk, dv, with_h0):
+    cfg = small(CONFIGS["C4"], B=B, T=T, H=H, d_k=dk, d_v=dv, seed=1500 + T + H)
+    x = make_inputs(cfg, with_dO=True, with_h0=with_h0)
+    xd = gu.to_dev(x)
+    o, ht, g, plan, ws, lf, lb = gu.gpu_training_step(cfg, xd, h0=xd.get("h0"), dht=xd.get("dht"), want_dh0=with_h0)
+    assert (lf, lb) == (1, 2)
+    oref, htref = gu.oracle_forward(cfg, x, h0=x.get("h0"))
+    ref = gu.oracle_backward(cfg, x, h0=x.get("h0"), dht=x.get("dht"))
+    pairs = {"o": (o, oref), "ht": (ht, htref)}
+    pairs.update({n: (g[n], ref[r]) for n, r in gu.GRAD_NAMES.items() if g.get(n) is not None and np.linalg.norm(ref[r]) > 0})
+    gu.assert_close({n: gu.rel_l2(a, r) for n, (a, r) in pairs.items()},
+                    {n: gu.row_err(a, r) for n, (a, r) in pairs.items()}, cfg.dtype, cfg)
+    # without the states the forward left: recomputed, same bits; and a forward that saves nothing gives the same output
+    g2, plan2 = gu.gpu_backward(cfg, xd, h0=xd.get("h0"), dht=xd.get("dht"), want_dh0=with_h0)
+    assert plan2.last_launch_count == 3
+    o2, ht2, plan3 = gu.gpu_forward(cfg, xd, h0=xd.get("h0"))
+    assert plan3.forward_workspace_bytes > 0 and torch.equal(o, o2) and torch.equal(ht, ht2)
+    for n, t in g.items():
+        if t is not None:
+            assert torch.equal(t, g2[n]), n
+    # a caller that brings no workspace is served by the kernel that needs none
+    o3 = torch.empty_like(o)
+    api.sla_forward(plan3, xd["q"], xd["k"], xd["v"], xd["log_decay"], xd["gq_logits"], xd["gk_logits"], beta=xd["beta"],
+                    h0=xd.get("h0"), o=o3, workspace=torch.empty(16, dtype=torch.uint8, device="cuda"))
+    torch.cuda.synchronize()
+    plan3.poll()
+    assert gu.rel_l2(o3, oref) <= 1e-2
+
+
+def test_chunk_parallel_packed_batch_gives_the_bits_of_its_sequences_alone():
+    lens = [1100, 1, 1088, 64, 1300]
+    cu = [0] + list(np.cumsum(lens))
+    cfg = small(CONFIGS["C4"], B=1, T=cu[-1], H=2, seed=1600)
+    x = gu.to_dev(make_inputs(cfg, with_dO=True))
+    names = ("q", "k", "v", "log_decay", "gq_logits", "gk_logits")
+    plan = api.sla_plan_create(cfg.variant, cfg.dtype, 1, cfg.T, cfg.H, 128, 128, flags=api.SLA_FLAG_SAVE_FOR_BACKWARD)
+    plan.set_sequences(cu)
+    ws = plan.workspace(backward=True)
+    ht = torch.empty((len(lens), cfg.H, 128, 128), device="cuda")
+    o, _ = api.sla_forward(plan, *(x[n] for n in names), beta=x["beta"], ht=ht, workspace=ws)
+    g = api.sla_backward(plan, *(x[n] for n in names), x["dO"], beta=x["beta"], workspace=ws)
+    torch.cuda.synchronize()
+    plan.poll()
+    for s, (a, b) in enumerate(zip(cu, cu[1:])):
+        if b - a <= 1024:                                   # (alone, a short sequence takes the other kernels)
+            continue
+        c1 = small(cfg, T=b - a)
+        xs = {n: (None if t is None else t[:, a:b].clone()) for n, t in x.items()}
+        o1, ht1, g1, *_ = gu.gpu_training_step(c1, xs)
+        assert torch.equal(o1, o[:, a:b]) and torch.equal(ht1, ht[s:s + 1])
+        for n, t in g1.items():
+            if t is not None:
+                assert torch.equal(t, g[n][:, a:b]), n
