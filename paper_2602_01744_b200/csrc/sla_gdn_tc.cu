@@ -125,8 +125,9 @@ k_gdn_fwd_tc(const __grid_constant__ CUtensorMap gm_q, const __grid_constant__ C
     const uint32_t tmem = *reinterpret_cast<volatile uint32_t *>(sm + OFF_TMEM);
 
     if (warp == 8) {
-        // ---------------- MMA issue (one lane) ----------------
-        if (lane == 0) {
+        // ---------------- MMA issue (the warp walks the loop together, one lane issues) ----------------
+        {
+            const bool leader = elect_lane();
             constexpr uint32_t ID_64 = idesc_bf16(64, 64, 0, 0);     // K-major x K-major
             constexpr uint32_t ID_N = idesc_bf16(64, 128, 0, 1);     // K-major x MN-major
             constexpr uint32_t ID_S = idesc_bf16(128, 128, 1, 1);    // MN-major x MN-major
@@ -141,47 +142,55 @@ k_gdn_fwd_tc(const __grid_constant__ CUtensorMap gm_q, const __grid_constant__ C
                 wait(SREADY, par);                     // S_n: fp32 in TMEM, bf16 in shared memory
                 if (failed) break;
                 tc_fence_after();
+                if (leader)
 #pragma unroll
                 for (int kk = 0; kk < 8; ++kk)         // K K^T
                     tc_mma_bf16(tmem + COL_KK, kK + kstep_kmajor(kk, HALF_BF16), kK + kstep_kmajor(kk, HALF_BF16), ID_64, kk > 0);
+                if (leader)
 #pragma unroll
                 for (int kk = 0; kk < 8; ++kk)         // (scale Gq Gam q) K^T
                     tc_mma_bf16(tmem + COL_QK, kQ + kstep_kmajor(kk, HALF_BF16), kK + kstep_kmajor(kk, HALF_BF16), ID_64, kk > 0);
-                tc_commit(bar(BAR_1));
+                if (leader) tc_commit(bar(BAR_1));
                 if (n > 0) wait(OSTAGED + ((n - 1) & 1), ((n - 1) >> 1) & 1);   // O of chunk n-1 has been read out
                 if (failed) break;
+                if (leader)
 #pragma unroll
                 for (int kk = 0; kk < 8; ++kk)         // O = (scale Gq Gam q) S
                     tc_mma_bf16(tmem + COL_O, kQ + kstep_kmajor(kk, HALF_BF16), mS + kstep_mnmajor(kk), ID_N, kk > 0);
                 wait(TREADY, par);                     // bf16 T and Pq in shared memory; K K^T, q K^T read out
                 if (failed) break;
                 tc_fence_after();
+                if (leader)
 #pragma unroll
                 for (int kk = 0; kk < 4; ++kk)         // W = T (beta Gam K)
                     tc_mma_bf16(tmem + COL_W, kT + kstep_kmajor(kk, 0), mKB + kstep_mnmajor(kk), ID_N, kk > 0);
+                if (leader)
 #pragma unroll
                 for (int kk = 0; kk < 4; ++kk)         // U0 = T (beta Gk V)
                     tc_mma_bf16(tmem + COL_U, kT + kstep_kmajor(kk, 0), mV + kstep_mnmajor(kk), ID_N, kk > 0);
-                tc_commit(bar(BAR_2));
+                if (leader) tc_commit(bar(BAR_2));
                 wait(WREADY, par);                     // -W as bf16 in the q buffer
                 if (failed) break;
                 tc_fence_after();
+                if (leader)
 #pragma unroll
                 for (int kk = 0; kk < 8; ++kk)         // U = U0 - W S
                     tc_mma_bf16(tmem + COL_U, kQ + kstep_kmajor(kk, HALF_BF16), mS + kstep_mnmajor(kk), ID_N, 1);
-                tc_commit(bar(BAR_3));
+                if (leader) tc_commit(bar(BAR_3));
                 wait(UREADY, par);                     // U as bf16 in the k buffer
                 if (failed) break;
                 tc_fence_after();
+                if (leader)
 #pragma unroll
                 for (int kk = 0; kk < 4; ++kk)         // O += Pq U
                     tc_mma_bf16(tmem + COL_O, kPQ + kstep_kmajor(kk, 0), mU + kstep_mnmajor(kk), ID_N, 1);
+                if (leader)
 #pragma unroll
                 for (int kk = 0; kk < 4; ++kk)         // S += (e^{-b} K)^T U
                     tc_mma_bf16(tmem + COL_S, mKE + kstep_mnmajor(kk), mU + kstep_mnmajor(kk), ID_S, 1);
-                tc_commit(bar(BAR_4));
+                if (leader) tc_commit(bar(BAR_4));
             }
-            tc_commit(bar(DRAIN));
+            if (leader) tc_commit(bar(DRAIN));
             mbar_wait_bounded(bar(DRAIN), 0, nullptr, 20000000ull);
         }
     } else if (warp == 13) {

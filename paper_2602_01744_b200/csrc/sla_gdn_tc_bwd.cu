@@ -138,8 +138,9 @@ k_gdn_bwd_tc(const __grid_constant__ CUtensorMap gm_q, const __grid_constant__ C
     // chunks are visited in the order n = NT-1 ... 0; k = NT-1-n is the visit number that drives every barrier parity
 
     if (warp == 8) {
-        // ---------------- MMA issue (one lane) ----------------
-        if (lane == 0) {
+        // ---------------- MMA issue (the warp walks the loop together, one lane issues) ----------------
+        {
+            const bool leader = elect_lane();
             constexpr uint32_t I64 = idesc_bf16(64, 64, 0, 0);        // K-major x K-major, 64 x 64
             constexpr uint32_t IKK = idesc_bf16(64, 128, 0, 0);       // K-major x K-major
             constexpr uint32_t IKM = idesc_bf16(64, 128, 0, 1);       // K-major x MN-major
@@ -168,80 +169,100 @@ k_gdn_bwd_tc(const __grid_constant__ CUtensorMap gm_q, const __grid_constant__ C
                 wait(OPR, par);
                 if (failed) break;
                 tc_fence_after();
+                if (leader)
 #pragma unroll
                 for (int kk = 0; kk < 8; ++kk) tc_mma_bf16(tmem + R1, kK + k8(kk, HALF_BF16), kK + k8(kk, HALF_BF16), I64, kk > 0);
+                if (leader)
 #pragma unroll
                 for (int kk = 0; kk < 8; ++kk) tc_mma_bf16(tmem + R1 + 64, kQ + k8(kk, HALF_BF16), kK + k8(kk, HALF_BF16), I64, kk > 0);
+                if (leader)
 #pragma unroll
                 for (int kk = 0; kk < 4; ++kk) tc_mma_bf16(tmem + R2, kT1 + k8(kk, 0), mK + kstep_mnmajor(kk), IKM, kk > 0);
+                if (leader)
 #pragma unroll
                 for (int kk = 0; kk < 4; ++kk) tc_mma_bf16(tmem + R3, kT2 + k8(kk, 0), mV + kstep_mnmajor(kk), IKM, kk > 0);
-                tc_commit(bar(C1));
+                if (leader) tc_commit(bar(C1));
                 // ---- group 2: dU = Ke dZ + Pq^T dO ; dPq = dO U^T ; ak1 = U dZ^T ----
                 wait(S1R, par);
                 wait(FULL_DO, par);
                 wait(FULL_U, par);
                 if (failed) break;
                 tc_fence_after();
+                if (leader)
 #pragma unroll
                 for (int kk = 0; kk < 8; ++kk) tc_mma_bf16(tmem + R1, kKE + k8(kk, HALF_BF16), mDZ + kstep_mnmajor(kk), IKM, kk > 0);
+                if (leader)
 #pragma unroll
                 for (int kk = 0; kk < 4; ++kk) tc_mma_bf16(tmem + R1, mPQ + kstep_mnmajor(kk), mDO + kstep_mnmajor(kk), IMM, 1);
+                if (leader)
 #pragma unroll
                 for (int kk = 0; kk < 8; ++kk) tc_mma_bf16(tmem + R2, kDO + k8(kk, HALF_BF16), kU + k8(kk, HALF_BF16), I64, kk > 0);
+                if (leader)
 #pragma unroll
                 for (int kk = 0; kk < 8; ++kk) tc_mma_bf16(tmem + R3, kU + k8(kk, HALF_BF16), kDZ + k8(kk, STATE_HALF), IKK, kk > 0);
-                tc_commit(bar(C2));
+                if (leader) tc_commit(bar(C2));
                 // ---- group 3: dW = dU S^T ; aq = dO S^T + dPq Ke ; ak1 += dPq^T Qg ; dS += Qg^T dO - W^T dU ----
                 wait(S2R, par);
                 wait(FULL_S, par);
                 if (failed) break;
                 tc_fence_after();
+                if (leader)
 #pragma unroll
                 for (int kk = 0; kk < 8; ++kk) tc_mma_bf16(tmem + R1, kDU + k8(kk, HALF_BF16), kS + k8(kk, STATE_HALF), IKK, kk > 0);
+                if (leader)
 #pragma unroll
                 for (int kk = 0; kk < 8; ++kk) tc_mma_bf16(tmem + R2, kDO + k8(kk, HALF_BF16), kS + k8(kk, STATE_HALF), IKK, kk > 0);
+                if (leader)
 #pragma unroll
                 for (int kk = 0; kk < 4; ++kk) tc_mma_bf16(tmem + R2, kDP + k8(kk, 0), mKE + kstep_mnmajor(kk), IKM, 1);
+                if (leader)
 #pragma unroll
                 for (int kk = 0; kk < 4; ++kk) tc_mma_bf16(tmem + R3, mDP + kstep_mnmajor(kk), mQ + kstep_mnmajor(kk), IMM, 1);
+                if (leader)
 #pragma unroll
                 for (int kk = 0; kk < 4; ++kk) tc_mma_bf16(tmem + R0, mQ + kstep_mnmajor(kk), mDO + kstep_mnmajor(kk), ISS, 1);
+                if (leader)
 #pragma unroll
                 for (int kk = 0; kk < 4; ++kk) tc_mma_bf16(tmem + R0, mWN + kstep_mnmajor(kk), mDU + kstep_mnmajor(kk), ISS, 1);
-                tc_commit(bar(C3));
+                if (leader) tc_commit(bar(C3));
                 // ---- group 4: dKbg = T^T dW ; dVb = T^T dU ----
                 wait(S3R, par);
                 if (failed) break;
                 tc_fence_after();
+                if (leader)
 #pragma unroll
                 for (int kk = 0; kk < 4; ++kk) tc_mma_bf16(tmem + R1, mT + kstep_mnmajor(kk), mDW + kstep_mnmajor(kk), IMM, kk > 0);
+                if (leader)
 #pragma unroll
                 for (int kk = 0; kk < 4; ++kk) tc_mma_bf16(tmem + R2, mT + kstep_mnmajor(kk), mDU + kstep_mnmajor(kk), IMM, kk > 0);
-                tc_commit(bar(C4));
+                if (leader) tc_commit(bar(C4));
                 // ---- group 5: dL = dKbg (-W)^T + dVb (-U0)^T ----
                 wait(S4R, par);
                 if (failed) break;
                 tc_fence_after();
+                if (leader)
 #pragma unroll
                 for (int kk = 0; kk < 8; ++kk) tc_mma_bf16(tmem + R2, kDK + k8(kk, HALF_BF16), kWN + k8(kk, HALF_BF16), I64, kk > 0);
+                if (leader)
 #pragma unroll
                 for (int kk = 0; kk < 8; ++kk) tc_mma_bf16(tmem + R2, kDV + k8(kk, HALF_BF16), kU0 + k8(kk, HALF_BF16), I64, 1);
-                tc_commit(bar(C5));
-                tc_commit(bar(SFREE));
+                if (leader) tc_commit(bar(C5));
+                if (leader) tc_commit(bar(SFREE));
                 // ---- group 6: dKbg += dL Ke ; ak1 += (beta Gam dL)^T K ----
                 wait(S5R, par);
                 if (failed) break;
                 tc_fence_after();
+                if (leader)
 #pragma unroll
                 for (int kk = 0; kk < 4; ++kk) tc_mma_bf16(tmem + R1, kDL + k8(kk, 0), mKE + kstep_mnmajor(kk), IKM, 1);
+                if (leader)
 #pragma unroll
                 for (int kk = 0; kk < 4; ++kk) tc_mma_bf16(tmem + R3, mT + kstep_mnmajor(kk), mK + kstep_mnmajor(kk), IMM, 1);
-                tc_commit(bar(C6));
-                tc_commit(bar(KFREE));
+                if (leader) tc_commit(bar(C6));
+                if (leader) tc_commit(bar(KFREE));
                 wait(S6R, par);                        // the accumulators have been read out before the next chunk reuses them
             }
-            tc_commit(bar(DRAIN));
+            if (leader) tc_commit(bar(DRAIN));
             mbar_wait_bounded(bar(DRAIN), 0, nullptr, 20000000ull);
         }
     } else if (warp == 13) {

@@ -135,8 +135,9 @@ k_gla_fwd_tc(const __grid_constant__ CUtensorMap gm_q, const __grid_constant__ C
     const uint32_t tmem = *reinterpret_cast<volatile uint32_t *>(sm + OFF_TMEM);
 
     if (warp == W_MMA) {
-        // ---------------- MMA issue (one lane) ----------------
-        if (lane == 0) {
+        // ---------------- MMA issue (the warp walks the loop together, one lane issues) ----------------
+        {
+            const bool leader = elect_lane();
             constexpr uint32_t ID_A = idesc_bf16(64, 64, 0, 0);      // qh (K-major) x kh (K-major)
             constexpr uint32_t ID_O = idesc_bf16(64, 128, 0, 1);     // qh x S, A x V (B operand MN-major)
             constexpr uint32_t ID_Z = idesc_bf16(128, 128, 1, 1);    // kh^T (MN-major) x V (MN-major)
@@ -146,10 +147,11 @@ k_gla_fwd_tc(const __grid_constant__ CUtensorMap gm_q, const __grid_constant__ C
                 if (n > 0) wait(ATAKEN, (n - 1) & 1);                // A_{n-1} has been read out of tensor memory
                 if (failed) return;
                 tc_fence_after();
+                if (leader)
 #pragma unroll
                 for (int kk = 0; kk < 8; ++kk)
                     tc_mma_bf16(tmem + COL_A, (desc_kmajor(sQ) + kstep_kmajor(kk, HALF_BF16)), (desc_kmajor(sK) + kstep_kmajor(kk, HALF_BF16)), ID_A, kk > 0);
-                tc_commit(bar(BAR_A));
+                if (leader) tc_commit(bar(BAR_A));
             };
             issue_a(0);
             for (int n = 0; n < NT && !failed; ++n) {
@@ -163,26 +165,29 @@ k_gla_fwd_tc(const __grid_constant__ CUtensorMap gm_q, const __grid_constant__ C
                 if (failed) break;
                 tc_fence_after();
                 // the recurrence: S += kh^T V and O = qh S_n; their commit releases the rescale
+                if (leader)
 #pragma unroll
                 for (int kk = 0; kk < 4; ++kk)
                     tc_mma_bf16(tmem + COL_S, (desc_mnmajor(sK, HALF_BF16) + kstep_mnmajor(kk)), (desc_mnmajor(sV, HALF_BF16) + kstep_mnmajor(kk)), ID_Z, 1);
+                if (leader)
 #pragma unroll
                 for (int kk = 0; kk < 8; ++kk)
                     tc_mma_bf16(tO, (desc_kmajor(sQ) + kstep_kmajor(kk, HALF_BF16)), (desc_mnmajor(base + OFF_S, STATE_HALF) + kstep_mnmajor(kk)), ID_O, kk > 0);
-                tc_commit(bar(BAR_Z));
-                tc_commit(bar(QKFREE + n % 3));        // (same event, own barrier: the TMA lane may look at it much later)
+                if (leader) tc_commit(bar(BAR_Z));
+                if (leader) tc_commit(bar(QKFREE + n % 3));        // (same event, own barrier: the TMA lane may look at it much later)
                 // beside the rescale: A of the next chunk, then A V of this one
                 if (n + 1 < NT) issue_a(n + 1);
                 wait(AREADY, par);                     // masked A_n is in shared memory
                 if (failed) break;
                 tc_fence_after();
+                if (leader)
 #pragma unroll
                 for (int kk = 0; kk < 4; ++kk)         // O += A V
                     tc_mma_bf16(tO, (desc_kmajor(base + OFF_A) + kstep_kmajor(kk, 0)), (desc_mnmajor(sV, HALF_BF16) + kstep_mnmajor(kk)), ID_O, 1);
-                tc_commit(bar(BAR_O + (n & 1)));
+                if (leader) tc_commit(bar(BAR_O + (n & 1)));
             }
             // let the tensor core finish before TMEM goes away (after an abort some of its work may still be queued)
-            tc_commit(bar(DRAIN));
+            if (leader) tc_commit(bar(DRAIN));
             mbar_wait_bounded(bar(DRAIN), 0, nullptr, 20000000ull);
         }
     } else if (warp == W_TMA) {

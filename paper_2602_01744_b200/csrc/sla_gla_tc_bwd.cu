@@ -141,8 +141,9 @@ k_gla_states_tc(const __grid_constant__ CUtensorMap gm_k, const __grid_constant_
     uint8_t *img0 = p.simg + slot * STATE_BF16;                       // (image mode: one segment, NT = p.NT)
 
     if (warp == 8) {
-        // ---------------- MMA issue (one lane) ----------------
-        if (lane == 0) {
+        // ---------------- MMA issue (the warp walks the loop together, one lane issues) ----------------
+        {
+            const bool leader = elect_lane();
             constexpr uint32_t ID_Z = idesc_bf16(128, 128, 1, 1);    // kh^T (MN-major) x V (MN-major)
             for (int n = 0; n < NT; ++n) {
                 const uint32_t sK = base + OFF_K + (n % 3) * TILE_BF16, sV = base + OFF_V + (n & 1) * TILE_BF16;
@@ -152,14 +153,15 @@ k_gla_states_tc(const __grid_constant__ CUtensorMap gm_k, const __grid_constant_
                 if (failed) break;
                 tc_fence_after();
                 const uint64_t dK = desc_mnmajor(sK, HALF_BF16), dV = desc_mnmajor(sV, HALF_BF16);
+                if (leader)
 #pragma unroll
                 for (int kk = 0; kk < 4; ++kk)         // S += kh^T V
                     tc_mma_bf16(tmem, dK + kstep_mnmajor(kk), dV + kstep_mnmajor(kk), ID_Z, 1);
-                tc_commit(bar(BAR_Z));
-                tc_commit(bar(KFREE + n % 3));         // (same event on per-buffer barriers for the TMA lane)
-                tc_commit(bar(VFREE + (n & 1)));
+                if (leader) tc_commit(bar(BAR_Z));
+                if (leader) tc_commit(bar(KFREE + n % 3));         // (same event on per-buffer barriers for the TMA lane)
+                if (leader) tc_commit(bar(VFREE + (n & 1)));
             }
-            tc_commit(bar(DRAIN));
+            if (leader) tc_commit(bar(DRAIN));
             mbar_wait_bounded(bar(DRAIN), 0, nullptr, 20000000ull);
         }
     } else if (warp == 11) {
@@ -437,8 +439,13 @@ k_gla_bwd_tc(const __grid_constant__ CUtensorMap gm_q, const __grid_constant__ C
     // chunks are visited in the order n = NT-1 ... 0; k = NT-1-n is the visit number that drives every barrier parity
 
     if (warp == 8) {
-        // ---------------- MMA issue (one lane) ----------------
-        if (lane == 0) {
+        // ---------------- MMA issue (the warp walks the loop together, one lane issues) ----------------
+        {
+            const bool leader = elect_lane();
+            // (the whole warp gives up together: it votes below)
+            auto wait = [&](int i, uint32_t parity) {
+                if (!failed && !__all_sync(0xffffffffu, mbar_wait_bounded(bar(i), parity, abort_flag))) { failed = true; *abort_flag = 1; }
+            };
             constexpr uint32_t ID_A = idesc_bf16(64, 64, 0, 0);
             constexpr uint32_t ID_KK = idesc_bf16(128, 64, 0, 0), ID_MK = idesc_bf16(128, 64, 1, 0),
                                ID_MM = idesc_bf16(128, 64, 1, 1), ID_S = idesc_bf16(128, 128, 1, 1);
@@ -457,6 +464,7 @@ k_gla_bwd_tc(const __grid_constant__ CUtensorMap gm_q, const __grid_constant__ C
                 wait(FULL_DO, par);
                 if (failed) break;
                 tc_fence_after();
+                if (leader)
 #pragma unroll
                 for (int kk = 0; kk < 8; ++kk)         // dA = dO V^T
                     tc_mma_bf16(tmem + COL_DA, kDO + kstep_kmajor(kk, HALF_BF16), kV + kstep_kmajor(kk, HALF_BF16), ID_A, kk > 0);
@@ -464,6 +472,7 @@ k_gla_bwd_tc(const __grid_constant__ CUtensorMap gm_q, const __grid_constant__ C
                 auto issue_sdo = [&]() {               // dqh^T = S_n dO^T ...
                     if (k > 0) wait(OUT1, (k - 1) & 1);    // dqh^T, dkh^T of the previous chunk have been read out (long ago)
                     tc_fence_after();
+                    if (leader)
 #pragma unroll
                     for (int kk = 0; kk < 8; ++kk)
                         tc_mma_bf16(tmem + COL_DQ, kS + kstep_kmajor(kk, STATE_HALF), kDO + kstep_kmajor(kk, HALF_BF16), ID_KK, kk > 0);
@@ -471,17 +480,19 @@ k_gla_bwd_tc(const __grid_constant__ CUtensorMap gm_q, const __grid_constant__ C
                 };
                 {   // whichever comes first: S_n landed, or the prologue done
                     const uint64_t t0 = globaltimer_ns();
-                    for (uint32_t it = 0; !failed && !mbar_test_wait(bar(OPR), par); ++it) {
-                        if (!sdo_done && mbar_test_wait(bar(FULL_S), par)) issue_sdo();
-                        if ((it & 63u) == 63u && (*abort_flag || globaltimer_ns() - t0 > 2000000000ull)) { failed = true; *abort_flag = 1; }
+                    for (uint32_t it = 0; !failed && !__all_sync(0xffffffffu, mbar_test_wait(bar(OPR), par)); ++it) {
+                        if (!sdo_done && __all_sync(0xffffffffu, mbar_test_wait(bar(FULL_S), par))) issue_sdo();
+                        const bool late = (it & 63u) == 63u && (*abort_flag || globaltimer_ns() - t0 > 2000000000ull);
+                        if (__any_sync(0xffffffffu, late)) { failed = true; *abort_flag = 1; }
                     }
                 }
                 if (failed) break;
                 tc_fence_after();
+                if (leader)
 #pragma unroll
                 for (int kk = 0; kk < 8; ++kk)         // A = qh kh^T
                     tc_mma_bf16(tmem + COL_A, kQ + kstep_kmajor(kk, HALF_BF16), kK + kstep_kmajor(kk, HALF_BF16), ID_A, kk > 0);
-                tc_commit(bar(BAR_A));
+                if (leader) tc_commit(bar(BAR_A));
                 if (!sdo_done) {
                     wait(FULL_S, par);
                     if (failed) break;
@@ -491,29 +502,32 @@ k_gla_bwd_tc(const __grid_constant__ CUtensorMap gm_q, const __grid_constant__ C
                 wait(ZREADY, par);                     // dZ: fp32 in TMEM, bf16 in shared memory
                 if (failed) break;
                 tc_fence_after();
+                if (leader)
 #pragma unroll
                 for (int kk = 0; kk < 8; ++kk) {       // three independent accumulation chains, interleaved
                     tc_mma_bf16(tmem + COL_DK, kDZ + kstep_kmajor(kk, STATE_HALF), kV + kstep_kmajor(kk, HALF_BF16), ID_KK, kk > 0);   // dkh^T = dZ V^T ...
                     tc_mma_bf16(tmem + COL_DV, mDZ + kstep_mnmajor(kk), kK + kstep_kmajor(kk, HALF_BF16), ID_MK, kk > 0);            // dV^T = dZ^T kh^T ...
                     if (kk < 4) tc_mma_bf16(tmem + COL_DS, mQ + kstep_mnmajor(kk), mDO + kstep_mnmajor(kk), ID_S, 1);                // dS_n = dZ + qh^T dO
                 }
-                tc_commit(bar(BAR_DS));                // dS_n is complete (and S_n dO^T has read S_n)
+                if (leader) tc_commit(bar(BAR_DS));                // dS_n is complete (and S_n dO^T has read S_n)
                 wait(AREADY, par);                     // masked A, dA in shared memory
                 if (failed) break;
                 tc_fence_after();
+                if (leader)
 #pragma unroll
                 for (int kk = 0; kk < 4; ++kk) {       // ... + kh^T dA^T  and  ... + qh^T dA, interleaved
                     tc_mma_bf16(tmem + COL_DQ, mK + kstep_mnmajor(kk), kDA + kstep_kmajor(kk, 0), ID_MK, 1);
                     tc_mma_bf16(tmem + COL_DK, mQ + kstep_mnmajor(kk), mDA + kstep_mnmajor(kk), ID_MM, 1);
                 }
-                tc_commit(bar(BAR_M1));
+                if (leader) tc_commit(bar(BAR_M1));
+                if (leader)
 #pragma unroll
                 for (int kk = 0; kk < 4; ++kk)         // ... + dO^T A
                     tc_mma_bf16(tmem + COL_DV, mDO + kstep_mnmajor(kk), mA + kstep_mnmajor(kk), ID_MM, 1);
-                tc_commit(bar(BAR_M2));
-                tc_commit(bar(DOFREE));                // (same event, for the TMA lane)
+                if (leader) tc_commit(bar(BAR_M2));
+                if (leader) tc_commit(bar(DOFREE));                // (same event, for the TMA lane)
             }
-            tc_commit(bar(DRAIN));
+            if (leader) tc_commit(bar(DRAIN));
             mbar_wait_bounded(bar(DRAIN), 0, nullptr, 20000000ull);
         }
     } else if (warp == 13) {
