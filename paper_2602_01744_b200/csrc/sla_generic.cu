@@ -108,24 +108,30 @@ k_gdn_prepare(Dims d, const TIO *__restrict__ k, const TIO *__restrict__ v,
         bs[i] = ok ? bcum[row] : 0.f;
         bt[i] = ok ? beta[row] : 0.f;
     }
-    for (int idx = threadIdx.x; idx < CMAX * d.dk; idx += blockDim.x) {
-        int i = idx / d.dk, dd = idx % d.dk;
-        Ks[i * ldk + dd] = i < cn ? ldf(k, tok_row(d, b, t0 + i, h) * d.dk + dd) : 0.f;
-    }
+    fill_rows(Ks, ldk, k, CMAX, cn, d.dk, [&](int i) { return tok_row(d, b, t0 + i, h) * d.dk; });
     __syncthreads();
     for (int idx = threadIdx.x; idx < CMAX * d.dk; idx += blockDim.x) {
         int i = idx / d.dk, dd = idx % d.dk;
         Xs[i * ldx + dd] = bt[i] * expf(bs[i]) * Ks[i * ldk + dd];
     }
-    for (int idx = threadIdx.x; idx < CMAX * d.dv; idx += blockDim.x) {
-        int i = idx / d.dv, j = idx % d.dv;
-        float val = 0.f;
-        if (i < cn) {
-            size_t row = tok_row(d, b, t0 + i, h);
-            val = bt[i] * Gk[row] * ldf(v, row * d.dv + j);
-        }
-        Xs[i * ldx + d.dk + j] = val;
-    }
+    const int v4 = d.dv >> 2;
+    struct In { float4 v; float g; };
+    fill(CMAX * v4,
+        [&](int idx) {
+            const int i = idx / v4;
+            In x{make_float4(0.f, 0.f, 0.f, 0.f), 0.f};
+            if (i < cn) {
+                const size_t row = tok_row(d, b, t0 + i, h);
+                x.v = ldf4(v, row * d.dv + 4 * (idx - i * v4));
+                x.g = Gk[row];
+            }
+            return x;
+        },
+        [&](int idx, const In &x) {
+            const int i = idx / v4;
+            const float f = bt[i] * x.g;
+            put4(Xs + i * ldx + d.dk + 4 * (idx - i * v4), make_float4(f * x.v.x, f * x.v.y, f * x.v.z, f * x.v.w));
+        });
     for (int idx = threadIdx.x; idx < CMAX * CMAX; idx += blockDim.x) {
         int i = idx % CMAX, j = idx / CMAX;
         float acc = 0.f;
@@ -155,87 +161,189 @@ k_gdn_prepare(Dims d, const TIO *__restrict__ k, const TIO *__restrict__ v,
 }
 
 // ------------------------------------------------------------------------------------------
-// a4: inter-chunk state pass.  grid (dv/VS, B*H); thread dd owns row dd of a [dk x VS] slice of S.
-// Stores the state before every chunk (slot n) and the final state (slot NT, and ht).
-// GDN: also turns U0 into U = U0 - W S in place.
+// a4 for GDN: inter-chunk state pass, chunk after chunk.  grid (dv/VS, B*H), 256 threads on a [dk x VS] slice of S.  Stores
+// the state before every chunk (slot n) and the final state (slot NT, and ht), and U = U0 - W S.
+// Serial over the chunks, so what counts is the time of one: four neighbouring columns a thread (float4 reads of the
+// shared operand) and the next chunk's tiles in flight in registers while this one computes (28 -> 4.4 us a chunk at d = 64).
 template <typename TIO>
-__global__ void __launch_bounds__(128)
-k_state_scan(Dims d, const TIO *__restrict__ k, const TIO *__restrict__ v,
-             const float *__restrict__ Gk, const float *__restrict__ bcum,
+__global__ void __launch_bounds__(256)
+k_state_scan(Dims d, const TIO *__restrict__ k, const float *__restrict__ bcum,
              const float *__restrict__ h0, float *__restrict__ states, float *__restrict__ ht,
              const float *__restrict__ Wws, const float *__restrict__ U0ws, float *__restrict__ Uws) {
     extern __shared__ float sm[];
-    int vs0 = blockIdx.x * VS, bh = blockIdx.y, b = bh / d.H, h = bh % d.H;
-    int ldk = d.dk + 1, lds = VS + 1;
-    float *Kb = sm;                         // [CMAX][ldk]  k~ * exp(b_last - b)
-    float *Vs = Kb + CMAX * ldk;            // [CMAX][VS]   V (or U) slice
-    float *Ws = Vs + CMAX * VS;             // [CMAX][ldk]  GDN only
-    float *Ss = Ws + CMAX * ldk;            // [dk][lds]    GDN only
-    const int dd = threadIdx.x;
-    const bool own = dd < d.dk;
-    const bool gdn = d.variant == SLA_GDN;
-    float S[VS];
+    const int vs0 = blockIdx.x * VS, bh = blockIdx.y, b = bh / d.H, h = bh % d.H, ldk = d.dk + 1, tid = threadIdx.x;
+    float *Ss = sm;                         // [dk][VS]
+    float *Vs = Ss + d.dk * VS;             // [CMAX][VS]   U0, then U
+    float *es = Vs + CMAX * VS;             // [CMAX]       e^{b_last - b}
+    float *Ks = es + CMAX;                  // [CMAX][ldk]
+    float *Ws = Ks + CMAX * ldk;            // [CMAX][ldk]
+    const int i0 = tid >> 2, jq = 4 * (tid & 3), w4 = d.dk >> 2;   // this thread's token and state rows (i0, i0 + 64), its columns
+    float4 S[2];
 #pragma unroll
-    for (int j = 0; j < VS; ++j)
-        S[j] = (own && h0) ? h0[((size_t)bh * d.dk + dd) * d.dv + vs0 + j] : 0.f;
-
+    for (int x = 0; x < 2; ++x) {
+        const int dd = i0 + 64 * x;
+        S[x] = (dd < d.dk && h0) ? ldf4(h0, ((size_t)bh * d.dk + dd) * d.dv + vs0 + jq) : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+    float4 kr[8], wr[8], ur;
+    float br = 0.f, bl = 0.f;
+    auto fetch = [&](int n) {
+        const int t0 = n * d.C, cn = min(d.C, d.T - t0);
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            const int idx = tid + 256 * u, i = idx / w4;
+            if (i >= cn) continue;
+            const size_t o = tok_row(d, b, t0 + i, h) * d.dk + 4 * (idx - i * w4);
+            kr[u] = ldf4(k, o);
+            wr[u] = ldf4(Wws, o);
+        }
+        if (i0 < cn) ur = ldf4(U0ws, tok_row(d, b, t0 + i0, h) * d.dv + vs0 + jq);
+        if (tid < cn) br = bcum[tok_row(d, b, t0 + tid, h)];
+        bl = bcum[tok_row(d, b, t0 + cn - 1, h)];
+    };
+    fetch(0);
     for (int n = 0; n < d.NT; ++n) {
-        int t0 = n * d.C, cn = min(d.C, d.T - t0);
-        if (own) {
-            float *dst = states + state_off(d, bh, n, d.NT + 1) + (size_t)dd * d.dv + vs0;
+        const int t0 = n * d.C, cn = min(d.C, d.T - t0);
+        const float dec = expf(bl);
 #pragma unroll
-            for (int j = 0; j < VS; ++j) dst[j] = S[j];
-            if (gdn)
+        for (int x = 0; x < 2; ++x) {
+            const int dd = i0 + 64 * x;
+            if (dd >= d.dk) continue;
+            *reinterpret_cast<float4 *>(states + state_off(d, bh, n, d.NT + 1) + (size_t)dd * d.dv + vs0 + jq) = S[x];
+            *reinterpret_cast<float4 *>(Ss + dd * VS + jq) = S[x];
+        }
 #pragma unroll
-                for (int j = 0; j < VS; ++j) Ss[dd * lds + j] = S[j];
+        for (int u = 0; u < 8; ++u) {
+            const int idx = tid + 256 * u, i = idx / w4, o = i * ldk + 4 * (idx - i * w4);
+            if (i >= cn) continue;
+            put4(Ks + o, kr[u]);
+            put4(Ws + o, wr[u]);
         }
-        size_t row_last = tok_row(d, b, t0 + cn - 1, h);
-        for (int idx = threadIdx.x; idx < cn * d.dk; idx += blockDim.x) {
-            int i = idx / d.dk, c = idx % d.dk;
-            size_t row = tok_row(d, b, t0 + i, h);
-            float e = expf(bcum_at(d, bcum, row_last, c) - bcum_at(d, bcum, row, c));
-            float gk = gdn ? 1.f : Gk[row];
-            Kb[i * ldk + c] = gk * ldf(k, row * d.dk + c) * e;
-            if (gdn) Ws[i * ldk + c] = Wws[row * d.dk + c];
-        }
-        for (int idx = threadIdx.x; idx < cn * VS; idx += blockDim.x) {
-            int i = idx / VS, j = idx % VS;
-            size_t row = tok_row(d, b, t0 + i, h);
-            Vs[idx] = gdn ? U0ws[row * d.dv + vs0 + j] : ldf(v, row * d.dv + vs0 + j);
+        if (tid < cn) es[tid] = expf(bl - br);
+        float4 acc = ur;
+        __syncthreads();
+        if (n + 1 < d.NT) fetch(n + 1);
+        if (i0 < cn) {
+#pragma unroll 4
+            for (int c = 0; c < d.dk; ++c) {
+                const float w = -Ws[i0 * ldk + c];
+                const float4 sv = *reinterpret_cast<const float4 *>(Ss + c * VS + jq);
+                acc.x = fmaf(w, sv.x, acc.x); acc.y = fmaf(w, sv.y, acc.y); acc.z = fmaf(w, sv.z, acc.z); acc.w = fmaf(w, sv.w, acc.w);
+            }
+            *reinterpret_cast<float4 *>(Vs + i0 * VS + jq) = acc;
+            *reinterpret_cast<float4 *>(Uws + tok_row(d, b, t0 + i0, h) * d.dv + vs0 + jq) = acc;
         }
         __syncthreads();
-        if (gdn) {
-            for (int idx = threadIdx.x; idx < cn * VS; idx += blockDim.x) {
-                int i = idx % cn, j = idx / cn;
-                float acc = Vs[i * VS + j];
-                for (int c = 0; c < d.dk; ++c) acc = fmaf(-Ws[i * ldk + c], Ss[c * lds + j], acc);
-                Vs[i * VS + j] = acc;
-                Uws[tok_row(d, b, t0 + i, h) * d.dv + vs0 + j] = acc;
-            }
-            __syncthreads();
-        }
-        if (own) {
-            float dec = expf(bcum_at(d, bcum, row_last, dd));
 #pragma unroll
-            for (int j = 0; j < VS; ++j) S[j] *= dec;
+        for (int x = 0; x < 2; ++x) {
+            const int dd = i0 + 64 * x;
+            if (dd >= d.dk) continue;
+            S[x].x *= dec; S[x].y *= dec; S[x].z *= dec; S[x].w *= dec;
+#pragma unroll 4
             for (int i = 0; i < cn; ++i) {
-                float kb = Kb[i * ldk + dd];
-#pragma unroll
-                for (int j = 0; j < VS; ++j) S[j] = fmaf(kb, Vs[i * VS + j], S[j]);
+                const float kb = Ks[i * ldk + dd] * es[i];
+                const float4 u = *reinterpret_cast<const float4 *>(Vs + i * VS + jq);
+                S[x].x = fmaf(kb, u.x, S[x].x); S[x].y = fmaf(kb, u.y, S[x].y); S[x].z = fmaf(kb, u.z, S[x].z); S[x].w = fmaf(kb, u.w, S[x].w);
             }
         }
         __syncthreads();
     }
-    if (own) {
-        float *dst = states + state_off(d, bh, d.NT, d.NT + 1) + (size_t)dd * d.dv + vs0;
 #pragma unroll
-        for (int j = 0; j < VS; ++j) dst[j] = S[j];
-        if (ht) {
-            float *hdst = ht + ((size_t)bh * d.dk + dd) * d.dv + vs0;
+    for (int x = 0; x < 2; ++x) {
+        const int dd = i0 + 64 * x;
+        if (dd >= d.dk) continue;
+        *reinterpret_cast<float4 *>(states + state_off(d, bh, d.NT, d.NT + 1) + (size_t)dd * d.dv + vs0 + jq) = S[x];
+        if (ht) *reinterpret_cast<float4 *>(ht + ((size_t)bh * d.dk + dd) * d.dv + vs0 + jq) = S[x];
+    }
+}
+
+// ------------------------------------------------------------------------------------------
+// a4 for RETNET / GLA, whose state transition is a diagonal: what a chunk adds to the state, and to the state gradient,
+// does not depend on the state, so those products run in parallel over the chunks and only an elementwise recurrence
+// is left for the walk along the sequence (k_state_fold).  One CTA per sequence walking the chunks through shared memory
+// took 19 us a chunk; at 2 x 1000 x 4 heads of 64 both kernels together take 20 us where the scan took 300 (reverse: 250).
+// GRAD = false: KV_n = (Gk k e^{b_last - b})^T V into state slot n + 1;  GRAD = true: qh^T dO into slot n - 1 of the state
+// gradients (n = 0: into dh0, if wanted).  grid (NT, B*H, ceil(dk / 64)).
+template <typename TIO, bool GRAD>
+__global__ void __launch_bounds__(256)
+k_chunk_outer(Dims d, const TIO *__restrict__ x, const TIO *__restrict__ y, const float *__restrict__ gate, const float *__restrict__ bcum,
+              float *__restrict__ out, float *__restrict__ dh0) {
+    extern __shared__ float sm[];
+    const int n = blockIdx.x, bh = blockIdx.y, b = bh / d.H, h = bh % d.H, r0 = 64 * blockIdx.z, nr = min(64, d.dk - r0);
+    float *dst = !GRAD ? out + state_off(d, bh, n + 1, d.NT + 1) : n > 0 ? out + state_off(d, bh, n - 1, d.NT) : dh0 ? dh0 + state_off(d, bh, 0, 1) : nullptr;
+    if (!dst) return;
+    const int t0 = n * d.C, cn = min(d.C, d.T - t0), ldv = d.dv + 1;
+    float *Xs = sm;                          // [CMAX][65]
+    float *Ys = Xs + CMAX * 65;              // [CMAX][ldv]
+    const size_t row_last = tok_row(d, b, t0 + cn - 1, h);
+    struct In { float4 x, b, bl; float g; };
+    const int w4 = nr >> 2;
+    fill<2>(cn * w4,
+        [&](int idx) {
+            const int i = idx / w4, c = r0 + 4 * (idx - i * w4);
+            const size_t row = tok_row(d, b, t0 + i, h);
+            In v;
+            v.x = ldf4(x, row * d.dk + c);
+            v.b = bcum_at4(d, bcum, row, c);
+            v.g = GRAD ? d.scale * gate[row] : gate[row];
+            v.bl = GRAD ? v.b : bcum_at4(d, bcum, row_last, c);
+            return v;
+        },
+        [&](int idx, const In &v) {
+            const int i = idx / w4;
+            const float4 e = GRAD ? v.b : make_float4(v.bl.x - v.b.x, v.bl.y - v.b.y, v.bl.z - v.b.z, v.bl.w - v.b.w);
+            put4(Xs + i * 65 + 4 * (idx - i * w4), make_float4(v.g * v.x.x * expf(e.x), v.g * v.x.y * expf(e.y), v.g * v.x.z * expf(e.z), v.g * v.x.w * expf(e.w)));
+        });
+    fill_rows(Ys, ldv, y, cn, cn, d.dv, [&](int i) { return tok_row(d, b, t0 + i, h) * d.dv; });
+    __syncthreads();
+    const int ty = threadIdx.x >> 5, tx = threadIdx.x & 31;
+    float acc[8][4];
+    zero_acc(acc);
+    tile_gemm<4>(acc, Xs, 1, 65, Ys, ldv, 1, cn, d.dv, ty, tx);
 #pragma unroll
-            for (int j = 0; j < VS; ++j) hdst[j] = S[j];
+    for (int r = 0; r < 8; ++r) {
+        const int i = ty + 8 * r;
+        if (i >= nr) continue;
+#pragma unroll
+        for (int cb = 0; cb < 4; ++cb) {
+            const int j = tx + 32 * cb;
+            if (j < d.dv) dst[(size_t)(r0 + i) * d.dv + j] = acc[r][cb];
         }
     }
+}
+
+// The walk along the sequence, one thread per state element, in place over what k_chunk_outer left:
+// GRAD = false: S_0 = h0, S_{n+1} = e^{b_last} S_n + KV_n (slot n: the state before chunk n; the last also to ht);
+// GRAD = true, in reverse: slot NT-1 = dht, slot n-1 = e^{b_last,n} slot n + (qh^T dO)_n (n = 0: dh0).
+template <bool GRAD>
+__global__ void __launch_bounds__(256)
+k_state_fold(Dims d, const float *__restrict__ bcum, const float *__restrict__ first, float *__restrict__ st, float *__restrict__ last) {
+    const int sz = d.dk * d.dv, e = blockIdx.x * blockDim.x + threadIdx.x, bh = blockIdx.y, b = bh / d.H, h = bh % d.H;
+    if (e >= sz) return;
+    const int c = e / d.dv, NT = d.NT, slots = GRAD ? NT : NT + 1;
+    float *p = st + (size_t)bh * slots * sz + e;
+    auto dec = [&](int n) { return bcum_at(d, bcum, tok_row(d, b, min((n + 1) * d.C, d.T) - 1, h), c); };
+    float S = first ? first[(size_t)bh * sz + e] : 0.f;
+    constexpr int U = 8;                     // chunks whose reads are in flight together
+    for (int m0 = 0; m0 < NT; m0 += U) {
+        float add[U], dc[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int m = m0 + u, n = GRAD ? NT - 1 - m : m;
+            add[u] = dc[u] = 0.f;
+            if (m >= NT) continue;
+            dc[u] = dec(n);
+            add[u] = !GRAD ? p[(size_t)(n + 1) * sz] : n > 0 ? p[(size_t)(n - 1) * sz] : last ? last[(size_t)bh * sz + e] : 0.f;
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int m = m0 + u, n = GRAD ? NT - 1 - m : m;
+            if (m >= NT) continue;
+            p[(size_t)n * sz] = S;
+            S = fmaf(expf(dc[u]), S, add[u]);
+        }
+    }
+    if (!GRAD) p[(size_t)NT * sz] = S;
+    if (last) last[(size_t)bh * sz + e] = S;
 }
 
 // ------------------------------------------------------------------------------------------
@@ -258,18 +366,11 @@ k_output(Dims d, const TIO *__restrict__ q, const TIO *__restrict__ k, const TIO
     const bool gdn = d.variant == SLA_GDN;
 
     load_qk_hat(d, q, k, Gq, Gk, bcum, b, h, t0, cn, Qs, Ks, ldk);
-    for (int idx = threadIdx.x; idx < CMAX * d.dv; idx += blockDim.x) {
-        int i = idx / d.dv, j = idx % d.dv;
-        float val = 0.f;
-        if (i < cn) {
-            size_t row = tok_row(d, b, t0 + i, h);
-            val = gdn ? Uws[row * d.dv + j] : ldf(v, row * d.dv + j);
-        }
-        Vs[i * ldv + j] = val;
-    }
+    auto vrow = [&](int i) { return tok_row(d, b, t0 + i, h) * d.dv; };
+    if (gdn) fill_rows(Vs, ldv, Uws, CMAX, cn, d.dv, vrow);
+    else fill_rows(Vs, ldv, v, CMAX, cn, d.dv, vrow);
     const float *Sg = states + state_off(d, bh, n, d.NT + 1);
-    for (int idx = threadIdx.x; idx < d.dk * d.dv; idx += blockDim.x)
-        Ss[(idx / d.dv) * ldv + idx % d.dv] = Sg[idx];
+    fill_rows(Ss, ldv, Sg, d.dk, d.dk, d.dv, [&](int i) { return (size_t)i * d.dv; });
     __syncthreads();
 
     {
@@ -303,109 +404,127 @@ k_output(Dims d, const TIO *__restrict__ q, const TIO *__restrict__ k, const TIO
 }
 
 // ------------------------------------------------------------------------------------------
-// backward, state-gradient pass (reverse chunk order).  grid (dv/VS, B*H); thread dd owns row dd of
-// a [dk x VS] slice of dS.  Stores dS entering each chunk from the right (slot n = gradient w.r.t.
-// the state after chunk n).  RETNET/GLA: dS' = diag(exp(b_last)) dS + qh^T dO.
-// GDN: dU = Pq^T dO + diag(E) K dS ;  dS' = exp(b_last) dS + qh^T dO - W^T dU   (dU stored).
+// backward for GDN, state-gradient pass (reverse chunk order).  grid (dv/VS, B*H), 256 threads on a [dk x VS] slice of dS.
+// Stores dS entering each chunk from the right (slot n = gradient w.r.t. the state after chunk n) and
+//   dU = Pq^T dO + diag(E) K dS ;  dS' = exp(b_last) dS + qh^T dO - W^T dU.
+// Thread layout and reason as in k_state_scan (52 -> 11 us a chunk at d = 64).
 template <typename TIO>
-__global__ void __launch_bounds__(128)
+__global__ void __launch_bounds__(256)
 k_dstate_scan(Dims d, const TIO *__restrict__ q, const TIO *__restrict__ k, const TIO *__restrict__ dO,
               const float *__restrict__ Gq, const float *__restrict__ bcum,
               const float *__restrict__ dht, float *__restrict__ dstates, float *__restrict__ dh0,
               const float *__restrict__ Wws, float *__restrict__ dUws) {
     extern __shared__ float sm[];
-    int vs0 = blockIdx.x * VS, bh = blockIdx.y, b = bh / d.H, h = bh % d.H;
-    int ldk = d.dk + 1, lds = VS + 1, lda = CMAX + 1;
-    float *Qs = sm;                          // [CMAX][ldk]  qh
-    float *dOs = Qs + CMAX * ldk;            // [CMAX][VS]
-    float *Ks = dOs + CMAX * VS;             // GDN: [CMAX][ldk]  k*exp(-b)
-    float *Ws = Ks + CMAX * ldk;             // GDN: [CMAX][ldk]
-    float *Ps = Ws + CMAX * ldk;             // GDN: [CMAX][lda]  Pq
-    float *dSs = Ps + CMAX * lda;            // GDN: [dk][lds]
-    float *dUs = dSs + d.dk * lds;           // GDN: [CMAX][VS]
-    const int dd = threadIdx.x;
-    const bool own = dd < d.dk;
-    const bool gdn = d.variant == SLA_GDN;
-    float dS[VS];
+    const int vs0 = blockIdx.x * VS, bh = blockIdx.y, b = bh / d.H, h = bh % d.H, ldk = d.dk + 1, lda = CMAX + 1, tid = threadIdx.x;
+    float *dSs = sm;                         // [dk][VS]
+    float *dOs = dSs + d.dk * VS;            // [CMAX][VS]
+    float *dUs = dOs + CMAX * VS;            // [CMAX][VS]
+    float *Qs = dUs + CMAX * VS;             // [CMAX][ldk]  qh
+    float *Ks = Qs + CMAX * ldk;             // [CMAX][ldk]  k*exp(-b)
+    float *Ws = Ks + CMAX * ldk;             // [CMAX][ldk]
+    float *Ps = Ws + CMAX * ldk;             // [CMAX][lda]  Pq
+    const int i0 = tid >> 2, jq = 4 * (tid & 3), w4 = d.dk >> 2, ty = tid >> 5, tx = tid & 31;
+    float4 dS[2];
 #pragma unroll
-    for (int j = 0; j < VS; ++j)
-        dS[j] = (own && dht) ? dht[((size_t)bh * d.dk + dd) * d.dv + vs0 + j] : 0.f;
-
+    for (int x = 0; x < 2; ++x) {
+        const int dd = i0 + 64 * x;
+        dS[x] = (dd < d.dk && dht) ? ldf4(dht, ((size_t)bh * d.dk + dd) * d.dv + vs0 + jq) : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+    struct In { float4 q, k, w; float b, g; };
     for (int n = d.NT - 1; n >= 0; --n) {
-        int t0 = n * d.C, cn = min(d.C, d.T - t0);
-        if (own) {
-            float *dst = dstates + state_off(d, bh, n, d.NT) + (size_t)dd * d.dv + vs0;
+        const int t0 = n * d.C, cn = min(d.C, d.T - t0);
 #pragma unroll
-            for (int j = 0; j < VS; ++j) dst[j] = dS[j];
-            if (gdn)
-#pragma unroll
-                for (int j = 0; j < VS; ++j) dSs[dd * lds + j] = dS[j];
+        for (int x = 0; x < 2; ++x) {
+            const int dd = i0 + 64 * x;
+            if (dd >= d.dk) continue;
+            *reinterpret_cast<float4 *>(dstates + state_off(d, bh, n, d.NT) + (size_t)dd * d.dv + vs0 + jq) = dS[x];
+            *reinterpret_cast<float4 *>(dSs + dd * VS + jq) = dS[x];
         }
-        size_t row_last = tok_row(d, b, t0 + cn - 1, h);
-        for (int idx = threadIdx.x; idx < CMAX * d.dk; idx += blockDim.x) {
-            int i = idx / d.dk, c = idx % d.dk;
-            float qv = 0.f, kv = 0.f, wv = 0.f;
-            if (i < cn) {
-                size_t row = tok_row(d, b, t0 + i, h);
-                float bb = bcum_at(d, bcum, row, c);
-                qv = d.scale * Gq[row] * ldf(q, row * d.dk + c) * expf(bb);
-                if (gdn) {
-                    kv = ldf(k, row * d.dk + c) * expf(-bb);
-                    wv = Wws[row * d.dk + c];
+        const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+        fill<4>(CMAX * w4,
+            [&](int idx) {
+                const int i = idx / w4;
+                In x{zero, zero, zero, 0.f, 0.f};
+                if (i < cn) {
+                    const size_t row = tok_row(d, b, t0 + i, h), o = row * d.dk + 4 * (idx - i * w4);
+                    x.q = ldf4(q, o);
+                    x.k = ldf4(k, o);
+                    x.w = ldf4(Wws, o);
+                    x.b = bcum[row];
+                    x.g = Gq[row];
                 }
-            }
-            Qs[i * ldk + c] = qv;
-            if (gdn) { Ks[i * ldk + c] = kv; Ws[i * ldk + c] = wv; }
-        }
-        for (int idx = threadIdx.x; idx < CMAX * VS; idx += blockDim.x) {
-            int i = idx / VS, j = idx % VS;
-            dOs[idx] = i < cn ? ldf(dO, tok_row(d, b, t0 + i, h) * d.dv + vs0 + j) : 0.f;
+                return x;
+            },
+            [&](int idx, const In &x) {
+                const int i = idx / w4, o = i * ldk + 4 * (idx - i * w4);
+                const float g = d.scale * x.g, e = expf(x.b), m = expf(-x.b);
+                put4(Qs + o, make_float4(g * x.q.x * e, g * x.q.y * e, g * x.q.z * e, g * x.q.w * e));
+                put4(Ks + o, make_float4(x.k.x * m, x.k.y * m, x.k.z * m, x.k.w * m));
+                put4(Ws + o, x.w);
+            });
+        *reinterpret_cast<float4 *>(dOs + i0 * VS + jq) = i0 < cn ? ldf4(dO, tok_row(d, b, t0 + i0, h) * d.dv + vs0 + jq) : zero;
+        const float dec = expf(bcum[tok_row(d, b, t0 + cn - 1, h)]);
+        __syncthreads();
+        {
+            float a[8][2];
+            zero_acc(a);
+            tile_gemm<2>(a, Qs, ldk, 1, Ks, 1, ldk, d.dk, CMAX, ty, tx);
+#pragma unroll
+            for (int r = 0; r < 8; ++r)
+#pragma unroll
+                for (int cb = 0; cb < 2; ++cb) {
+                    const int i = ty + 8 * r, j = tx + 32 * cb;
+                    Ps[i * lda + j] = (j <= i && i < cn) ? a[r][cb] : 0.f;
+                }
         }
         __syncthreads();
-        float dec = own ? expf(bcum_at(d, bcum, row_last, dd)) : 0.f;
-        if (gdn) {
-            float elast = expf(bcum[row_last]);
-            for (int idx = threadIdx.x; idx < CMAX * CMAX; idx += blockDim.x) {
-                int i = idx % CMAX, j = idx / CMAX;
-                float acc = 0.f;
-                if (j <= i && i < cn)
-                    for (int c = 0; c < d.dk; ++c) acc = fmaf(Qs[i * ldk + c], Ks[j * ldk + c], acc);
-                Ps[i * lda + j] = acc;
+        if (i0 < cn) {
+            float4 acc = zero, acc2 = zero;
+#pragma unroll 4
+            for (int i2 = i0; i2 < cn; ++i2) {
+                const float pv = Ps[i2 * lda + i0];
+                const float4 g = *reinterpret_cast<const float4 *>(dOs + i2 * VS + jq);
+                acc.x = fmaf(pv, g.x, acc.x); acc.y = fmaf(pv, g.y, acc.y); acc.z = fmaf(pv, g.z, acc.z); acc.w = fmaf(pv, g.w, acc.w);
             }
-            __syncthreads();
-            for (int idx = threadIdx.x; idx < cn * VS; idx += blockDim.x) {
-                int i = idx % cn, j = idx / cn;
-                float acc = 0.f;
-                for (int i2 = i; i2 < cn; ++i2) acc = fmaf(Ps[i2 * lda + i], dOs[i2 * VS + j], acc);
-                float acc2 = 0.f;
-                for (int c = 0; c < d.dk; ++c) acc2 = fmaf(Ks[i * ldk + c], dSs[c * lds + j], acc2);
-                acc = fmaf(elast, acc2, acc);
-                dUs[i * VS + j] = acc;
-                dUws[tok_row(d, b, t0 + i, h) * d.dv + vs0 + j] = acc;
+#pragma unroll 4
+            for (int c = 0; c < d.dk; ++c) {
+                const float kv = Ks[i0 * ldk + c];
+                const float4 sv = *reinterpret_cast<const float4 *>(dSs + c * VS + jq);
+                acc2.x = fmaf(kv, sv.x, acc2.x); acc2.y = fmaf(kv, sv.y, acc2.y); acc2.z = fmaf(kv, sv.z, acc2.z); acc2.w = fmaf(kv, sv.w, acc2.w);
             }
-            __syncthreads();
+            acc.x = fmaf(dec, acc2.x, acc.x); acc.y = fmaf(dec, acc2.y, acc.y); acc.z = fmaf(dec, acc2.z, acc.z); acc.w = fmaf(dec, acc2.w, acc.w);
+            *reinterpret_cast<float4 *>(dUs + i0 * VS + jq) = acc;
+            *reinterpret_cast<float4 *>(dUws + tok_row(d, b, t0 + i0, h) * d.dv + vs0 + jq) = acc;
         }
-        if (own) {
+        __syncthreads();
 #pragma unroll
-            for (int j = 0; j < VS; ++j) dS[j] *= dec;
+        for (int x = 0; x < 2; ++x) {
+            const int dd = i0 + 64 * x;
+            if (dd >= d.dk) continue;
+            float4 v = dS[x];
+            v.x *= dec; v.y *= dec; v.z *= dec; v.w *= dec;
+#pragma unroll 4
             for (int i = 0; i < cn; ++i) {
-                float qv = Qs[i * ldk + dd];
-#pragma unroll
-                for (int j = 0; j < VS; ++j) dS[j] = fmaf(qv, dOs[i * VS + j], dS[j]);
+                const float qv = Qs[i * ldk + dd];
+                const float4 g = *reinterpret_cast<const float4 *>(dOs + i * VS + jq);
+                v.x = fmaf(qv, g.x, v.x); v.y = fmaf(qv, g.y, v.y); v.z = fmaf(qv, g.z, v.z); v.w = fmaf(qv, g.w, v.w);
             }
-            if (gdn)
-                for (int i = 0; i < cn; ++i) {
-                    float wv = Ws[i * ldk + dd];
-#pragma unroll
-                    for (int j = 0; j < VS; ++j) dS[j] = fmaf(-wv, dUs[i * VS + j], dS[j]);
-                }
+#pragma unroll 4
+            for (int i = 0; i < cn; ++i) {
+                const float wv = -Ws[i * ldk + dd];
+                const float4 u = *reinterpret_cast<const float4 *>(dUs + i * VS + jq);
+                v.x = fmaf(wv, u.x, v.x); v.y = fmaf(wv, u.y, v.y); v.z = fmaf(wv, u.z, v.z); v.w = fmaf(wv, u.w, v.w);
+            }
+            dS[x] = v;
         }
         __syncthreads();
     }
-    if (own && dh0) {
-        float *dst = dh0 + ((size_t)bh * d.dk + dd) * d.dv + vs0;
+    if (dh0) {
 #pragma unroll
-        for (int j = 0; j < VS; ++j) dst[j] = dS[j];
+        for (int x = 0; x < 2; ++x) {
+            const int dd = i0 + 64 * x;
+            if (dd < d.dk) *reinterpret_cast<float4 *>(dh0 + ((size_t)bh * d.dk + dd) * d.dv + vs0 + jq) = dS[x];
+        }
     }
 }
 
@@ -438,20 +557,11 @@ k_grads_lin(Dims d, const TIO *__restrict__ q, const TIO *__restrict__ k, const 
     size_t row_last = tok_row(d, b, t0 + cn - 1, h);
 
     load_qk_hat(d, q, k, Gq, Gk, bcum, b, h, t0, cn, Qs, Ks, ldk);
-    for (int idx = threadIdx.x; idx < CMAX * d.dv; idx += blockDim.x) {
-        int i = idx / d.dv, j = idx % d.dv;
-        float vv = 0.f, gg = 0.f;
-        if (i < cn) {
-            size_t row = tok_row(d, b, t0 + i, h);
-            vv = ldf(v, row * d.dv + j);
-            gg = ldf(dO, row * d.dv + j);
-        }
-        Vs[i * ldv + j] = vv;
-        dOs[i * ldv + j] = gg;
-    }
+    auto vrow = [&](int i) { return tok_row(d, b, t0 + i, h) * d.dv; };
+    fill_rows(Vs, ldv, v, CMAX, cn, d.dv, vrow);
+    fill_rows(dOs, ldv, dO, CMAX, cn, d.dv, vrow);
     const float *Sg = states + state_off(d, bh, n, d.NT + 1);
-    for (int idx = threadIdx.x; idx < d.dk * d.dv; idx += blockDim.x)
-        Ss[(idx / d.dv) * ldv + idx % d.dv] = Sg[idx];
+    fill_rows(Ss, ldv, Sg, d.dk, d.dk, d.dv, [&](int i) { return (size_t)i * d.dv; });
     __syncthreads();
     {
         float a1[8][2], a2[8][2];
@@ -584,13 +694,14 @@ size_t smem_prepare(const Dims &d) {
     return sizeof(float) * (CMAX * (d.dk + 1) + CMAX * (CMAX + 1) + CMAX * (d.dk + d.dv) + 2 * CMAX);
 }
 size_t smem_scan(const Dims &d) {
-    return sizeof(float) * (2 * CMAX * (d.dk + 1) + CMAX * VS + d.dk * (VS + 1));
+    return sizeof(float) * (2 * CMAX * (d.dk + 1) + CMAX * VS + d.dk * VS + CMAX);
 }
+size_t smem_outer(const Dims &d) { return sizeof(float) * CMAX * (65 + d.dv + 1); }
 size_t smem_output(const Dims &d) {
     return sizeof(float) * (2 * CMAX * (d.dk + 1) + CMAX * (d.dv + 1) + CMAX * (CMAX + 1) + d.dk * (d.dv + 1));
 }
 size_t smem_dscan(const Dims &d) {
-    return sizeof(float) * (3 * CMAX * (d.dk + 1) + 2 * CMAX * VS + CMAX * (CMAX + 1) + d.dk * (VS + 1));
+    return sizeof(float) * (3 * CMAX * (d.dk + 1) + 2 * CMAX * VS + CMAX * (CMAX + 1) + d.dk * VS);
 }
 size_t smem_grads_lin(const Dims &d) {
     return sizeof(float) * (2 * CMAX * (d.dk + 1) + 2 * CMAX * (d.dv + 1) + 2 * CMAX * (CMAX + 1) +
@@ -641,10 +752,18 @@ int forward_t(const Dims &d, const Workspace &w, const FwdArgs &a, bool write_o,
         tr.mark("gdn_prepare");
         ++launches;
     }
-    dim3 slices(d.dv / VS, d.B * d.H);
-    k_state_scan<TIO><<<slices, 128, smem_scan(d), st>>>(d, k, v, Gk, bcum, a.h0, states, a.ht, Wws, U0ws, Uws);
-    tr.mark("state_scan");
-    ++launches;
+    if (d.variant == SLA_GDN) {
+        dim3 slices(d.dv / VS, d.B * d.H);
+        k_state_scan<TIO><<<slices, 256, smem_scan(d), st>>>(d, k, bcum, a.h0, states, a.ht, Wws, U0ws, Uws);
+        tr.mark("state_scan");
+        ++launches;
+    } else {
+        k_chunk_outer<TIO, false><<<dim3(d.NT, d.B * d.H, (d.dk + 63) / 64), 256, smem_outer(d), st>>>(d, k, v, Gk, bcum, states, nullptr);
+        tr.mark("chunk_outer");
+        k_state_fold<false><<<dim3((d.dk * d.dv + 255) / 256, d.B * d.H), 256, 0, st>>>(d, bcum, a.h0, states, a.ht);
+        tr.mark("state_fold");
+        launches += 2;
+    }
     if (write_o) {
         k_output<TIO><<<tiles, 256, smem_output(d), st>>>(d, q, k, v, Gq, Gk, bcum, states, Uws, (TIO *)a.o);
         tr.mark("output");
@@ -660,11 +779,12 @@ int backward_lin_t(const Dims &d, const Workspace &w, const BwdArgs &a, cudaStre
     float *dstates = ws + w.dstates, *dGq = ws + w.dGq, *dGk = ws + w.dGk;
     int launches = 0;
     const TIO *q = (const TIO *)a.q, *k = (const TIO *)a.k, *v = (const TIO *)a.v, *dO = (const TIO *)a.dO;
-    dim3 tiles(d.NT, d.B * d.H), slices(d.dv / VS, d.B * d.H);
-    k_dstate_scan<TIO><<<slices, 128, smem_dscan(d), st>>>(d, q, k, dO, Gq, bcum, a.dht, dstates, a.dh0,
-                                                           nullptr, nullptr);
-    tr.mark("dstate_scan");
-    ++launches;
+    dim3 tiles(d.NT, d.B * d.H);
+    k_chunk_outer<TIO, true><<<dim3(d.NT, d.B * d.H, (d.dk + 63) / 64), 256, smem_outer(d), st>>>(d, q, dO, Gq, bcum, dstates, a.dh0);
+    tr.mark("chunk_outer");
+    k_state_fold<true><<<dim3((d.dk * d.dv + 255) / 256, d.B * d.H), 256, 0, st>>>(d, bcum, a.dht, dstates, a.dh0);
+    tr.mark("state_fold");
+    launches += 2;
     k_grads_lin<TIO><<<tiles, 256, smem_grads_lin(d), st>>>(d, q, k, v, dO, Gq, Gk, bcum, states, dstates,
                                                             (TIO *)a.dq, (TIO *)a.dk, (TIO *)a.dv,
                                                             a.dlog_decay, dGq, dGk);
@@ -680,6 +800,7 @@ template <typename TIO> bool configure_t() {
     ok &= set_smem(k_gdn_prepare<TIO>, smem_prepare(d));
     ok &= set_smem(k_state_scan<TIO>, smem_scan(d));
     ok &= set_smem(k_output<TIO>, smem_output(d));
+    ok &= set_smem(k_chunk_outer<TIO, false>, smem_outer(d)) && set_smem(k_chunk_outer<TIO, true>, smem_outer(d));
     ok &= set_smem(k_dstate_scan<TIO>, smem_dscan(d));
     ok &= set_smem(k_grads_lin<TIO>, smem_grads_lin(d));
     return ok;
@@ -706,11 +827,11 @@ int generic_backward(const Dims &d, const Workspace &w, const BwdArgs &a, cudaSt
         float *ws = a.ws;
         dim3 slices(d.dv / VS, d.B * d.H);
         if (d.io_bf16)
-            k_dstate_scan<__nv_bfloat16><<<slices, 128, smem_dscan(d), st>>>(
+            k_dstate_scan<__nv_bfloat16><<<slices, 256, smem_dscan(d), st>>>(
                 d, (const __nv_bfloat16 *)a.q, (const __nv_bfloat16 *)a.k, (const __nv_bfloat16 *)a.dO, ws + w.Gq,
                 ws + w.bcum, a.dht, ws + w.dstates, a.dh0, ws + w.W, ws + w.dU);
         else
-            k_dstate_scan<float><<<slices, 128, smem_dscan(d), st>>>(
+            k_dstate_scan<float><<<slices, 256, smem_dscan(d), st>>>(
                 d, (const float *)a.q, (const float *)a.k, (const float *)a.dO, ws + w.Gq, ws + w.bcum, a.dht,
                 ws + w.dstates, a.dh0, ws + w.W, ws + w.dU);
         tr.mark("dstate_scan");

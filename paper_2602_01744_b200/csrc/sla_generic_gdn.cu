@@ -42,17 +42,9 @@ k_gdn_bwd_solve(Dims d, const TIO *__restrict__ k, const TIO *__restrict__ v,
         bs[i] = bcum[row];
         bt[i] = i < cn ? beta[row] : 0.f;
     }
-    for (int idx = threadIdx.x; idx < CMAX * d.dk; idx += blockDim.x) {
-        int i = idx / d.dk, c = idx % d.dk;
-        Ks[i * ldk + c] = i < cn ? ldf(k, tok_row(d, b, t0 + i, h) * d.dk + c) : 0.f;
-    }
-    for (int idx = threadIdx.x; idx < CMAX * d.dv; idx += blockDim.x) {
-        int i = idx / d.dv, j = idx % d.dv;
-        dUs[i * ldv + j] = i < cn ? dUws[tok_row(d, b, t0 + i, h) * d.dv + j] : 0.f;
-    }
-    const float *Sg = states + state_off(d, bh, n, d.NT + 1);
-    for (int idx = threadIdx.x; idx < d.dk * d.dv; idx += blockDim.x)
-        Ss[(idx / d.dv) * ldv + idx % d.dv] = Sg[idx];
+    fill_rows(Ks, ldk, k, CMAX, cn, d.dk, [&](int i) { return tok_row(d, b, t0 + i, h) * d.dk; });
+    fill_rows(dUs, ldv, dUws, CMAX, cn, d.dv, [&](int i) { return tok_row(d, b, t0 + i, h) * d.dv; });
+    fill_rows(Ss, ldv, states + state_off(d, bh, n, d.NT + 1), d.dk, d.dk, d.dv, [&](int i) { return (size_t)i * d.dv; });
     __syncthreads();
     for (int idx = threadIdx.x; idx < CMAX * CMAX; idx += blockDim.x) {
         int i = idx % CMAX, j = idx / CMAX;
@@ -143,10 +135,7 @@ k_gdn_grads(Dims d, const TIO *__restrict__ q, const TIO *__restrict__ k, const 
     const int ty = threadIdx.x >> 5, tx = threadIdx.x & 31;
 
     auto load_tile = [&](float *dst, const float *src, int width) {
-        for (int idx = threadIdx.x; idx < CMAX * width; idx += blockDim.x) {
-            int i = idx / width, c = idx % width;
-            dst[i * ldt + c] = i < cn ? src[tok_row(d, b, t0 + i, h) * width + c] : 0.f;
-        }
+        fill_rows(dst, ldt, src, CMAX, cn, width, [&](int i) { return tok_row(d, b, t0 + i, h) * width; });
     };
     for (int i = threadIdx.x; i < CMAX; i += blockDim.x) {
         size_t row = tok_row(d, b, t0 + min(i, cn - 1), h);
@@ -174,21 +163,28 @@ k_gdn_grads(Dims d, const TIO *__restrict__ q, const TIO *__restrict__ k, const 
     }
     __syncthreads();
     // phase B operands: T0 = q~ (gated, scaled, no decay), T1 = K, T2 = dO, T3 = U
-    for (int idx = threadIdx.x; idx < CMAX * d.dk; idx += blockDim.x) {
-        int i = idx / d.dk, c = idx % d.dk;
-        float qv = 0.f, kv = 0.f;
-        if (i < cn) {
-            size_t row = tok_row(d, b, t0 + i, h);
-            qv = d.scale * Gq[row] * ldf(q, row * d.dk + c);
-            kv = ldf(k, row * d.dk + c);
-        }
-        T0[i * ldt + c] = qv;
-        T1[i * ldt + c] = kv;
+    {
+        struct In { float4 q, k; float g; };
+        const int w4 = d.dk >> 2;
+        fill<2>(CMAX * w4,
+            [&](int idx) {
+                const int i = idx / w4;
+                In x{make_float4(0.f, 0.f, 0.f, 0.f), make_float4(0.f, 0.f, 0.f, 0.f), 0.f};
+                if (i < cn) {
+                    const size_t row = tok_row(d, b, t0 + i, h), o = row * d.dk + 4 * (idx - i * w4);
+                    x.q = ldf4(q, o);
+                    x.k = ldf4(k, o);
+                    x.g = d.scale * Gq[row];
+                }
+                return x;
+            },
+            [&](int idx, const In &x) {
+                const int i = idx / w4, o = i * ldt + 4 * (idx - i * w4);
+                put4(T0 + o, make_float4(x.g * x.q.x, x.g * x.q.y, x.g * x.q.z, x.g * x.q.w));
+                put4(T1 + o, x.k);
+            });
     }
-    for (int idx = threadIdx.x; idx < CMAX * d.dv; idx += blockDim.x) {
-        int i = idx / d.dv, j = idx % d.dv;
-        T2[i * ldt + j] = i < cn ? ldf(dO, tok_row(d, b, t0 + i, h) * d.dv + j) : 0.f;
-    }
+    fill_rows(T2, ldt, dO, CMAX, cn, d.dv, [&](int i) { return tok_row(d, b, t0 + i, h) * d.dv; });
     load_tile(T3, Uws, d.dv);
     __syncthreads();
     {
