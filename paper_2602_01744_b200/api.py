@@ -119,15 +119,17 @@ def _check(call: str, status: int):
         raise SLAError(call, status, lib().sla_status_string(status).decode())
 
 
+# A small decode step takes the GPU 5 us, so what the binding costs per call is what a serving loop sees: pointers go as plain
+# integers (ctypes converts them to the declared void * itself) and the stream handle comes without a Stream object around it.
 def _ptr(t):
     if t is None:
         return None
     assert t.is_cuda and t.is_contiguous(), "tensors must be contiguous CUDA tensors"
-    return ctypes.c_void_p(t.data_ptr())
+    return t.data_ptr()
 
 
 def _stream():
-    return ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
+    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
 
 
 class Plan:
@@ -143,6 +145,7 @@ class Plan:
                lib().sla_plan_workspace_bytes(self.handle, ctypes.byref(f), ctypes.byref(b)))
         self.forward_workspace_bytes, self.backward_workspace_bytes = f.value, b.value
         self.io_torch = torch.bfloat16 if self.desc.io_dtype == SLA_BF16 else torch.float32
+        self.heads, self.width_v = self.desc.H, self.desc.d_v
 
     def close(self):
         h = getattr(self, "handle", None)
@@ -254,13 +257,14 @@ def sla_backward(plan: Plan, q, k, v, log_decay, gq_logits, gk_logits, dO, beta=
 def sla_decode_step(plan: Plan, q_t, k_t, v_t, log_decay_t, gq_logits_t, gk_logits_t, state, beta_t=None,
                     o_t=None):
     """One recurrent step on `state` ([Bdec,H,d_k,d_v] fp32, updated in place).  Returns o_t."""
-    d = plan.desc
     Bdec = q_t.shape[0]
     if o_t is None:
-        o_t = torch.empty((Bdec, d.H, d.d_v), dtype=plan.io_torch, device=q_t.device)
-    _check("sla_decode_step", lib().sla_decode_step(
+        o_t = torch.empty((Bdec, plan.heads, plan.width_v), dtype=plan.io_torch, device=q_t.device)
+    status = (_lib or lib()).sla_decode_step(
         plan.handle, Bdec, _ptr(q_t), _ptr(k_t), _ptr(v_t), _ptr(log_decay_t), _ptr(beta_t),
-        _ptr(gq_logits_t), _ptr(gk_logits_t), _ptr(state), _ptr(o_t), _stream()))
+        _ptr(gq_logits_t), _ptr(gk_logits_t), _ptr(state), _ptr(o_t), _stream())
+    if status:
+        _check("sla_decode_step", status)
     return o_t
 
 
