@@ -176,18 +176,26 @@ k_gate_scores_bwd(long n_tok, int H, int d, int hpc, const TIO *__restrict__ q, 
     for (int e = 0; e < N; ++e) dst[e] = acc[e];
 }
 
-// dW[c,h] = sum over the CTAs' partial sums (stored [h][c]): one warp per element, lane l adds the partials of CTAs
-// l, l+32, .. in order, then the lanes are folded in a fixed tree - the same bits on every run.  grid (H*d/8, 2 sides).
-__global__ void k_gate_scores_dw(int n_cta, int H, int d, const float *__restrict__ partial, float *__restrict__ dWq,
-                                 float *__restrict__ dWk) {
-    const int i = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31, n = H * d;
-    if (i >= n) return;
-    const float *src = partial + (size_t)blockIdx.y * n_cta * n + i;
+// dW[c,h] = sum over the CTAs' partial sums (stored [h][c]).  A warp reads 32 neighbouring elements of one CTA; warp s of the
+// block adds the CTAs s, s + DW_WARPS, .. in order and the warps' sums are added in order: the same bits on every run.
+// (One element a warp, its lanes on 32 CTAs, fetched a 32-byte sector for every 4 bytes.)  grid (H*d/32, 2 sides).
+constexpr int DW_WARPS = 32;
+__global__ void __launch_bounds__(32 * DW_WARPS) k_gate_scores_dw(int n_cta, int H, int d, const float *__restrict__ partial, float *__restrict__ dWq,
+                                                                  float *__restrict__ dWk) {
+    __shared__ float sm[DW_WARPS][33];
+    const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5, n = H * d, i = blockIdx.x * 32 + lane;
+    const float *src = partial + (size_t)blockIdx.y * n_cta * n;
     float acc = 0.f;
-    for (int c = lane; c < n_cta; c += 32) acc += src[(size_t)c * n];
+    if (i < n) {
+#pragma unroll 8
+        for (int c = wp; c < n_cta; c += DW_WARPS) acc += src[(size_t)c * n + i];
+    }
+    sm[wp][lane] = acc;
+    __syncthreads();
+    if (wp != 0 || i >= n) return;
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    if (lane == 0) (blockIdx.y ? dWk : dWq)[(size_t)(i % d) * H + i / d] = acc;
+    for (int x = 1; x < DW_WARPS; ++x) acc += sm[x][lane];
+    (blockIdx.y ? dWk : dWq)[(size_t)(i % d) * H + i / d] = acc;
 }
 
 int score_ctas(long n_tok) {
@@ -236,8 +244,8 @@ int gate_scores_backward(const Dims &d, const void *q, const void *k, const floa
         k_gate_scores_bwd<float><<<grid, threads, 0, st>>>(n_tok, d.H, d.dk, hpc, (const float *)q, (const float *)k, Wq, Wk, dlq,
                                                            dlk, (float *)dq, (float *)dk, ws);
     tr.mark("gate_scores_bwd");
-    dim3 g2((d.H * d.dk + 7) / 8, 2);
-    k_gate_scores_dw<<<g2, 256, 0, st>>>(ctas, d.H, d.dk, ws, dWq, dWk);
+    dim3 g2((d.H * d.dk + 31) / 32, 2);
+    k_gate_scores_dw<<<g2, 32 * DW_WARPS, 0, st>>>(ctas, d.H, d.dk, ws, dWq, dWk);
     tr.mark("gate_scores_dw");
     return cudaGetLastError() == cudaSuccess ? 2 : -1;
 }

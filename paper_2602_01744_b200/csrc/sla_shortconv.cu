@@ -62,6 +62,14 @@ struct ConvDims { int T, H, d, K, per, hpc; float eps; };   // per: tokens of on
 // taps of this thread's channels, padded at the front to KMAX: y_t = sum_j wt[j] x[t-3+j]
 template <int N>
 __device__ __forceinline__ void load_taps(const float *w, int c0, int K, bool live, float (&wt)[KMAX][N]) {
+    if (K == KMAX) {         // a channel's taps are one 16-byte vector
+#pragma unroll
+        for (int e = 0; e < N; ++e) {
+            const float4 v = live ? __ldg(reinterpret_cast<const float4 *>(w) + c0 + e) : make_float4(0.f, 0.f, 0.f, 0.f);
+            wt[0][e] = v.x; wt[1][e] = v.y; wt[2][e] = v.z; wt[3][e] = v.w;
+        }
+        return;
+    }
 #pragma unroll
     for (int j = 0; j < KMAX; ++j)
 #pragma unroll
@@ -426,17 +434,31 @@ k_shortconv_bwd_blocks(ConvDims cd, int B, const __nv_bfloat16 *__restrict__ x, 
     }
 }
 
-// dw[c, j] = sum over the CTAs' partial sums: one warp per element, lane l adds the partials of CTAs l, l+32, .. in
-// order, then the lanes are folded in a fixed tree (same bits on every run)
-__global__ void k_shortconv_dw(int n_cta, int C, int K, const float *__restrict__ partial, float *__restrict__ dw) {
-    const int i = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-    if (i >= C * K) return;
-    const int c = i / K, j = i % K + (KMAX - K);
-    float acc = 0.f;
-    for (int n = lane; n < n_cta; n += 32) acc += partial[((size_t)n * C + c) * KMAX + j];
+// dw[c, j] = sum over the CTAs' partial sums.  A warp reads 32 channels' taps of one CTA as whole 512-byte runs (one element
+// a warp, its lanes on 32 CTAs, took a 32-byte sector per lane); warp s of the block adds the CTAs s, s + DW_WARPS, .. in
+// order and the warps' sums are added in order: the same bits on every run.
+constexpr int DW_WARPS = 16;
+__global__ void __launch_bounds__(32 * DW_WARPS) k_shortconv_dw(int n_cta, int C, int K, const float *__restrict__ partial, float *__restrict__ dw) {
+    __shared__ float4 sm[DW_WARPS][32];
+    const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5, c = blockIdx.x * 32 + lane;
+    float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (c < C) {
+#pragma unroll 8
+        for (int n = wp; n < n_cta; n += DW_WARPS) {
+            const float4 v = *reinterpret_cast<const float4 *>(partial + ((size_t)n * C + c) * KMAX);
+            acc.x += v.x; acc.y += v.y; acc.z += v.z; acc.w += v.w;
+        }
+    }
+    sm[wp][lane] = acc;
+    __syncthreads();
+    if (wp != 0 || c >= C) return;
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    if (lane == 0) dw[i] = acc;
+    for (int x = 1; x < DW_WARPS; ++x) {
+        const float4 v = sm[x][lane];
+        acc.x += v.x; acc.y += v.y; acc.z += v.z; acc.w += v.w;
+    }
+    const float r[KMAX] = {acc.x, acc.y, acc.z, acc.w};
+    for (int t = 0; t < K; ++t) dw[(size_t)c * K + t] = r[KMAX - K + t];
 }
 
 int tokens_per_cta(const Dims &d) {       // about four CTAs per SM, slices of at least 32 tokens
@@ -516,7 +538,7 @@ int shortconv_backward(const Dims &d, int width, int K, bool normalize, float ep
         if (normalize) k_shortconv_bwd_blocks<true><<<g, threads4, 0, st>>>(cd4, d.B, (const __nv_bfloat16 *)x, w, (const __nv_bfloat16 *)dout, (__nv_bfloat16 *)dx, ws);
         else k_shortconv_bwd_blocks<false><<<g, threads4, 0, st>>>(cd4, d.B, (const __nv_bfloat16 *)x, w, (const __nv_bfloat16 *)dout, (__nv_bfloat16 *)dx, ws);
         tr.mark("shortconv_bwd");
-        k_shortconv_dw<<<(C * K + 7) / 8, 256, 0, st>>>((int)g.x, C, K, ws, dw);
+        k_shortconv_dw<<<(C + 31) / 32, 32 * DW_WARPS, 0, st>>>((int)g.x, C, K, ws, dw);
         tr.mark("shortconv_dw");
         return cudaGetLastError() == cudaSuccess ? 2 : -1;
     }
@@ -533,7 +555,7 @@ int shortconv_backward(const Dims &d, int width, int K, bool normalize, float ep
     }
 #undef SLA_LAUNCH_BWD
     tr.mark("shortconv_bwd");
-    k_shortconv_dw<<<(C * K + 7) / 8, 256, 0, st>>>((int)(grid.x * grid.y), C, K, ws, dw);
+    k_shortconv_dw<<<(C + 31) / 32, 32 * DW_WARPS, 0, st>>>((int)(grid.x * grid.y), C, K, ws, dw);
     tr.mark("shortconv_dw");
     return cudaGetLastError() == cudaSuccess ? 2 : -1;
 }
