@@ -137,11 +137,10 @@ sla_status sla_plan_create(sla_plan **out, const sla_desc *desc) {
     if ((uint64_t)desc->B * desc->H > 65535u) return SLA_ERR_UNSUPPORTED;   // grid.y limit
     if (!(desc->scale == desc->scale)) return SLA_ERR_INVALID_ARG;
 
-    int dev = 0;
-    cudaDeviceProp prop;
+    int dev = 0, major = 0;                          // (one attribute: the whole property record takes the driver 7 ms and more)
     if (cudaGetDevice(&dev) != cudaSuccess) return SLA_ERR_CUDA;
-    if (cudaGetDeviceProperties(&prop, dev) != cudaSuccess) return SLA_ERR_CUDA;
-    if (prop.major != 10) return SLA_ERR_ARCH;
+    if (cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, dev) != cudaSuccess) return SLA_ERR_CUDA;
+    if (major != 10) return SLA_ERR_ARCH;
     if (sla::generic_configure() != 0 || sla::gdn_configure() != 0 || sla::gla_tc_configure() != 0 ||
         sla::gla_tc_bwd_configure() != 0 || sla::gdn_tc_configure() != 0 ||
         sla::gdn_tc_bwd_configure() != 0 || sla::decode_configure() != 0 || sla::out_proj_configure() != 0)
