@@ -109,12 +109,6 @@ __device__ __forceinline__ int next_chunk(const ChunkParams &p, int slot, int st
     return min(slot, p.slots);
 }
 
-// Rows r, r + 8 (r = 16 quarter + lane / 4), columns col0 + 8i + 2 (lane % 4) + {0, 1} of a swizzled tile of 64-column
-// halves: the places tmem_ld_frag* hands a thread.  Byte offset of column block i in row r; row r + 8 is 1024 further.
-__device__ __forceinline__ uint32_t frag_off(int quarter, int lane, int col0, int i) {
-    const uint32_t r = 16 * quarter + (lane >> 2), cb = (col0 >> 3) + i;
-    return (cb >> 3) * HALF_BF16 + swz(r, cb & 7) + (lane & 3) * 4;
-}
 // K extent of 128 (8 steps of 16) or 64 (4), unrolled: a rolled loop costs the issuing lane about 130 cycles a step
 template <class F>
 __device__ __forceinline__ void ksteps(bool wide, F step) {
@@ -124,11 +118,6 @@ __device__ __forceinline__ void ksteps(bool wide, F step) {
 #pragma unroll
         for (int kk = 4; kk < 8; ++kk) step(kk);
     }
-}
-// every writing thread has fenced; one arrival per warp
-__device__ __forceinline__ void warp_arrive(uint32_t bar, int lane) {
-    __syncwarp();
-    if (lane == 0) mbar_arrive(bar);
 }
 // loads still in flight when a wait gave up get time to land before shared memory is used for other things
 __device__ __forceinline__ void let_copies_land() {
@@ -1202,6 +1191,15 @@ __device__ __forceinline__ void bgrad_chunks(const CUtensorMap &gm_q, const CUte
         // ---------------- compute warps ----------------
         const int qr = warp & 3, ch = warp >> 2, r = 16 * qr + (lane >> 2);
         const uint32_t tq = tmem + ((uint32_t)(32 * qr) << 16);
+        // this thread's words of a tile: rows r, r + 8 of its eight column blocks
+        auto read_tile = [&](uint32_t tile, uint32_t (&w)[16]) {
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                const uint32_t off = tile + frag_off(qr, lane, 64 * ch, i);
+                w[2 * i] = *reinterpret_cast<const uint32_t *>(sm + off);
+                w[2 * i + 1] = *reinterpret_cast<const uint32_t *>(sm + off + 1024);
+            }
+        };
         // row sums of (fragment * tile) over this warp's 64 columns; lanes of a quad share a row
         auto quad_store = [&](float a0, float a1, float *dst) {
 #pragma unroll
@@ -1221,14 +1219,16 @@ __device__ __forceinline__ void bgrad_chunks(const CUtensorMap &gm_q, const CUte
             wait(FV, par);
             const float fq0 = sc[SC_FQ * C + r], fq1 = sc[SC_FQ * C + r + 8], bg0 = sc[SC_BG * C + r], bg1 = sc[SC_BG * C + r + 8];
             wait(FQ, par);
+            uint32_t tw[16];                           // (read whole, then written: no read is moved above a write of these tiles)
+            read_tile(OFF_Q, tw);
 #pragma unroll
             for (int i = 0; i < 8; ++i) {
                 const uint32_t off = frag_off(qr, lane, 64 * ch, i);
-                uint32_t *x0 = reinterpret_cast<uint32_t *>(sm + OFF_Q + off), *x1 = reinterpret_cast<uint32_t *>(sm + OFF_Q + off + 1024);
-                const float2 y0 = unpack_bf16(*x0), y1 = unpack_bf16(*x1);
-                *x0 = pack_bf16(fq0 * y0.x, fq0 * y0.y);
-                *x1 = pack_bf16(fq1 * y1.x, fq1 * y1.y);
+                const float2 y0 = unpack_bf16(tw[2 * i]), y1 = unpack_bf16(tw[2 * i + 1]);
+                *reinterpret_cast<uint32_t *>(sm + OFF_Q + off) = pack_bf16(fq0 * y0.x, fq0 * y0.y);
+                *reinterpret_cast<uint32_t *>(sm + OFF_Q + off + 1024) = pack_bf16(fq1 * y1.x, fq1 * y1.y);
             }
+            read_tile(OFF_V, tw);
             wait(C1, par);
             tc_fence_after();
             {
@@ -1242,7 +1242,7 @@ __device__ __forceinline__ void bgrad_chunks(const CUtensorMap &gm_q, const CUte
                     for (int i = 0; i < 8; ++i) {
                         const uint32_t off = frag_off(qr, lane, 64 * ch, i);
                         uint32_t *x0 = reinterpret_cast<uint32_t *>(sm + OFF_V + off), *x1 = reinterpret_cast<uint32_t *>(sm + OFF_V + off + 1024);
-                        const float2 y0 = unpack_bf16(*x0), y1 = unpack_bf16(*x1);
+                        const float2 y0 = unpack_bf16(tw[2 * i]), y1 = unpack_bf16(tw[2 * i + 1]);
                         a0 = fmaf(v[4 * i], y0.x, a0);     a0 = fmaf(v[4 * i + 1], y0.y, a0);
                         a1 = fmaf(v[4 * i + 2], y1.x, a1); a1 = fmaf(v[4 * i + 3], y1.y, a1);
                         *reinterpret_cast<uint32_t *>(sm + OFF_DR + off) = pack_bf16(v[4 * i], v[4 * i + 1]);
@@ -1290,12 +1290,13 @@ __device__ __forceinline__ void bgrad_chunks(const CUtensorMap &gm_q, const CUte
                 warp_arrive(bar(E2R), lane);
                 float v[32], a0 = 0.f, a1 = 0.f;
                 tmem_ld_frag8(tq + TM_Q + 64 * ch, v);
+                read_tile(OFF_Q, tw);
                 tmem_wait_ld();
 #pragma unroll
                 for (int i = 0; i < 8; ++i) {
                     const uint32_t off = frag_off(qr, lane, 64 * ch, i);
                     uint32_t *x0 = reinterpret_cast<uint32_t *>(sm + OFF_Q + off), *x1 = reinterpret_cast<uint32_t *>(sm + OFF_Q + off + 1024);
-                    const float2 y0 = unpack_bf16(*x0), y1 = unpack_bf16(*x1);
+                    const float2 y0 = unpack_bf16(tw[2 * i]), y1 = unpack_bf16(tw[2 * i + 1]);
                     a0 = fmaf(v[4 * i], y0.x, a0);     a0 = fmaf(v[4 * i + 1], y0.y, a0);
                     a1 = fmaf(v[4 * i + 2], y1.x, a1); a1 = fmaf(v[4 * i + 3], y1.y, a1);
                     *x0 = pack_bf16(fq0 * v[4 * i], fq0 * v[4 * i + 1]);
@@ -1313,6 +1314,7 @@ __device__ __forceinline__ void bgrad_chunks(const CUtensorMap &gm_q, const CUte
                 float v[32], y[32], a0 = 0.f, a1 = 0.f, e0 = 0.f, e1 = 0.f;
                 tmem_ld_frag8(tq + TM_K + 64 * ch, v);
                 tmem_ld_frag8(tq + TM_R + 64 * ch, y);
+                read_tile(OFF_K, tw);
                 tmem_wait_ld();
                 tc_fence_before();
                 warp_arrive(bar(TFREE), lane);
@@ -1320,7 +1322,7 @@ __device__ __forceinline__ void bgrad_chunks(const CUtensorMap &gm_q, const CUte
                 for (int i = 0; i < 8; ++i) {
                     const uint32_t off = frag_off(qr, lane, 64 * ch, i);
                     uint32_t *x0 = reinterpret_cast<uint32_t *>(sm + OFF_K + off), *x1 = reinterpret_cast<uint32_t *>(sm + OFF_K + off + 1024);
-                    const float2 k0 = unpack_bf16(*x0), k1 = unpack_bf16(*x1);
+                    const float2 k0 = unpack_bf16(tw[2 * i]), k1 = unpack_bf16(tw[2 * i + 1]);
                     a0 = fmaf(v[4 * i], k0.x, a0);     a0 = fmaf(v[4 * i + 1], k0.y, a0);
                     a1 = fmaf(v[4 * i + 2], k1.x, a1); a1 = fmaf(v[4 * i + 3], k1.y, a1);
                     e0 = fmaf(y[4 * i], k0.x, e0);     e0 = fmaf(y[4 * i + 1], k0.y, e0);

@@ -34,6 +34,18 @@ __device__ __forceinline__ uint64_t desc_mnmajor(uint32_t tile, uint32_t mn_stri
 }
 __device__ __forceinline__ constexpr uint64_t kstep_mnmajor(uint32_t kk) { return (kk * 2048) >> 4; }
 
+// Rows r, r + 8 (r = 16 quarter + lane / 4), columns col0 + 8i + 2 (lane % 4) + {0, 1} of a swizzled tile of 64-column
+// halves: the places tmem_ld_frag* hands a thread.  Byte offset of column block i in row r; row r + 8 is 1024 further.
+__device__ __forceinline__ uint32_t frag_off(int quarter, int lane, int col0, int i) {
+    const uint32_t r = 16 * quarter + (lane >> 2), cb = (col0 >> 3) + i;
+    return (cb >> 3) * HALF_BF16 + swz(r, cb & 7) + (lane & 3) * 4;
+}
+// every writing thread has fenced; one arrival per warp
+__device__ __forceinline__ void warp_arrive(uint32_t bar, int lane) {
+    __syncwarp();
+    if (lane == 0) ptx::mbar_arrive(bar);
+}
+
 typedef CUresult (*EncodeFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *,
                              const cuuint64_t *, const cuuint32_t *, const cuuint32_t *, CUtensorMapInterleave,
                              CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
@@ -139,12 +151,15 @@ constexpr float LOG2E = 1.4426950408889634f;
 //   b_i = inclusive cumulative log-decay (kept in log2 units), two-level: per-8-row sums, then a running sum
 //   qh_i = gq_i * q_i * 2^{b_i}   (gq_i = scale*Gq_i)      kh_i = gk_i * k_i * 2^{-b_i}
 // written over q and k in place (the swizzled tiles are the MMA operands); eblast[d] = 2^{b_last,d}.
-// With WITH_E also leaves the tile e2[i][d] = (bf16 gq_i 2^{b_i}, bf16 gk_i 2^{-b_i}), 4 bytes per element, rows of 512 B,
-// unswizzled: the factors that turn dqh, dkh into dq, dk.  Thread (rg = warp, cj = lane) owns rows 8rg..8rg+7,
+// With WITH_E also leaves the tile e2[i][d] = (bf16 gq_i 2^{b_i}, bf16 gk_i 2^{-b_i}), 4 bytes per element, rows of 512 B with
+// their 16-byte chunks swizzled (e2_off): the factors that turn dqh, dkh into dq, dk.  Thread (rg = warp, cj = lane) owns rows 8rg..8rg+7,
 // columns 4cj..4cj+3.
 // tot: [8][128] floats of scratch.  status: the plan's device status word (a chunk whose cumulative log-decay is
 // beyond the representable range raises STATUS_RANGE there).
 constexpr uint32_t TOT_BYTES = 8 * D * 4;
+// byte offset of 16-byte chunk `chunk` (0..31) of row `row` in a [64][128] tile of 4-byte elements: the gradient epilogue reads 32
+// bytes of each of eight rows at once, which without the swizzle all sit in the same banks
+__device__ __forceinline__ uint32_t e2_off(uint32_t row, uint32_t chunk) { return row * (D * 4) + ((chunk ^ ((row & 3) << 1)) << 4); }
 struct NoHook { __device__ __forceinline__ void operator()() const {} };
 // Softmax-RetNet runs on the same kernels: with gs == nullptr the chunk's log-decay tile is not read but generated,
 // log_gamma on each of the chunk's cn tokens (all key dimensions alike).
@@ -174,25 +189,38 @@ __device__ __forceinline__ void chunk_prologue(uint8_t *q_tile, uint8_t *k_tile,
     named_bar_sync(bar_id, NCOMPUTE);
     tile_read();                                // every thread has read its rows: the log-decay tile may be overwritten
     float bsum[4] = {0.f, 0.f, 0.f, 0.f};
-    for (int g = 0; g < rg; ++g) {
-        const float4 a = *reinterpret_cast<const float4 *>(tot + g * D + 4 * cj);
+#pragma unroll
+    for (int g = 0; g < 7; ++g) {               // (unrolled: the reads overlap)
+        const float4 a = g < rg ? *reinterpret_cast<const float4 *>(tot + g * D + 4 * cj) : make_float4(0.f, 0.f, 0.f, 0.f);
         bsum[0] += a.x; bsum[1] += a.y; bsum[2] += a.z; bsum[3] += a.w;
     }
 #pragma unroll
     for (int e = 0; e < 4; ++e) bsum[e] *= LOG2E;
     // columns 4cj..4cj+3 = 8 bytes of a bf16 row: half cj>>4, 16-byte chunk (cj&15)>>1, upper or lower 8 bytes
     const uint32_t half = cj >> 4, chunk = (cj & 15) >> 1, sub = (cj & 1) * 8;
+    // rows in batches whose reads are all in flight before the first write over them (no read is moved above a write of these
+    // tiles); the backward pass has the registers for whole batches of eight
+    constexpr int RB = WITH_E ? 8 : 2;
+    uint2 qr[RB], kr[RB];
 #pragma unroll
     for (int rr = 0; rr < 8; ++rr) {
         const int r = 8 * rg + rr;
+        if (rr % RB == 0) {
+#pragma unroll
+            for (int x = 0; x < RB; ++x) {
+                const uint32_t o = half * HALF_BF16 + swz(r + x, chunk) + sub;
+                kr[x] = *reinterpret_cast<const uint2 *>(k_tile + o);
+                if (WITH_Q) qr[x] = *reinterpret_cast<const uint2 *>(q_tile + o);
+            }
+        }
         const float4 g = gl[rr];
         bsum[0] = fmaf(g.x, LOG2E, bsum[0]); bsum[1] = fmaf(g.y, LOG2E, bsum[1]);
         bsum[2] = fmaf(g.z, LOG2E, bsum[2]); bsum[3] = fmaf(g.w, LOG2E, bsum[3]);
         const float gq = WITH_Q ? gq_s[r] : 0.f, gk = gk_s[r];
         const uint32_t off = half * HALF_BF16 + swz(r, chunk) + sub;
-        uint2 qv, kv = *reinterpret_cast<uint2 *>(k_tile + off);
+        uint2 qv, kv = kr[rr % RB];
         uint4 e2v;
-        if (WITH_Q) qv = *reinterpret_cast<uint2 *>(q_tile + off);
+        if (WITH_Q) qv = qr[rr % RB];
         uint32_t *qw = reinterpret_cast<uint32_t *>(&qv), *kw = reinterpret_cast<uint32_t *>(&kv);
         uint32_t *e2w = reinterpret_cast<uint32_t *>(&e2v);
 #pragma unroll
@@ -212,7 +240,7 @@ __device__ __forceinline__ void chunk_prologue(uint8_t *q_tile, uint8_t *k_tile,
         }
         *reinterpret_cast<uint2 *>(k_tile + off) = kv;
         if (WITH_Q) *reinterpret_cast<uint2 *>(q_tile + off) = qv;
-        if (WITH_E) *reinterpret_cast<uint4 *>(e2_tile + r * (D * 4) + cj * 16) = e2v;
+        if (WITH_E) *reinterpret_cast<uint4 *>(e2_tile + e2_off(r, cj)) = e2v;
     }
     if (rg == 7) {
 #pragma unroll

@@ -9,13 +9,19 @@
 //   k_gla_bwd_tc      reverse order.  Carries dS (fp32, TMEM).  Per chunk, with qh = scale*Gq*q*e^b,
 //                     kh = Gk*k*e^-b, dZ = diag(e^{b_last}) dS_{n+1}:
 //                       A = tril(qh kh^T)            dA = tril(dO V^T)
-//                       dqh^T = kh^T dA^T + S_n dO^T        (128 x 64: key dimension x token)
-//                       dkh^T = qh^T dA   + dZ V^T
-//                       dV^T  = dO^T A    + dZ^T kh^T
-//                       dS_n  = dZ + qh^T dO
-//                     The three gradient tiles are produced transposed so that one thread owns one key (value)
-//                     dimension and walks the tokens: the log-decay gradient is the in-chunk suffix sum of
-//                     qh*dqh - kh*dkh plus rowsum(dS_{n+1} * S_{n+1}) carried from the chunk to the right.
+//                       dqh = dA kh   + dO S_n^T
+//                       dkh = dA^T qh + V dZ^T
+//                       dV  = A^T dO  + kh dZ
+//                       dS_n = dZ + qh^T dO
+//                     The gradient tiles are 64 x 128, token by feature, read out in the 16x256b form: a thread holds pairs
+//                     of neighbouring features, so operands and results move in 4-byte words, a token's sum over the features
+//                     takes two shuffles, and every thread has work.  (Produced transposed, one thread walked 32 tokens of
+//                     one feature in 2-byte words and every token sum was a 31-shuffle transpose.  Alone, Softmax-GLA then Softmax-RetNet,
+//                     8 x 4096 tokens x 16 heads: 403 and 380 us so, 397 and 354 us now.)  The kernel is bound by the serial
+//                     passes of a chunk, about 9,500 cycles of which the prologue and the gradient read-out, each limited by
+//                     instruction issue of eight warps, take 2,600 and 2,100; the tensor core is idle for most of it.
+//                     The log-decay gradient is the in-chunk suffix sum of qh*dqh - kh*dkh, taken over an fp32 tile in the
+//                     place of the factors, plus rowsum(dS_{n+1} * S_{n+1}) carried from the chunk to the right.
 //                     Gate gradients leave as the products Gq*dGq = sum_d qh*dqh, Gk*dGk = sum_d kh*dkh per
 //                     (token, head); the softmax backward over heads runs afterwards on [B,T,H].
 // Few long sequences (at least three segments per sequence fit the SMs): gla_tc_backward_segmented runs both sweeps
@@ -321,15 +327,14 @@ constexpr uint32_t OFF_TOT = OFF_DA + HALF_BF16;        // prologue scratch
 constexpr uint32_t OFF_EB = OFF_TOT + TOT_BYTES;        // [128] 2^{b_last}
 constexpr uint32_t OFF_GATE = OFF_EB + D * 4;           // [4][2][64]: scale*Gq, Gk of four chunks
 constexpr uint32_t OFF_R = OFF_GATE + 4 * 2 * C * 4;    // [2 buffers][2 column halves][128] rowsum(dS*S) partials
-constexpr uint32_t OFF_UP = OFF_R + 4 * D * 4;          // [128] suffix total of the upper 32 tokens
-constexpr uint32_t OFF_RED = OFF_UP + D * 4;            // [2][8 warps][32] gate partial sums
-constexpr uint32_t OFF_BAR = OFF_RED + 2 * 8 * 32 * 4;
+constexpr uint32_t OFF_RED = OFF_R + 4 * D * 4;            // [2][2 column halves][64] gate partial sums
+constexpr uint32_t OFF_BAR = OFF_RED + 2 * 2 * C * 4;
 constexpr uint32_t OFF_TMEM = OFF_BAR + 32 * 8;         // TMEM base address, then the abort flag
 constexpr uint32_t SMEM_BYTES = OFF_TMEM + 16 + 1024;
-constexpr uint32_t COL_DS = 0, COL_A = 128, COL_DA = 192, COL_DQ = 256, COL_DK = 320, COL_DV = 384, TMEM_COLS = 512;
+constexpr uint32_t COL_DS = 0, COL_A = 128, COL_DA = 192, COL_DV = 128 /* once A and dA are read */, COL_DQ = 256, COL_DK = 384, TMEM_COLS = 512;
 constexpr int NTHREADS = NCOMPUTE + 32 + NGATE + 32;    // warps 0..7 compute, 8 MMA issue, 9..12 gates, 13 TMA
 enum Bar { FULL_G = 0, FULL_QK, FULL_V, FULL_DO, FULL_S, OPR, GREADY /*[4]*/, GFREE = GREADY + 4 /*[4]*/, ZREADY = GFREE + 4,
-           AREADY, OUT1, OUT2, SNFREE, INIT_DONE, DGFREE, BAR_A, BAR_M1, BAR_M2, DOFREE, INIT_FULL, DRAIN, BAR_DS, NBAR };
+           AREADY, OUT1, OUT2, SNFREE, INIT_DONE, DVREAD, DGFREE, BAR_A, BAR_M1, BAR_M2, DOFREE, INIT_FULL, DRAIN, BAR_DS, NBAR };
 static_assert(SMEM_BYTES <= 232448, "shared memory budget");
 static_assert(NBAR <= 32, "barrier slots");
 }  // namespace st2
@@ -346,21 +351,6 @@ struct BwdParams {
     const CUtensorMap *vmaps;
     int dk, dv;             // head widths, each 128 or 64 (the upper half of a 128-wide tile is then zero padding)
 };
-
-// Sum v[j] over the 32 lanes for every j: afterwards lane l holds the total of v[l] in v[0].
-__device__ __forceinline__ float warp_transpose_sum(float (&v)[32], int lane) {
-#pragma unroll
-    for (int off = 16; off >= 1; off >>= 1) {
-        const bool upper = (lane & off) != 0;
-#pragma unroll
-        for (int j = 0; j < off; ++j) {
-            const float send = upper ? v[j] : v[j + off];
-            const float keep = upper ? v[j + off] : v[j];
-            v[j] = keep + __shfl_xor_sync(0xffffffffu, send, off);
-        }
-    }
-    return v[0];
-}
 
 // Chunks in reverse order.  Per chunk n the compute warps run: prologue -> dZ = diag(2^{b_last}) dS_{n+1} -> causal
 // mask of A and dA -> gradient tiles out of TMEM.  The MMA lane issues each product as soon as its operands exist:
@@ -401,7 +391,6 @@ k_gla_bwd_tc(const __grid_constant__ CUtensorMap gm_q, const __grid_constant__ C
     float *eblast = reinterpret_cast<float *>(sm + OFF_EB);
     float *gate_s = reinterpret_cast<float *>(sm + OFF_GATE);
     float *Rs = reinterpret_cast<float *>(sm + OFF_R);
-    float *up = reinterpret_cast<float *>(sm + OFF_UP);
     float *red = reinterpret_cast<float *>(sm + OFF_RED);
     volatile int *abort_flag = reinterpret_cast<volatile int *>(sm + OFF_TMEM + 8);
     bool failed = false;
@@ -415,8 +404,9 @@ k_gla_bwd_tc(const __grid_constant__ CUtensorMap gm_q, const __grid_constant__ C
     if (tid == 0) {
         *abort_flag = 0;
         for (int i = 0; i < NBAR; ++i) {
-            const bool all = i == OPR || (i >= GFREE && i <= INIT_DONE);
-            mbar_init(bar(i), all ? NCOMPUTE : (i >= GREADY && i < GFREE) ? NGATE / 32 : 1);
+            const bool all = i == INIT_DONE || (i >= GFREE && i < ZREADY);
+            const bool warps = i == OPR || (i >= ZREADY && i <= SNFREE) || i == DVREAD;                        // one arrival per warp
+            mbar_init(bar(i), all ? NCOMPUTE : warps ? NCOMPUTE / 32 : (i >= GREADY && i < GFREE) ? NGATE / 32 : 1);
         }
         fence_mbar_init();
         tma_prefetch_desc(&tm_q);
@@ -447,8 +437,8 @@ k_gla_bwd_tc(const __grid_constant__ CUtensorMap gm_q, const __grid_constant__ C
                 if (!failed && !__all_sync(0xffffffffu, mbar_wait_bounded(bar(i), parity, abort_flag))) { failed = true; *abort_flag = 1; }
             };
             constexpr uint32_t ID_A = idesc_bf16(64, 64, 0, 0);
-            constexpr uint32_t ID_KK = idesc_bf16(128, 64, 0, 0), ID_MK = idesc_bf16(128, 64, 1, 0),
-                               ID_MM = idesc_bf16(128, 64, 1, 1), ID_S = idesc_bf16(128, 128, 1, 1);
+            constexpr uint32_t ID_KK = idesc_bf16(64, 128, 0, 0), ID_KM = idesc_bf16(64, 128, 0, 1),
+                               ID_MM = idesc_bf16(64, 128, 1, 1), ID_S = idesc_bf16(128, 128, 1, 1);
             const uint64_t kS = desc_kmajor(base + OFF_S), kDZ = desc_kmajor(base + OFF_DZ),
                            mDZ = desc_mnmajor(base + OFF_DZ, STATE_HALF), mA = desc_mnmajor(base + OFF_A, HALF_BF16),
                            kDA = desc_kmajor(base + OFF_DA), mDA = desc_mnmajor(base + OFF_DA, HALF_BF16);
@@ -462,6 +452,7 @@ k_gla_bwd_tc(const __grid_constant__ CUtensorMap gm_q, const __grid_constant__ C
                 // dA = dO V^T and S_n dO^T need no prologue: they are issued while the compute warps still scale q and k
                 wait(FULL_V, par);
                 wait(FULL_DO, par);
+                if (k > 0) wait(DVREAD, (k - 1) & 1);  // dV of the previous chunk, in the columns of A and dA, has been read out
                 if (failed) break;
                 tc_fence_after();
                 if (leader)
@@ -469,13 +460,13 @@ k_gla_bwd_tc(const __grid_constant__ CUtensorMap gm_q, const __grid_constant__ C
                 for (int kk = 0; kk < 8; ++kk)         // dA = dO V^T
                     tc_mma_bf16(tmem + COL_DA, kDO + kstep_kmajor(kk, HALF_BF16), kV + kstep_kmajor(kk, HALF_BF16), ID_A, kk > 0);
                 bool sdo_done = false;
-                auto issue_sdo = [&]() {               // dqh^T = S_n dO^T ...
-                    if (k > 0) wait(OUT1, (k - 1) & 1);    // dqh^T, dkh^T of the previous chunk have been read out (long ago)
+                auto issue_sdo = [&]() {               // dqh = dO S_n^T ...
+                    if (k > 0) wait(OUT1, (k - 1) & 1);    // dqh, dkh of the previous chunk have been read out (long ago)
                     tc_fence_after();
                     if (leader)
 #pragma unroll
                     for (int kk = 0; kk < 8; ++kk)
-                        tc_mma_bf16(tmem + COL_DQ, kS + kstep_kmajor(kk, STATE_HALF), kDO + kstep_kmajor(kk, HALF_BF16), ID_KK, kk > 0);
+                        tc_mma_bf16(tmem + COL_DQ, kDO + kstep_kmajor(kk, HALF_BF16), kS + kstep_kmajor(kk, STATE_HALF), ID_KK, kk > 0);
                     sdo_done = true;
                 };
                 {   // whichever comes first: S_n landed, or the prologue done
@@ -498,15 +489,14 @@ k_gla_bwd_tc(const __grid_constant__ CUtensorMap gm_q, const __grid_constant__ C
                     if (failed) break;
                     issue_sdo();
                 }
-                if (k > 0) wait(OUT2, (k - 1) & 1);    // dV^T and dS of the previous chunk have been read out
+                if (k > 0) wait(OUT2, (k - 1) & 1);    // dS of the previous chunk has been read out
                 wait(ZREADY, par);                     // dZ: fp32 in TMEM, bf16 in shared memory
                 if (failed) break;
                 tc_fence_after();
                 if (leader)
 #pragma unroll
-                for (int kk = 0; kk < 8; ++kk) {       // three independent accumulation chains, interleaved
-                    tc_mma_bf16(tmem + COL_DK, kDZ + kstep_kmajor(kk, STATE_HALF), kV + kstep_kmajor(kk, HALF_BF16), ID_KK, kk > 0);   // dkh^T = dZ V^T ...
-                    tc_mma_bf16(tmem + COL_DV, mDZ + kstep_mnmajor(kk), kK + kstep_kmajor(kk, HALF_BF16), ID_MK, kk > 0);            // dV^T = dZ^T kh^T ...
+                for (int kk = 0; kk < 8; ++kk) {       // two independent accumulation chains, interleaved
+                    tc_mma_bf16(tmem + COL_DK, kV + kstep_kmajor(kk, HALF_BF16), kDZ + kstep_kmajor(kk, STATE_HALF), ID_KK, kk > 0);   // dkh = V dZ^T ...
                     if (kk < 4) tc_mma_bf16(tmem + COL_DS, mQ + kstep_mnmajor(kk), mDO + kstep_mnmajor(kk), ID_S, 1);                // dS_n = dZ + qh^T dO
                 }
                 if (leader) tc_commit(bar(BAR_DS));                // dS_n is complete (and S_n dO^T has read S_n)
@@ -515,15 +505,19 @@ k_gla_bwd_tc(const __grid_constant__ CUtensorMap gm_q, const __grid_constant__ C
                 tc_fence_after();
                 if (leader)
 #pragma unroll
-                for (int kk = 0; kk < 4; ++kk) {       // ... + kh^T dA^T  and  ... + qh^T dA, interleaved
-                    tc_mma_bf16(tmem + COL_DQ, mK + kstep_mnmajor(kk), kDA + kstep_kmajor(kk, 0), ID_MK, 1);
-                    tc_mma_bf16(tmem + COL_DK, mQ + kstep_mnmajor(kk), mDA + kstep_mnmajor(kk), ID_MM, 1);
+                for (int kk = 0; kk < 8; ++kk)         // dV = kh dZ ... (A and dA have been read; before M1, after which dk goes over kh)
+                    tc_mma_bf16(tmem + COL_DV, kK + kstep_kmajor(kk, HALF_BF16), mDZ + kstep_mnmajor(kk), ID_KM, kk > 0);
+                if (leader)
+#pragma unroll
+                for (int kk = 0; kk < 4; ++kk) {       // ... + dA kh  and  ... + dA^T qh, interleaved
+                    tc_mma_bf16(tmem + COL_DQ, kDA + kstep_kmajor(kk, 0), mK + kstep_mnmajor(kk), ID_KM, 1);
+                    tc_mma_bf16(tmem + COL_DK, mDA + kstep_mnmajor(kk), mQ + kstep_mnmajor(kk), ID_MM, 1);
                 }
                 if (leader) tc_commit(bar(BAR_M1));
                 if (leader)
 #pragma unroll
-                for (int kk = 0; kk < 4; ++kk)         // ... + dO^T A
-                    tc_mma_bf16(tmem + COL_DV, mDO + kstep_mnmajor(kk), mA + kstep_mnmajor(kk), ID_MM, 1);
+                for (int kk = 0; kk < 4; ++kk)         // ... + A^T dO
+                    tc_mma_bf16(tmem + COL_DV, mA + kstep_mnmajor(kk), mDO + kstep_mnmajor(kk), ID_MM, 1);
                 if (leader) tc_commit(bar(BAR_M2));
                 if (leader) tc_commit(bar(DOFREE));                // (same event, for the TMA lane)
             }
@@ -627,7 +621,8 @@ k_gla_bwd_tc(const __grid_constant__ CUtensorMap gm_q, const __grid_constant__ C
         // ---------------- compute warps ----------------
         const uint32_t lane_base = (uint32_t)(32 * (warp & 3)) << 16;
         const int wh = warp >> 2;                       // column half (state passes) / token half (gradient tiles)
-        const int row = 32 * (warp & 3) + lane;         // TMEM lane = key (value) dimension owned by this thread
+        const int row = 32 * (warp & 3) + lane;         // state row of this thread (its TMEM lane)
+        const int qr = warp & 3, tr = 16 * qr + (lane >> 2);       // gradient tiles: tokens tr, tr + 8
         const bool retnet = p.log_gamma != nullptr;
         const float lgam = retnet ? p.log_gamma[h] : 0.f;
 
@@ -680,7 +675,7 @@ k_gla_bwd_tc(const __grid_constant__ CUtensorMap gm_q, const __grid_constant__ C
                                            ScalarDecay{lgam, min(C, p.T - t0)});
             }
             fence_proxy_async();
-            mbar_arrive(bar(OPR));
+            warp_arrive(bar(OPR), lane);
             mbar_arrive(bar(GFREE + (k & 3)));
 
             // ---- dZ = diag(2^{b_last}) dS_{n+1}: fp32 back into TMEM (dS_n accumulates on it), bf16 operand copy ----
@@ -705,44 +700,27 @@ k_gla_bwd_tc(const __grid_constant__ CUtensorMap gm_q, const __grid_constant__ C
             }
             fence_proxy_async();
             tc_fence_before();
-            mbar_arrive(bar(ZREADY));
+            warp_arrive(bar(ZREADY), lane);
 
-            // ---- A, dA: TMEM -> causal mask -> bf16 -> shared memory (row i of an M=64 tile sits in lane 32*(i/16) + i%16) ----
+            // ---- A, dA: TMEM -> causal mask -> bf16 -> shared memory ----
             wait(BAR_A, par);
             tc_fence_after();
             {
-                // rows 16q..16q+15 of this warp: a block of 8 columns c is empty for c >= 2q+2, full for c < 2q
-                const int q4 = warp & 3, i = 16 * q4 + lane;
-                const uint32_t col = wh ? COL_DA : COL_A;
                 uint8_t *dst = sm + (wh ? OFF_DA : OFF_A);
-                float v0[32], v1[32];
-                tmem_ld32(tmem + lane_base + col, v0);
-                tmem_ld32(tmem + lane_base + col + 32, v1);
+                float v[32];
+                tmem_ld_frag8(tmem + lane_base + (wh ? COL_DA : COL_A), v);
                 tmem_wait_ld();
-                if (lane < 16) {
-#define SLA_MASK_BLOCK(V, CL, CB)                                                                                          \
-    {                                                                                                                      \
-        uint4 w = make_uint4(0u, 0u, 0u, 0u);                                                                              \
-        if ((CB) < 2 * q4 + 2) {                                                                                           \
-            const int j0 = 8 * (CB);                                                                                       \
-            const bool full = (CB) < 2 * q4;                                                                               \
-            w.x = pack_bf16(full || j0 + 0 <= i ? V[8 * (CL) + 0] : 0.f, full || j0 + 1 <= i ? V[8 * (CL) + 1] : 0.f);     \
-            w.y = pack_bf16(full || j0 + 2 <= i ? V[8 * (CL) + 2] : 0.f, full || j0 + 3 <= i ? V[8 * (CL) + 3] : 0.f);     \
-            w.z = pack_bf16(full || j0 + 4 <= i ? V[8 * (CL) + 4] : 0.f, full || j0 + 5 <= i ? V[8 * (CL) + 5] : 0.f);     \
-            w.w = pack_bf16(full || j0 + 6 <= i ? V[8 * (CL) + 6] : 0.f, full || j0 + 7 <= i ? V[8 * (CL) + 7] : 0.f);     \
-        }                                                                                                                  \
-        *reinterpret_cast<uint4 *>(dst + swz(i, (CB))) = w;                                                                \
-    }
 #pragma unroll
-                    for (int c = 0; c < 4; ++c) SLA_MASK_BLOCK(v0, c, c)
-#pragma unroll
-                    for (int c = 0; c < 4; ++c) SLA_MASK_BLOCK(v1, c, 4 + c)
-#undef SLA_MASK_BLOCK
+                for (int i = 0; i < 8; ++i) {
+                    const int j = 8 * i + 2 * (lane & 3);
+                    const uint32_t off = frag_off(qr, lane, 0, i);
+                    *reinterpret_cast<uint32_t *>(dst + off) = pack_bf16(j <= tr ? v[4 * i] : 0.f, j + 1 <= tr ? v[4 * i + 1] : 0.f);
+                    *reinterpret_cast<uint32_t *>(dst + off + 1024) = pack_bf16(j <= tr + 8 ? v[4 * i + 2] : 0.f, j + 1 <= tr + 8 ? v[4 * i + 3] : 0.f);
                 }
             }
             fence_proxy_async();
             tc_fence_before();
-            mbar_arrive(bar(AREADY));
+            warp_arrive(bar(AREADY), lane);
 
             // ---- R_{n-1} = rowsum(dS_n * S_n), while the tensor core works on the products with the masked tiles ----
             // (it feeds the log-decay gradient only: Softmax-RetNet, whose decay is a constant, has none and skips it)
@@ -755,82 +733,115 @@ k_gla_bwd_tc(const __grid_constant__ CUtensorMap gm_q, const __grid_constant__ C
                 tmem_wait_ld();
                 Rs[((n & 1) ^ 1) * 2 * D + wh * D + row] = rowdot_part(v0, 0) + rowdot_part(v1, 1);
             }
-            mbar_arrive(bar(SNFREE));                   // S_n is no longer needed: the next image may land
+            warp_arrive(bar(SNFREE), lane);                   // S_n is no longer needed: the next image may land
 
-            // ---- dqh^T, dkh^T: this thread owns key dimension `row` and tokens 32*wh .. 32*wh+31 ----
+            // ---- dqh, dkh: tokens tr, tr + 8, pairs of features of column half wh ----
             wait(BAR_M1, par);
             tc_fence_after();
-            const float *Rcur = Rs + (n & 1) * 2 * D;
-            float sfx[32];
             {
-                float dqh[32], dkh[32];
-                tmem_ld32(tmem + lane_base + COL_DQ + 32 * wh, dqh);
-                tmem_ld32(tmem + lane_base + COL_DK + 32 * wh, dkh);
-                tmem_wait_ld();
-                const uint32_t dhalf = (uint32_t)(row >> 6) * HALF_BF16, dchunk = (uint32_t)(row & 63) >> 3, dbyte = (row & 7) * 2;
-                float run = 0.f;
+                float sq0 = 0.f, sq1 = 0.f, sk0 = 0.f, sk1 = 0.f;
+                // the pair's factors (gq 2^b, gk 2^-b), 8 bytes; qh dqh - kh dkh of the pair goes in their place
+                auto e2_at = [&](int hf, int y) {
+                    return sm + OFF_E2 + e2_off(tr + 8 * (y & 1), 16 * wh + 8 * hf + 2 * (y >> 1) + ((lane & 3) >> 1)) + 8 * (lane & 1);
+                };
 #pragma unroll
-                for (int ii = 31; ii >= 0; --ii) {
-                    const int i = 32 * wh + ii;
-                    const uint32_t off = dhalf + swz(i, dchunk) + dbyte;
-                    __nv_bfloat16 *qp = reinterpret_cast<__nv_bfloat16 *>(qk + off);
-                    __nv_bfloat16 *kp = reinterpret_cast<__nv_bfloat16 *>(qk + TILE_BF16 + off);
-                    const float2 ee = unpack_bf16(*reinterpret_cast<const uint32_t *>(sm + OFF_E2 + i * (D * 4) + row * 4));
-                    const float pq = __bfloat162float(*qp) * dqh[ii], pk = __bfloat162float(*kp) * dkh[ii];
-                    run += pq - pk;
-                    sfx[ii] = run;
-                    *qp = __float2bfloat16_rn(ee.x * dqh[ii]);       // dq = scale Gq 2^b dqh   (over qh, for the store)
-                    *kp = __float2bfloat16_rn(ee.y * dkh[ii]);       // dk = Gk 2^-b dkh
-                    dqh[ii] = pq;
-                    dkh[ii] = pk;
+                for (int hf = 0; hf < 2; ++hf) {       // 32 features at a time; every read of a batch is in flight before its first
+                    float dqh[16], dkh[16];            // write (the compiler moves no read above a write of these tiles: 2490 cycles)
+                    uint32_t qw[8], kw[8];
+                    uint2 ew[8];
+                    tmem_ld_frag4(tmem + lane_base + COL_DQ + 64 * wh + 32 * hf, dqh);
+                    tmem_ld_frag4(tmem + lane_base + COL_DK + 64 * wh + 32 * hf, dkh);
+#pragma unroll
+                    for (int y = 0; y < 8; ++y) {      // feature block y / 2, token tr + 8 (y % 2)
+                        const uint32_t off = frag_off(qr, lane, 64 * wh + 32 * hf, y >> 1) + 1024 * (y & 1);
+                        qw[y] = *reinterpret_cast<const uint32_t *>(qk + off);
+                        kw[y] = *reinterpret_cast<const uint32_t *>(qk + TILE_BF16 + off);
+                        ew[y] = *reinterpret_cast<const uint2 *>(e2_at(hf, y));
+                    }
+                    tmem_wait_ld();
+#pragma unroll
+                    for (int y = 0; y < 8; ++y) {
+                        const uint32_t off = frag_off(qr, lane, 64 * wh + 32 * hf, y >> 1) + 1024 * (y & 1);
+                        const float2 ea = unpack_bf16(ew[y].x), eb = unpack_bf16(ew[y].y), qv = unpack_bf16(qw[y]), kv = unpack_bf16(kw[y]);
+                        const float a0 = dqh[2 * y], a1 = dqh[2 * y + 1], c0 = dkh[2 * y], c1 = dkh[2 * y + 1];
+                        const float pq0 = qv.x * a0, pq1 = qv.y * a1, pk0 = kv.x * c0, pk1 = kv.y * c1;
+                        if (!retnet) *reinterpret_cast<float2 *>(e2_at(hf, y)) = make_float2(pq0 - pk0, pq1 - pk1);
+                        if ((y & 1) == 0) { sq0 += pq0 + pq1; sk0 += pk0 + pk1; } else { sq1 += pq0 + pq1; sk1 += pk0 + pk1; }
+                        *reinterpret_cast<uint32_t *>(qk + off) = pack_bf16(ea.x * a0, eb.x * a1);                // dq = scale Gq 2^b dqh   (over qh, for the store)
+                        *reinterpret_cast<uint32_t *>(qk + TILE_BF16 + off) = pack_bf16(ea.y * c0, eb.y * c1);    // dk = Gk 2^-b dkh
+                    }
                 }
-                if (wh == 1) up[row] = run + Rcur[row] + Rcur[D + row];
-                const float sq = warp_transpose_sum(dqh, lane);
-                const float sk = warp_transpose_sum(dkh, lane);
-                red[warp * 32 + lane] = sq;
-                red[8 * 32 + warp * 32 + lane] = sk;
+#pragma unroll
+                for (int o = 1; o < 4; o <<= 1) {      // a token's features: four lanes, two column halves
+                    sq0 += __shfl_xor_sync(0xffffffffu, sq0, o); sq1 += __shfl_xor_sync(0xffffffffu, sq1, o);
+                    sk0 += __shfl_xor_sync(0xffffffffu, sk0, o); sk1 += __shfl_xor_sync(0xffffffffu, sk1, o);
+                }
+                if ((lane & 3) == 0) {
+                    red[wh * C + tr] = sq0;
+                    red[wh * C + tr + 8] = sq1;
+                    red[(2 + wh) * C + tr] = sk0;
+                    red[(2 + wh) * C + tr + 8] = sk1;
+                }
             }
             fence_proxy_async();
             tc_fence_before();
-            mbar_arrive(bar(OUT1));
+            warp_arrive(bar(OUT1), lane);
 
-            // ---- dV^T -> dv tile; dlog_decay tile; gate products ----
+            // ---- dV -> dv tile; dlog_decay tile; gate products ----
             wait(BAR_M2, par);
             tc_fence_after();
             {
-                float dvt[32];
-                tmem_ld32(tmem + lane_base + COL_DV + 32 * wh, dvt);
+                float v[32];
+                tmem_ld_frag8(tmem + lane_base + COL_DV + 64 * wh, v);
                 tmem_wait_ld();
-                const uint32_t dhalf = (uint32_t)(row >> 6) * HALF_BF16, dchunk = (uint32_t)(row & 63) >> 3, dbyte = (row & 7) * 2;
+                tc_fence_before();
+                warp_arrive(bar(DVREAD), lane);
 #pragma unroll
-                for (int ii = 0; ii < 32; ++ii)
-                    *reinterpret_cast<__nv_bfloat16 *>(sm + OFF_A + dhalf + swz(32 * wh + ii, dchunk) + dbyte) =
-                        __float2bfloat16_rn(dvt[ii]);
+                for (int i = 0; i < 8; ++i) {
+                    const uint32_t off = frag_off(qr, lane, 64 * wh, i);
+                    *reinterpret_cast<uint32_t *>(sm + OFF_A + off) = pack_bf16(v[4 * i], v[4 * i + 1]);
+                    *reinterpret_cast<uint32_t *>(sm + OFF_A + off + 1024) = pack_bf16(v[4 * i + 2], v[4 * i + 3]);
+                }
             }
-            named_bar_sync(1, NCOMPUTE);                // up, red and the R partials are complete
-            {   // log-decay gradient: in-chunk suffix sum + what flows in from the right of the chunk
-                const float offs = wh == 1 ? Rcur[row] + Rcur[D + row] : up[row];
-                float *dgt = reinterpret_cast<float *>(sm + OFF_DZ);
+            float *dgt = reinterpret_cast<float *>(sm + OFF_DZ);
+            named_bar_sync(1, NCOMPUTE);                // qh dqh - kh dkh, red and the R partials are complete
+            if (!retnet) {   // log-decay gradient (a constant decay has none): in-chunk suffix sum + what flows in from the right.
+                // Warp g owns tokens 8g .. 8g+7, a lane four features (16-byte accesses, whole rows a warp); a group's total
+                // goes in the place of the group's first row (each lane has read what it writes over)
+                const float *Rcur = Rs + (n & 1) * 2 * D;
+                float4 sfx[8], run = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-                for (int ii = 0; ii < 32; ++ii) dgt[(32 * wh + ii) * D + row] = sfx[ii] + offs;
+                for (int ii = 0; ii < 8; ++ii) sfx[ii] = *reinterpret_cast<const float4 *>(sm + OFF_E2 + e2_off(8 * warp + ii, lane));
+#pragma unroll
+                for (int ii = 7; ii >= 0; --ii) {
+                    run.x += sfx[ii].x; run.y += sfx[ii].y; run.z += sfx[ii].z; run.w += sfx[ii].w;
+                    sfx[ii] = run;
+                }
+                *reinterpret_cast<float4 *>(sm + OFF_E2 + e2_off(8 * warp, lane)) = run;
+                named_bar_sync(1, NCOMPUTE);
+                const float4 ra = *reinterpret_cast<const float4 *>(Rcur + 4 * lane), rb = *reinterpret_cast<const float4 *>(Rcur + D + 4 * lane);
+                float4 offs = make_float4(ra.x + rb.x, ra.y + rb.y, ra.z + rb.z, ra.w + rb.w);
+#pragma unroll
+                for (int g = 7; g > 0; --g) {
+                    const float4 a = g > warp ? *reinterpret_cast<const float4 *>(sm + OFF_E2 + e2_off(8 * g, lane)) : make_float4(0.f, 0.f, 0.f, 0.f);
+                    offs.x += a.x; offs.y += a.y; offs.z += a.z; offs.w += a.w;
+                }
+#pragma unroll
+                for (int ii = 0; ii < 8; ++ii)
+                    *reinterpret_cast<float4 *>(dgt + (8 * warp + ii) * D + 4 * lane) =
+                        make_float4(sfx[ii].x + offs.x, sfx[ii].y + offs.y, sfx[ii].z + offs.z, sfx[ii].w + offs.w);
             }
             if (tid < C) {   // Gq*dGq and Gk*dGk of token tid: sum over the four key-dimension quarters
                 const int cn = min(C, p.T - t0);
                 if (tid < cn) {
-                    const int w0 = 4 * (tid >> 5), l = tid & 31;
-                    float sq = 0.f, sk = 0.f;
-#pragma unroll
-                    for (int w = 0; w < 4; ++w) {
-                        sq += red[(w0 + w) * 32 + l];
-                        sk += red[8 * 32 + (w0 + w) * 32 + l];
-                    }
+                    const float sq = red[tid] + red[C + tid], sk = red[2 * C + tid] + red[3 * C + tid];
                     p.pq[(tokb + t0 + tid) * p.H + h] = sq;
                     p.pk[(tokb + t0 + tid) * p.H + h] = sk;
                 }
             }
             fence_proxy_async();
             tc_fence_before();
-            mbar_arrive(bar(OUT2));
+            warp_arrive(bar(OUT2), lane);
         }
 
         if (p.dh0) {   // dS_0, fp32 (the last chunk's MMAs were waited for above)
