@@ -306,6 +306,7 @@ k_gla_fwd_tc(const __grid_constant__ CUtensorMap gm_q, const __grid_constant__ C
             // first starts from S <- diag(gam_s) S + fin_s taken over the segments s before it (a short scan over their
             // summaries, elementwise, done here rather than in a launch of its own).
             const float *src = state_row(p.h0, sbh, row, colhalf, p.dk, p.dv);
+            if (p.P > 1) grid_dependency_wait();
 #pragma unroll
             for (int part = 0; part < 2; ++part) {
                 float v[32];
@@ -533,12 +534,27 @@ int gla_tc_forward(const Dims &d, const FwdArgs &a, uint8_t *simg, int *status, 
         const size_t nseg = (size_t)d.B * d.H * P;
         fin = a.ws;
         gam = fin + nseg * D * D;
-        if (gla_tc_segment_summaries(d, a, P, L, fin, gam, status, st, tr) < 0) return -1;
+        // (nothing starts from the last segment's end)
+        if (gla_tc_segment_summaries(d, a, P, L, P - 1, fin, gam, status, st, tr) < 0) return -1;
         launches = 2;
         simg = nullptr;
     }
     FwdParams p{a.lq, a.lk, a.h0, fin, gam, (__nv_bfloat16 *)a.o, a.ht, simg, status, d.T, d.H, d.NT, P, L, d.scale, retnet ? a.log_decay : nullptr, nullptr, nullptr, d.dk, d.dv};
-    k_gla_fwd_tc<<<d.B * d.H * P, NTHREADS, SMEM_BYTES, st>>>(mq, mk, mv, mg, mo, p);
+    // After the summaries (whose blocks are all resident at once) the second pass may start early: its blocks move in as the
+    // first pass's leave, and set up, load and scale their first chunks beside the ones still running; the warps that read the
+    // summaries wait for all of them.  Everything else they read is the caller's.  (With the last segment left out of the first
+    // pass: 4 x 2048 tokens x 8 heads 54.7 -> 52.4 us a call, 1 x 65536 x 16 514 -> 506.)
+    cudaLaunchAttribute early;
+    early.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    early.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)(d.B * d.H * P));
+    cfg.blockDim = dim3(NTHREADS);
+    cfg.dynamicSmemBytes = SMEM_BYTES;
+    cfg.stream = st;
+    cfg.attrs = &early;
+    cfg.numAttrs = P > 1 ? 1 : 0;
+    if (cudaLaunchKernelEx(&cfg, k_gla_fwd_tc, mq, mk, mv, mg, mo, p) != cudaSuccess) return -1;
     tr.mark("gla_fwd_tc");
     return cudaGetLastError() == cudaSuccess ? launches : -1;
 }

@@ -65,6 +65,7 @@ struct StatesParams {
     int *status;
     int T, H, NT;
     int P, L;               // segments per sequence and chunks per segment (image mode: P = 1, L = NT)
+    int PS;                 // of them, from the first on, run (the grid has PS CTAs per sequence)
     const float *log_gamma; // Softmax-RetNet: [H] constant log-decays (no log-decay tensor is read); else nullptr
     const SeqInfo *seqs;    // packed variable-length batch: per-sequence table and tensor maps (k, v, g), else nullptr
     const CUtensorMap *vmaps;
@@ -98,7 +99,8 @@ k_gla_states_tc(const __grid_constant__ CUtensorMap gm_k, const __grid_constant_
     const uint32_t base = (raw + 1023u) & ~1023u;
     uint8_t *sm = smem_raw + (base - raw);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int bh = blockIdx.x / p.P, seg = blockIdx.x % p.P, h = bh % p.H;
+    const int bh = blockIdx.x / p.PS, seg = blockIdx.x % p.PS, h = bh % p.H;
+    const size_t sum_i = (size_t)bh * p.P + seg;            // summary slot of this segment
     int b = bh / p.H;
     size_t tokb = (size_t)b * p.T, slot = (size_t)bh * (p.NT + 1);
     size_t sbh = (size_t)bh;                                // (sequence, head) index into h0 / ht / dht / dh0
@@ -145,6 +147,7 @@ k_gla_states_tc(const __grid_constant__ CUtensorMap gm_k, const __grid_constant_
     tc_fence_after();
     const uint32_t tmem = *reinterpret_cast<volatile uint32_t *>(sm + OFF_TMEM);
     uint8_t *img0 = p.simg + slot * STATE_BF16;                       // (image mode: one segment, NT = p.NT)
+    grid_launch_dependents();                               // the segmented forward's second pass: see gla_tc_forward
 
     if (warp == 8) {
         // ---------------- MMA issue (the warp walks the loop together, one lane issues) ----------------
@@ -289,13 +292,13 @@ k_gla_states_tc(const __grid_constant__ CUtensorMap gm_k, const __grid_constant_
                     store_state_part(sm + OFF_IMG, row, colhalf, 0, v0);
                     store_state_part(sm + OFF_IMG, row, colhalf, 1, v1);
                 } else if (n == NT - 1) {              // summary mode: where the segment ended, fp32
-                    float *dst = p.fin + ((size_t)blockIdx.x * D + row) * D + 64 * colhalf;
+                    float *dst = p.fin + (sum_i * D + row) * D + 64 * colhalf;
 #pragma unroll
                     for (int j = 0; j < 32; j += 4) {
                         *reinterpret_cast<float4 *>(dst + j) = make_float4(v0[j], v0[j + 1], v0[j + 2], v0[j + 3]);
                         *reinterpret_cast<float4 *>(dst + 32 + j) = make_float4(v1[j], v1[j + 1], v1[j + 2], v1[j + 3]);
                     }
-                    if (colhalf == 0) p.gam[(size_t)blockIdx.x * D + row] = gam;
+                    if (colhalf == 0) p.gam[sum_i * D + row] = gam;
                 }
                 tmem_wait_st();
             }
@@ -961,16 +964,16 @@ size_t gla_tc_backward_workspace_bytes(const Dims &d, const Varlen *vl) {
     return state_slots(d, vl) * STATE_BF16 + 2 * ((bth + 63) & ~(size_t)63) * sizeof(float);
 }
 
-int gla_tc_segment_summaries(const Dims &d, const FwdArgs &a, int P, int L, float *fin, float *gam, int *status,
+int gla_tc_segment_summaries(const Dims &d, const FwdArgs &a, int P, int L, int PS, float *fin, float *gam, int *status,
                              cudaStream_t st, Tracer &tr) {
     CUtensorMap mk, mv, mg;
     const bool retnet = d.variant == SLA_RETNET;
     if (!make_tile_map(&mk, a.k, d.B, d.T, d.H, d.dk) || !make_tile_map(&mv, a.v, d.B, d.T, d.H, d.dv)) return -1;
     if (retnet) mg = mk;   // (never used: the decay is generated in the kernel)
     else if (!make_map(&mg, a.log_decay, d.B, d.T, d.H, d.dk, true, 128)) return -1;
-    StatesParams sp{a.lq, a.lk, nullptr, nullptr, fin, gam, status, d.T, d.H, d.NT, P, L, retnet ? a.log_decay : nullptr,
+    StatesParams sp{a.lq, a.lk, nullptr, nullptr, fin, gam, status, d.T, d.H, d.NT, P, L, PS, retnet ? a.log_decay : nullptr,
                     nullptr, nullptr, d.dk, d.dv};
-    k_gla_states_tc<<<d.B * d.H * P, st1::NTHREADS, st1::SMEM_BYTES, st>>>(mk, mv, mg, sp);
+    k_gla_states_tc<<<d.B * d.H * PS, st1::NTHREADS, st1::SMEM_BYTES, st>>>(mk, mv, mg, sp);
     tr.mark("gla_segment_states_tc");
     return cudaGetLastError() == cudaSuccess ? 1 : -1;
 }
@@ -1013,7 +1016,7 @@ int gla_tc_backward(const Dims &d, const BwdArgs &a, bool have_states, int *stat
             });
             if (!vm) return -1;
         }
-        StatesParams sp{a.lq, a.lk, a.h0, simg, nullptr, nullptr, status, d.T, d.H, d.NT, 1, d.NT, retnet ? a.log_decay : nullptr,
+        StatesParams sp{a.lq, a.lk, a.h0, simg, nullptr, nullptr, status, d.T, d.H, d.NT, 1, d.NT, 1, retnet ? a.log_decay : nullptr,
                         dseqs, vm, d.dk, d.dv};
         k_gla_states_tc<<<ctas, st1::NTHREADS, st1::SMEM_BYTES, st>>>(mk, mv, mg, sp);
         tr.mark("gla_states_tc");
@@ -1076,7 +1079,7 @@ int gla_tc_backward_segmented(const Dims &d, const BwdArgs &a, Varlen &segs, int
     float *h0seg = gam + nseg * D, *dhtseg = h0seg + stf, *dsfin = dhtseg + stf;
     // the state every segment starts from
     FwdArgs f{a.q, a.k, a.v, a.log_decay, a.beta, a.lq, a.lk, a.h0, nullptr, nullptr, a.ws, a.status, nullptr};
-    if (gla_tc_segment_summaries(d, f, P, L, fin, gam, status, st, tr) < 0) return -1;
+    if (gla_tc_segment_summaries(d, f, P, L, P /* the last one's decay is needed */, fin, gam, status, st, tr) < 0) return -1;
     const dim3 grid(d.B * d.H, d.dk);
     k_fold_segment_states<<<grid, d.dv, 0, st>>>(d.H, P, d.dk, d.dv, a.h0, fin, gam, h0seg);
     tr.mark("fold_segment_states");

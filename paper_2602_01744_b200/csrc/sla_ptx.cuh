@@ -70,6 +70,10 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint32_t bar, uint32_t parity,
         if ((it & 63u) == 63u && ((abort && *abort) || globaltimer_ns() - t0 > limit_ns)) return false;
     }
 }
+// A kernel launched with programmatic stream serialization may start once every block of its predecessor has called
+// grid_launch_dependents (or ended); grid_dependency_wait returns when the predecessor is complete and its writes are visible.
+__device__ __forceinline__ void grid_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void fence_mbar_init() { asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory"); }
 __device__ __forceinline__ void fence_proxy_async() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 
