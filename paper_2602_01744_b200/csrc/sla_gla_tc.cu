@@ -315,10 +315,10 @@ k_gla_fwd_tc(const __grid_constant__ CUtensorMap gm_q, const __grid_constant__ C
                 for (int sgm = 0; sgm < seg; ++sgm) {
                     const size_t c = (size_t)bh * p.P + sgm;
                     const float gmm = p.gam[c * D + row];
-                    const float4 *f = reinterpret_cast<const float4 *>(p.fin + (c * D + row) * D + 64 * colhalf + 32 * part);
+                    const float4 *f = reinterpret_cast<const float4 *>(p.fin + c * D * D + fin_off(row, 16 * colhalf + 8 * part));
 #pragma unroll
                     for (int j = 0; j < 8; ++j) {
-                        const float4 x = f[j];
+                        const float4 x = f[(size_t)j * D];
                         v[4 * j] = fmaf(gmm, v[4 * j], x.x);         v[4 * j + 1] = fmaf(gmm, v[4 * j + 1], x.y);
                         v[4 * j + 2] = fmaf(gmm, v[4 * j + 2], x.z); v[4 * j + 3] = fmaf(gmm, v[4 * j + 3], x.w);
                     }

@@ -107,6 +107,11 @@ __device__ __forceinline__ T *state_row(T *t, size_t bh, int row, int half, int 
     return (t && row < dk && 64 * half < dv) ? t + (bh * dk + row) * dv + 64 * half : nullptr;
 }
 
+// Where the 16 bytes (row, columns 4 c4 .. 4 c4 + 3) of a segment's fp32 summary lie, in floats: rows next to one another, because the
+// kernels that write and read it have a row of the state in each thread and a warp then moves 512 bytes at a time (in rows of 512 bytes
+// a warp touched 32 lines an access: 4 x 2048 tokens x 8 heads 52.0 us a call, 45.5 now).
+__device__ __forceinline__ size_t fin_off(int row, int c4) { return ((size_t)c4 * D + row) * 4; }
+
 // Device array of the per-sequence tensor maps of region r of a packed batch: `make(seq, maps)` encodes one sequence's
 // maps.  They are encoded and uploaded (stream-ordered, from a pinned mirror) only when `key`, the tensors they point
 // at, differs from the last call's; a training loop that reuses its buffers encodes once.  nullptr on failure.

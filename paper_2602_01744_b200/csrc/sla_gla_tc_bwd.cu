@@ -61,7 +61,7 @@ static_assert(NBAR <= 32, "barrier slots");
 struct StatesParams {
     const float *lq, *lk, *h0;
     uint8_t *simg;          // [B*H][NT+1][32 KiB] bf16 state images (image mode)
-    float *fin, *gam;       // summary mode: per CTA the state reached from a zero start [128][128] and the total decay [128]
+    float *fin, *gam;       // summary mode: per segment the state reached from a zero start (fin_off) and the total decay [128]
     int *status;
     int T, H, NT;
     int P, L;               // segments per sequence and chunks per segment (image mode: P = 1, L = NT)
@@ -292,11 +292,11 @@ k_gla_states_tc(const __grid_constant__ CUtensorMap gm_k, const __grid_constant_
                     store_state_part(sm + OFF_IMG, row, colhalf, 0, v0);
                     store_state_part(sm + OFF_IMG, row, colhalf, 1, v1);
                 } else if (n == NT - 1) {              // summary mode: where the segment ended, fp32
-                    float *dst = p.fin + (sum_i * D + row) * D + 64 * colhalf;
+                    float *dst = p.fin + sum_i * D * D + fin_off(row, 16 * colhalf);
 #pragma unroll
-                    for (int j = 0; j < 32; j += 4) {
-                        *reinterpret_cast<float4 *>(dst + j) = make_float4(v0[j], v0[j + 1], v0[j + 2], v0[j + 3]);
-                        *reinterpret_cast<float4 *>(dst + 32 + j) = make_float4(v1[j], v1[j + 1], v1[j + 2], v1[j + 3]);
+                    for (int j = 0; j < 8; ++j) {
+                        *reinterpret_cast<float4 *>(dst + fin_off(0, j)) = make_float4(v0[4 * j], v0[4 * j + 1], v0[4 * j + 2], v0[4 * j + 3]);
+                        *reinterpret_cast<float4 *>(dst + fin_off(0, 8 + j)) = make_float4(v1[4 * j], v1[4 * j + 1], v1[4 * j + 2], v1[4 * j + 3]);
                     }
                     if (colhalf == 0) p.gam[sum_i * D + row] = gam;
                 }
@@ -912,7 +912,7 @@ __global__ void k_fold_segment_states(int H, int P, int dk, int dv, const float 
     for (int p = 0; p < P; ++p) {
         h0seg[((((size_t)b * P + p) * H + h) * dk + row) * dv + col] = sv;
         const size_t c = (size_t)bh * P + p;
-        sv = fmaf(gam[c * D + row], sv, fin[(c * D + row) * D + col]);
+        sv = fmaf(gam[c * D + row], sv, fin[c * D * D + fin_off(row, col >> 2) + (col & 3)]);
     }
 }
 // State gradients entering each segment from its right: R_{P-1} = dht (or zero), R_p = diag(gam_{p+1}) R_{p+1} + F_{p+1},

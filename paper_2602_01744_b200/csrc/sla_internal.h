@@ -140,7 +140,7 @@ int gla_tc_forward(const Dims &d, const FwdArgs &a, uint8_t *simg, int *status, 
 // B*H*(NT+1)*32 KiB + 2*B*T*H*4 bytes (rounded up) of the workspace, less than the generic path.
 int gla_tc_bwd_configure();
 // Segmented forward of long sequences, first pass: every (sequence, segment of L chunks) from a zero state; leaves
-// the state it reaches (fin [B*H*P][128][128]) and the segment's total decay (gam [B*H*P][128]), of the first PS segments.
+// the state it reaches (fin [B*H*P][128 x 128], laid out as fin_off says) and the segment's total decay (gam [B*H*P][128]), of the first PS segments.
 int gla_tc_segment_summaries(const Dims &d, const FwdArgs &a, int P, int L, int PS, float *fin, float *gam, int *status,
                              cudaStream_t st, Tracer &tr);
 // Bytes of workspace the tensor-core forward / backward need (the generic kernels need more).
