@@ -310,8 +310,7 @@ k_gla_fwd_tc(const __grid_constant__ CUtensorMap gm_q, const __grid_constant__ C
 #pragma unroll
             for (int part = 0; part < 2; ++part) {
                 float v[32];
-#pragma unroll
-                for (int j = 0; j < 32; ++j) v[j] = src ? src[32 * part + j] : 0.f;
+                load_state32(src ? src + 32 * part : nullptr, v);
                 for (int sgm = 0; sgm < seg; ++sgm) {
                     const size_t c = (size_t)bh * p.P + sgm;
                     const float gmm = p.gam[c * D + row];
@@ -424,16 +423,24 @@ k_gla_fwd_tc(const __grid_constant__ CUtensorMap gm_q, const __grid_constant__ C
         }
 
         if (p.ht && seg == p.P - 1) {   // final state, fp32 (each thread reads back what it wrote in the last rescale)
-            float *dst = state_row(p.ht, sbh, row, colhalf, p.dk, p.dv);
+            // through shared memory (every product of the CTA has been read out, the q, k buffers are free), so that a warp writes
+            // whole rows (4 x 2048 tokens x 8 heads: 46.4 -> 43.6 us a call)
+            const uint32_t R = OFF_QK + row * (D * 4);
 #pragma unroll
             for (int part = 0; part < 2; ++part) {
                 float v[32];
                 tmem_ld32(tmem + lane_base + COL_S + 64 * colhalf + 32 * part, v);
                 tmem_wait_ld();
 #pragma unroll
-                for (int j = 0; j < 32; j += 4)
-                    if (dst) *reinterpret_cast<float4 *>(dst + 32 * part + j) = make_float4(v[j], v[j + 1], v[j + 2], v[j + 3]);
+                for (int j = 0; j < 8; ++j)
+                    *reinterpret_cast<float4 *>(sm + R + (((16 * colhalf + 8 * part + j) ^ lane) << 4)) =
+                        make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
             }
+            named_bar_sync(1, NCOMPUTE);
+            float *dst = p.ht + sbh * p.dk * p.dv + 4 * lane;
+            if (4 * lane < p.dv)
+                for (int r = warp; r < p.dk; r += NCOMPUTE / 32)
+                    *reinterpret_cast<float4 *>(dst + (size_t)r * p.dv) = *reinterpret_cast<const float4 *>(sm + OFF_QK + r * (D * 4) + ((lane ^ (r & 31)) << 4));
         }
     }
     if (failed) atomicOr(p.status, STATUS_TIMEOUT);

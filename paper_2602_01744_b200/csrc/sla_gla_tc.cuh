@@ -107,6 +107,22 @@ __device__ __forceinline__ T *state_row(T *t, size_t bh, int row, int half, int 
     return (t && row < dk && 64 * half < dv) ? t + (bh * dk + row) * dv + 64 * half : nullptr;
 }
 
+// 32 floats of a caller's state row (any 4-byte alignment), zeros if there is none.  Lanes hold different rows, so an access costs
+// a line a lane whatever its width: 16 bytes at a time where the row allows it (4 x 2048 tokens x 8 heads from a given state: 55.5 us a
+// call a word at a time, 46 so, with the final state written as below).
+__device__ __forceinline__ void load_state32(const float *src, float (&v)[32]) {
+    if (src && reinterpret_cast<uintptr_t>(src) % 16 == 0) {
+#pragma unroll
+        for (int j = 0; j < 32; j += 4) {
+            const float4 x = *reinterpret_cast<const float4 *>(src + j);
+            v[j] = x.x; v[j + 1] = x.y; v[j + 2] = x.z; v[j + 3] = x.w;
+        }
+    } else {
+#pragma unroll
+        for (int j = 0; j < 32; ++j) v[j] = src ? src[j] : 0.f;
+    }
+}
+
 // Where the 16 bytes (row, columns 4 c4 .. 4 c4 + 3) of a segment's fp32 summary lie, in floats: rows next to one another, because the
 // kernels that write and read it have a row of the state in each thread and a warp then moves 512 bytes at a time (in rows of 512 bytes
 // a warp touched 32 lines an access: 4 x 2048 tokens x 8 heads 52.0 us a call, 45.5 now).

@@ -245,8 +245,7 @@ k_gla_states_tc(const __grid_constant__ CUtensorMap gm_k, const __grid_constant_
 #pragma unroll
             for (int part = 0; part < 2; ++part) {
                 float v[32];
-#pragma unroll
-                for (int j = 0; j < 32; ++j) v[j] = src ? src[32 * part + j] : 0.f;
+                load_state32(src ? src + 32 * part : nullptr, v);
                 tmem_st32(tmem + lane_base + 64 * colhalf + 32 * part, v);
                 if (images) store_state_part(img0, row, colhalf, part, v);
             }
@@ -653,8 +652,7 @@ k_gla_bwd_tc(const __grid_constant__ CUtensorMap gm_q, const __grid_constant__ C
 #pragma unroll
             for (int part = 0; part < 2; ++part) {
                 float v[32];
-#pragma unroll
-                for (int j = 0; j < 32; ++j) v[j] = src ? src[32 * part + j] : 0.f;
+                load_state32(src ? src + 32 * part : nullptr, v);
                 tmem_st32(tmem + lane_base + COL_DS + 64 * wh + 32 * part, v);
                 if (p.dht) rpart += rowdot_part(v, part);
             }
