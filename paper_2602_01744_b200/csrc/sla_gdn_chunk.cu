@@ -685,8 +685,7 @@ __device__ __forceinline__ void scan_item(int item, const CUtensorMap &gm_q, con
         float S[32];
         {
             const float *src = state_row(p.h0, s.sbh, row, sl, p.dk, p.dv);
-#pragma unroll
-            for (int j = 0; j < 32; ++j) S[j] = src ? src[32 * ch + j] : 0.f;
+            load_state32(src ? src + 32 * ch : nullptr, S);
         }
         store_slice(sm + OFF_S, row, ch, S);
         fence_proxy_async();
@@ -930,8 +929,7 @@ __device__ __forceinline__ void bscan_item(int item, const CUtensorMap &gm_q, co
         float S[32];                                   // dS of the state after the current chunk
         {
             const float *src = state_row(p.dht, s.sbh, row, sl, p.dk, p.dv);
-#pragma unroll
-            for (int j = 0; j < 32; ++j) S[j] = src ? src[32 * ch + j] : 0.f;
+            load_state32(src ? src + 32 * ch : nullptr, S);
         }
         float e = scalars(0)[SC_GAM * C + C - 1];
         for (int x = 0; x < NT; ++x) {

@@ -261,8 +261,7 @@ k_gdn_fwd_tc(const __grid_constant__ CUtensorMap gm_q, const __grid_constant__ C
 #pragma unroll
             for (int part = 0; part < 2; ++part) {
                 float v[32];
-#pragma unroll
-                for (int j = 0; j < 32; ++j) v[j] = src ? src[32 * part + j] : 0.f;
+                load_state32(src ? src + 32 * part : nullptr, v);
                 tmem_st32(tmem + lane_base + COL_S + 64 * colhalf + 32 * part, v);
 #pragma unroll
                 for (int c = 0; c < 4; ++c) {

@@ -428,11 +428,8 @@ k_gdn_bwd_tc(const __grid_constant__ CUtensorMap gm_q, const __grid_constant__ C
             float v0[32], v1[32];
             if (p.dht) wait(INIT_FULL, 0);
             const float *src = state_row(p.dht, sbh, row, ch, p.dk, p.dv);
-#pragma unroll
-            for (int j = 0; j < 32; ++j) {
-                v0[j] = src ? src[j] : 0.f;
-                v1[j] = src ? src[32 + j] : 0.f;
-            }
+            load_state32(src, v0);
+            load_state32(src ? src + 32 : nullptr, v1);
             tmem_st32(tmem + lane_base + R0 + 64 * ch, v0);
             tmem_st32(tmem + lane_base + R0 + 64 * ch + 32, v1);
             const float part = p.dht ? state_dot(v0, v1) : 0.f;
