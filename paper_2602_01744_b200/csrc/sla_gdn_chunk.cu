@@ -1524,13 +1524,28 @@ int chunk_sm_count() {
 
 }  // namespace
 
-// The chunk-parallel form needs records in memory and a grid-wide barrier; it pays from the number of chunks on at which
-// its shorter serial chain outweighs them.  Short, small batches stay on the kernels that need no workspace.
+// The chunk-parallel form needs records in memory and a grid-wide barrier; its serial chain is a seventh of the one-CTA kernels' (1.1
+// against 7 us a chunk of the longest sequence).  Above the line, one-CTA against chunk-parallel, 128-wide heads, B x T x H: forward
+// 1 x 1088 x 4 123 / 39 us, 4 x 512 x 16 64 / 39, 1 x 2048 x 4 223 / 57; training step 382 / 84, 221 / 106, 698 / 127.  Below it
+// (1 x 1024 x 4: 111 forward, 4 x 256 x 16: 35) stay the calls whose forward pass is promised to need no workspace, although the longer
+// ones of them would gain too.
 bool gdn_chunk_selected(const Dims &d, const Varlen *vl) {
     const bool packed = vl && vl->n_seq;
     const int longest = packed ? vl->seqs[0].NT : d.NT;          // (the table is kept longest sequence first)
     const long chunks = packed ? (vl->slots - vl->n_seq) * d.H : (long)d.B * d.H * d.NT;
     return longest > 16 || chunks > 256;
+}
+
+// A forward pass that keeps no records gains nothing from the chunk-parallel form where every sequence is short (up to 8 chunks) and
+// the sequences fill the SMs by themselves, to four fifths of a whole number of waves or more.  One-CTA against chunk-parallel:
+// 8 x 512 x 16 63.6 / 67.8 us, 18 x 512 x 16 127.4 / 131.7, 64 x 128 x 16 146 / 162; but 12 x 512 x 16 (two waves, 65 % filled)
+// 123.5 / 96.1 and 8 x 1024 x 16 121.2 / 110.9.
+bool gdn_chunk_forward_selected(const Dims &d, const Varlen *vl) {
+    if (!gdn_chunk_selected(d, vl)) return false;
+    const bool packed = vl && vl->n_seq;
+    const int longest = packed ? vl->seqs[0].NT : d.NT;
+    const long seqs = packed ? (long)vl->n_seq * d.H : (long)d.B * d.H, sms = chunk_sm_count(), waves = (seqs + sms - 1) / sms;
+    return longest > 8 || 5 * seqs < 4 * waves * sms;
 }
 
 int gdn_chunk_configure() {

@@ -169,6 +169,7 @@ int gdn_tc_backward(const Dims &d, const BwdArgs &a, bool have_records, int *sta
 // Chunk-parallel form of the same (sla_gdn_chunk.cu): per-chunk records prepared and consumed in parallel, two products a
 // chunk on the serial chain.  gdn_tc_forward / gdn_tc_backward take it where gdn_chunk_selected says so.
 bool gdn_chunk_selected(const Dims &d, const Varlen *vl);
+bool gdn_chunk_forward_selected(const Dims &d, const Varlen *vl);             // ... for a forward pass that keeps no records
 int gdn_chunk_configure();
 size_t gdn_chunk_forward_workspace_bytes(const Dims &d, const Varlen *vl);     // records of a forward that saves nothing
 size_t gdn_chunk_record_bytes(const Dims &d, const Varlen *vl);                // records of a training step

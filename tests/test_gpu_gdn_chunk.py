@@ -15,7 +15,8 @@ pytestmark = pytest.mark.gpu
 # head widths; the batch that just passes 256 chunks
 @pytest.mark.parametrize("B,T,H,dk,dv,with_h0", [(1, 1025, 1, 128, 128, True), (1, 1151, 3, 128, 128, False), (20, 64, 16, 128, 128, True),
                                                  (10, 65, 16, 128, 128, True), (2, 1090, 2, 64, 64, True), (1, 1100, 5, 64, 128, True),
-                                                 (1, 1100, 5, 128, 64, False), (1, 1280, 16, 64, 64, True)])
+                                                 (1, 1100, 5, 128, 64, False), (1, 1280, 16, 64, 64, True),
+                                                 (9, 128, 16, 128, 128, True)])   # the last: forward alone on the one-CTA kernel
 def test_chunk_parallel_step_matches_the_oracle(B, T, H, dk, dv, with_h0):
     cfg = small(CONFIGS["C4"], B=B, T=T, H=H, d_k=dk, d_v=dv, seed=1500 + T + H)
     x = make_inputs(cfg, with_dO=True, with_h0=with_h0)
