@@ -107,19 +107,14 @@ __device__ __forceinline__ T *state_row(T *t, size_t bh, int row, int half, int 
     return (t && row < dk && 64 * half < dv) ? t + (bh * dk + row) * dv + 64 * half : nullptr;
 }
 
-// 32 floats of a caller's state row (any 4-byte alignment), zeros if there is none.  Lanes hold different rows, so an access costs
-// a line a lane whatever its width: 16 bytes at a time where the row allows it (4 x 2048 tokens x 8 heads from a given state: 55.5 us a
-// call a word at a time, 46 so, with the final state written as below).
+// 32 floats of a caller's state row (state tensors are 16-byte aligned), zeros if there is none.  Lanes hold different rows, so an
+// access costs a line a lane whatever its width (4 x 2048 tokens x 8 heads from a given state: 55.5 us a call a word at a time, 46 in
+// 16-byte pieces, with the final state written by rows).
 __device__ __forceinline__ void load_state32(const float *src, float (&v)[32]) {
-    if (src && reinterpret_cast<uintptr_t>(src) % 16 == 0) {
 #pragma unroll
-        for (int j = 0; j < 32; j += 4) {
-            const float4 x = *reinterpret_cast<const float4 *>(src + j);
-            v[j] = x.x; v[j + 1] = x.y; v[j + 2] = x.z; v[j + 3] = x.w;
-        }
-    } else {
-#pragma unroll
-        for (int j = 0; j < 32; ++j) v[j] = src ? src[j] : 0.f;
+    for (int j = 0; j < 32; j += 4) {
+        const float4 x = src ? *reinterpret_cast<const float4 *>(src + j) : make_float4(0.f, 0.f, 0.f, 0.f);
+        v[j] = x.x; v[j + 1] = x.y; v[j + 2] = x.z; v[j + 3] = x.w;
     }
 }
 

@@ -15,8 +15,7 @@ pytestmark = pytest.mark.gpu
 # head widths; the batch that just passes 256 chunks
 @pytest.mark.parametrize("B,T,H,dk,dv,with_h0", [(1, 1025, 1, 128, 128, True), (1, 1151, 3, 128, 128, False), (20, 64, 16, 128, 128, True),
                                                  (10, 65, 16, 128, 128, True), (2, 1090, 2, 64, 64, True), (1, 1100, 5, 64, 128, True),
-                                                 (1, 1100, 5, 128, 64, False), (1, 1280, 16, 64, 64, True),
-                                                 (9, 128, 16, 128, 128, True)])   # the last: forward alone on the one-CTA kernel
+                                                 (1, 1100, 5, 128, 64, False), (1, 1280, 16, 64, 64, True)])
 def test_chunk_parallel_step_matches_the_oracle(B, T, H, dk, dv, with_h0):
     cfg = small(CONFIGS["C4"], B=B, T=T, H=H, d_k=dk, d_v=dv, seed=1500 + T + H)
     x = make_inputs(cfg, with_dO=True, with_h0=with_h0)
@@ -70,3 +69,20 @@ def test_chunk_parallel_packed_batch_gives_the_bits_of_its_sequences_alone():
         for n, t in g1.items():
             if t is not None:
                 assert torch.equal(t, g[n][:, a:b]), n
+
+
+# sequences of up to 8 chunks that fill the SMs (to four fifths of whole waves: 144 and 288 sequences; 128 of 9 chunks and 160 of 2 do not
+# count): a forward pass alone needs no workspace, a training step over the same tensors is chunk-parallel all the same
+@pytest.mark.parametrize("B,T,H,alone", [(9, 128, 16, True), (18, 512, 16, True), (8, 513, 16, False), (10, 128, 16, False)])
+def test_short_sequences_that_fill_the_chip_run_forward_without_workspace(B, T, H, alone):
+    cfg = small(CONFIGS["C4"], B=B, T=T, H=H, seed=1700 + B)
+    x = make_inputs(cfg, with_dO=True, with_h0=True)
+    xd = gu.to_dev(x)
+    o, ht, g, plan, ws, lf, lb = gu.gpu_training_step(cfg, xd, h0=xd["h0"])
+    assert (lf, lb) == (1, 2)
+    o2, ht2, plan2 = gu.gpu_forward(cfg, xd, h0=xd["h0"])
+    assert (plan2.forward_workspace_bytes == 0) == alone
+    oref, htref = gu.oracle_forward(cfg, x, h0=x["h0"])
+    pairs = {"o": (o, oref), "ht": (ht, htref), "o2": (o2, oref), "ht2": (ht2, htref)}
+    gu.assert_close({n: gu.rel_l2(a, r) for n, (a, r) in pairs.items()},
+                    {n: gu.row_err(a, r) for n, (a, r) in pairs.items()}, cfg.dtype, cfg)
