@@ -17,11 +17,14 @@
 //   Te = diag(e^{-b}) T      T2 = Te diag(beta Gk)      We = Te diag(beta Gam) K
 // and the forward's operands enter the tensor core as they stand in memory: no tile is rescaled, which leaves the two
 // serial products a chunk (We S and K^T Ue), one 64x64 and one 128x64 accumulator read between them.
-// Gradients (chain rule, X = dUe):  dR = Te^T X,  dA = tril(dO Ue^T),  P = strict_tril(dR Ue^T),  M = -beta Gam P,
+// Gradients (chain rule, X = dUe):  dR = Te^T X (T's unit diagonal in fp32, only the part below it as bf16),  dA = tril(dO Ue^T),  P = strict_tril(dR Ue^T),  M = -beta Gam P,
 //   aq = dO S^T + dA K               dq = fq aq               dv = beta Gk dR
 //   kd = Ue dZ^T + dA^T Qg + M^T K   Y = dR S^T + P K         dk = kd - beta Gam Y
 //   dbeta = Gk (dR.v) - Gam (k.Y)    db = Qg.aq - k.kd - beta Gam (k.Y)  (+ <dS', S'> on the last row)
 //   dlog_decay = suffix sum of db;   Gq dGq = Qg.aq,  Gk dGk = beta Gk (dR.v)
+// T's diagonal is one, but e^{-b} is not a bf16 number: with the whole of Te as the operand dR's dominant term was rounded once more than
+// in the one-CTA kernels, which hold T itself (dv 4.00e-3 against 3.60e-3 on feature-map keys, and 3.41e-3 with the diagonal in fp32,
+// which costs the training step 1 %: 4 x 4096 x 16 heads 512 -> 517 us).
 // Qg.aq and k.kd cancel in the suffix sum, so both sides take the same rounded Qg and the same rounded dA.
 #include "sla_gla_tc.cuh"
 
@@ -39,9 +42,10 @@ using namespace tc;
 struct Rec {
     uint32_t bytes, s, u, te, w, a, sc, t2, du, dz;
 };
-constexpr uint32_t SC_BYTES = 2048;                  // [5][64] floats, then at float 384 the 16 partial sums of <dS', S'>
-enum Sc { SC_FQ = 0, SC_BG, SC_FV, SC_GAM, SC_GK, SC_NARR };
+constexpr uint32_t SC_BYTES = 2048;                  // [6][64] floats, then at float 384 the 16 partial sums of <dS', S'>
+enum Sc { SC_FQ = 0, SC_BG, SC_FV, SC_GAM, SC_GK, SC_IG, SC_NARR };
 constexpr uint32_t SC_LOAD = SC_NARR * C * 4, SC_DOT = 384;
+static_assert(SC_NARR * C <= SC_DOT && (SC_DOT + 16) * 4 <= SC_BYTES, "scalars of a record");
 constexpr uint32_t PREP_BYTES = TILE_BF16 + HALF_BF16 + SC_BYTES + HALF_BF16;                        // We | A | scalars | T2
 constexpr Rec REC_INFER = {PREP_BYTES, 0, 0, 0, 0, TILE_BF16, TILE_BF16 + HALF_BF16, TILE_BF16 + HALF_BF16 + SC_BYTES, 0, 0};
 constexpr uint32_t R_U = STATE_BF16, R_TE = R_U + TILE_BF16, R_W = R_TE + HALF_BF16, R_A = R_W + TILE_BF16, R_SC = R_A + HALF_BF16,
@@ -134,7 +138,7 @@ constexpr int LDL = 68;                                 // row stride (floats) o
 constexpr uint32_t MAT = 64 * LDL * 4;                  // 17 KiB
 constexpr uint32_t OFF_Q = 0;                           // q tile -> fp32 T -> We staged
 constexpr uint32_t OFF_K = OFF_Q + MAT;
-constexpr uint32_t OFF_L = OFF_K + TILE_BF16;           // fp32 L -> Te | T2 (bf16)
+constexpr uint32_t OFF_L = OFF_K + TILE_BF16;           // fp32 L -> Te below its diagonal | T2 (bf16)
 constexpr uint32_t OFF_A = OFF_L + MAT;                 // bf16 A
 constexpr uint32_t OFF_TW = OFF_A + HALF_BF16;          // bf16 -Te diag(beta Gam)
 constexpr uint32_t OFF_X = OFF_TW + HALF_BF16;          // [4 warps][32][8] block-product scratch
@@ -225,8 +229,8 @@ __device__ __forceinline__ void prep_worker(const CUtensorMap &gm_q, const CUten
         if (tid >= C) {
             const int t = tid - C;
             const float b = s_b[t], beta = s_beta[t], gam = __expf(b);
-            const float fq = s_fq[t] * gam, bg = beta * gam, fv = beta * s_gk[t];
-            s_ig[t] = __expf(-b);
+            const float fq = s_fq[t] * gam, bg = beta * gam, fv = beta * s_gk[t], ig = __expf(-b);
+            s_ig[t] = ig;
             s_fq[t] = fq;
             s_bg[t] = bg;
             s_fv[t] = fv;
@@ -236,6 +240,7 @@ __device__ __forceinline__ void prep_worker(const CUtensorMap &gm_q, const CUten
             out[SC_FV * C + t] = fv;
             out[SC_GAM * C + t] = gam;
             out[SC_GK * C + t] = s_gk[t];
+            out[SC_IG * C + t] = ig;
             if (t == C - 1 && b < -SLA_MAX_CHUNK_DECAY) atomicOr(p.status, STATUS_RANGE);
         }
         sync();
@@ -338,7 +343,7 @@ __device__ __forceinline__ void prep_worker(const CUtensorMap &gm_q, const CUten
             }
         }
         sync();
-        {   // Te, T2 over L; -Te diag(beta Gam): thread = (row i, every other 16-byte chunk)
+        {   // Te without its diagonal, T2 over L; -Te diag(beta Gam): thread = (row i, every other 16-byte chunk)
             const int i = tid >> 1;
             const float gi = s_ig[i];
 #pragma unroll
@@ -364,6 +369,7 @@ __device__ __forceinline__ void prep_worker(const CUtensorMap &gm_q, const CUten
                 *reinterpret_cast<uint4 *>(sm + OFF_L + HALF_BF16 + swz(i, ch)) = t2;
                 *reinterpret_cast<uint4 *>(sm + OFF_TW + swz(i, ch)) = tn;
             }
+            if ((tid & 1) == ((i >> 3) & 1)) *reinterpret_cast<__nv_bfloat16 *>(sm + OFF_L + swz(i, i >> 3) + 2 * (i & 7)) = __float2bfloat16_rn(0.f);
         }
         fence_proxy_async();
         tc_fence_before();
@@ -1052,7 +1058,7 @@ __device__ __forceinline__ void bgrad_chunks(const CUtensorMap &gm_q, const CUte
             tc_fence_after();
             if (leader) {
 #pragma unroll
-                for (int kk = 0; kk < 4; ++kk) tc_mma_bf16(tmem + TM_R, mTE + kstep_mnmajor(kk), mX + kstep_mnmajor(kk), ID_DR, kk > 0);   // dR = Te^T X
+                for (int kk = 0; kk < 4; ++kk) tc_mma_bf16(tmem + TM_R, mTE + kstep_mnmajor(kk), mX + kstep_mnmajor(kk), ID_DR, kk > 0);   // dR = Te^T X, but for the diagonal
                 ksteps(wide, [&](int kk) {                        // dA = dO Ue^T
                     tc_mma_bf16(tmem + TM_A, kDO + kstep_kmajor(kk, HALF_BF16), kU + kstep_kmajor(kk, HALF_BF16), ID_64, kk > 0);
                 });
@@ -1105,11 +1111,13 @@ __device__ __forceinline__ void bgrad_chunks(const CUtensorMap &gm_q, const CUte
             const uint8_t *rec = p.rec + (size_t)slot * p.L.bytes;
             mbar_expect_tx(bar(FA), HALF_BF16 + TILE_BF16 + nh * (HALF_BF16 + HALF_BF16 + STATE_HALF + STATE_HALF));
             bulk_load(base + OFF_TE, rec + p.L.te, HALF_BF16, bar(FA));
-            bulk_load(base + OFF_X, rec + p.L.du, nh * HALF_BF16, bar(FA));
             tma_load_5d(base + OFF_DO, mp(s, 3, &gm_do), 0, n * C, 0, s.h, s.b, bar(FA));
             bulk_load(base + OFF_DZ, rec + p.L.dz, nh * STATE_HALF, bar(FA));
         };
-        auto load_a2 = [&](int slot) {
+        auto load_x = [&](int slot) {                              // (X: the compute warps read it, too)
+            if (leader) bulk_load(base + OFF_X, p.rec + (size_t)slot * p.L.bytes + p.L.du, nh * HALF_BF16, bar(FA));
+        };
+        auto load_a2 = [&](int slot) {                             // ... and what the later ones read as well
             if (!leader) return;
             const uint8_t *rec = p.rec + (size_t)slot * p.L.bytes;
             bulk_load(base + OFF_U, rec + p.L.u, nh * HALF_BF16, bar(FA));
@@ -1140,6 +1148,7 @@ __device__ __forceinline__ void bgrad_chunks(const CUtensorMap &gm_q, const CUte
         int slot = next_chunk(p, blockIdx.x, step, s);
         if (slot < p.slots) {
             load_a1(s, slot);
+            load_x(slot);
             load_a2(slot);
             load_v(s, slot, 0);
             load_k(s, slot);
@@ -1155,6 +1164,7 @@ __device__ __forceinline__ void bgrad_chunks(const CUtensorMap &gm_q, const CUte
                 const uint8_t *rec = p.rec + (size_t)sl2 * p.L.bytes;
                 bulk_prefetch_l2(rec + p.L.s, nh * STATE_HALF);
                 bulk_prefetch_l2(rec + p.L.u, nh * HALF_BF16);
+                bulk_prefetch_l2(rec + p.L.du, nh * HALF_BF16);
                 tma_prefetch_l2_5d(mp(sn, 2, &gm_v), 0, n2 * C, 0, sn.h, sn.b);
                 tma_prefetch_l2_5d(mp(sn, 0, &gm_q), 0, n2 * C, 0, sn.h, sn.b);
                 tma_prefetch_l2_5d(mp(sn, 1, &gm_k), 0, n2 * C, 0, sn.h, sn.b);
@@ -1165,6 +1175,7 @@ __device__ __forceinline__ void bgrad_chunks(const CUtensorMap &gm_q, const CUte
             wait(E1R, par);                        // dv staged over v
             if (failed) break;
             store(mp(s, 6, &gm_dv), OFF_V, s, n);
+            if (more) load_x(sl2);
             wait(C2, par);
             if (failed) break;
             if (more) load_a2(sl2);
@@ -1227,12 +1238,15 @@ __device__ __forceinline__ void bgrad_chunks(const CUtensorMap &gm_q, const CUte
                 *reinterpret_cast<uint32_t *>(sm + OFF_Q + off + 1024) = pack_bf16(fq1 * y1.x, fq1 * y1.y);
             }
             read_tile(OFF_V, tw);
+            uint32_t xw[16];                           // X: T's unit diagonal is added to dR here, in fp32
+            wait(FA, par);
+            if (ch < nh) read_tile(OFF_X, xw);
             wait(C1, par);
             tc_fence_after();
             {
                 float a0 = 0.f, a1 = 0.f;
                 if (ch < nh) {
-                    const float fv0 = sc[SC_FV * C + r], fv1 = sc[SC_FV * C + r + 8];
+                    const float fv0 = sc[SC_FV * C + r], fv1 = sc[SC_FV * C + r + 8], ig0 = sc[SC_IG * C + r], ig1 = sc[SC_IG * C + r + 8];
                     float v[32];
                     tmem_ld_frag8(tq + TM_R + 64 * ch, v);
                     tmem_wait_ld();
@@ -1240,7 +1254,9 @@ __device__ __forceinline__ void bgrad_chunks(const CUtensorMap &gm_q, const CUte
                     for (int i = 0; i < 8; ++i) {
                         const uint32_t off = frag_off(qr, lane, 64 * ch, i);
                         uint32_t *x0 = reinterpret_cast<uint32_t *>(sm + OFF_V + off), *x1 = reinterpret_cast<uint32_t *>(sm + OFF_V + off + 1024);
-                        const float2 y0 = unpack_bf16(tw[2 * i]), y1 = unpack_bf16(tw[2 * i + 1]);
+                        const float2 y0 = unpack_bf16(tw[2 * i]), y1 = unpack_bf16(tw[2 * i + 1]), x2 = unpack_bf16(xw[2 * i]), x3 = unpack_bf16(xw[2 * i + 1]);
+                        v[4 * i] = fmaf(ig0, x2.x, v[4 * i]);         v[4 * i + 1] = fmaf(ig0, x2.y, v[4 * i + 1]);
+                        v[4 * i + 2] = fmaf(ig1, x3.x, v[4 * i + 2]); v[4 * i + 3] = fmaf(ig1, x3.y, v[4 * i + 3]);
                         a0 = fmaf(v[4 * i], y0.x, a0);     a0 = fmaf(v[4 * i + 1], y0.y, a0);
                         a1 = fmaf(v[4 * i + 2], y1.x, a1); a1 = fmaf(v[4 * i + 3], y1.y, a1);
                         *reinterpret_cast<uint32_t *>(sm + OFF_DR + off) = pack_bf16(v[4 * i], v[4 * i + 1]);
