@@ -17,6 +17,11 @@
 //   Te = diag(e^{-b}) T      T2 = Te diag(beta Gk)      We = Te diag(beta Gam) K
 // and the forward's operands enter the tensor core as they stand in memory: no tile is rescaled, which leaves the two
 // serial products a chunk (We S and K^T Ue), one 64x64 and one 128x64 accumulator read between them.
+// Range: e^b is kept as 2^k e^b, with 2^-k the power of two nearest to half a chunk's whole decay, and S, dS as 2^-k S, 2^k dS: the
+// formulas keep their form, every factor is exact (the bits are those of k = 0), and a state goes from one chunk's scale to the next one's
+// inside its decay.  At the decay limit the factors that bf16 operands carry (e^b in A and dUe, e^-b in T2 and Ue) then span e^-38 .. e^38.
+// With k = 0 A and dUe carried e^-76 = 1e-33: for dO of 1e-6, the size a mean-reduced loss leaves, their products were bf16 subnormals and dv
+// was off by 1.5 % (26 % at 1e-9; one-CTA kernels 1.0 and 3.5 %; 0.3 % now at every scale).
 // Gradients (chain rule, X = dUe):  dR = Te^T X (T's unit diagonal in fp32, only the part below it as bf16),  dA = tril(dO Ue^T),  P = strict_tril(dR Ue^T),  M = -beta Gam P,
 //   aq = dO S^T + dA K               dq = fq aq               dv = beta Gk dR
 //   kd = Ue dZ^T + dA^T Qg + M^T K   Y = dR S^T + P K         dk = kd - beta Gam Y
@@ -42,10 +47,10 @@ using namespace tc;
 struct Rec {
     uint32_t bytes, s, u, te, w, a, sc, t2, du, dz;
 };
-constexpr uint32_t SC_BYTES = 2048;                  // [6][64] floats, then at float 384 the 16 partial sums of <dS', S'>
+constexpr uint32_t SC_BYTES = 2048;                  // [6][64] floats, at float 384 (2^k e^{b_last}, 2^-k), at float 388 the 16 partial sums of <dS', S'>
 enum Sc { SC_FQ = 0, SC_BG, SC_FV, SC_GAM, SC_GK, SC_IG, SC_NARR };
-constexpr uint32_t SC_LOAD = SC_NARR * C * 4, SC_DOT = 384;
-static_assert(SC_NARR * C <= SC_DOT && (SC_DOT + 16) * 4 <= SC_BYTES, "scalars of a record");
+constexpr uint32_t SC_END = SC_NARR * C, SC_DOT = SC_END + 4, SC_LOAD = SC_DOT * 4;
+static_assert(SC_LOAD % 16 == 0 && (SC_DOT + 16) * 4 <= SC_BYTES, "scalars of a record");
 constexpr uint32_t PREP_BYTES = TILE_BF16 + HALF_BF16 + SC_BYTES + HALF_BF16;                        // We | A | scalars | T2
 constexpr Rec REC_INFER = {PREP_BYTES, 0, 0, 0, 0, TILE_BF16, TILE_BF16 + HALF_BF16, TILE_BF16 + HALF_BF16 + SC_BYTES, 0, 0};
 constexpr uint32_t R_U = STATE_BF16, R_TE = R_U + TILE_BF16, R_W = R_TE + HALF_BF16, R_A = R_W + TILE_BF16, R_SC = R_A + HALF_BF16,
@@ -228,8 +233,10 @@ __device__ __forceinline__ void prep_worker(const CUtensorMap &gm_q, const CUten
         sync();
         if (tid >= C) {
             const int t = tid - C;
-            const float b = s_b[t], beta = s_beta[t], gam = __expf(b);
-            const float fq = s_fq[t] * gam, bg = beta * gam, fv = beta * s_gk[t], ig = __expf(-b);
+            const float b = s_b[t], beta = s_beta[t];
+            const int k = min(max(__float2int_rn(s_b[C - 1] * (-0.5f * LOG2E)), -60), 60);
+            const float up = __int_as_float((127 + k) << 23), down = __int_as_float((127 - k) << 23);          // 2^k, 2^-k
+            const float gam = __expf(b) * up, fq = s_fq[t] * gam, bg = beta * gam, fv = beta * s_gk[t], ig = __expf(-b) * down;
             s_ig[t] = ig;
             s_fq[t] = fq;
             s_bg[t] = bg;
@@ -241,7 +248,10 @@ __device__ __forceinline__ void prep_worker(const CUtensorMap &gm_q, const CUten
             out[SC_GAM * C + t] = gam;
             out[SC_GK * C + t] = s_gk[t];
             out[SC_IG * C + t] = ig;
-            if (t == C - 1 && b < -SLA_MAX_CHUNK_DECAY) atomicOr(p.status, STATUS_RANGE);
+            if (t == C - 1) {
+                *reinterpret_cast<float2 *>(out + SC_END) = make_float2(gam, down);
+                if (b < -SLA_MAX_CHUNK_DECAY) atomicOr(p.status, STATUS_RANGE);
+            }
         }
         sync();
         wait(bM1, par);
@@ -496,6 +506,7 @@ __device__ __forceinline__ void scan_item(int item, const CUtensorMap &gm_q, con
     };
     scan_barriers(bars, first);
     auto scalars = [&](int n) { return reinterpret_cast<const float *>(rec0 + (size_t)n * p.L.bytes + p.L.sc); };
+    auto end_of = [&](int n) { return *reinterpret_cast<const float2 *>(scalars(n) + SC_END); };
 
     if (warp == 8) {
         // ---------------- MMA issue ----------------
@@ -689,17 +700,19 @@ __device__ __forceinline__ void scan_item(int item, const CUtensorMap &gm_q, con
         const int qr = warp & 3, ch = warp >> 2, row = 32 * qr + lane;
         const uint32_t tq = tmem + ((uint32_t)(32 * qr) << 16);
         float S[32];
+        float2 e = end_of(0);
         {
             const float *src = state_row(p.h0, s.sbh, row, sl, p.dk, p.dv);
             load_state32(src ? src + 32 * ch : nullptr, S);
+#pragma unroll
+            for (int j = 0; j < 32; ++j) S[j] *= e.y;
         }
         store_slice(sm + OFF_S, row, ch, S);
         fence_proxy_async();
         warp_arrive(bar(SREADY), lane);
-        float e = scalars(0)[SC_GAM * C + C - 1];
         for (int n = 0; n < NT; ++n) {
             const int x = n & 1;
-            const float en = scalars(n + 1 < NT ? n + 1 : n)[SC_GAM * C + C - 1];
+            const float2 en = end_of(n + 1 < NT ? n + 1 : n);
             wait(C1, n & 1);
             tc_fence_after();
             {
@@ -717,8 +730,9 @@ __device__ __forceinline__ void scan_item(int item, const CUtensorMap &gm_q, con
                 float v[32];
                 tmem_ld32(tq + TM_D + 32 * ch, v);
                 tmem_wait_ld();
+                const float dec = n + 1 < NT ? e.x * en.y : e.x;     // (the final state leaves unscaled)
 #pragma unroll
-                for (int j = 0; j < 32; ++j) S[j] = e * (S[j] + v[j]);
+                for (int j = 0; j < 32; ++j) S[j] = dec * (S[j] + v[j]);
             }
             if (p.save && n >= 1) wait(SAVED + (x ^ 1), ((n - 1) >> 1) & 1);         // S_{n-1} and Ue of chunk n-1 have left their buffers
             store_slice(sm + OFF_S + (x ^ 1) * SLICE, row, ch, S);
@@ -764,6 +778,7 @@ __device__ __forceinline__ void bscan_item(int item, const CUtensorMap &gm_q, co
     scan_barriers(bars, first);
     // chunks are visited in the order n = NT-1 ... 0; x = NT-1-n is the visit number that drives buffers and parities
     auto scalars = [&](int x) { return reinterpret_cast<const float *>(rec0 + (size_t)(NT - 1 - x) * p.L.bytes + p.L.sc); };
+    auto end_of = [&](int x) { return *reinterpret_cast<const float2 *>(scalars(x) + SC_END); };
 
     if (warp == 8) {
         // ---------------- MMA issue ----------------
@@ -937,7 +952,8 @@ __device__ __forceinline__ void bscan_item(int item, const CUtensorMap &gm_q, co
             const float *src = state_row(p.dht, s.sbh, row, sl, p.dk, p.dv);
             load_state32(src ? src + 32 * ch : nullptr, S);
         }
-        float e = scalars(0)[SC_GAM * C + C - 1];
+        float2 e = end_of(0);
+        float d = 1.f;                                 // 2^-k of the chunk visited before (the gradient of the final state comes unscaled)
         for (int x = 0; x < NT; ++x) {
             const int y = x & 1;
             const uint32_t ph = (x >> 1) & 1;
@@ -945,8 +961,9 @@ __device__ __forceinline__ void bscan_item(int item, const CUtensorMap &gm_q, co
             float part = 0.f;
             {   // dZ = e^{b_last} dS' as an operand; <dS', S'> beside the first product
                 float z[32];
+                const float dec = e.x * d;             // (here and not where e is read: the read is under way until now)
 #pragma unroll
-                for (int j = 0; j < 32; ++j) z[j] = e * S[j];
+                for (int j = 0; j < 32; ++j) z[j] = dec * S[j];
                 store_slice(sm + OFF_Z + y * SLICE, row, ch, z);
                 fence_proxy_async();
                 tc_fence_before();
@@ -970,7 +987,8 @@ __device__ __forceinline__ void bscan_item(int item, const CUtensorMap &gm_q, co
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
             if (lane == 0) const_cast<float *>(scalars(x))[SC_DOT + 8 * sl + warp] = part;
-            e = scalars(x + 1 < NT ? x + 1 : x)[SC_GAM * C + C - 1];
+            d = e.y;
+            e = end_of(x + 1 < NT ? x + 1 : x);
             wait(C1, x & 1);
             tc_fence_after();
             {
@@ -994,7 +1012,8 @@ __device__ __forceinline__ void bscan_item(int item, const CUtensorMap &gm_q, co
         }
         if (float *dst = state_row(p.dh0, s.sbh, row, sl, p.dk, p.dv)) {
 #pragma unroll
-            for (int j = 0; j < 32; j += 4) *reinterpret_cast<float4 *>(dst + 32 * ch + j) = make_float4(S[j], S[j + 1], S[j + 2], S[j + 3]);
+            for (int j = 0; j < 32; j += 4)
+                *reinterpret_cast<float4 *>(dst + 32 * ch + j) = make_float4(d * S[j], d * S[j + 1], d * S[j + 2], d * S[j + 3]);
         }
     }
 }

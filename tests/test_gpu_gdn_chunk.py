@@ -110,3 +110,28 @@ def test_chunk_parallel_gradients_are_as_exact_as_the_one_cta_kernels():
         assert not torch.equal(whole, alone), n             # (two kernels, not one compared with itself)
         e_whole, e_alone = gu.rel_l2(whole, r), gu.rel_l2(alone, r)
         assert e_whole <= 1.03 * e_alone, (n, e_whole, e_alone)
+
+
+@pytest.mark.parametrize("strongest", [-1.0, -1.15, -1.9])      # every token -1.0 or -1.15 (74 a chunk of 64); -1.9: uniform in -1.9 .. 0
+@pytest.mark.parametrize("loss_scale", [1.0, 1e-3, 1e-6, 1e-9])
+def test_strong_decay_keeps_gradients_of_any_scale(strongest, loss_scale):
+    """Close to the decay limit of 76 a chunk, gradients as a mean-reduced loss hands them in: the pass is linear in (dO, dht), so the errors relative
+    to the oracle's results must not depend on their scale."""
+    cfg = small(CONFIGS["C4"], B=1, T=1100, H=3, seed=1660)
+    xh = make_inputs(cfg, with_dO=True, with_h0=True)
+    if strongest < -1.5:
+        xh["log_decay"] = strongest * torch.rand(xh["log_decay"].shape, generator=torch.Generator().manual_seed(1661))
+    else:
+        xh["log_decay"].fill_(strongest)
+    xh["dO"], xh["dht"] = (xh["dO"].float() * loss_scale).to(torch.bfloat16), xh["dht"] * loss_scale
+    x = gu.to_dev(xh)
+    o, ht, g, plan, ws, lf, lb = gu.gpu_training_step(cfg, x, h0=x["h0"], dht=x["dht"], want_dh0=True)
+    assert (lf, lb) == (1, 2)
+    oref, htref = gu.oracle_forward(cfg, xh, h0=xh["h0"])
+    ref = gu.oracle_backward(cfg, xh, h0=xh["h0"], dht=xh["dht"])
+    # dh0 is e^-1200 and below: zero in fp32, and so are the oracle's
+    pairs = {"o": (o, oref), "ht": (ht, htref)}
+    pairs.update({n: (g[n], ref[r]) for n, r in gu.GRAD_NAMES.items() if g.get(n) is not None and n != "dh0"})
+    errs = {n: gu.rel_l2(a, r) for n, (a, r) in pairs.items()}
+    gu.assert_close(errs, {n: gu.row_err(a, r) for n, (a, r) in pairs.items()}, cfg.dtype, cfg)
+    assert float(g["dh0"].abs().max()) == 0.0 or gu.rel_l2(g["dh0"], ref["dh0"]) <= 1e-2
