@@ -138,16 +138,16 @@ sla_status sla_plan_create(sla_plan **out, const sla_desc *desc) {
     if (!(desc->scale == desc->scale)) return SLA_ERR_INVALID_ARG;
 
     int dev = 0, major = 0;                          // (one attribute: the whole property record takes the driver 7 ms and more)
-    if (cudaGetDevice(&dev) != cudaSuccess) return SLA_ERR_CUDA;
-    if (cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, dev) != cudaSuccess) return SLA_ERR_CUDA;
+    if (cudaGetDevice(&dev) != cudaSuccess) return sla::cuda_error();
+    if (cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, dev) != cudaSuccess) return sla::cuda_error();
     if (major != 10) return SLA_ERR_ARCH;
     if (sla::generic_configure() != 0 || sla::gdn_configure() != 0 || sla::gla_tc_configure() != 0 ||
         sla::gla_tc_bwd_configure() != 0 || sla::gdn_tc_configure() != 0 ||
         sla::gdn_tc_bwd_configure() != 0 || sla::decode_configure() != 0 || sla::out_proj_configure() != 0)
-        return SLA_ERR_CUDA;
+        return sla::cuda_error();
 
     sla_plan *p = new (std::nothrow) sla_plan();
-    if (!p) return SLA_ERR_CUDA;
+    if (!p) return sla::cuda_error();
     sla::Dims &d = p->dims;
     d.variant = desc->variant;
     d.io_bf16 = desc->io_dtype == SLA_BF16;
@@ -166,7 +166,7 @@ sla_status sla_plan_create(sla_plan **out, const sla_desc *desc) {
             if (!varlen_to_device(p->segs)) {
                 varlen_release(p->segs);
                 delete p;
-                return SLA_ERR_CUDA;
+                return sla::cuda_error();
             }
         }
     }
@@ -178,7 +178,7 @@ sla_status sla_plan_create(sla_plan **out, const sla_desc *desc) {
         cudaMemset(p->d_status, 0, sizeof(int)) != cudaSuccess) {
         if (p->d_status) cudaFree(p->d_status);
         delete p;
-        return SLA_ERR_CUDA;
+        return sla::cuda_error();
     }
     *out = p;
     return SLA_OK;
@@ -225,7 +225,7 @@ sla_status sla_plan_set_sequences(sla_plan *plan, const int32_t *cu_seqlens, int
     if (!varlen_to_device(v)) {
         varlen_release(v);
         plan_workspace_sizes(plan);
-        return SLA_ERR_CUDA;
+        return sla::cuda_error();
     }
     plan_workspace_sizes(plan);
     return SLA_OK;
@@ -241,7 +241,7 @@ sla_status sla_plan_workspace_bytes(const sla_plan *plan, size_t *fwd, size_t *b
 sla_status sla_plan_poll(sla_plan *plan) {
     if (!plan) return SLA_ERR_INVALID_ARG;
     int v = 0;
-    if (cudaMemcpy(&v, plan->d_status, sizeof(int), cudaMemcpyDeviceToHost) != cudaSuccess) return SLA_ERR_CUDA;
+    if (cudaMemcpy(&v, plan->d_status, sizeof(int), cudaMemcpyDeviceToHost) != cudaSuccess) return sla::cuda_error();
     if (v != 0) {
         cudaMemset(plan->d_status, 0, sizeof(int));
         return (v & sla::STATUS_TIMEOUT) ? SLA_ERR_TIMEOUT : SLA_ERR_RANGE;
@@ -254,7 +254,7 @@ int32_t sla_plan_last_launch_count(const sla_plan *plan) { return plan ? plan->l
 sla_status sla_plan_selftest_timeout(sla_plan *plan, void *cuda_stream) {
     if (!plan) return SLA_ERR_INVALID_ARG;
     k_selftest_bounded_wait<<<1, 32, 0, (cudaStream_t)cuda_stream>>>(plan->d_status, 2000000ull);   // 2 ms
-    return cudaGetLastError() == cudaSuccess ? SLA_OK : SLA_ERR_CUDA;
+    return cudaGetLastError() == cudaSuccess ? SLA_OK : sla::cuda_error();
 }
 
 sla_status sla_plan_set_kernel_timing(sla_plan *plan, int32_t enable) {
@@ -268,10 +268,10 @@ sla_status sla_plan_set_kernel_timing(sla_plan *plan, int32_t enable) {
 sla_status sla_plan_kernel_timing_collect(sla_plan *plan, int32_t *n_kernels) {
     if (!plan || !n_kernels) return SLA_ERR_INVALID_ARG;
     sla::Tracer &t = plan->tracer;
-    if (t.used && cudaEventSynchronize(t.pool[t.used - 1]) != cudaSuccess) return SLA_ERR_CUDA;
+    if (t.used && cudaEventSynchronize(t.pool[t.used - 1]) != cudaSuccess) return sla::cuda_error();
     for (const auto &r : t.recs) {
         float ms = 0.f;
-        if (cudaEventElapsedTime(&ms, t.pool[r.e0], t.pool[r.e1]) != cudaSuccess) return SLA_ERR_CUDA;
+        if (cudaEventElapsedTime(&ms, t.pool[r.e0], t.pool[r.e1]) != cudaSuccess) return sla::cuda_error();
         bool found = false;
         for (auto &a : plan->agg)
             if (!strcmp(a.first, r.name)) { a.second.first += 1; a.second.second += ms; found = true; break; }
@@ -305,7 +305,7 @@ sla_status sla_forward(sla_plan *plan, const void *q, const void *k, const void 
         const size_t bytes = (size_t)d.B * d.H * d.dk * d.dv * sizeof(float);
         cudaError_t e = h0 ? cudaMemcpyAsync(ht, h0, bytes, cudaMemcpyDeviceToDevice, (cudaStream_t)cuda_stream)
                            : cudaMemsetAsync(ht, 0, bytes, (cudaStream_t)cuda_stream);
-        return e == cudaSuccess ? SLA_OK : SLA_ERR_CUDA;
+        return e == cudaSuccess ? SLA_OK : sla::cuda_error();
     }
     if (!q || !k || !v || !log_decay || !gq_logits || !gk_logits || !o) return SLA_ERR_INVALID_ARG;
     if (d.variant == SLA_GDN && !beta) return SLA_ERR_INVALID_ARG;
@@ -331,7 +331,7 @@ sla_status sla_forward(sla_plan *plan, const void *q, const void *k, const void 
                 ? sla::gdn_tc_forward(d, a, save ? sla::gdn_tc_records(a.ws) : nullptr, plan->d_status,
                                       (cudaStream_t)cuda_stream, plan->tracer)
                 : sla::generic_forward(d, plan->ws, a, true, (cudaStream_t)cuda_stream, plan->tracer);
-    if (n < 0) return SLA_ERR_CUDA;
+    if (n < 0) return sla::cuda_error();
     plan->last_launches = n;
     if (save) {
         sla_plan::Saved &sv = plan->saved;
@@ -358,7 +358,7 @@ sla_status sla_backward(sla_plan *plan, const void *q, const void *k, const void
         const size_t bytes = (size_t)d.B * d.H * d.dk * d.dv * sizeof(float);
         cudaError_t e = dht ? cudaMemcpyAsync(dh0, dht, bytes, cudaMemcpyDeviceToDevice, (cudaStream_t)cuda_stream)
                             : cudaMemsetAsync(dh0, 0, bytes, (cudaStream_t)cuda_stream);
-        return e == cudaSuccess ? SLA_OK : SLA_ERR_CUDA;
+        return e == cudaSuccess ? SLA_OK : sla::cuda_error();
     }
     if (!q || !k || !v || !log_decay || !gq_logits || !gk_logits || !dO || !dq || !dk || !dv ||
         !dgq_logits || !dgk_logits)
@@ -393,7 +393,7 @@ sla_status sla_backward(sla_plan *plan, const void *q, const void *k, const void
                 ? sla::gdn_tc_backward(d, a, have, plan->d_status, (cudaStream_t)cuda_stream, plan->tracer)
                 : sla::generic_backward(d, plan->ws, a, (cudaStream_t)cuda_stream, plan->tracer);
     if (n == -2) return SLA_ERR_UNSUPPORTED;
-    if (n < 0) return SLA_ERR_CUDA;
+    if (n < 0) return sla::cuda_error();
     plan->last_launches = n;
     return SLA_OK;
 }
@@ -418,7 +418,7 @@ sla_status sla_shortconv_forward(sla_plan *plan, const void *x, const float *w, 
     plan->tracer.start((cudaStream_t)cuda_stream);
     int n = sla::shortconv_forward(dm, d, K, normalize != 0, SLA_SHORTCONV_EPS, x, w, out, (cudaStream_t)cuda_stream,
                                    plan->tracer);
-    if (n < 0) return SLA_ERR_CUDA;
+    if (n < 0) return sla::cuda_error();
     plan->last_launches = n;
     return SLA_OK;
 }
@@ -433,7 +433,7 @@ sla_status sla_shortconv_backward(sla_plan *plan, const void *x, const float *w,
     if (!dw || !aligned16(dw)) return SLA_ERR_INVALID_ARG;
     if (dm.B == 0 || dm.T == 0)
         return cudaMemsetAsync(dw, 0, (size_t)dm.H * d * K * sizeof(float), (cudaStream_t)cuda_stream) == cudaSuccess
-                   ? SLA_OK : SLA_ERR_CUDA;
+                   ? SLA_OK : sla::cuda_error();
     if (!x || !w || !dout || !dx) return SLA_ERR_INVALID_ARG;
     const void *ptrs[] = {x, w, dout, dx, workspace};
     for (const void *p : ptrs)
@@ -442,7 +442,7 @@ sla_status sla_shortconv_backward(sla_plan *plan, const void *x, const float *w,
     plan->tracer.start((cudaStream_t)cuda_stream);
     int n = sla::shortconv_backward(dm, d, K, normalize != 0, SLA_SHORTCONV_EPS, x, w, dout, dx, dw, (float *)workspace,
                                     (cudaStream_t)cuda_stream, plan->tracer);
-    if (n < 0) return SLA_ERR_CUDA;
+    if (n < 0) return sla::cuda_error();
     plan->last_launches = n;
     return SLA_OK;
 }
@@ -461,7 +461,7 @@ sla_status sla_out_proj_forward(sla_plan *plan, const void *o, const void *w_o, 
     plan->tracer.start((cudaStream_t)cuda_stream);
     int n = sla::out_proj_forward((long)d.B * d.T, d.H * d.dv, d_model, o, w_o, y, plan->d_status, (cudaStream_t)cuda_stream,
                                   plan->tracer);
-    if (n < 0) return SLA_ERR_CUDA;
+    if (n < 0) return sla::cuda_error();
     plan->last_launches = n;
     return SLA_OK;
 }
@@ -475,13 +475,13 @@ sla_status sla_out_proj_backward(sla_plan *plan, const void *o, const void *w_o,
     if (!dw_o || !aligned16(dw_o)) return SLA_ERR_INVALID_ARG;
     if (d.B == 0 || d.T == 0)           // no tokens: the weight gradient is zero
         return cudaMemsetAsync(dw_o, 0, (size_t)d.H * d.dv * d_model * sizeof(float), (cudaStream_t)cuda_stream) == cudaSuccess
-                   ? SLA_OK : SLA_ERR_CUDA;
+                   ? SLA_OK : sla::cuda_error();
     if (!o || !w_o || !dy || !d_o || !aligned16(o) || !aligned16(w_o) || !aligned16(dy) || !aligned16(d_o))
         return SLA_ERR_INVALID_ARG;
     plan->tracer.start((cudaStream_t)cuda_stream);
     int n = sla::out_proj_backward((long)d.B * d.T, d.H * d.dv, d_model, o, w_o, dy, d_o, dw_o, plan->d_status,
                                    (cudaStream_t)cuda_stream, plan->tracer);
-    if (n < 0) return SLA_ERR_CUDA;
+    if (n < 0) return sla::cuda_error();
     plan->last_launches = n;
     return SLA_OK;
 }
@@ -504,7 +504,7 @@ sla_status sla_gate_scores_forward(sla_plan *plan, const void *q, const void *k,
         if (!aligned16(p)) return SLA_ERR_INVALID_ARG;
     plan->tracer.start((cudaStream_t)cuda_stream);
     int n = sla::gate_scores_forward(d, q, k, w_gq, w_gk, gq_logits, gk_logits, (cudaStream_t)cuda_stream, plan->tracer);
-    if (n < 0) return SLA_ERR_CUDA;
+    if (n < 0) return sla::cuda_error();
     plan->last_launches = n;
     return SLA_OK;
 }
@@ -521,7 +521,7 @@ sla_status sla_gate_scores_backward(sla_plan *plan, const void *q, const void *k
         const size_t wb = (size_t)d.dk * d.H * sizeof(float);
         if (cudaMemsetAsync(dw_gq, 0, wb, (cudaStream_t)cuda_stream) != cudaSuccess ||
             cudaMemsetAsync(dw_gk, 0, wb, (cudaStream_t)cuda_stream) != cudaSuccess)
-            return SLA_ERR_CUDA;
+            return sla::cuda_error();
         return SLA_OK;
     }
     if (!q || !k || !w_gq || !w_gk || !dgq_logits || !dgk_logits || !dq || !dk) return SLA_ERR_INVALID_ARG;
@@ -532,7 +532,7 @@ sla_status sla_gate_scores_backward(sla_plan *plan, const void *q, const void *k
     plan->tracer.start((cudaStream_t)cuda_stream);
     int n = sla::gate_scores_backward(d, q, k, w_gq, w_gk, dgq_logits, dgk_logits, dq, dk, dw_gq, dw_gk,
                                       (float *)workspace, (cudaStream_t)cuda_stream, plan->tracer);
-    if (n < 0) return SLA_ERR_CUDA;
+    if (n < 0) return sla::cuda_error();
     plan->last_launches = n;
     return SLA_OK;
 }
@@ -554,7 +554,7 @@ sla_status sla_decode_steps(sla_plan *plan, int32_t Bdec, int32_t n_tokens, cons
     sla::DecArgs a{q, k, v, log_decay, beta, gq_logits, gk_logits, state, o, Bdec, n_tokens};
     plan->tracer.start((cudaStream_t)cuda_stream);
     int n = sla::decode_step(d, a, plan->d_status, (cudaStream_t)cuda_stream, plan->tracer);
-    if (n < 0) return SLA_ERR_CUDA;
+    if (n < 0) return sla::cuda_error();
     plan->last_launches = n;
     return SLA_OK;
 }

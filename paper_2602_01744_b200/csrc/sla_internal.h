@@ -16,6 +16,13 @@ namespace sla {
 constexpr int STATUS_TIMEOUT = 1;    // a bounded wait expired
 constexpr int STATUS_RANGE = 2;      // a chunk's cumulative log-decay went below -SLA_MAX_CHUNK_DECAY
 
+// What a call whose CUDA call failed returns.  The runtime keeps such an error until it is asked for: taken back here, or the next call,
+// whose own launches succeed, would find it and report it again.
+inline sla_status cuda_error() {
+    cudaGetLastError();
+    return SLA_ERR_CUDA;
+}
+
 struct Dims {
     int variant;      // sla_variant
     int io_bf16;      // 1: q,k,v,o are bf16, 0: fp32

@@ -22,7 +22,7 @@ sla_status scratch_for_current_device(int dev, void **out) {
     std::lock_guard<std::mutex> lock(g_mu);
     if (!g_scratch_addr[dev]) {
         void *p = nullptr;
-        if (cudaGetSymbolAddress(&p, g_noalloc_scratch) != cudaSuccess || !p) return SLA_ERR_CUDA;
+        if (cudaGetSymbolAddress(&p, g_noalloc_scratch) != cudaSuccess || !p) return sla::cuda_error();
         g_scratch_addr[dev] = p;
     }
     *out = g_scratch_addr[dev];
@@ -49,7 +49,7 @@ extern "C" sla_status sla_forward_noalloc(sla_plan *plan, const void *q, const v
     // The built-in scratch has a fixed size: larger problems must use sla_forward with a caller workspace.
     if (plan->ws.fwd_floats * sizeof(float) > kScratchBytes) return SLA_ERR_WORKSPACE;
     int dev = -1;
-    if (cudaGetDevice(&dev) != cudaSuccess) return SLA_ERR_CUDA;
+    if (cudaGetDevice(&dev) != cudaSuccess) return sla::cuda_error();
     if (dev != plan->device) return SLA_ERR_INVALID_ARG;
     void *scratch = nullptr;
     sla_status s = scratch_for_current_device(dev, &scratch);
@@ -59,7 +59,7 @@ extern "C" sla_status sla_forward_noalloc(sla_plan *plan, const void *q, const v
     sla::FwdArgs a{q, k, v, log_decay, beta, gq_logits, gk_logits, h0, o, ht, (float *)scratch, plan->d_status};
     plan->tracer.start((cudaStream_t)cuda_stream);
     int n = sla::generic_forward(d, plan->ws, a, true, (cudaStream_t)cuda_stream, plan->tracer);
-    if (n < 0) return SLA_ERR_CUDA;
+    if (n < 0) return sla::cuda_error();
     plan->last_launches = n;
     return SLA_OK;
 }
