@@ -82,6 +82,12 @@ static void plan_workspace_sizes(sla_plan *p) {
     }
     if ((p->flags & SLA_FLAG_SAVE_FOR_BACKWARD) && forward_can_save(*p) && p->bwd_bytes > p->fwd_bytes)
         p->fwd_bytes = p->bwd_bytes;     // the forward writes into the backward pass's workspace layout
+    p->fwd_least = p->fwd_bytes;
+    p->bwd_least = p->bwd_bytes;
+    if (sla::gdn_tc_supported(d) && !generic) {      // its one-CTA kernels keep smaller records, and none in a forward pass alone
+        p->bwd_least = sla::gdn_tc_one_cta_workspace_bytes(d, &p->varlen);
+        p->fwd_least = (p->flags & SLA_FLAG_SAVE_FOR_BACKWARD) ? p->bwd_least : 0;
+    }
 }
 
 static void varlen_release(sla::Varlen &v) {
@@ -312,23 +318,20 @@ sla_status sla_forward(sla_plan *plan, const void *q, const void *k, const void 
     const void *ptrs[] = {q, k, v, log_decay, beta, gq_logits, gk_logits, h0, o, ht, workspace};
     for (const void *p : ptrs)
         if (!aligned16(p)) return SLA_ERR_INVALID_ARG;
-    if (plan->fwd_bytes > 0 && (!workspace || workspace_bytes < plan->fwd_bytes)) {
-        // Softmax-GatedDeltaNet has a kernel that needs none: a caller without scratch gets that one
-        const bool scratch_free = sla::gdn_tc_supported(d) && !(plan->flags & (SLA_FLAG_FORCE_GENERIC | SLA_FLAG_SAVE_FOR_BACKWARD));
-        if (!scratch_free) return SLA_ERR_WORKSPACE;
-        workspace = nullptr;
-    }
+    if (!workspace) workspace_bytes = 0;
+    if (workspace_bytes < plan->fwd_least) return SLA_ERR_WORKSPACE;
     sla::FwdArgs a{q, k, v, log_decay, beta, gq_logits, gk_logits, h0, o, ht, (float *)workspace, plan->d_status,
                    plan->varlen.n_seq ? &plan->varlen : nullptr};
     plan->tracer.start((cudaStream_t)cuda_stream);
     const bool generic = plan->flags & SLA_FLAG_FORCE_GENERIC;
     const bool save = (plan->flags & SLA_FLAG_SAVE_FOR_BACKWARD) && forward_can_save(*plan);
+    const bool chunked = !generic && sla::gdn_tc_supported(d) && sla::gdn_tc_chunked(d, &plan->varlen, save, workspace_bytes);
     plan->saved.valid = false;
     int n = (!generic && sla::gla_tc_supported(d))
                 ? sla::gla_tc_forward(d, a, save ? sla::gla_tc_state_images(a.ws) : nullptr, plan->d_status,
                                       (cudaStream_t)cuda_stream, plan->tracer)
             : (!generic && sla::gdn_tc_supported(d))
-                ? sla::gdn_tc_forward(d, a, save ? sla::gdn_tc_records(a.ws) : nullptr, plan->d_status,
+                ? sla::gdn_tc_forward(d, a, save ? sla::gdn_tc_records(a.ws) : nullptr, chunked, plan->d_status,
                                       (cudaStream_t)cuda_stream, plan->tracer)
                 : sla::generic_forward(d, plan->ws, a, true, (cudaStream_t)cuda_stream, plan->tracer);
     if (n < 0) return sla::cuda_error();
@@ -337,7 +340,7 @@ sla_status sla_forward(sla_plan *plan, const void *q, const void *k, const void 
         sla_plan::Saved &sv = plan->saved;
         sv.valid = true;
         sv.ws = workspace; sv.q = q; sv.k = k; sv.v = v; sv.log_decay = log_decay; sv.beta = beta;
-        sv.lq = gq_logits; sv.lk = gk_logits; sv.h0 = h0; sv.stream = cuda_stream;
+        sv.lq = gq_logits; sv.lk = gk_logits; sv.h0 = h0; sv.stream = cuda_stream; sv.chunked = chunked;
     }
     return SLA_OK;
 }
@@ -371,7 +374,8 @@ sla_status sla_backward(sla_plan *plan, const void *q, const void *k, const void
                           dlog_decay, dbeta, dgq_logits, dgk_logits, dh0, workspace};
     for (const void *p : ptrs)
         if (!aligned16(p)) return SLA_ERR_INVALID_ARG;
-    if (plan->bwd_bytes > 0 && (!workspace || workspace_bytes < plan->bwd_bytes)) return SLA_ERR_WORKSPACE;
+    if (!workspace) workspace_bytes = 0;
+    if (workspace_bytes < plan->bwd_least) return SLA_ERR_WORKSPACE;
     sla::BwdArgs a{q, k, v, log_decay, beta, gq_logits, gk_logits, h0, dO, dht, dq, dk, dv,
                    dlog_decay, dbeta, dgq_logits, dgk_logits, dh0, (float *)workspace, plan->d_status,
                    plan->varlen.n_seq ? &plan->varlen : nullptr};
@@ -379,8 +383,9 @@ sla_status sla_backward(sla_plan *plan, const void *q, const void *k, const void
     const bool generic = plan->flags & SLA_FLAG_FORCE_GENERIC;
     // the states (GLA) or per-chunk records (GDN) are taken from the workspace only if the last sla_forward of this plan
     // left them there for exactly these inputs, on this stream; anything else recomputes them
+    const bool chunked = !generic && sla::gdn_tc_supported(d) && sla::gdn_tc_chunked(d, &plan->varlen, true, workspace_bytes);
     sla_plan::Saved &sv = plan->saved;
-    const bool have = sv.valid && sv.ws == workspace && sv.q == q && sv.k == k && sv.v == v && sv.log_decay == log_decay &&
+    const bool have = sv.valid && sv.chunked == chunked && sv.ws == workspace && sv.q == q && sv.k == k && sv.v == v && sv.log_decay == log_decay &&
                       sv.beta == beta && sv.lq == gq_logits && sv.lk == gk_logits && sv.h0 == h0 && sv.stream == cuda_stream;
     // a backward pass that recomputes writes its own states into `workspace`: whatever an earlier forward left there
     // (for other inputs) is gone, and must not be taken for valid by a later call
@@ -390,7 +395,7 @@ sla_status sla_backward(sla_plan *plan, const void *q, const void *k, const void
             : (!generic && sla::gla_tc_supported(d))
                 ? sla::gla_tc_backward(d, a, have, plan->d_status, (cudaStream_t)cuda_stream, plan->tracer)
             : (!generic && sla::gdn_tc_supported(d))
-                ? sla::gdn_tc_backward(d, a, have, plan->d_status, (cudaStream_t)cuda_stream, plan->tracer)
+                ? sla::gdn_tc_backward(d, a, have, chunked, plan->d_status, (cudaStream_t)cuda_stream, plan->tracer)
                 : sla::generic_backward(d, plan->ws, a, (cudaStream_t)cuda_stream, plan->tracer);
     if (n == -2) return SLA_ERR_UNSUPPORTED;
     if (n < 0) return sla::cuda_error();

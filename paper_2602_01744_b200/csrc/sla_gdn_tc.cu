@@ -588,6 +588,10 @@ int gdn_tc_configure() {
 size_t gdn_tc_forward_workspace_bytes(const Dims &d, const Varlen *vl) {
     return gdn_chunk_forward_selected(d, vl) ? gdn_chunk_forward_workspace_bytes(d, vl) : 0;
 }
+bool gdn_tc_chunked(const Dims &d, const Varlen *vl, bool records, size_t ws_bytes) {
+    return records ? gdn_chunk_selected(d, vl) && ws_bytes >= gdn_tc_backward_workspace_bytes(d, vl)
+                   : gdn_chunk_forward_selected(d, vl) && ws_bytes >= gdn_chunk_forward_workspace_bytes(d, vl);
+}
 
 // per-sequence tensor maps of a packed batch (q, k, v and, when given, o) into region `r`
 static const CUtensorMap *gdn_varlen_maps(const Dims &d, const FwdArgs &a, int r, cudaStream_t st) {
@@ -620,9 +624,8 @@ int gdn_tc_forward_save(const Dims &d, const FwdArgs &a, uint8_t *save, int *sta
 }
 
 // Forward; with `save` not null it also leaves the per-chunk records for a later gradient sweep over the same inputs.
-// Without a workspace (a.ws null) every shape runs on the one-CTA-per-sequence kernel.
-int gdn_tc_forward(const Dims &d, const FwdArgs &a, uint8_t *save, int *status, cudaStream_t st, Tracer &tr) {
-    if (save ? gdn_chunk_selected(d, a.vl) : a.ws && gdn_chunk_forward_selected(d, a.vl))
+int gdn_tc_forward(const Dims &d, const FwdArgs &a, uint8_t *save, bool chunked, int *status, cudaStream_t st, Tracer &tr) {
+    if (chunked)
         return gdn_chunk_forward(d, a, save ? save : reinterpret_cast<uint8_t *>(a.ws), save != nullptr, status, st, tr);
     CUtensorMap mq, mk, mv, mo;
     if (!make_tile_map(&mq, a.q, d.B, d.T, d.H, d.dk) || !make_tile_map(&mk, a.k, d.B, d.T, d.H, d.dk) ||

@@ -791,15 +791,19 @@ static size_t record_slots(const Dims &d, const Varlen *vl) {
     return (vl && vl->n_seq) ? (size_t)vl->slots * d.H : (size_t)d.B * d.H * (d.NT + 1);
 }
 
-size_t gdn_tc_backward_workspace_bytes(const Dims &d, const Varlen *vl) {
+static size_t with_gate_sums(const Dims &d, size_t records) {
     const size_t bth = (size_t)d.B * d.T * d.H;
-    return (gdn_chunk_selected(d, vl) ? gdn_chunk_record_bytes(d, vl) : record_slots(d, vl) * REC_BYTES) + 2 * ((bth + 63) & ~(size_t)63) * sizeof(float);
+    return records + 2 * ((bth + 63) & ~(size_t)63) * sizeof(float);
+}
+size_t gdn_tc_one_cta_workspace_bytes(const Dims &d, const Varlen *vl) { return with_gate_sums(d, record_slots(d, vl) * REC_BYTES); }
+size_t gdn_tc_backward_workspace_bytes(const Dims &d, const Varlen *vl) {
+    return gdn_chunk_selected(d, vl) ? with_gate_sums(d, gdn_chunk_record_bytes(d, vl)) : gdn_tc_one_cta_workspace_bytes(d, vl);
 }
 
 uint8_t *gdn_tc_records(float *ws) { return reinterpret_cast<uint8_t *>(ws); }
 
-int gdn_tc_backward(const Dims &d, const BwdArgs &a, bool have_records, int *status, cudaStream_t st, Tracer &tr) {
-    if (gdn_chunk_selected(d, a.vl)) return gdn_chunk_backward(d, a, have_records, status, st, tr);
+int gdn_tc_backward(const Dims &d, const BwdArgs &a, bool have_records, bool chunked, int *status, cudaStream_t st, Tracer &tr) {
+    if (chunked) return gdn_chunk_backward(d, a, have_records, status, st, tr);
     CUtensorMap mq, mk, mv, mdo, mdq, mdk, mdv;
     if (!make_tile_map(&mq, a.q, d.B, d.T, d.H, d.dk) || !make_tile_map(&mk, a.k, d.B, d.T, d.H, d.dk) ||
         !make_tile_map(&mv, a.v, d.B, d.T, d.H, d.dv) || !make_tile_map(&mdo, a.dO, d.B, d.T, d.H, d.dv) ||

@@ -166,15 +166,20 @@ int gla_tc_backward_segmented(const Dims &d, const BwdArgs &a, Varlen &segs, int
 bool gdn_tc_supported(const Dims &d);
 int gdn_tc_configure();
 size_t gdn_tc_forward_workspace_bytes(const Dims &d, const Varlen *vl = nullptr);
-int gdn_tc_forward(const Dims &d, const FwdArgs &a, uint8_t *save, int *status, cudaStream_t st, Tracer &tr);
+// chunked: the chunk-parallel form; see gdn_tc_chunked
+int gdn_tc_forward(const Dims &d, const FwdArgs &a, uint8_t *save, bool chunked, int *status, cudaStream_t st, Tracer &tr);
 uint8_t *gdn_tc_records(float *ws);        // where in the backward workspace the per-chunk records sit
 int gdn_tc_forward_save(const Dims &d, const FwdArgs &a, uint8_t *save, int *status, cudaStream_t st, Tracer &tr);
 // backward: forward sweep in save mode (per-chunk S_n, U, T records), reverse gradient sweep, gate softmax backward
 int gdn_tc_bwd_configure();
 size_t gdn_tc_backward_workspace_bytes(const Dims &d, const Varlen *vl = nullptr);
-int gdn_tc_backward(const Dims &d, const BwdArgs &a, bool have_records, int *status, cudaStream_t st, Tracer &tr);
+size_t gdn_tc_one_cta_workspace_bytes(const Dims &d, const Varlen *vl = nullptr);      // the least a training step runs with
+int gdn_tc_backward(const Dims &d, const BwdArgs &a, bool have_records, bool chunked, int *status, cudaStream_t st, Tracer &tr);
 // Chunk-parallel form of the same (sla_gdn_chunk.cu): per-chunk records prepared and consumed in parallel, two products a
-// chunk on the serial chain.  gdn_tc_forward / gdn_tc_backward take it where gdn_chunk_selected says so.
+// chunk on the serial chain.  gdn_tc_chunked: whether a call with ws_bytes of workspace takes it - the shape gains (gdn_chunk_selected,
+// gdn_chunk_forward_selected) and its records fit; with less the one-CTA kernels serve the call.  records: the call keeps
+// or reads them (a training step's forward, every backward).
+bool gdn_tc_chunked(const Dims &d, const Varlen *vl, bool records, size_t ws_bytes);
 bool gdn_chunk_selected(const Dims &d, const Varlen *vl);
 bool gdn_chunk_forward_selected(const Dims &d, const Varlen *vl);             // ... for a forward pass that keeps no records
 int gdn_chunk_configure();
@@ -216,6 +221,7 @@ struct sla_plan {
     sla::Dims dims;
     sla::Workspace ws;          // carve-up for the generic kernels
     size_t fwd_bytes, bwd_bytes; // what the kernels this plan selects need (tensor-core plans need less than ws says)
+    size_t fwd_least, bwd_least; // the least that sla_forward / sla_backward accept (less than the above where slower kernels need less)
     uint32_t flags;
     int device;
     int *d_status;          // device status word (bounded waits report here)
@@ -226,6 +232,7 @@ struct sla_plan {
         const void *ws = nullptr, *q = nullptr, *k = nullptr, *v = nullptr, *log_decay = nullptr, *beta = nullptr, *lq = nullptr,
                    *lk = nullptr, *h0 = nullptr;
         void *stream = nullptr;
+        bool chunked = false;       // Softmax-GatedDeltaNet: in which of the two forms
     } saved;
     sla::Varlen varlen;     // sla_plan_set_sequences: packed variable-length batch (n_seq == 0: regular batch)
     sla::Varlen segs;       // tensor-core GLA / RetNet plans with few long sequences: the segments the backward runs in

@@ -135,3 +135,58 @@ def test_strong_decay_keeps_gradients_of_any_scale(strongest, loss_scale):
     errs = {n: gu.rel_l2(a, r) for n, (a, r) in pairs.items()}
     gu.assert_close(errs, {n: gu.row_err(a, r) for n, (a, r) in pairs.items()}, cfg.dtype, cfg)
     assert float(g["dh0"].abs().max()) == 0.0 or gu.rel_l2(g["dh0"], ref["dh0"]) <= 1e-2
+
+
+def _one_cta_bytes(seq_chunks, tokens, H):
+    """The least workspace of a training step (include/sla.h, sla_plan_workspace_bytes)."""
+    return sum(c + 1 for c in seq_chunks) * H * (56 << 10) + 2 * ((tokens * H * 4 + 255) & ~255)
+
+
+@pytest.mark.parametrize("lens", [(1100,), (1025, 70, 1)])       # one sequence; a packed batch
+def test_a_workspace_for_the_one_cta_kernels_is_still_enough_for_a_training_step(lens):
+    H, T = 3, sum(lens)
+    cfg = small(CONFIGS["C4"], B=1, T=T, H=H, seed=1670)
+    xh = make_inputs(cfg, with_dO=True)
+    x = gu.to_dev(xh)
+    args = (x["q"], x["k"], x["v"], x["log_decay"], x["gq_logits"], x["gk_logits"])
+    plan = api.sla_plan_create(cfg.variant, cfg.dtype, 1, T, H, 128, 128, flags=api.SLA_FLAG_SAVE_FOR_BACKWARD)
+    cu = [0] + list(np.cumsum(lens))
+    if len(lens) > 1:
+        plan.set_sequences(cu)
+    least = _one_cta_bytes([(n + 63) // 64 for n in lens], T, H)
+    assert least < plan.backward_workspace_bytes
+    arena = gu.Guarded.for_sizes([least])
+    ws = arena.take(least)
+    o, _ = api.sla_forward(plan, *args, beta=x["beta"], workspace=ws)
+    assert plan.last_launch_count == 1
+    g = api.sla_backward(plan, *args, x["dO"], beta=x["beta"], workspace=ws)
+    assert plan.last_launch_count == 2                           # read what the forward left
+    g2 = api.sla_backward(plan, *args, x["dO"], beta=x["beta"], workspace=torch.empty_like(ws))
+    assert plan.last_launch_count == 3
+    # what the fast kernels left in a larger workspace is not taken for these kernels' records, nor the other way round
+    big = plan.workspace(backward=True)
+    api.sla_forward(plan, *args, beta=x["beta"], workspace=big)
+    g3 = api.sla_backward(plan, *args, x["dO"], beta=x["beta"], workspace=big[:least])
+    assert plan.last_launch_count == 3
+    api.sla_forward(plan, *args, beta=x["beta"], workspace=big[:least])
+    fast = api.sla_backward(plan, *args, x["dO"], beta=x["beta"], workspace=big)
+    assert plan.last_launch_count == 3
+    fast2 = api.sla_backward(plan, *args, x["dO"], beta=x["beta"])
+    torch.cuda.synchronize()
+    plan.poll()
+    arena.check()
+    parts = [({n: t if t is None else t[:, a:b] for n, t in xh.items()}, small(cfg, T=b - a)) for a, b in zip(cu, cu[1:])]
+    refs = [gu.oracle_backward(c, p) for p, c in parts]
+    pairs = {"o": (o, np.concatenate([gu.oracle_forward(c, p)[0] for p, c in parts], 1))}
+    for n, r in gu.GRAD_NAMES.items():
+        if g.get(n) is None:
+            continue
+        assert torch.equal(g[n], g2[n]) and torch.equal(g[n], g3[n]) and torch.equal(fast[n], fast2[n]), n
+        pairs[n] = (g[n], np.concatenate([ref[r] for ref in refs], 1))
+        pairs[n + " fast"] = (fast[n], pairs[n][1])
+    gu.assert_close({n: gu.rel_l2(a, r) for n, (a, r) in pairs.items()}, {n: gu.row_err(a, r) for n, (a, r) in pairs.items()}, cfg.dtype, cfg)
+    for call in (lambda w: api.sla_forward(plan, *args, beta=x["beta"], o=o, workspace=w),
+                 lambda w: api.sla_backward(plan, *args, x["dO"], beta=x["beta"], workspace=w)):
+        with pytest.raises(api.SLAError) as e:
+            call(big[:least - 1])
+        assert e.value.status == 3                               # SLA_ERR_WORKSPACE
