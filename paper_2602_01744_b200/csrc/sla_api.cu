@@ -161,6 +161,7 @@ sla_status sla_plan_create(sla_plan **out, const sla_desc *desc) {
     d.dk = desc->d_k; d.dv = desc->d_v; d.C = desc->chunk;
     d.NT = (desc->T + desc->chunk - 1) / desc->chunk;
     d.scale = desc->scale;
+    d.coop_sms = sla::gdn_tc_supported(d) && !(desc->flags & SLA_FLAG_FORCE_GENERIC) ? sla::gdn_chunk_sms() : 0;
     p->ws = sla::plan_workspace(d);
     p->flags = desc->flags;
     // few long sequences on the tensor-core GLA / RetNet kernels: the table of segments the backward runs in
@@ -325,7 +326,7 @@ sla_status sla_forward(sla_plan *plan, const void *q, const void *k, const void 
     plan->tracer.start((cudaStream_t)cuda_stream);
     const bool generic = plan->flags & SLA_FLAG_FORCE_GENERIC;
     const bool save = (plan->flags & SLA_FLAG_SAVE_FOR_BACKWARD) && forward_can_save(*plan);
-    const bool chunked = !generic && sla::gdn_tc_supported(d) && sla::gdn_tc_chunked(d, &plan->varlen, save, workspace_bytes);
+    bool chunked = !generic && sla::gdn_tc_supported(d) && sla::gdn_tc_chunked(d, &plan->varlen, save, workspace_bytes);
     plan->saved.valid = false;
     int n = (!generic && sla::gla_tc_supported(d))
                 ? sla::gla_tc_forward(d, a, save ? sla::gla_tc_state_images(a.ws) : nullptr, plan->d_status,
@@ -383,13 +384,14 @@ sla_status sla_backward(sla_plan *plan, const void *q, const void *k, const void
     const bool generic = plan->flags & SLA_FLAG_FORCE_GENERIC;
     // the states (GLA) or per-chunk records (GDN) are taken from the workspace only if the last sla_forward of this plan
     // left them there for exactly these inputs, on this stream; anything else recomputes them
-    const bool chunked = !generic && sla::gdn_tc_supported(d) && sla::gdn_tc_chunked(d, &plan->varlen, true, workspace_bytes);
+    bool chunked = !generic && sla::gdn_tc_supported(d) && sla::gdn_tc_chunked(d, &plan->varlen, true, workspace_bytes);
     sla_plan::Saved &sv = plan->saved;
     const bool have = sv.valid && sv.chunked == chunked && sv.ws == workspace && sv.q == q && sv.k == k && sv.v == v && sv.log_decay == log_decay &&
                       sv.beta == beta && sv.lq == gq_logits && sv.lk == gk_logits && sv.h0 == h0 && sv.stream == cuda_stream;
     // a backward pass that recomputes writes its own states into `workspace`: whatever an earlier forward left there
     // (for other inputs) is gone, and must not be taken for valid by a later call
     if (!have && sv.ws == workspace) sv.valid = false;
+    const bool chunked_records = have && chunked;
     int n = (!generic && sla::gla_tc_supported(d) && !a.vl && plan->segs.n_seq)
                 ? sla::gla_tc_backward_segmented(d, a, plan->segs, plan->d_status, (cudaStream_t)cuda_stream, plan->tracer)
             : (!generic && sla::gla_tc_supported(d))
@@ -397,6 +399,7 @@ sla_status sla_backward(sla_plan *plan, const void *q, const void *k, const void
             : (!generic && sla::gdn_tc_supported(d))
                 ? sla::gdn_tc_backward(d, a, have, chunked, plan->d_status, (cudaStream_t)cuda_stream, plan->tracer)
                 : sla::generic_backward(d, plan->ws, a, (cudaStream_t)cuda_stream, plan->tracer);
+    if (chunked_records && !chunked) sv.valid = false;   // (the one-CTA kernels stepped in and wrote records of their own there)
     if (n == -2) return SLA_ERR_UNSUPPORTED;
     if (n < 0) return sla::cuda_error();
     plan->last_launches = n;

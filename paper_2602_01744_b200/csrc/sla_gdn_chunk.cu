@@ -32,6 +32,7 @@
 // which costs the training step 1 %: 4 x 4096 x 16 heads 512 -> 517 us).
 // Qg.aq and k.kd cancel in the suffix sum, so both sides take the same rounded Qg and the same rounded dA.
 #include "sla_gla_tc.cuh"
+#include "sla_gdn_route.h"
 
 #include <algorithm>
 #include <cooperative_groups.h>
@@ -1551,36 +1552,32 @@ bool chunk_maps(const Dims &d, Varlen *vl, int r, const MapSpec (&spec)[N], CUte
     return *dev != nullptr;
 }
 
-int chunk_sm_count() {
-    int dev = 0, n = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 0;
-    return n;
-}
-
 }  // namespace
 
-// The chunk-parallel form needs records in memory and a grid-wide barrier; its serial chain is a seventh of the one-CTA kernels' (1.1
-// against 7 us a chunk of the longest sequence).  Above the line, one-CTA against chunk-parallel, 128-wide heads, B x T x H: forward
-// 1 x 1088 x 4 123 / 39 us, 4 x 512 x 16 64 / 39, 1 x 2048 x 4 223 / 57; training step 382 / 84, 221 / 106, 698 / 127.  Below it
-// (1 x 1024 x 4: 111 forward, 4 x 256 x 16: 35) stay the calls whose forward pass is promised to need no workspace, although the longer
-// ones of them would gain too.
-bool gdn_chunk_selected(const Dims &d, const Varlen *vl) {
-    const bool packed = vl && vl->n_seq;
-    const int longest = packed ? vl->seqs[0].NT : d.NT;          // (the table is kept longest sequence first)
-    const long chunks = packed ? (vl->slots - vl->n_seq) * d.H : (long)d.B * d.H * d.NT;
-    return longest > 16 || chunks > 256;
+static gdn::Load chunk_load(const Dims &d, const Varlen *vl) {
+    if (vl && vl->n_seq) return {vl->seqs[0].NT, (vl->slots - vl->n_seq) * d.H, (long)vl->n_seq * d.H, d.coop_sms};      // (kept longest first)
+    return {d.NT, (long)d.B * d.H * d.NT, (long)d.B * d.H, d.coop_sms};
+}
+bool gdn_chunk_selected(const Dims &d, const Varlen *vl) { return gdn::chunk_parallel(chunk_load(d, vl)); }
+bool gdn_chunk_forward_selected(const Dims &d, const Varlen *vl) { return gdn::chunk_parallel_forward(chunk_load(d, vl)); }
+
+int gdn_chunk_sms() {
+    int dev = 0, sms = 0, coop = 0, fwd = 0, bwd = 0;
+    if (cudaGetDevice(&dev) == cudaSuccess && cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess &&
+        cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) == cudaSuccess &&
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&fwd, k_gdn_chunk_fwd, scn::NTHREADS, kn::FWD_SMEM) == cudaSuccess &&
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bwd, k_gdn_chunk_bwd, scn::NTHREADS, kn::BWD_SMEM) == cudaSuccess)
+        return coop && fwd > 0 && bwd > 0 ? sms : 0;
+    cudaGetLastError();
+    return 0;
 }
 
-// A forward pass that keeps no records gains nothing from the chunk-parallel form where every sequence is short (up to 8 chunks) and
-// the sequences fill the SMs by themselves, to four fifths of a whole number of waves or more.  One-CTA against chunk-parallel:
-// 8 x 512 x 16 63.6 / 67.8 us, 18 x 512 x 16 127.4 / 131.7, 64 x 128 x 16 146 / 162; but 12 x 512 x 16 (two waves, 65 % filled)
-// 123.5 / 96.1 and 8 x 1024 x 16 121.2 / 110.9.
-bool gdn_chunk_forward_selected(const Dims &d, const Varlen *vl) {
-    if (!gdn_chunk_selected(d, vl)) return false;
-    const bool packed = vl && vl->n_seq;
-    const int longest = packed ? vl->seqs[0].NT : d.NT;
-    const long seqs = packed ? (long)vl->n_seq * d.H : (long)d.B * d.H, sms = chunk_sm_count(), waves = (seqs + sms - 1) / sms;
-    return longest > 8 || 5 * seqs < 4 * waves * sms;
+// One of the two kernels on a cooperative grid of at most one CTA per SM
+static int launch_cooperative(const void *kernel, long grid, void **args, uint32_t smem, cudaStream_t st) {
+    const cudaError_t e = cudaLaunchCooperativeKernel(kernel, dim3((unsigned)grid), dim3(scn::NTHREADS), args, smem, st);
+    if (e != cudaErrorCooperativeLaunchTooLarge && e != cudaErrorNotSupported) return e == cudaSuccess ? 0 : -1;
+    cudaGetLastError();
+    return gdn::REFUSED;
 }
 
 int gdn_chunk_configure() {
@@ -1618,9 +1615,9 @@ int gdn_chunk_forward(const Dims &d, const FwdArgs &a, uint8_t *rec, bool save, 
     CUtensorMap m[4];
     if (!chunk_maps(d, vl, a.o ? 0 : 1, spec, m, &p.vmaps, st)) return -1;
     const long items = (long)(vl ? vl->n_seq : d.B) * d.H * (d.dv / 64);
-    const long grid = std::min<long>(chunk_sm_count(), std::max<long>((p.slots + pr::NWORK - 1) / pr::NWORK, items));
+    const long grid = std::min<long>(d.coop_sms, std::max<long>((p.slots + pr::NWORK - 1) / pr::NWORK, items));
     void *args[] = {&m[0], &m[1], &m[2], &m[3], &p};
-    if (cudaLaunchCooperativeKernel((void *)k_gdn_chunk_fwd, dim3((unsigned)grid), dim3(scn::NTHREADS), args, kn::FWD_SMEM, st) != cudaSuccess) return -1;
+    if (const int e = launch_cooperative((const void *)k_gdn_chunk_fwd, grid, args, kn::FWD_SMEM, st)) return e;
     tr.mark(a.o ? "gdn_chunk_fwd" : "gdn_chunk_records");
     return cudaGetLastError() == cudaSuccess ? 1 : -1;
 }
@@ -1633,7 +1630,7 @@ int gdn_chunk_backward(const Dims &d, const BwdArgs &a, bool have_records, int *
     int n = 0;
     if (!have_records) {
         n = gdn_chunk_forward(d, f, rec, true, status, st, tr);
-        if (n < 0) return -1;
+        if (n < 0) return n;
     }
     ChunkParams p = chunk_params(d, f, rec, true, status);
     p.dht = a.dht; p.dh0 = a.dh0;
@@ -1645,9 +1642,9 @@ int gdn_chunk_backward(const Dims &d, const BwdArgs &a, bool have_records, int *
     CUtensorMap m[8];
     if (!chunk_maps(d, vl, 2, spec, m, &p.vmaps, st)) return -1;
     const long items = (long)(vl ? vl->n_seq : d.B) * d.H * (d.dv / 64);
-    const long grid = std::min<long>(chunk_sm_count(), std::max<long>(p.slots, items));
+    const long grid = std::min<long>(d.coop_sms, std::max<long>(p.slots, items));
     void *args[] = {&m[0], &m[1], &m[2], &m[3], &m[4], &m[5], &m[6], &m[7], &p};
-    if (cudaLaunchCooperativeKernel((void *)k_gdn_chunk_bwd, dim3((unsigned)grid), dim3(scn::NTHREADS), args, kn::BWD_SMEM, st) != cudaSuccess) return -1;
+    if (const int e = launch_cooperative((const void *)k_gdn_chunk_bwd, grid, args, kn::BWD_SMEM, st)) return e;
     tr.mark("gdn_chunk_bwd");
     if (gate_bwd_prod(a.lq, a.lk, p.pq, p.pk, a.dlq, a.dlk, (long)d.B * d.T, d.H, st) < 0) return -1;
     tr.mark("gate_bwd");

@@ -12,6 +12,7 @@
 // blocks by forward substitution, off-diagonal blocks level by level) and handed to the tensor core as bf16.
 // One CTA per (batch, head) sequence; roles as in the GLA kernels: MMA lane, TMA lane, gate warps, compute warps.
 #include "sla_gla_tc.cuh"
+#include "sla_gdn_route.h"
 
 namespace sla {
 namespace {
@@ -623,10 +624,7 @@ int gdn_tc_forward_save(const Dims &d, const FwdArgs &a, uint8_t *save, int *sta
     return cudaGetLastError() == cudaSuccess ? 1 : -1;
 }
 
-// Forward; with `save` not null it also leaves the per-chunk records for a later gradient sweep over the same inputs.
-int gdn_tc_forward(const Dims &d, const FwdArgs &a, uint8_t *save, bool chunked, int *status, cudaStream_t st, Tracer &tr) {
-    if (chunked)
-        return gdn_chunk_forward(d, a, save ? save : reinterpret_cast<uint8_t *>(a.ws), save != nullptr, status, st, tr);
+static int gdn_one_cta_forward(const Dims &d, const FwdArgs &a, uint8_t *save, int *status, cudaStream_t st, Tracer &tr) {
     CUtensorMap mq, mk, mv, mo;
     if (!make_tile_map(&mq, a.q, d.B, d.T, d.H, d.dk) || !make_tile_map(&mk, a.k, d.B, d.T, d.H, d.dk) ||
         !make_tile_map(&mv, a.v, d.B, d.T, d.H, d.dv) || !make_tile_map(&mo, a.o, d.B, d.T, d.H, d.dv))
@@ -639,6 +637,13 @@ int gdn_tc_forward(const Dims &d, const FwdArgs &a, uint8_t *save, bool chunked,
     k_gdn_fwd_tc<<<vl ? a.vl->n_seq * d.H : d.B * d.H, gd::NTHREADS, gd::SMEM_BYTES, st>>>(mq, mk, mv, mo, p);
     tr.mark("gdn_fwd_tc");
     return cudaGetLastError() == cudaSuccess ? 1 : -1;
+}
+
+// Forward; with `save` not null it also leaves the per-chunk records for a later gradient sweep over the same inputs.
+int gdn_tc_forward(const Dims &d, const FwdArgs &a, uint8_t *save, bool &chunked, int *status, cudaStream_t st, Tracer &tr) {
+    return gdn::run(chunked,
+        [&] { return gdn_chunk_forward(d, a, save ? save : reinterpret_cast<uint8_t *>(a.ws), save != nullptr, status, st, tr); },
+        [&] { return gdn_one_cta_forward(d, a, save, status, st, tr); });
 }
 
 }  // namespace sla

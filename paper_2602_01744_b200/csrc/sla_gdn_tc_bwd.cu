@@ -17,6 +17,7 @@
 // produce from the accumulators stage by stage (six MMA groups per chunk).  Buffers and TMEM regions are reused as
 // their contents die, see the maps below.
 #include "sla_gla_tc.cuh"
+#include "sla_gdn_route.h"
 
 namespace sla {
 namespace {
@@ -802,8 +803,7 @@ size_t gdn_tc_backward_workspace_bytes(const Dims &d, const Varlen *vl) {
 
 uint8_t *gdn_tc_records(float *ws) { return reinterpret_cast<uint8_t *>(ws); }
 
-int gdn_tc_backward(const Dims &d, const BwdArgs &a, bool have_records, bool chunked, int *status, cudaStream_t st, Tracer &tr) {
-    if (chunked) return gdn_chunk_backward(d, a, have_records, status, st, tr);
+static int gdn_one_cta_backward(const Dims &d, const BwdArgs &a, bool have_records, int *status, cudaStream_t st, Tracer &tr) {
     CUtensorMap mq, mk, mv, mdo, mdq, mdk, mdv;
     if (!make_tile_map(&mq, a.q, d.B, d.T, d.H, d.dk) || !make_tile_map(&mk, a.k, d.B, d.T, d.H, d.dk) ||
         !make_tile_map(&mv, a.v, d.B, d.T, d.H, d.dv) || !make_tile_map(&mdo, a.dO, d.B, d.T, d.H, d.dv) ||
@@ -837,6 +837,12 @@ int gdn_tc_backward(const Dims &d, const BwdArgs &a, bool have_records, bool chu
     if (gate_bwd_prod(a.lq, a.lk, pq, pk, a.dlq, a.dlk, (long)d.B * d.T, d.H, st) < 0) return -1;
     tr.mark("gate_bwd");
     return cudaGetLastError() == cudaSuccess ? (have_records ? 2 : 3) : -1;
+}
+
+int gdn_tc_backward(const Dims &d, const BwdArgs &a, bool have_records, bool &chunked, int *status, cudaStream_t st, Tracer &tr) {
+    const bool records_of_chunks = chunked;
+    return gdn::run(chunked, [&] { return gdn_chunk_backward(d, a, have_records, status, st, tr); },
+        [&] { return gdn_one_cta_backward(d, a, have_records && !records_of_chunks, status, st, tr); });
 }
 
 }  // namespace sla

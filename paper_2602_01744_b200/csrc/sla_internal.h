@@ -28,6 +28,7 @@ struct Dims {
     int io_bf16;      // 1: q,k,v,o are bf16, 0: fp32
     int B, T, H, dk, dv, C, NT;
     float scale;
+    int coop_sms;     // SMs that the chunk-parallel Gated-DeltaNet kernels' cooperative grid can fill; 0: not available (or not needed)
 };
 
 // Packed variable-length batches (B = 1: sequences one after another along T, the state reset at every boundary,
@@ -166,15 +167,15 @@ int gla_tc_backward_segmented(const Dims &d, const BwdArgs &a, Varlen &segs, int
 bool gdn_tc_supported(const Dims &d);
 int gdn_tc_configure();
 size_t gdn_tc_forward_workspace_bytes(const Dims &d, const Varlen *vl = nullptr);
-// chunked: the chunk-parallel form; see gdn_tc_chunked
-int gdn_tc_forward(const Dims &d, const FwdArgs &a, uint8_t *save, bool chunked, int *status, cudaStream_t st, Tracer &tr);
+// chunked: in the chunk-parallel form (see gdn_tc_chunked); false afterwards if the one-CTA kernels had to step in
+int gdn_tc_forward(const Dims &d, const FwdArgs &a, uint8_t *save, bool &chunked, int *status, cudaStream_t st, Tracer &tr);
 uint8_t *gdn_tc_records(float *ws);        // where in the backward workspace the per-chunk records sit
 int gdn_tc_forward_save(const Dims &d, const FwdArgs &a, uint8_t *save, int *status, cudaStream_t st, Tracer &tr);
 // backward: forward sweep in save mode (per-chunk S_n, U, T records), reverse gradient sweep, gate softmax backward
 int gdn_tc_bwd_configure();
 size_t gdn_tc_backward_workspace_bytes(const Dims &d, const Varlen *vl = nullptr);
 size_t gdn_tc_one_cta_workspace_bytes(const Dims &d, const Varlen *vl = nullptr);      // the least a training step runs with
-int gdn_tc_backward(const Dims &d, const BwdArgs &a, bool have_records, bool chunked, int *status, cudaStream_t st, Tracer &tr);
+int gdn_tc_backward(const Dims &d, const BwdArgs &a, bool have_records, bool &chunked, int *status, cudaStream_t st, Tracer &tr);
 // Chunk-parallel form of the same (sla_gdn_chunk.cu): per-chunk records prepared and consumed in parallel, two products a
 // chunk on the serial chain.  gdn_tc_chunked: whether a call with ws_bytes of workspace takes it - the shape gains (gdn_chunk_selected,
 // gdn_chunk_forward_selected) and its records fit; with less the one-CTA kernels serve the call.  records: the call keeps
@@ -183,8 +184,10 @@ bool gdn_tc_chunked(const Dims &d, const Varlen *vl, bool records, size_t ws_byt
 bool gdn_chunk_selected(const Dims &d, const Varlen *vl);
 bool gdn_chunk_forward_selected(const Dims &d, const Varlen *vl);             // ... for a forward pass that keeps no records
 int gdn_chunk_configure();
+int gdn_chunk_sms();                                                           // Dims::coop_sms of the current device
 size_t gdn_chunk_forward_workspace_bytes(const Dims &d, const Varlen *vl);     // records of a forward that saves nothing
 size_t gdn_chunk_record_bytes(const Dims &d, const Varlen *vl);                // records of a training step
+// These two also return gdn::REFUSED (sla_gdn_route.h).
 int gdn_chunk_forward(const Dims &d, const FwdArgs &a, uint8_t *rec, bool save, int *status, cudaStream_t st, Tracer &tr);
 int gdn_chunk_backward(const Dims &d, const BwdArgs &a, bool have_records, int *status, cudaStream_t st, Tracer &tr);
 int gate_bwd_prod(const float *lq, const float *lk, const float *pq, const float *pk, float *dlq, float *dlk, long n_tok,
