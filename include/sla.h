@@ -175,7 +175,7 @@ sla_status sla_forward(sla_plan *plan,
  * flowing into the final state).  Outputs, written in full (not accumulated): dq, dk, dv
  * (io dtype); dlog_decay fp32 in the shape of log_decay (must be NULL for RETNET, whose gamma_h
  * is a constant); dbeta fp32 [B,T,H] (GDN, else NULL); dgq_logits, dgk_logits fp32 [B,T,H];
- * dh0 fp32 or NULL.  dgq_logits and dgk_logits must not alias each other.
+ * dh0 fp32 or NULL (dh0 may be the buffer of dht).  dgq_logits and dgk_logits must not alias each other.
  */
 sla_status sla_backward(sla_plan *plan,
                         const void *q, const void *k, const void *v,

@@ -262,8 +262,8 @@ k_state_scan(Dims d, const TIO *__restrict__ k, const float *__restrict__ bcum,
 // is left for the walk along the sequence (k_state_fold).  One CTA per sequence walking the chunks through shared memory
 // took 19 us a chunk; at 2 x 1000 x 4 heads of 64 both kernels together take 20 us where the scan took 300 (reverse: 250).
 // GRAD = false: KV_n = (Gk k e^{b_last - b})^T V into state slot n + 1;  GRAD = true: qh^T dO into slot n - 1 of the state
-// gradients (n = 0: into dh0, if wanted).  grid (NT, B*H, ceil(dk / 64)).
-template <typename TIO, bool GRAD>
+// gradients (n = 0: into dh0 - ADD: on top of what is there - if wanted).  grid (NT, B*H, ceil(dk / 64)).
+template <typename TIO, bool GRAD, bool ADD = false>
 __global__ void __launch_bounds__(256)
 k_chunk_outer(Dims d, const TIO *__restrict__ x, const TIO *__restrict__ y, const float *__restrict__ gate, const float *__restrict__ bcum,
               float *__restrict__ out, float *__restrict__ dh0) {
@@ -306,17 +306,19 @@ k_chunk_outer(Dims d, const TIO *__restrict__ x, const TIO *__restrict__ y, cons
 #pragma unroll
         for (int cb = 0; cb < 4; ++cb) {
             const int j = tx + 32 * cb;
-            if (j < d.dv) dst[(size_t)(r0 + i) * d.dv + j] = acc[r][cb];
+            float *e = dst + (size_t)(r0 + i) * d.dv + j;
+            if (j < d.dv) *e = ADD ? *e + acc[r][cb] : acc[r][cb];
         }
     }
 }
 
 // The walk along the sequence, one thread per state element, in place over what k_chunk_outer left:
 // GRAD = false: S_0 = h0, S_{n+1} = e^{b_last} S_n + KV_n (slot n: the state before chunk n; the last also to ht);
-// GRAD = true, in reverse: slot NT-1 = dht, slot n-1 = e^{b_last,n} slot n + (qh^T dO)_n (n = 0: dh0).
+// GRAD = true, in reverse: slot NT-1 = dht, slot n-1 = e^{b_last,n} slot n + (qh^T dO)_n (n = 0: dh0, whose product lies in prod0 or,
+// nullptr, comes later).  first and last may be one buffer.
 template <bool GRAD>
 __global__ void __launch_bounds__(256)
-k_state_fold(Dims d, const float *__restrict__ bcum, const float *__restrict__ first, float *__restrict__ st, float *__restrict__ last) {
+k_state_fold(Dims d, const float *__restrict__ bcum, const float *first, float *__restrict__ st, float *last, const float *prod0) {
     const int sz = d.dk * d.dv, e = blockIdx.x * blockDim.x + threadIdx.x, bh = blockIdx.y, b = bh / d.H, h = bh % d.H;
     if (e >= sz) return;
     const int c = e / d.dv, NT = d.NT, slots = GRAD ? NT : NT + 1;
@@ -332,7 +334,7 @@ k_state_fold(Dims d, const float *__restrict__ bcum, const float *__restrict__ f
             add[u] = dc[u] = 0.f;
             if (m >= NT) continue;
             dc[u] = dec(n);
-            add[u] = !GRAD ? p[(size_t)(n + 1) * sz] : n > 0 ? p[(size_t)(n - 1) * sz] : last ? last[(size_t)bh * sz + e] : 0.f;
+            add[u] = !GRAD ? p[(size_t)(n + 1) * sz] : n > 0 ? p[(size_t)(n - 1) * sz] : prod0 ? prod0[(size_t)bh * sz + e] : 0.f;
         }
 #pragma unroll
         for (int u = 0; u < U; ++u) {
@@ -760,7 +762,7 @@ int forward_t(const Dims &d, const Workspace &w, const FwdArgs &a, bool write_o,
     } else {
         k_chunk_outer<TIO, false><<<dim3(d.NT, d.B * d.H, (d.dk + 63) / 64), 256, smem_outer(d), st>>>(d, k, v, Gk, bcum, states, nullptr);
         tr.mark("chunk_outer");
-        k_state_fold<false><<<dim3((d.dk * d.dv + 255) / 256, d.B * d.H), 256, 0, st>>>(d, bcum, a.h0, states, a.ht);
+        k_state_fold<false><<<dim3((d.dk * d.dv + 255) / 256, d.B * d.H), 256, 0, st>>>(d, bcum, a.h0, states, a.ht, nullptr);
         tr.mark("state_fold");
         launches += 2;
     }
@@ -780,11 +782,19 @@ int backward_lin_t(const Dims &d, const Workspace &w, const BwdArgs &a, cudaStre
     int launches = 0;
     const TIO *q = (const TIO *)a.q, *k = (const TIO *)a.k, *v = (const TIO *)a.v, *dO = (const TIO *)a.dO;
     dim3 tiles(d.NT, d.B * d.H);
-    k_chunk_outer<TIO, true><<<dim3(d.NT, d.B * d.H, (d.dk + 63) / 64), 256, smem_outer(d), st>>>(d, q, dO, Gq, bcum, dstates, a.dh0);
+    // dh0 may be dht's own buffer: the first chunk's product must not go there before dht has been read
+    const bool in_place = a.dh0 && a.dh0 == a.dht;
+    float *prod0 = in_place ? nullptr : a.dh0;
+    k_chunk_outer<TIO, true><<<dim3(d.NT, d.B * d.H, (d.dk + 63) / 64), 256, smem_outer(d), st>>>(d, q, dO, Gq, bcum, dstates, prod0);
     tr.mark("chunk_outer");
-    k_state_fold<true><<<dim3((d.dk * d.dv + 255) / 256, d.B * d.H), 256, 0, st>>>(d, bcum, a.dht, dstates, a.dh0);
+    k_state_fold<true><<<dim3((d.dk * d.dv + 255) / 256, d.B * d.H), 256, 0, st>>>(d, bcum, a.dht, dstates, a.dh0, prod0);
     tr.mark("state_fold");
     launches += 2;
+    if (in_place) {
+        k_chunk_outer<TIO, true, true><<<dim3(1, d.B * d.H, (d.dk + 63) / 64), 256, smem_outer(d), st>>>(d, q, dO, Gq, bcum, nullptr, a.dh0);
+        tr.mark("chunk_outer");
+        ++launches;
+    }
     k_grads_lin<TIO><<<tiles, 256, smem_grads_lin(d), st>>>(d, q, k, v, dO, Gq, Gk, bcum, states, dstates,
                                                             (TIO *)a.dq, (TIO *)a.dk, (TIO *)a.dv,
                                                             a.dlog_decay, dGq, dGk);
@@ -800,7 +810,8 @@ template <typename TIO> bool configure_t() {
     ok &= set_smem(k_gdn_prepare<TIO>, smem_prepare(d));
     ok &= set_smem(k_state_scan<TIO>, smem_scan(d));
     ok &= set_smem(k_output<TIO>, smem_output(d));
-    ok &= set_smem(k_chunk_outer<TIO, false>, smem_outer(d)) && set_smem(k_chunk_outer<TIO, true>, smem_outer(d));
+    ok &= set_smem(k_chunk_outer<TIO, false>, smem_outer(d)) && set_smem(k_chunk_outer<TIO, true>, smem_outer(d)) &&
+          set_smem(k_chunk_outer<TIO, true, true>, smem_outer(d));
     ok &= set_smem(k_dstate_scan<TIO>, smem_dscan(d));
     ok &= set_smem(k_grads_lin<TIO>, smem_grads_lin(d));
     return ok;
