@@ -146,6 +146,7 @@ class Plan:
         self.forward_workspace_bytes, self.backward_workspace_bytes = f.value, b.value
         self.io_torch = torch.bfloat16 if self.desc.io_dtype == SLA_BF16 else torch.float32
         self.heads, self.width_v = self.desc.H, self.desc.d_v
+        self._slots = B * (-(-T // chunk) + 1)                 # chunks and one more, over the sequences
 
     def close(self):
         h = getattr(self, "handle", None)
@@ -169,6 +170,8 @@ class Plan:
         _check("sla_plan_workspace_bytes", lib().sla_plan_workspace_bytes(self.handle, ctypes.byref(f), ctypes.byref(b)))
         self.forward_workspace_bytes, self.backward_workspace_bytes = f.value, b.value
         self.n_seq = n
+        lens = [b - a for a, b in zip(cu, cu[1:])] or [self.desc.T] * self.desc.B
+        self._slots = sum(-(-t // self.desc.chunk) + 1 for t in lens)
 
     def poll(self):
         _check("sla_plan_poll", lib().sla_plan_poll(self.handle))
@@ -200,6 +203,23 @@ class Plan:
         n = self.backward_workspace_bytes if backward else self.forward_workspace_bytes
         return torch.empty(max(n, 16), dtype=torch.uint8, device=device)
 
+    def scratch(self, backward, device):
+        """The workspace of a call that brings none.  Where memory is too short for the fast Softmax-GatedDeltaNet kernels' (130 or 34 KiB a
+        chunk and head), the least that sla_plan_workspace_bytes documents: 56 KiB and the gate sums, or nothing."""
+        try:
+            return self.workspace(backward, device)
+        except torch.OutOfMemoryError:
+            d = self.desc
+            if (d.variant != SLA_GDN or d.io_dtype != SLA_BF16 or d.flags & SLA_FLAG_FORCE_GENERIC or d.chunk != 64
+                    or not {d.d_k, d.d_v} <= {64, 128}):
+                raise
+            n = 0
+            if backward or d.flags & SLA_FLAG_SAVE_FOR_BACKWARD:
+                n = self._slots * d.H * (56 << 10) + 2 * ((d.B * d.T * d.H * 4 + 255) // 256 * 256)
+            if n >= (self.backward_workspace_bytes if backward else self.forward_workspace_bytes):
+                raise
+            return torch.empty(max(n, 16), dtype=torch.uint8, device=device)
+
 
 def sla_plan_create(variant, io_dtype, B, T, H, d_k, d_v, chunk=64, scale=1.0, flags=0) -> Plan:
     return Plan(variant, io_dtype, B, T, H, d_k, d_v, chunk, scale, flags)
@@ -212,7 +232,7 @@ def sla_forward(plan: Plan, q, k, v, log_decay, gq_logits, gk_logits, beta=None,
     if o is None:
         o = torch.empty((d.B, d.T, d.H, d.d_v), dtype=plan.io_torch, device=q.device)
     if workspace is None:
-        workspace = plan.workspace(False, q.device)
+        workspace = plan.scratch(False, q.device)
     _check("sla_forward", lib().sla_forward(
         plan.handle, _ptr(q), _ptr(k), _ptr(v), _ptr(log_decay), _ptr(beta), _ptr(gq_logits),
         _ptr(gk_logits), _ptr(h0), _ptr(o), _ptr(ht), _ptr(workspace), workspace.numel(), _stream()))
@@ -245,7 +265,7 @@ def sla_backward(plan: Plan, q, k, v, log_decay, gq_logits, gk_logits, dO, beta=
             dh0=torch.empty((getattr(plan, "n_seq", 0) or d.B, d.H, d.d_k, d.d_v), dtype=torch.float32, device=dev) if want_dh0 else None,
         )
     if workspace is None:
-        workspace = plan.workspace(True, dev)
+        workspace = plan.scratch(True, dev)
     _check("sla_backward", lib().sla_backward(
         plan.handle, _ptr(q), _ptr(k), _ptr(v), _ptr(log_decay), _ptr(beta), _ptr(gq_logits),
         _ptr(gk_logits), _ptr(h0), _ptr(dO), _ptr(dht), _ptr(out["dq"]), _ptr(out["dk"]), _ptr(out["dv"]),

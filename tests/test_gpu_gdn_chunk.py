@@ -190,3 +190,31 @@ def test_a_workspace_for_the_one_cta_kernels_is_still_enough_for_a_training_step
         with pytest.raises(api.SLAError) as e:
             call(big[:least - 1])
         assert e.value.status == 3                               # SLA_ERR_WORKSPACE
+
+
+@pytest.mark.parametrize("lens", [[1100], [1088, 70]])
+def test_calls_without_a_workspace_fit_where_the_large_one_does_not(lens, monkeypatch):
+    """The binding allocates the scratch of a call that brings none; where the fast kernels' does not fit, the slower kernels' serves the call."""
+    cfg = small(CONFIGS["C4"], B=1, T=sum(lens), H=2, seed=1640)
+    x = gu.to_dev(make_inputs(cfg, with_dO=True))
+    args = (x["q"], x["k"], x["v"], x["log_decay"], x["gq_logits"], x["gk_logits"])
+    plan = api.sla_plan_create(cfg.variant, cfg.dtype, 1, cfg.T, 2, 128, 128)
+    if len(lens) > 1:
+        plan.set_sequences([0, *np.cumsum(lens).tolist()])
+    o, _ = api.sla_forward(plan, *args, beta=x["beta"])
+    g = api.sla_backward(plan, *args, x["dO"], beta=x["beta"])
+
+    def short_of_memory(self, backward=False, device="cuda"):
+        raise torch.OutOfMemoryError
+
+    monkeypatch.setattr(api.Plan, "workspace", short_of_memory)
+    assert plan.scratch(True, "cuda").numel() == _one_cta_bytes([(n + 63) // 64 for n in lens], cfg.T, 2)
+    o2, _ = api.sla_forward(plan, *args, beta=x["beta"])
+    g2 = api.sla_backward(plan, *args, x["dO"], beta=x["beta"])
+    with pytest.raises(torch.OutOfMemoryError):                  # (no smaller form)
+        api.sla_plan_create("gla", "bf16", 1, 2048, 2, 128, 128).scratch(True, "cuda")
+    torch.cuda.synchronize()
+    plan.poll()
+    for n, t in [("o", o)] + list(g.items()):                    # two roundings to bf16 and the kernels' own, 4e-3 each, apart
+        if t is not None:
+            assert gu.rel_l2(o2 if n == "o" else g2[n], t.double().cpu().numpy()) <= 1e-2, n
