@@ -192,6 +192,89 @@ def test_a_workspace_for_the_one_cta_kernels_is_still_enough_for_a_training_step
         assert e.value.status == 3                               # SLA_ERR_WORKSPACE
 
 
+@pytest.mark.parametrize("dk,dv", [(128, 128), (64, 128)])
+def test_chunk_parallel_packed_batch_with_states_matches_the_oracle(dk, dv):
+    """Every sequence of a packed batch, the one-chunk ones too: the kernels keep the table longest first, the caller's h0, ht, dht and dh0 are in
+    the caller's order.  The packed tensors are compared whole (a one-token sequence is a single dot product)."""
+    lens, H = [64, 1100, 1, 300, 1088, 65], 3
+    cu = [0] + list(np.cumsum(lens))
+    cfg = small(CONFIGS["C4"], B=1, T=cu[-1], H=H, d_k=dk, d_v=dv, seed=1610)
+    xh = make_inputs(cfg, with_dO=True)
+    gen = torch.Generator().manual_seed(1611)
+    h0, dht = (torch.randn(len(lens), H, dk, dv, generator=gen) * 0.1 for _ in range(2))
+    x = gu.to_dev(xh)
+    args = (x["q"], x["k"], x["v"], x["log_decay"], x["gq_logits"], x["gk_logits"])
+    plan = api.sla_plan_create(cfg.variant, cfg.dtype, 1, cfg.T, H, dk, dv, flags=api.SLA_FLAG_SAVE_FOR_BACKWARD)
+    plan.set_sequences(cu)
+    ws, h0d, dhtd = plan.workspace(backward=True), h0.cuda(), dht.cuda()
+    ht = torch.full_like(h0d, float("nan"))
+    o, _ = api.sla_forward(plan, *args, beta=x["beta"], h0=h0d, ht=ht, workspace=ws)
+    g = api.sla_backward(plan, *args, x["dO"], beta=x["beta"], h0=h0d, dht=dhtd, want_dh0=True, workspace=ws)
+    assert plan.last_launch_count == 2
+    torch.cuda.synchronize()
+    plan.poll()
+    refs = {}
+    for s, (a, b) in enumerate(zip(cu, cu[1:])):
+        c1, xs = small(cfg, T=b - a), {n: t if t is None else t[:, a:b] for n, t in xh.items()}
+        oref, htref = gu.oracle_forward(c1, xs, h0=h0[s:s + 1])
+        ref = gu.oracle_backward(c1, xs, h0=h0[s:s + 1], dht=dht[s:s + 1])
+        for n, r in [("o", oref), ("ht", htref)] + [(n, ref[r]) for n, r in gu.GRAD_NAMES.items() if g.get(n) is not None]:
+            refs.setdefault(n, []).append(r)
+    pairs = {n: (o if n == "o" else ht if n == "ht" else g[n], np.concatenate(r, 0 if n in ("ht", "dh0") else 1)) for n, r in refs.items()}
+    gu.assert_close({n: gu.rel_l2(a, r) for n, (a, r) in pairs.items()}, {n: gu.row_err(a, r) for n, (a, r) in pairs.items()}, cfg.dtype, cfg)
+
+
+def test_chunk_parallel_records_serve_several_backwards_and_no_other_inputs():
+    cfg = small(CONFIGS["C4"], B=1, T=1100, H=2, seed=1620)
+    x = gu.to_dev(make_inputs(cfg, with_dO=True))
+    o, ht, g, plan, ws, lf, lb = gu.gpu_training_step(cfg, x)
+    args = (x["q"], x["k"], x["v"], x["log_decay"], x["gq_logits"], x["gk_logits"])
+    again = api.sla_backward(plan, *args, x["dO"], beta=x["beta"], workspace=ws)
+    assert plan.last_launch_count == 2                           # (the gradient of another loss, say: same records)
+    moved = api.sla_backward(plan, args[0], x["k"].clone(), *args[2:], x["dO"], beta=x["beta"], workspace=ws)
+    assert plan.last_launch_count == 3
+    # a forward pass alone with exactly the bytes it asks for
+    alone = api.sla_plan_create(cfg.variant, cfg.dtype, 1, cfg.T, 2, 128, 128)
+    arena = gu.Guarded.for_sizes([alone.forward_workspace_bytes])
+    o2, _ = api.sla_forward(alone, *args, beta=x["beta"], workspace=arena.take(alone.forward_workspace_bytes))
+    torch.cuda.synchronize()
+    plan.poll()
+    alone.poll()
+    arena.check()
+    assert torch.equal(o, o2)
+    for n, t in g.items():
+        if t is not None:
+            assert torch.equal(t, again[n]) and torch.equal(t, moved[n]), n
+
+
+# the chunk-parallel kernels (cooperative launches) and the segmented Softmax-GLA forward (its second pass starts early)
+@pytest.mark.parametrize("base,T", [("C4", 1100), ("C4", 300), ("C2", 2048)])
+def test_a_training_step_is_captured_and_replayed(base, T):
+    cfg = small(CONFIGS[base], B=1, T=T, H=3, seed=1630 + T)
+    x = gu.to_dev(make_inputs(cfg, with_dO=True, with_h0=True))
+    o, ht, g, plan, ws, lf, lb = gu.gpu_training_step(cfg, x, h0=x["h0"], dht=x["dht"], want_dh0=True)
+    args = (x["q"], x["k"], x["v"], x["log_decay"], x["gq_logits"], x["gk_logits"])
+    o2, ht2 = torch.empty_like(o), torch.empty_like(ht)
+    out = {n: None if t is None else torch.empty_like(t) for n, t in g.items()}
+    if plan.desc.T == 2048:                                      # (its tensor maps are uploaded by the first call with these buffers)
+        api.sla_backward(plan, *args, x["dO"], beta=x["beta"], h0=x["h0"], dht=x["dht"], workspace=ws, out=out)
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        api.sla_forward(plan, *args, beta=x["beta"], h0=x["h0"], o=o2, ht=ht2, workspace=ws)
+        api.sla_backward(plan, *args, x["dO"], beta=x["beta"], h0=x["h0"], dht=x["dht"], workspace=ws, out=out)
+    for _ in range(2):
+        for t in (o2, ht2, ws, *(t for t in out.values() if t is not None)):
+            t.fill_(0)
+        graph.replay()
+        torch.cuda.synchronize()
+        plan.poll()
+        assert torch.equal(o, o2) and torch.equal(ht, ht2)
+        for n, t in g.items():
+            if t is not None:
+                assert torch.equal(t, out[n]), n
+
+
 @pytest.mark.parametrize("lens", [[1100], [1088, 70]])
 def test_calls_without_a_workspace_fit_where_the_large_one_does_not(lens, monkeypatch):
     """The binding allocates the scratch of a call that brings none; where the fast kernels' does not fit, the slower kernels' serves the call."""

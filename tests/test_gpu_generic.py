@@ -119,14 +119,15 @@ def _with_decay(cfg, per_step, **kw):
     return x
 
 
-@pytest.mark.parametrize("variant,dtype,flags", [("gla", "bf16", 0), ("gdn", "bf16", 0), ("gla", "fp32", GEN),
-                                                 ("gdn", "fp32", GEN), ("retnet", "fp32", GEN)])
-def test_decay_beyond_the_chunk_range_is_reported(variant, dtype, flags):
+@pytest.mark.parametrize("variant,dtype,flags,T", [("gla", "bf16", 0, 130), ("gdn", "bf16", 0, 130), ("gla", "fp32", GEN, 130),
+                                                   ("gdn", "fp32", GEN, 130), ("retnet", "fp32", GEN, 130),
+                                                   ("gdn", "bf16", 0, 1100)])             # (1100: chunk-parallel)
+def test_decay_beyond_the_chunk_range_is_reported(variant, dtype, flags, T):
     """log_decay = -2 per token puts the cumulative log-decay of a 64-token chunk at -128, beyond what the
     e^{b} e^{-b} split can carry: the call completes, sla_plan_poll answers SLA_ERR_RANGE once, and the same plan
     works again on inputs inside the range."""
     base = {"retnet": CONFIGS["C0"], "gla": CONFIGS["C2"], "gdn": CONFIGS["C4"]}[variant]
-    cfg = small(base, B=1, T=130, H=2, d_k=128, d_v=128, dtype=dtype, seed=950, backward=True)
+    cfg = small(base, B=1, T=T, H=2, d_k=128, d_v=128, dtype=dtype, seed=950, backward=True)
     plan = api.sla_plan_create(cfg.variant, cfg.dtype, cfg.B, cfg.T, cfg.H, cfg.d_k, cfg.d_v, cfg.chunk, cfg.scale, flags)
     args = lambda x: (x["q"], x["k"], x["v"], x["log_decay"], x["gq_logits"], x["gk_logits"])
     xs = gu.to_dev(_with_decay(cfg, -2.0, with_dO=True))

@@ -135,11 +135,11 @@ def test_saved_states_are_used_only_for_the_same_inputs_and_never_change_the_res
                 assert torch.equal(t, other[n]), n
 
 
-@pytest.mark.parametrize("base", ["C2", "C4"])
-def test_saved_states_are_not_reused_once_another_backward_has_overwritten_them(base):
+@pytest.mark.parametrize("base,T", [("C2", 300), ("C4", 300), ("C4", 1100)])             # (1100: chunk-parallel Softmax-GDN)
+def test_saved_states_are_not_reused_once_another_backward_has_overwritten_them(base, T):
     """forward(A) leaves A's chunk states in the workspace; a backward for OTHER contents through the same workspace
     recomputes and overwrites them; a backward for A's pointers afterwards must recompute too (not read B's states)."""
-    cfg_a = small(CONFIGS[base], B=2, T=300, H=4, seed=911)
+    cfg_a = small(CONFIGS[base], B=2, T=T, H=4, seed=911)
     cfg_b = small(cfg_a, seed=912)
     xa_host, xb_host = make_inputs(cfg_a, with_dO=True), make_inputs(cfg_b, with_dO=True)
     xa, xb = gu.to_dev(xa_host), gu.to_dev(xb_host)
@@ -171,7 +171,8 @@ def test_saved_states_are_not_reused_once_another_backward_has_overwritten_them(
 
 
 @pytest.mark.parametrize("base,T,d", [("C2", 200, 128), ("C2", 64, 128), ("C4", 200, 128), ("C4", 65, 128),
-                                      ("C2", 200, 64), ("C2", 65, 64), ("C4", 200, 64)])
+                                      ("C2", 200, 64), ("C2", 65, 64), ("C4", 200, 64),
+                                      ("C4", 1025, 128), ("C4", 1151, 64)])             # (from 17 chunks on: chunk-parallel Softmax-GDN)
 def test_nothing_is_written_outside_the_buffers_handed_in(base, T, d):
     """In place of a memory checker: outputs and workspace are carved out of one pattern-filled arena with guard bands
     around each; after a training step and a recomputing backward no guard byte may differ, every output element must
