@@ -69,7 +69,8 @@ typedef enum { SLA_FP32 = 0, SLA_BF16 = 1 } sla_dtype;
 #define SLA_FLAG_SAVE_FOR_BACKWARD 2u
 /* Training plans: sla_forward also leaves in its workspace what the chunkwise backward pass would
  * otherwise recompute first (Softmax-GLA: the state before every chunk; Softmax-GDN: per chunk the
- * state, the corrected values U and the inverse T of the WY form).  sla_plan_workspace_bytes then
+ * state and the chunk's factors of the WY form - the inverse T, the corrected values U and, on the chunk-parallel kernels, the
+ * query-key products, W = T (beta Gam K) and the per-token factors, beside room for the state gradients).  sla_plan_workspace_bytes then
  * reports the backward size for the forward too.  A following sla_backward on the same plan that is
  * given the same workspace, the same q, k, v, log_decay, beta, logits and h0 pointers and the same
  * stream as that sla_forward uses what was left and skips its recomputation; any other call

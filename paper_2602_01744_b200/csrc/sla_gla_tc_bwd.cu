@@ -16,8 +16,8 @@
 //                     The gradient tiles are 64 x 128, token by feature, read out in the 16x256b form: a thread holds pairs
 //                     of neighbouring features, so operands and results move in 4-byte words, a token's sum over the features
 //                     takes two shuffles, and every thread has work.  (Produced transposed, one thread walked 32 tokens of
-//                     one feature in 2-byte words and every token sum was a 31-shuffle transpose.  Alone, Softmax-GLA then Softmax-RetNet,
-//                     8 x 4096 tokens x 16 heads: 403 and 380 us so, 397 and 354 us now.)  The kernel is bound by the serial
+//                     one feature in 2-byte words and every token sum was a 31-shuffle transpose.  Alone, 8 x 4096 tokens x 16 heads:
+//                     Softmax-RetNet 380 us so, 354 now; Softmax-GLA 403 and 397, within what its runs differ by.)  The kernel is bound by the serial
 //                     passes of a chunk, about 9,500 cycles of which the prologue and the gradient read-out, each limited by
 //                     instruction issue of eight warps, take 2,600 and 2,100; the tensor core is idle for most of it.
 //                     The log-decay gradient is the in-chunk suffix sum of qh*dqh - kh*dkh, taken over an fp32 tile in the
@@ -355,10 +355,11 @@ struct BwdParams {
 };
 
 // Chunks in reverse order.  Per chunk n the compute warps run: prologue -> dZ = diag(2^{b_last}) dS_{n+1} -> causal
-// mask of A and dA -> gradient tiles out of TMEM.  The MMA lane issues each product as soon as its operands exist:
-// A, dA and S_n dO^T after the prologue; dZ V^T, dZ^T kh^T and qh^T dO after the dZ pass; only the three products
-// with the masked tiles wait for the mask.  All four gradient tensors leave through staged TMA stores (rows past T
-// are clipped by the tensor map).
+// mask of A and dA -> gradient tiles out of TMEM.  The MMA warp issues each product as soon as its operands exist:
+// dA and dO S_n^T beside the prologue, A after it; V dZ^T and qh^T dO after the dZ pass; the three products with the
+// masked tiles after the mask.  kh dZ waits for the mask too: dV takes over the columns of A and dA, which AREADY says have been
+// read (and DVREAD that the next chunk's dA may come there); it is issued before the masked products, after whose commit dk is
+// written over kh.  All four gradient tensors leave through staged TMA stores (rows past T are clipped by the tensor map).
 __global__ void __launch_bounds__(st2::NTHREADS, 1)
 k_gla_bwd_tc(const __grid_constant__ CUtensorMap gm_q, const __grid_constant__ CUtensorMap gm_k,
              const __grid_constant__ CUtensorMap gm_v, const __grid_constant__ CUtensorMap gm_do,
@@ -622,7 +623,7 @@ k_gla_bwd_tc(const __grid_constant__ CUtensorMap gm_q, const __grid_constant__ C
     } else {
         // ---------------- compute warps ----------------
         const uint32_t lane_base = (uint32_t)(32 * (warp & 3)) << 16;
-        const int wh = warp >> 2;                       // column half (state passes) / token half (gradient tiles)
+        const int wh = warp >> 2;                       // column half, of the state and of the gradient tiles
         const int row = 32 * (warp & 3) + lane;         // state row of this thread (its TMEM lane)
         const int qr = warp & 3, tr = 16 * qr + (lane >> 2);       // gradient tiles: tokens tr, tr + 8
         const bool retnet = p.log_gamma != nullptr;
@@ -832,7 +833,7 @@ k_gla_bwd_tc(const __grid_constant__ CUtensorMap gm_q, const __grid_constant__ C
                     *reinterpret_cast<float4 *>(dgt + (8 * warp + ii) * D + 4 * lane) =
                         make_float4(sfx[ii].x + offs.x, sfx[ii].y + offs.y, sfx[ii].z + offs.z, sfx[ii].w + offs.w);
             }
-            if (tid < C) {   // Gq*dGq and Gk*dGk of token tid: sum over the four key-dimension quarters
+            if (tid < C) {   // Gq*dGq and Gk*dGk of token tid: sum over the two column halves
                 const int cn = min(C, p.T - t0);
                 if (tid < cn) {
                     const float sq = red[tid] + red[C + tid], sk = red[2 * C + tid] + red[3 * C + tid];
