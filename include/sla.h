@@ -114,7 +114,8 @@ sla_status sla_plan_set_sequences(sla_plan *plan, const int32_t *cu_seqlens, int
  * plan selects; 0 means none is needed and the workspace pointer may then be NULL).  A bf16 Softmax-GatedDeltaNet plan
  * with a sequence of more than 16 chunks, or more than 256 chunks x heads, reports the size for its fast kernels: 130 KiB per chunk
  * and head for a backward pass (and a forward pass that saves for it), 34 KiB for a forward pass alone.  It also accepts
- * less, and then runs on slower kernels: a backward pass (and a forward pass that saves) from 56 KiB per chunk and head on, a forward pass
+ * less (and reports less where the smaller size serves it as well: sequences of one or two chunks that fill the GPU),
+ * and then runs on slower kernels: a backward pass (and a forward pass that saves) from 56 KiB per chunk and head on, a forward pass
  * alone with any workspace or none.  (Each sequence counts as one chunk more than it has; 8 bytes per token and head, each of
  * two arrays rounded up to 256 bytes, come on top of the 130 and the 56 KiB.) */
 sla_status sla_plan_workspace_bytes(const sla_plan *plan, size_t *forward_bytes, size_t *backward_bytes);

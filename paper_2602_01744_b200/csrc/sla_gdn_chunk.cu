@@ -1555,10 +1555,10 @@ bool chunk_maps(const Dims &d, Varlen *vl, int r, const MapSpec (&spec)[N], CUte
 }  // namespace
 
 static gdn::Load chunk_load(const Dims &d, const Varlen *vl) {
-    if (vl && vl->n_seq) return {vl->seqs[0].NT, (vl->slots - vl->n_seq) * d.H, (long)vl->n_seq * d.H, d.coop_sms};      // (kept longest first)
-    return {d.NT, (long)d.B * d.H * d.NT, (long)d.B * d.H, d.coop_sms};
+    if (vl && vl->n_seq) return {vl->seqs[0].NT, (vl->slots - vl->n_seq) * d.H, (long)vl->n_seq * d.H, d.coop_sms, d.dv > 64};      // (kept longest first)
+    return {d.NT, (long)d.B * d.H * d.NT, (long)d.B * d.H, d.coop_sms, d.dv > 64};
 }
-bool gdn_chunk_selected(const Dims &d, const Varlen *vl) { return gdn::chunk_parallel(chunk_load(d, vl)); }
+bool gdn_chunk_selected(const Dims &d, const Varlen *vl) { return gdn::chunk_parallel_step(chunk_load(d, vl)); }
 bool gdn_chunk_forward_selected(const Dims &d, const Varlen *vl) { return gdn::chunk_parallel_forward(chunk_load(d, vl)); }
 
 int gdn_chunk_sms() {

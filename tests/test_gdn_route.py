@@ -11,6 +11,7 @@ SRC = r"""
 #include "sla_gdn_route.h"
 using namespace sla::gdn;
 extern "C" int train(long longest, long chunks, long seqs, long sms) { return chunk_parallel({longest, chunks, seqs, sms}); }
+extern "C" int step(long longest, long chunks, long seqs, long sms, int wide) { return chunk_parallel_step({longest, chunks, seqs, sms, wide != 0}); }
 extern "C" int forward(long longest, long chunks, long seqs, long sms) { return chunk_parallel_forward({longest, chunks, seqs, sms}); }
 // the answers of the two forms' launches; returns the call's, and in *form 1 if the chunk-parallel form ran, in *calls how many were tried
 extern "C" int call(int chunked, int chunk_answer, int one_cta_answer, int *form, int *calls) {
@@ -32,6 +33,7 @@ def route(tmp_path_factory):
     L = ctypes.CDLL(str(d / "route.so"))
     for f in (L.train, L.forward):
         f.argtypes = [ctypes.c_long] * 4
+    L.step.argtypes = [ctypes.c_long] * 4 + [ctypes.c_int]
     return L
 
 
@@ -46,6 +48,14 @@ def test_without_a_cooperative_grid_every_call_stays_on_the_one_cta_kernels(rout
                                                 ((2, 288, 144), 1, 0), ((1, 65535, 65535), 1, 0)])
 def test_the_rules_lines(route, load, train, forward):
     assert (route.train(*load, 148), route.forward(*load, 148)) == (train, forward)
+
+
+# a step of one chunk a sequence, or of two in one wave, where the sequences fill the SMs: 128-wide values, 64-wide ones
+@pytest.mark.parametrize("load,wide,narrow", [((1, 257, 257), 0, 1), ((1, 8192, 8192), 0, 1), ((1, 320, 320), 1, 1), ((2, 288, 144), 0, 1), ((2, 320, 160), 1, 1),
+                                              ((2, 576, 288), 1, 1), ((3, 432, 144), 1, 1), ((1, 256, 256), 0, 0), ((17, 17, 1), 1, 1)])
+def test_steps_over_sequences_of_a_chunk_or_two(route, load, wide, narrow):
+    assert (route.step(*load, 148, 1), route.step(*load, 148, 0)) == (wide, narrow)
+    assert not route.step(*load, 0, 1)
 
 
 def test_a_refused_cooperative_launch_leaves_the_call_to_the_one_cta_kernels(route):

@@ -72,7 +72,8 @@ def test_chunk_parallel_packed_batch_gives_the_bits_of_its_sequences_alone():
 
 
 # sequences of up to 8 chunks that fill the SMs (to four fifths of whole waves: 144 and 288 sequences; 128 of 9 chunks and 160 of 2 do not
-# count): a forward pass alone needs no workspace, a training step over the same tensors is chunk-parallel all the same
+# count): a forward pass alone needs no workspace, a training step over the same tensors is chunk-parallel all the same (from two chunks in
+# more than one wave on)
 @pytest.mark.parametrize("B,T,H,alone", [(9, 128, 16, True), (18, 512, 16, True), (8, 513, 16, False), (10, 128, 16, False)])
 def test_short_sequences_that_fill_the_chip_run_forward_without_workspace(B, T, H, alone):
     cfg = small(CONFIGS["C4"], B=B, T=T, H=H, seed=1700 + B)
