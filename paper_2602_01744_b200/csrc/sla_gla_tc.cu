@@ -14,7 +14,7 @@
 // A and O are 64-row accumulators, which occupy only the lower 16 lanes of each warp's quarter of TMEM: the 16x256b loads hand
 // them to all 32 threads of a warp as pairs of neighbouring columns, where a load of one lane a thread leaves half the threads
 // without work and twice the instructions to the others (1 x 65536 tokens x 16 heads: 345 -> 307 us for this kernel, with one
-// mbarrier arrival a warp instead of 32; 8 x 4096 x 16: 188 -> 183 us, Softmax-RetNet 172 -> 165 us).
+// mbarrier arrival a warp instead of 32; 8 x 4096 x 16: 188 -> 183 us, Softmax-RetNet 172 -> 165 us; 156 with its prologue by rows).
 // The state never leaves the SM: fp32 in TMEM (Eq. 12's S), bf16 copy in shared memory as MMA operand.
 #include "sla_gla_tc.cuh"
 
@@ -61,7 +61,7 @@ struct FwdParams {
     int T, H, NT;
     int P, L;                       // segments per sequence and chunks per segment (P = 1: L = NT)
     float scale;
-    const float *log_gamma;         // Softmax-RetNet: [H] constant log-decays (no log-decay tensor is read); else nullptr
+    const float *log_gamma;         // SCALAR: [H] constant log-decays (no log-decay tensor is read)
     const SeqInfo *seqs;            // packed variable-length batch: per-sequence table and tensor maps (q, k, v, g, o), else nullptr
     const CUtensorMap *vmaps;
     int dk, dv;             // head widths, each 128 or 64 (the upper half of a 128-wide tile is then zero padding)
@@ -75,6 +75,8 @@ struct FwdParams {
 //   warps 17..20       head-softmax gates (Eq. 4) up to four chunks ahead, one thread per (token, gate)
 // The prologue of chunk n+1.. runs beside the mask / rescale / store work of chunk n, so the shared-memory,
 // special-function and FMA phases of the two groups overlap instead of following one another.
+// SCALAR: Softmax-RetNet, whose gate warps fold the constant decay into the gates and whose prologue only scales rows.
+template <bool SCALAR>
 __global__ void __launch_bounds__(NTHREADS, 1)
 k_gla_fwd_tc(const __grid_constant__ CUtensorMap gm_q, const __grid_constant__ CUtensorMap gm_k,
              const __grid_constant__ CUtensorMap gm_v, const __grid_constant__ CUtensorMap gm_g,
@@ -262,11 +264,15 @@ k_gla_fwd_tc(const __grid_constant__ CUtensorMap gm_q, const __grid_constant__ C
         const int g = tid - 32 * W_GATE, t = g & (C - 1);
         const float *l = g < C ? p.lq : p.lk;
         const float mult = g < C ? p.scale : 1.f;
+        const float lg = SCALAR ? (g < C ? LOG2E : -LOG2E) * p.log_gamma[h] : 0.f;
         for (int n = 0; n < NT; ++n) {
             if (n >= 4) wait_relaxed(GFREE + (n & 3), ((n >> 2) - 1) & 1);
             if (failed) break;
             const int cn = min(C, p.T - (n0 + n) * C);
-            chunk_gate(l + (tokb + (size_t)(n0 + n) * C) * p.H, p.H, cn, h, mult, gate_s + (n & 3) * 2 * C + (g < C ? 0 : C), t);
+            const float *lc = l + (tokb + (size_t)(n0 + n) * C) * p.H;
+            float *dst = gate_s + (n & 3) * 2 * C + (g < C ? 0 : C);
+            if (SCALAR) chunk_gate_by(lc, p.H, cn, h, DecayFactor{mult, lg}, dst, t);
+            else chunk_gate(lc, p.H, cn, h, mult, dst, t);
             __syncwarp();
             if (lane == 0) mbar_arrive(bar(GREADY + (n & 3)));
         }
@@ -277,21 +283,24 @@ k_gla_fwd_tc(const __grid_constant__ CUtensorMap gm_q, const __grid_constant__ C
             mbar_expect_tx(bar(FULL_G), TILE_G);
             tma_load_4d(base + OFF_G, &tm_g, 0, h, (n0 + n) * C, b, bar(FULL_G));
         };
-        const bool retnet = p.log_gamma != nullptr;
-        const float lgam = retnet ? p.log_gamma[h] : 0.f;
-        if (ptid == 0 && !retnet) load_g(0);
+        if (ptid == 0 && !SCALAR) load_g(0);
+        if (ptid == 0 && SCALAR) check_scalar_range(p.log_gamma[h], p.T, p.status);
         for (int n = 0; n < NT; ++n) {
             wait(GREADY + (n & 3), (n >> 2) & 1);
-            if (!retnet) wait(FULL_G, n & 1);
+            if (!SCALAR) wait(FULL_G, n & 1);
             wait(FULL_QK + n % 3, (n / 3) & 1);
             if (failed) break;
             uint8_t *qk = sm + OFF_QK + (n % 3) * QK_BYTES;
             const float *g = gate_s + (n & 3) * 2 * C;
             // eblast has four slots: these warps are never more than three chunks ahead of the rescale that reads one
-            chunk_prologue<true, false>(qk, qk + TILE_BF16, retnet ? nullptr : reinterpret_cast<const float *>(sm + OFF_G), tot, g, g + C,
-                                        eblast + (n & 3) * D, nullptr, p.status, ptid, 2,
-                                        [&]() { if (ptid == 0 && n + 1 < NT && !retnet) load_g(n + 1); },
-                                        ScalarDecay{lgam, min(C, p.T - (n0 + n) * C)});
+            if (SCALAR) {
+                scale_rows(qk, g, ptid);
+                scale_rows(qk + TILE_BF16, g + C, ptid);
+            } else {
+                chunk_prologue<true, false>(qk, qk + TILE_BF16, reinterpret_cast<const float *>(sm + OFF_G), tot, g, g + C,
+                                            eblast + (n & 3) * D, nullptr, p.status, ptid, 2,
+                                            [&]() { if (ptid == 0 && n + 1 < NT) load_g(n + 1); });
+            }
             fence_proxy_async();
             mbar_arrive(bar(OPR + n % 3));
             mbar_arrive(bar(GFREE + (n & 3)));
@@ -301,6 +310,7 @@ k_gla_fwd_tc(const __grid_constant__ CUtensorMap gm_q, const __grid_constant__ C
         const uint32_t lane_base = (uint32_t)(32 * (warp & 3)) << 16;   // this warp's TMEM lane quarter
         const int colhalf = warp >> 2;                                   // which 64 state / output columns
         const int row = 32 * (warp & 3) + lane;
+        const float lg = SCALAR ? LOG2E * p.log_gamma[h] : 0.f;
 
         {   // initial state: fp32 into TMEM, bf16 copy into shared memory (row = key dimension).  A segment that is not the
             // first starts from S <- diag(gam_s) S + fin_s taken over the segments s before it (a short scan over their
@@ -393,7 +403,7 @@ k_gla_fwd_tc(const __grid_constant__ CUtensorMap gm_q, const __grid_constant__ C
             tc_fence_after();
             if (p.simg) wait(SSAVED, par);             // the image store of S_n has read the operand copy
             {
-                const float e = eblast[(n & 3) * D + row];
+                const float e = SCALAR ? ex2f(lg * (float)min(C, p.T - (n0 + n) * C)) : eblast[(n & 3) * D + row];
 #pragma unroll
                 for (int part = 0; part < 2; ++part) {
                     float v[32];
@@ -476,15 +486,16 @@ void choose_segments(const Dims &d, int &P, int &L) {
 }  // namespace
 
 // Softmax-GLA (Eq. 12-13) and Softmax-RetNet (Eq. 10-11: the same recurrence with a constant decay per head, which the
-// kernels generate instead of reading a [B,T,H,d_k] tensor).
+// gate warps multiply into the gates instead of reading a [B,T,H,d_k] tensor).
 bool gla_tc_supported(const Dims &d) {
     return (d.variant == SLA_GLA || d.variant == SLA_RETNET) && d.io_bf16 && (d.dk == 128 || d.dk == 64) && (d.dv == 128 || d.dv == 64) && d.C == 64;
 }
 
 int gla_tc_configure() {
     if (!encode_fn()) return -1;
-    return cudaFuncSetAttribute(k_gla_fwd_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_BYTES) ==
-                   cudaSuccess ? 0 : -1;
+    constexpr cudaFuncAttribute A = cudaFuncAttributeMaxDynamicSharedMemorySize;
+    return cudaFuncSetAttribute(k_gla_fwd_tc<false>, A, (int)SMEM_BYTES) == cudaSuccess &&
+                   cudaFuncSetAttribute(k_gla_fwd_tc<true>, A, (int)SMEM_BYTES) == cudaSuccess ? 0 : -1;
 }
 
 // The backward runs the gradient sweep twice when it is cut into segments (once for the state gradients that leave
@@ -511,6 +522,7 @@ bool gla_tc_forward_can_save(const Dims &d, const Varlen *vl) {
 int gla_tc_forward(const Dims &d, const FwdArgs &a, uint8_t *simg, int *status, cudaStream_t st, Tracer &tr) {
     CUtensorMap mq, mk, mv, mg, mo;
     const bool retnet = d.variant == SLA_RETNET;
+    auto *const kernel = retnet ? k_gla_fwd_tc<true> : k_gla_fwd_tc<false>;
     if (a.vl && a.vl->n_seq) {          // packed batch: one CTA per (sequence, head), per-sequence tensor maps
         const void *key[] = {a.q, a.k, a.v, a.log_decay, a.o};
         const CUtensorMap *vm = varlen_maps(*a.vl, 0, key, 5, st, [&](const SeqInfo &si, CUtensorMap *m) {
@@ -525,7 +537,7 @@ int gla_tc_forward(const Dims &d, const FwdArgs &a, uint8_t *simg, int *status, 
         if (!vm || !make_tile_map(&mq, a.q, d.B, d.T, d.H, d.dk)) return -1;
         FwdParams p{a.lq, a.lk, a.h0, nullptr, nullptr, (__nv_bfloat16 *)a.o, a.ht, simg, status, d.T, d.H, d.NT, 1, d.NT, d.scale,
                     retnet ? a.log_decay : nullptr, a.vl->d_seqs, vm, d.dk, d.dv};
-        k_gla_fwd_tc<<<a.vl->n_seq * d.H, NTHREADS, SMEM_BYTES, st>>>(mq, mq, mq, mq, mq, p);
+        kernel<<<a.vl->n_seq * d.H, NTHREADS, SMEM_BYTES, st>>>(mq, mq, mq, mq, mq, p);
         tr.mark("gla_fwd_tc");
         return cudaGetLastError() == cudaSuccess ? 1 : -1;
     }
@@ -561,7 +573,7 @@ int gla_tc_forward(const Dims &d, const FwdArgs &a, uint8_t *simg, int *status, 
     cfg.stream = st;
     cfg.attrs = &early;
     cfg.numAttrs = P > 1 ? 1 : 0;
-    if (cudaLaunchKernelEx(&cfg, k_gla_fwd_tc, mq, mk, mv, mg, mo, p) != cudaSuccess) return -1;
+    if (cudaLaunchKernelEx(&cfg, kernel, mq, mk, mv, mg, mo, p) != cudaSuccess) return -1;
     tr.mark("gla_fwd_tc");
     return cudaGetLastError() == cudaSuccess ? launches : -1;
 }

@@ -162,8 +162,8 @@ __device__ __forceinline__ float ex2f(float x) {
 constexpr uint32_t NCOMPUTE = 256;      // compute threads (warps 0..7); they meet on named barrier 1
 constexpr float LOG2E = 1.4426950408889634f;
 
-// Chunk prologue, run by 256 threads (tid 0..255, meeting on named barrier bar_id) on one landed stage (the decay of Eq. 12, or of
-// Eq. 10 when gs is null, made chunk-local):
+// Chunk prologue of Softmax-GLA, run by 256 threads (tid 0..255, meeting on named barrier bar_id) on one landed stage (the decay of
+// Eq. 12 made chunk-local):
 //   b_i = inclusive cumulative log-decay (kept in log2 units), two-level: per-8-row sums, then a running sum
 //   qh_i = gq_i * q_i * 2^{b_i}   (gq_i = scale*Gq_i)      kh_i = gk_i * k_i * 2^{-b_i}
 // written over q and k in place (the swizzled tiles are the MMA operands); eblast[d] = 2^{b_last,d}.
@@ -177,14 +177,11 @@ constexpr uint32_t TOT_BYTES = 8 * D * 4;
 // bytes of each of eight rows at once, which without the swizzle all sit in the same banks
 __device__ __forceinline__ uint32_t e2_off(uint32_t row, uint32_t chunk) { return row * (D * 4) + ((chunk ^ ((row & 3) << 1)) << 4); }
 struct NoHook { __device__ __forceinline__ void operator()() const {} };
-// Softmax-RetNet runs on the same kernels: with gs == nullptr the chunk's log-decay tile is not read but generated,
-// log_gamma on each of the chunk's cn tokens (all key dimensions alike).
-struct ScalarDecay { float log_gamma = 0.f; int cn = 0; };
 template <bool WITH_Q, bool WITH_E, class Hook = NoHook>
 __device__ __forceinline__ void chunk_prologue(uint8_t *q_tile, uint8_t *k_tile, const float *gs, float *tot,
                                                const float *gq_s, const float *gk_s, float *eblast,
                                                uint8_t *e2_tile, int *status, int tid, int bar_id = 1,
-                                               Hook tile_read = Hook(), ScalarDecay sc = ScalarDecay()) {
+                                               Hook tile_read = Hook()) {
     using namespace ptx;
     const int rg = tid >> 5, cj = tid & 31;
     float4 gl[8];                               // this thread's log-decay rows: read once, kept for the second pass
@@ -192,12 +189,7 @@ __device__ __forceinline__ void chunk_prologue(uint8_t *q_tile, uint8_t *k_tile,
         float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
         for (int rr = 0; rr < 8; ++rr) {
-            if (gs) {
-                gl[rr] = *reinterpret_cast<const float4 *>(gs + (8 * rg + rr) * D + 4 * cj);
-            } else {                            // Eq. 10: one constant log-decay per head, none past the sequence end
-                const float v = 8 * rg + rr < sc.cn ? sc.log_gamma : 0.f;
-                gl[rr] = make_float4(v, v, v, v);
-            }
+            gl[rr] = *reinterpret_cast<const float4 *>(gs + (8 * rg + rr) * D + 4 * cj);
             acc.x += gl[rr].x; acc.y += gl[rr].y; acc.z += gl[rr].z; acc.w += gl[rr].w;
         }
         *reinterpret_cast<float4 *>(tot + rg * D + 4 * cj) = acc;
@@ -266,6 +258,37 @@ __device__ __forceinline__ void chunk_prologue(uint8_t *q_tile, uint8_t *k_tile,
     }
 }
 
+// Chunk prologue of Softmax-RetNet (Eq. 10: one constant log-decay per head).  All key dimensions of a token share one factor,
+// which the gate warps have already multiplied into its gates (DecayFactor): f_i = scale*Gq_i 2^{b_i} or Gk_i 2^{-b_i}, so a tile
+// becomes qh or kh by scaling its rows - no log-decay tile, no scan, no exponential an element.  256 threads, a thread every
+// fourth 16-byte chunk of one row (the rows of a pair start in opposite halves of a swizzled line: no bank is asked twice).
+__device__ __forceinline__ void scale_rows(uint8_t *tile, const float *f, int tid) {
+    using namespace ptx;
+    const int r = tid >> 2;
+    const float g = f[r];
+    uint8_t *at = tile + swz(r, (tid & 3) + 4 * (r & 1));
+#pragma unroll
+    for (int hf = 0; hf < 2; ++hf, at += HALF_BF16) {
+        uint8_t *other = reinterpret_cast<uint8_t *>(reinterpret_cast<uintptr_t>(at) ^ 64);      // the chunk four further (tiles are 1 KiB aligned)
+        uint4 v[2] = {*reinterpret_cast<const uint4 *>(at), *reinterpret_cast<const uint4 *>(other)};
+#pragma unroll
+        for (int x = 0; x < 2; ++x) {
+            uint32_t *w = reinterpret_cast<uint32_t *>(&v[x]);
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const float2 y = unpack_bf16(w[e]);
+                w[e] = pack_bf16(g * y.x, g * y.y);
+            }
+        }
+        *reinterpret_cast<uint4 *>(at) = v[0];
+        *reinterpret_cast<uint4 *>(other) = v[1];
+    }
+}
+// A sequence's first chunk is its longest: raises STATUS_RANGE if its cumulative log-decay is beyond the range of 2^{b}, 2^{-b}.
+__device__ __forceinline__ void check_scalar_range(float log_gamma, int T, int *status) {
+    if (log_gamma * (float)min(C, T) < -SLA_MAX_CHUNK_DECAY) atomicOr(status, STATUS_RANGE);
+}
+
 // Head-softmax gate (Eq. 4) of ONE token for head h: the H <= HP logits are fetched before the first use (one memory
 // round trip), then max, exp and sum run over registers.  Returns softmax(row[0..H))[h].
 template <int HP>
@@ -305,10 +328,19 @@ __device__ __forceinline__ void gate_fetch(const float *__restrict__ L, int cn, 
         x[i] = f / LPT < cn ? __ldg(reinterpret_cast<const float4 *>(L) + f) : make_float4(0.f, 0.f, 0.f, 0.f);
     }
 }
-// finish: softmax over the H/4 lanes of every token, dst[token] = mult * G[token][h].  Stage by stage over all of the
+// What a gate is multiplied with on its way out: a constant, or (a constant decay per head) also 2^{lg (token + 1)}.
+struct ConstFactor {
+    float mult;
+    __device__ __forceinline__ float operator()(int) const { return mult; }
+};
+struct DecayFactor {
+    float mult, lg;
+    __device__ __forceinline__ float operator()(int token) const { return mult * ex2f(lg * (float)(token + 1)); }
+};
+// finish: softmax over the H/4 lanes of every token, dst[token] = mult(token) * G[token][h].  Stage by stage over all of the
 // thread's float4s, so that the shuffles and exponentials of different tokens overlap.
-template <int LPT, int NTH>
-__device__ __forceinline__ void gate_finish(float4 (&x)[LPT * 64 / NTH], int cn, int h, float mult, float *dst, int t) {
+template <int LPT, int NTH, class Mult>
+__device__ __forceinline__ void gate_finish(float4 (&x)[LPT * 64 / NTH], int cn, int h, Mult mult, float *dst, int t) {
     constexpr int NF = LPT * 64 / NTH;
     float m[NF], sum[NF];
 #pragma unroll
@@ -335,28 +367,49 @@ __device__ __forceinline__ void gate_finish(float4 (&x)[LPT * 64 / NTH], int cn,
         for (int i = 0; i < NF; ++i) {
             const int token = (i * NTH + t) / LPT;
             const float eh = j == 0 ? x[i].x : j == 1 ? x[i].y : j == 2 ? x[i].z : x[i].w;
-            dst[token] = token < cn ? mult * __fdividef(eh, sum[i]) : 0.f;
+            dst[token] = token < cn ? mult(token) * __fdividef(eh, sum[i]) : 0.f;
         }
     }
 }
-template <int LPT, int NTH>
-__device__ __forceinline__ void chunk_gate_vec(const float *__restrict__ L, int cn, int h, float mult, float *dst, int t) {
+template <int LPT, int NTH, class Mult>
+__device__ __forceinline__ void chunk_gate_vec(const float *__restrict__ L, int cn, int h, Mult mult, float *dst, int t) {
     float4 x[LPT * 64 / NTH];
     gate_fetch<LPT, NTH>(L, cn, t, x);
-    gate_finish<LPT, NTH>(x, cn, h, mult, dst, t);
+    gate_finish<LPT, NTH, Mult>(x, cn, h, mult, dst, t);
 }
 // NTH = 64 (threads t = 0..63, two whole warps) or 32 (one warp) serve one gate of one chunk.
-template <int NTH = 64>
-__device__ __forceinline__ void chunk_gate(const float *L, int H, int cn, int h, float mult, float *dst, int t) {
+template <int NTH = 64, class Mult>
+__device__ __forceinline__ void chunk_gate_by(const float *L, int H, int cn, int h, Mult mult, float *dst, int t) {
     if (H == 16) chunk_gate_vec<4, NTH>(L, cn, h, mult, dst, t);
     else if (H == 8) chunk_gate_vec<2, NTH>(L, cn, h, mult, dst, t);
     else if (H == 4) chunk_gate_vec<1, NTH>(L, cn, h, mult, dst, t);
     else if (H == 32) chunk_gate_vec<8, NTH>(L, cn, h, mult, dst, t);
     else {
-        for (int i = t; i < C; i += NTH) dst[i] = i < cn ? mult * token_gate_any(L + (size_t)i * H, H, h) : 0.f;
+        for (int i = t; i < C; i += NTH) dst[i] = i < cn ? mult(i) * token_gate_any(L + (size_t)i * H, H, h) : 0.f;
     }
 }
+template <int NTH = 64>
+__device__ __forceinline__ void chunk_gate(const float *L, int H, int cn, int h, float mult, float *dst, int t) {
+    chunk_gate_by<NTH>(L, H, cn, h, ConstFactor{mult}, dst, t);
+}
 constexpr int NGATE = 128;   // gate threads: g < 64 -> scale*Gq of token g, g >= 64 -> Gk of token g-64
+
+// ---- the gradient sweep's parameters, Softmax-GLA (sla_gla_tc_bwd.cu) and Softmax-RetNet (sla_retnet_tc_bwd.cu) ----
+struct BwdParams {
+    const float *lq, *lk, *dht;
+    const uint8_t *simg;
+    float *pq, *pk, *dh0;          // pq = Gq*dGq, pk = Gk*dGk per (token, head)
+    int *status;
+    int T, H, NT;
+    float scale;
+    const float *log_gamma;         // Softmax-RetNet: [H] constant log-decays (no log-decay read, no log-decay gradient)
+    const SeqInfo *seqs;            // packed variable-length batch: per-sequence table and tensor maps (the nine below), else nullptr
+    const CUtensorMap *vmaps;       // q, k, v, dO, log-decay, dq, dk, dv, dlog_decay (Softmax-RetNet: neither of the decay's)
+    int dk, dv;             // head widths, each 128 or 64 (the upper half of a 128-wide tile is then zero padding)
+};
+// maps: q, k, v, dO, dq, dk, dv
+int retnet_tc_bwd_configure();
+void retnet_tc_bwd_launch(const CUtensorMap (&maps)[7], const BwdParams &p, int ctas, cudaStream_t st);
 
 }  // namespace tc
 }  // namespace sla

@@ -17,7 +17,8 @@
 //                     of neighbouring features, so operands and results move in 4-byte words, a token's sum over the features
 //                     takes two shuffles, and every thread has work.  (Produced transposed, one thread walked 32 tokens of
 //                     one feature in 2-byte words and every token sum was a 31-shuffle transpose.  Alone, 8 x 4096 tokens x 16 heads:
-//                     Softmax-RetNet 380 us so, 354 now; Softmax-GLA 403 and 397, within what its runs differ by.)  The kernel is bound by the serial
+//                     403 us so, 397 token by feature, 378 since Softmax-RetNet has a kernel of its own, sla_retnet_tc_bwd.cu, and its branches
+//                     no longer cost this one registers.)  The kernel is bound by the serial
 //                     passes of a chunk, about 9,500 cycles of which the prologue and the gradient read-out, each limited by
 //                     instruction issue of eight warps, take 2,600 and 2,100; the tensor core is idle for most of it.
 //                     The log-decay gradient is the in-chunk suffix sum of qh*dqh - kh*dkh, taken over an fp32 tile in the
@@ -66,7 +67,7 @@ struct StatesParams {
     int T, H, NT;
     int P, L;               // segments per sequence and chunks per segment (image mode: P = 1, L = NT)
     int PS;                 // of them, from the first on, run (the grid has PS CTAs per sequence)
-    const float *log_gamma; // Softmax-RetNet: [H] constant log-decays (no log-decay tensor is read); else nullptr
+    const float *log_gamma; // SCALAR: [H] constant log-decays (no log-decay tensor is read)
     const SeqInfo *seqs;    // packed variable-length batch: per-sequence table and tensor maps (k, v, g), else nullptr
     const CUtensorMap *vmaps;
     int dk, dv;             // head widths, each 128 or 64 (the upper half of a 128-wide tile is then zero padding)
@@ -90,6 +91,8 @@ __device__ __forceinline__ void store_state_part(uint8_t *img, int row, int colh
 // Summary mode (simg == nullptr) serves the segmented forward of long sequences: every CTA runs one segment of a
 // sequence from a zero state and leaves only where it ended and the segment's total decay; a scan over the segments
 // then gives every segment its true starting state.
+// SCALAR: Softmax-RetNet (its constant decay comes in with the gates; the prologue only scales rows).
+template <bool SCALAR>
 __global__ void __launch_bounds__(st1::NTHREADS, 1)
 k_gla_states_tc(const __grid_constant__ CUtensorMap gm_k, const __grid_constant__ CUtensorMap gm_v,
                 const __grid_constant__ CUtensorMap gm_g, StatesParams p) {
@@ -190,12 +193,11 @@ k_gla_states_tc(const __grid_constant__ CUtensorMap gm_k, const __grid_constant_
                 mbar_expect_tx(bf, TILE_BF16);
                 tma_load_5d(base + OFF_V + (n & 1) * TILE_BF16, &tm_v, 0, (n0 + n) * C, 0, h, b, bf);
             };
-            const bool retnet = p.log_gamma != nullptr;
-            for (int n = 0; n < 2 && n < NT && !retnet; ++n) load_g(n);
+            for (int n = 0; n < 2 && n < NT && !SCALAR; ++n) load_g(n);
             for (int n = 0; n < 3 && n < NT; ++n) load_k(n);
             for (int n = 0; n < 2 && n < NT; ++n) load_v(n);
             for (int n = 0; n < NT && !failed; ++n) {
-                if (n + 2 < NT && !retnet) {         // log-decay buffer: free once the prologue of chunk n is done
+                if (n + 2 < NT && !SCALAR) {         // log-decay buffer: free once the prologue of chunk n is done
                     wait(OPR + n % 3, (n / 3) & 1);
                     if (failed) break;
                     load_g(n + 2);
@@ -227,11 +229,14 @@ k_gla_states_tc(const __grid_constant__ CUtensorMap gm_k, const __grid_constant_
     } else if (warp >= 9) {
         // ---------------- gates (Gk only), up to four chunks ahead ----------------
         const int t = tid - (NCOMPUTE + 32);
+        const float lg = SCALAR ? -LOG2E * p.log_gamma[h] : 0.f;
         for (int n = 0; n < NT; ++n) {
             if (n >= 4) wait_relaxed(GFREE + (n & 3), ((n >> 2) - 1) & 1);
             if (failed) break;
             const int cn = min(C, p.T - (n0 + n) * C);
-            chunk_gate(p.lk + (tokb + (size_t)(n0 + n) * C) * p.H, p.H, cn, h, 1.f, gate_s + (n & 3) * C, t);
+            const float *lc = p.lk + (tokb + (size_t)(n0 + n) * C) * p.H;
+            if (SCALAR) chunk_gate_by(lc, p.H, cn, h, DecayFactor{1.f, lg}, gate_s + (n & 3) * C, t);
+            else chunk_gate(lc, p.H, cn, h, 1.f, gate_s + (n & 3) * C, t);
             __syncwarp();
             if (lane == 0) mbar_arrive(bar(GREADY + (n & 3)));
         }
@@ -254,16 +259,16 @@ k_gla_states_tc(const __grid_constant__ CUtensorMap gm_k, const __grid_constant_
         tc_fence_before();
         mbar_arrive(bar(SREADY));
 
-        const bool retnet = p.log_gamma != nullptr;
-        const float lgam = retnet ? p.log_gamma[h] : 0.f;
+        const float lg = SCALAR ? LOG2E * p.log_gamma[h] : 0.f;
+        if (SCALAR && tid == 0) check_scalar_range(p.log_gamma[h], p.T, p.status);
         auto prologue = [&](int n) {
             wait(GREADY + (n & 3), (n >> 2) & 1);
-            if (!retnet) wait(FULL_G + (n & 1), (n >> 1) & 1);
+            if (!SCALAR) wait(FULL_G + (n & 1), (n >> 1) & 1);
             wait(FULL_K + n % 3, (n / 3) & 1);
-            chunk_prologue<false, false>(nullptr, sm + OFF_K + (n % 3) * TILE_BF16,
-                                         retnet ? nullptr : reinterpret_cast<const float *>(sm + OFF_G + (n & 1) * TILE_G), tot, nullptr,
-                                         gate_s + (n & 3) * C, eblast + (n & 1) * D, nullptr, p.status, tid, 1, NoHook(),
-                                         ScalarDecay{lgam, min(C, p.T - (n0 + n) * C)});
+            uint8_t *kt = sm + OFF_K + (n % 3) * TILE_BF16;
+            if (SCALAR) scale_rows(kt, gate_s + (n & 3) * C, tid);
+            else chunk_prologue<false, false>(nullptr, kt, reinterpret_cast<const float *>(sm + OFF_G + (n & 1) * TILE_G), tot, nullptr,
+                                              gate_s + (n & 3) * C, eblast + (n & 1) * D, nullptr, p.status, tid);
             fence_proxy_async();
             mbar_arrive(bar(OPR + n % 3));
             mbar_arrive(bar(GFREE + (n & 3)));
@@ -275,7 +280,7 @@ k_gla_states_tc(const __grid_constant__ CUtensorMap gm_k, const __grid_constant_
             wait(BAR_Z, n & 1);
             tc_fence_after();
             {   // S_{n+1} = diag(2^{b_last}) (S_n + kh^T V): fp32 back into TMEM, bf16 image staged for slot n+1
-                const float e = eblast[(n & 1) * D + row];
+                const float e = SCALAR ? ex2f(lg * (float)min(C, p.T - (n0 + n) * C)) : eblast[(n & 1) * D + row];
                 gam *= e;
                 float v0[32], v1[32];
                 const uint32_t ta = tmem + lane_base + 64 * colhalf;
@@ -340,19 +345,6 @@ enum Bar { FULL_G = 0, FULL_QK, FULL_V, FULL_DO, FULL_S, OPR, GREADY /*[4]*/, GF
 static_assert(SMEM_BYTES <= 232448, "shared memory budget");
 static_assert(NBAR <= 32, "barrier slots");
 }  // namespace st2
-
-struct BwdParams {
-    const float *lq, *lk, *dht;
-    const uint8_t *simg;
-    float *pq, *pk, *dh0;          // pq = Gq*dGq, pk = Gk*dGk per (token, head)
-    int *status;
-    int T, H, NT;
-    float scale;
-    const float *log_gamma;         // Softmax-RetNet: [H] constant log-decays (no log-decay read, no log-decay gradient)
-    const SeqInfo *seqs;            // packed variable-length batch: per-sequence table and tensor maps (the nine below), else nullptr
-    const CUtensorMap *vmaps;
-    int dk, dv;             // head widths, each 128 or 64 (the upper half of a 128-wide tile is then zero padding)
-};
 
 // Chunks in reverse order.  Per chunk n the compute warps run: prologue -> dZ = diag(2^{b_last}) dS_{n+1} -> causal
 // mask of A and dA -> gradient tiles out of TMEM.  The MMA warp issues each product as soon as its operands exist:
@@ -552,12 +544,11 @@ k_gla_bwd_tc(const __grid_constant__ CUtensorMap gm_q, const __grid_constant__ C
                 mbar_expect_tx(bar(FULL_S), STATE_BF16);
                 bulk_load(base + OFF_S, img0 + (size_t)n * STATE_BF16, STATE_BF16, bar(FULL_S));
             };
-            const bool retnet = p.log_gamma != nullptr;
             if (p.dht) {                               // S_NT, for rowsum(dht * S_NT)
                 mbar_expect_tx(bar(INIT_FULL), STATE_BF16);
                 bulk_load(base + OFF_S, img0 + (size_t)NT * STATE_BF16, STATE_BF16, bar(INIT_FULL));
             }
-            if (!retnet) load_g(NT - 1);
+            load_g(NT - 1);
             load_qk(NT - 1, 0);
             load_vdo(NT - 1, 0);
             if (p.dht) wait(INIT_DONE, 0);             // the compute warps are done with S_NT
@@ -575,7 +566,7 @@ k_gla_bwd_tc(const __grid_constant__ CUtensorMap gm_q, const __grid_constant__ C
                     bulk_prefetch_l2(img0 + (size_t)(n - 1) * STATE_BF16, STATE_BF16);
                     wait(OPR, par);                    // prologue done: the log-decay buffer is free
                     if (failed) break;
-                    if (!retnet) load_g(n - 1);
+                    load_g(n - 1);
                     wait(DOFREE, par);                 // every MMA of the chunk is done: its (v, dO) buffer takes the next q, k
                     if (failed) break;
                     load_qk(n - 1, k + 1);
@@ -595,7 +586,7 @@ k_gla_bwd_tc(const __grid_constant__ CUtensorMap gm_q, const __grid_constant__ C
                 wait(OUT2, par);                       // dv, dlog_decay staged
                 if (failed) break;
                 tma_store_5d(&tm_dv, base + OFF_A, 0, n * C, 0, h, b);
-                if (!retnet) tma_store_4d(&tm_dg, base + OFF_DZ, 0, h, n * C, b);
+                tma_store_4d(&tm_dg, base + OFF_DZ, 0, h, n * C, b);
                 bulk_commit();
                 bulk_wait_read0();
                 mbar_arrive(bar(DGFREE));
@@ -626,8 +617,6 @@ k_gla_bwd_tc(const __grid_constant__ CUtensorMap gm_q, const __grid_constant__ C
         const int wh = warp >> 2;                       // column half, of the state and of the gradient tiles
         const int row = 32 * (warp & 3) + lane;         // state row of this thread (its TMEM lane)
         const int qr = warp & 3, tr = 16 * qr + (lane >> 2);       // gradient tiles: tokens tr, tr + 8
-        const bool retnet = p.log_gamma != nullptr;
-        const float lgam = retnet ? p.log_gamma[h] : 0.f;
 
         // rowsum(dS * S) over this thread's 64 columns, with dS in registers part by part
         auto rowdot_part = [&](const float (&v)[32], int part) {
@@ -668,13 +657,12 @@ k_gla_bwd_tc(const __grid_constant__ CUtensorMap gm_q, const __grid_constant__ C
             uint8_t *qk = sm + ((k & 1) ? OFF_Y : OFF_X);          // this chunk's q, k tiles
             // ---- prologue: cumulative decay, qh, kh in place, the (gq 2^b, gk 2^-b) tile ----
             wait(GREADY + (k & 3), (k >> 2) & 1);
-            if (!retnet) wait(FULL_G, par);
+            wait(FULL_G, par);
             wait(FULL_QK, par);
             {
                 const float *g = gate_s + (k & 3) * 2 * C;
-                chunk_prologue<true, true>(qk, qk + TILE_BF16, retnet ? nullptr : reinterpret_cast<const float *>(sm + OFF_G), tot, g, g + C,
-                                           eblast, sm + OFF_E2, p.status, tid, 1, NoHook(),
-                                           ScalarDecay{lgam, min(C, p.T - t0)});
+                chunk_prologue<true, true>(qk, qk + TILE_BF16, reinterpret_cast<const float *>(sm + OFF_G), tot, g, g + C,
+                                           eblast, sm + OFF_E2, p.status, tid);
             }
             fence_proxy_async();
             warp_arrive(bar(OPR), lane);
@@ -725,10 +713,9 @@ k_gla_bwd_tc(const __grid_constant__ CUtensorMap gm_q, const __grid_constant__ C
             warp_arrive(bar(AREADY), lane);
 
             // ---- R_{n-1} = rowsum(dS_n * S_n), while the tensor core works on the products with the masked tiles ----
-            // (it feeds the log-decay gradient only: Softmax-RetNet, whose decay is a constant, has none and skips it)
             wait(BAR_DS, par);
             tc_fence_after();
-            if (!retnet) {
+            {
                 float v0[32], v1[32];
                 tmem_ld32(tmem + lane_base + COL_DS + 64 * wh, v0);
                 tmem_ld32(tmem + lane_base + COL_DS + 64 * wh + 32, v1);
@@ -767,7 +754,7 @@ k_gla_bwd_tc(const __grid_constant__ CUtensorMap gm_q, const __grid_constant__ C
                         const float2 ea = unpack_bf16(ew[y].x), eb = unpack_bf16(ew[y].y), qv = unpack_bf16(qw[y]), kv = unpack_bf16(kw[y]);
                         const float a0 = dqh[2 * y], a1 = dqh[2 * y + 1], c0 = dkh[2 * y], c1 = dkh[2 * y + 1];
                         const float pq0 = qv.x * a0, pq1 = qv.y * a1, pk0 = kv.x * c0, pk1 = kv.y * c1;
-                        if (!retnet) *reinterpret_cast<float2 *>(e2_at(hf, y)) = make_float2(pq0 - pk0, pq1 - pk1);
+                        *reinterpret_cast<float2 *>(e2_at(hf, y)) = make_float2(pq0 - pk0, pq1 - pk1);
                         if ((y & 1) == 0) { sq0 += pq0 + pq1; sk0 += pk0 + pk1; } else { sq1 += pq0 + pq1; sk1 += pk0 + pk1; }
                         *reinterpret_cast<uint32_t *>(qk + off) = pack_bf16(ea.x * a0, eb.x * a1);                // dq = scale Gq 2^b dqh   (over qh, for the store)
                         *reinterpret_cast<uint32_t *>(qk + TILE_BF16 + off) = pack_bf16(ea.y * c0, eb.y * c1);    // dk = Gk 2^-b dkh
@@ -807,7 +794,7 @@ k_gla_bwd_tc(const __grid_constant__ CUtensorMap gm_q, const __grid_constant__ C
             }
             float *dgt = reinterpret_cast<float *>(sm + OFF_DZ);
             named_bar_sync(1, NCOMPUTE);                // qh dqh - kh dkh, red and the R partials are complete
-            if (!retnet) {   // log-decay gradient (a constant decay has none): in-chunk suffix sum + what flows in from the right.
+            {   // log-decay gradient: in-chunk suffix sum + what flows in from the right.
                 // Warp g owns tokens 8g .. 8g+7, a lane four features (16-byte accesses, whole rows a warp); a group's total
                 // goes in the place of the group's first row (each lane has read what it writes over)
                 const float *Rcur = Rs + (n & 1) * 2 * D;
@@ -930,11 +917,12 @@ __global__ void k_fold_segment_dstates(int H, int P, int dk, int dv, const float
 }  // namespace
 
 int gla_tc_bwd_configure() {
-    if (cudaFuncSetAttribute(k_gla_states_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)st1::SMEM_BYTES) != cudaSuccess)
+    if (cudaFuncSetAttribute(k_gla_states_tc<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)st1::SMEM_BYTES) != cudaSuccess ||
+        cudaFuncSetAttribute(k_gla_states_tc<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)st1::SMEM_BYTES) != cudaSuccess)
         return -1;
     if (cudaFuncSetAttribute(k_gla_bwd_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)st2::SMEM_BYTES) != cudaSuccess)
         return -1;
-    return 0;
+    return retnet_tc_bwd_configure();
 }
 
 // Softmax backward over the heads from the gate products P = G dG (shared by the GLA and GDN tensor-core paths).
@@ -972,7 +960,7 @@ int gla_tc_segment_summaries(const Dims &d, const FwdArgs &a, int P, int L, int 
     else if (!make_map(&mg, a.log_decay, d.B, d.T, d.H, d.dk, true, 128)) return -1;
     StatesParams sp{a.lq, a.lk, nullptr, nullptr, fin, gam, status, d.T, d.H, d.NT, P, L, PS, retnet ? a.log_decay : nullptr,
                     nullptr, nullptr, d.dk, d.dv};
-    k_gla_states_tc<<<d.B * d.H * PS, st1::NTHREADS, st1::SMEM_BYTES, st>>>(mk, mv, mg, sp);
+    (retnet ? k_gla_states_tc<true> : k_gla_states_tc<false>)<<<d.B * d.H * PS, st1::NTHREADS, st1::SMEM_BYTES, st>>>(mk, mv, mg, sp);
     tr.mark("gla_segment_states_tc");
     return cudaGetLastError() == cudaSuccess ? 1 : -1;
 }
@@ -1017,7 +1005,7 @@ int gla_tc_backward(const Dims &d, const BwdArgs &a, bool have_states, int *stat
         }
         StatesParams sp{a.lq, a.lk, a.h0, simg, nullptr, nullptr, status, d.T, d.H, d.NT, 1, d.NT, 1, retnet ? a.log_decay : nullptr,
                         dseqs, vm, d.dk, d.dv};
-        k_gla_states_tc<<<ctas, st1::NTHREADS, st1::SMEM_BYTES, st>>>(mk, mv, mg, sp);
+        (retnet ? k_gla_states_tc<true> : k_gla_states_tc<false>)<<<ctas, st1::NTHREADS, st1::SMEM_BYTES, st>>>(mk, mv, mg, sp);
         tr.mark("gla_states_tc");
     }
     const CUtensorMap *vm = nullptr;
@@ -1038,7 +1026,8 @@ int gla_tc_backward(const Dims &d, const BwdArgs &a, bool have_states, int *stat
         if (!vm) return -1;
     }
     BwdParams bp{a.lq, a.lk, a.dht, simg, pq, pk, a.dh0, status, d.T, d.H, d.NT, d.scale, retnet ? a.log_decay : nullptr, dseqs, vm, d.dk, d.dv};
-    k_gla_bwd_tc<<<ctas, st2::NTHREADS, st2::SMEM_BYTES, st>>>(mq, mk, mv, mdo, mg, mdq, mdk, mdv, mdg, bp);
+    if (retnet) retnet_tc_bwd_launch({mq, mk, mv, mdo, mdq, mdk, mdv}, bp, ctas, st);
+    else k_gla_bwd_tc<<<ctas, st2::NTHREADS, st2::SMEM_BYTES, st>>>(mq, mk, mv, mdo, mg, mdq, mdk, mdv, mdg, bp);
     tr.mark("gla_bwd_tc");
     if (gate_bwd_prod(a.lq, a.lk, pq, pk, a.dlq, a.dlk, (long)d.B * d.T, d.H, st) < 0) return -1;
     tr.mark("gate_bwd");
