@@ -17,25 +17,75 @@ namespace {
 using namespace detail;
 
 // ------------------------------------------------------------------------------------------
-// a1: head-softmax gates, HP lanes per token (HP = power of two >= H), max and sum by shuffles.
+// a1 + a2 in one launch (the two do not meet; a launch costs more than either).  Blocks 0 .. gate_blocks-1: head-softmax gates, HP
+// lanes per token (HP = power of two >= H), max and sum by shuffles, the two gates side by side.  The others: chunk-local
+// inclusive cumulative log-decay of one chunk of one (batch, head) sequence (Softmax-GLA, a lane four key dimensions) or of eight
+// (a warp each, by shuffles).  A chunk whose cumulative log-decay is beyond the range of the e^{b}, e^{-b} factors raises STATUS_RANGE.
 template <int HP>
-__global__ void k_gate_fwd(const float *__restrict__ lq, const float *__restrict__ lk,
-                           float *__restrict__ Gq, float *__restrict__ Gk, long n_tok, int H) {
-    const float *l = blockIdx.y ? lk : lq;
-    float *G = blockIdx.y ? Gk : Gq;
-    long gt = (long)blockIdx.x * blockDim.x + threadIdx.x;
-    long tok = gt / HP;
-    int h = (int)(gt % HP);
-    bool valid = tok < n_tok && h < H;
-    float x = valid ? l[tok * H + h] : -INFINITY;
-    float m = x;
+__global__ void __launch_bounds__(256)
+k_gates_decay(Dims d, const float *__restrict__ lq, const float *__restrict__ lk, float *__restrict__ Gq, float *__restrict__ Gk,
+              const float *__restrict__ log_decay, float *__restrict__ bcum, int gate_blocks, int *status) {
+    if ((int)blockIdx.x < gate_blocks) {
+        const long n_tok = (long)d.B * d.T, gt = (long)blockIdx.x * 256 + threadIdx.x, tok = gt / HP;
+        const int h = (int)(gt % HP);
+        const bool valid = tok < n_tok && h < d.H;
+        const float x0 = valid ? lq[tok * d.H + h] : -INFINITY, x1 = valid ? lk[tok * d.H + h] : -INFINITY;
+        float m0 = x0, m1 = x1;
 #pragma unroll
-    for (int o = HP / 2; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(FULL, m, o));
-    float e = valid ? expf(x - m) : 0.f;
-    float s = e;
+        for (int o = HP / 2; o > 0; o >>= 1) {
+            m0 = fmaxf(m0, __shfl_xor_sync(FULL, m0, o));
+            m1 = fmaxf(m1, __shfl_xor_sync(FULL, m1, o));
+        }
+        const float e0 = valid ? expf(x0 - m0) : 0.f, e1 = valid ? expf(x1 - m1) : 0.f;
+        float s0 = e0, s1 = e1;
 #pragma unroll
-    for (int o = HP / 2; o > 0; o >>= 1) s += __shfl_xor_sync(FULL, s, o);
-    if (valid) G[tok * H + h] = e / s;
+        for (int o = HP / 2; o > 0; o >>= 1) {
+            s0 += __shfl_xor_sync(FULL, s0, o);
+            s1 += __shfl_xor_sync(FULL, s1, o);
+        }
+        if (valid) {
+            Gq[tok * d.H + h] = e0 / s0;
+            Gk[tok * d.H + h] = e1 / s1;
+        }
+        return;
+    }
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, blk = (int)blockIdx.x - gate_blocks;
+    const long chunks = (long)d.B * d.H * d.NT;
+    const long c = d.variant == SLA_GLA ? blk : 8L * blk + w;
+    if (c >= chunks) return;
+    const int n = (int)(c % d.NT), bh = (int)(c / d.NT), b = bh / d.H, h = bh % d.H, t0 = n * d.C, cn = min(d.C, d.T - t0);
+    if (d.variant == SLA_GLA) {             // warp w the tokens 8w .. 8w+7 of all key dimensions, two levels
+        __shared__ float4 tot[8][32];
+        const bool live = 4 * lane < d.dk;
+        float4 g[8], run = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+            g[i] = live && 8 * w + i < cn ? ldf4(log_decay, tok_row(d, b, t0 + 8 * w + i, h) * d.dk + 4 * lane) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) { run.x += g[i].x; run.y += g[i].y; run.z += g[i].z; run.w += g[i].w; }
+        tot[w][lane] = run;
+        __syncthreads();
+        run = make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int x = 0; x < w; ++x) { const float4 a = tot[x][lane]; run.x += a.x; run.y += a.y; run.z += a.z; run.w += a.w; }
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            run.x += g[i].x; run.y += g[i].y; run.z += g[i].z; run.w += g[i].w;
+            if (live && 8 * w + i < cn) stf4(bcum, tok_row(d, b, t0 + 8 * w + i, h) * d.dk + 4 * lane, run);
+        }
+        if (w == 7 && live && fminf(fminf(run.x, run.y), fminf(run.z, run.w)) < -SLA_MAX_CHUNK_DECAY) atomicOr(status, STATUS_RANGE);
+        return;
+    }
+    auto at = [&](int i) { return i >= cn ? 0.f : d.variant == SLA_RETNET ? log_decay[h] : log_decay[tok_row(d, b, t0 + i, h)]; };
+    const float g0 = at(2 * lane), g1 = at(2 * lane + 1);      // lane l owns tokens 2l, 2l + 1
+    float incl = g0 + g1;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const float t = __shfl_up_sync(FULL, incl, o);
+        if (lane >= o) incl += t;
+    }
+    if (2 * lane < cn) bcum[tok_row(d, b, t0 + 2 * lane, h)] = incl - g1;
+    if (2 * lane + 1 < cn) bcum[tok_row(d, b, t0 + 2 * lane + 1, h)] = incl;
+    if (lane == 31 && incl < -SLA_MAX_CHUNK_DECAY) atomicOr(status, STATUS_RANGE);
 }
 
 // gate backward: dl_h = G_h (dG_h - sum_h' G_h' dG_h')
@@ -56,33 +106,6 @@ __global__ void k_gate_bwd(const float *__restrict__ Gq, const float *__restrict
 #pragma unroll
     for (int o = HP / 2; o > 0; o >>= 1) s += __shfl_xor_sync(FULL, s, o);
     if (valid) dl[tok * H + h] = g * (dg - s);
-}
-
-// ------------------------------------------------------------------------------------------
-// a2: chunk-local inclusive cumulative log-decay.  grid (NT, B*H).
-// A chunk whose cumulative log-decay is beyond the range of the e^{b}, e^{-b} factors raises STATUS_RANGE.
-__global__ void k_cumdecay(Dims d, const float *__restrict__ log_decay, float *__restrict__ bcum, int *status) {
-    int n = blockIdx.x, bh = blockIdx.y, b = bh / d.H, h = bh % d.H;
-    int t0 = n * d.C, cn = min(d.C, d.T - t0);
-    if (d.variant == SLA_GLA) {
-        for (int dd = threadIdx.x; dd < d.dk; dd += blockDim.x) {
-            float acc = 0.f;
-            for (int i = 0; i < cn; ++i) {
-                size_t idx = tok_row(d, b, t0 + i, h) * d.dk + dd;
-                acc += log_decay[idx];
-                bcum[idx] = acc;
-            }
-            if (acc < -SLA_MAX_CHUNK_DECAY) atomicOr(status, STATUS_RANGE);
-        }
-    } else if (threadIdx.x == 0) {
-        float acc = 0.f;
-        for (int i = 0; i < cn; ++i) {
-            size_t row = tok_row(d, b, t0 + i, h);
-            acc += (d.variant == SLA_RETNET) ? log_decay[h] : log_decay[row];
-            bcum[row] = acc;
-        }
-        if (acc < -SLA_MAX_CHUNK_DECAY) atomicOr(status, STATUS_RANGE);
-    }
 }
 
 // ------------------------------------------------------------------------------------------
@@ -271,9 +294,10 @@ k_chunk_outer(Dims d, const TIO *__restrict__ x, const TIO *__restrict__ y, cons
     const int n = blockIdx.x, bh = blockIdx.y, b = bh / d.H, h = bh % d.H, r0 = 64 * blockIdx.z, nr = min(64, d.dk - r0);
     float *dst = !GRAD ? out + state_off(d, bh, n + 1, d.NT + 1) : n > 0 ? out + state_off(d, bh, n - 1, d.NT) : dh0 ? dh0 + state_off(d, bh, 0, 1) : nullptr;
     if (!dst) return;
-    const int t0 = n * d.C, cn = min(d.C, d.T - t0), ldv = d.dv + 1;
-    float *Xs = sm;                          // [CMAX][65]
-    float *Ys = Xs + CMAX * 65;              // [CMAX][ldv]
+    const int t0 = n * d.C, cn = min(d.C, d.T - t0), ldv = pad4(d.dv);
+    constexpr int ldx = pad4(64);
+    float *Xs = sm;                          // [CMAX][ldx]
+    float *Ys = Xs + CMAX * ldx;             // [CMAX][ldv]
     const size_t row_last = tok_row(d, b, t0 + cn - 1, h);
     struct In { float4 x, b, bl; float g; };
     const int w4 = nr >> 2;
@@ -291,24 +315,37 @@ k_chunk_outer(Dims d, const TIO *__restrict__ x, const TIO *__restrict__ y, cons
         [&](int idx, const In &v) {
             const int i = idx / w4;
             const float4 e = GRAD ? v.b : make_float4(v.bl.x - v.b.x, v.bl.y - v.b.y, v.bl.z - v.b.z, v.bl.w - v.b.w);
-            put4(Xs + i * 65 + 4 * (idx - i * w4), make_float4(v.g * v.x.x * expf(e.x), v.g * v.x.y * expf(e.y), v.g * v.x.z * expf(e.z), v.g * v.x.w * expf(e.w)));
+            stf4(Xs, i * ldx + 4 * (idx - i * w4), make_float4(v.g * v.x.x * expf(e.x), v.g * v.x.y * expf(e.y), v.g * v.x.z * expf(e.z), v.g * v.x.w * expf(e.w)));
         });
     fill_rows(Ys, ldv, y, cn, cn, d.dv, [&](int i) { return tok_row(d, b, t0 + i, h) * d.dv; });
     __syncthreads();
-    const int ty = threadIdx.x >> 5, tx = threadIdx.x & 31;
-    float acc[8][4];
-    zero_acc(acc);
-    tile_gemm<4>(acc, Xs, 1, 65, Ys, ldv, 1, cn, d.dv, ty, tx);
+    const Tile t;
+    auto emit = [&](const auto &acc) {
+        if (4 * t.tr >= nr) return;
 #pragma unroll
-    for (int r = 0; r < 8; ++r) {
-        const int i = ty + 8 * r;
-        if (i >= nr) continue;
+        for (int a = 0; a < 4; ++a)
 #pragma unroll
-        for (int cb = 0; cb < 4; ++cb) {
-            const int j = tx + 32 * cb;
-            float *e = dst + (size_t)(r0 + i) * d.dv + j;
-            if (j < d.dv) *e = ADD ? *e + acc[r][cb] : acc[r][cb];
-        }
+            for (int blk = 0; blk < (int)(sizeof(acc[0]) / 16); ++blk) {
+                if (t.col(blk) >= d.dv) continue;
+                float *e = dst + (size_t)(r0 + 4 * t.tr + a) * d.dv + t.col(blk);
+                float4 v = make_float4(acc[a][4 * blk], acc[a][4 * blk + 1], acc[a][4 * blk + 2], acc[a][4 * blk + 3]);
+                if (ADD) {
+                    const float4 w = *reinterpret_cast<const float4 *>(e);
+                    v.x += w.x; v.y += w.y; v.z += w.z; v.w += w.w;
+                }
+                *reinterpret_cast<float4 *>(e) = v;
+            }
+    };
+    if (d.dv <= 64) {
+        float acc[4][4];
+        zero_acc(acc);
+        mm_outer<1>(acc, t, Xs, ldx, Ys, ldv, cn, nr, d.dv);
+        emit(acc);
+    } else {
+        float acc[4][8];
+        zero_acc(acc);
+        mm_outer<2>(acc, t, Xs, ldx, Ys, ldv, cn, nr, d.dv);
+        emit(acc);
     }
 }
 
@@ -358,14 +395,15 @@ k_output(Dims d, const TIO *__restrict__ q, const TIO *__restrict__ k, const TIO
     extern __shared__ float sm[];
     int n = blockIdx.x, bh = blockIdx.y, b = bh / d.H, h = bh % d.H;
     int t0 = n * d.C, cn = min(d.C, d.T - t0);
-    int ldk = d.dk + 1, ldv = d.dv + 1, lda = CMAX + 1;
+    const int ldk = pad4(d.dk), ldv = pad4(d.dv), cn4 = (cn + 3) & ~3;
+    constexpr int lda = pad4(CMAX);
     float *Qs = sm;
     float *Ks = Qs + CMAX * ldk;
     float *Vs = Ks + CMAX * ldk;
     float *As = Vs + CMAX * ldv;
     float *Ss = As + CMAX * lda;             // [dk][ldv]
-    const int ty = threadIdx.x >> 5, tx = threadIdx.x & 31;
     const bool gdn = d.variant == SLA_GDN;
+    const Tile t;
 
     load_qk_hat(d, q, k, Gq, Gk, bcum, b, h, t0, cn, Qs, Ks, ldk);
     auto vrow = [&](int i) { return tok_row(d, b, t0 + i, h) * d.dv; };
@@ -374,34 +412,40 @@ k_output(Dims d, const TIO *__restrict__ q, const TIO *__restrict__ k, const TIO
     const float *Sg = states + state_off(d, bh, n, d.NT + 1);
     fill_rows(Ss, ldv, Sg, d.dk, d.dk, d.dv, [&](int i) { return (size_t)i * d.dv; });
     __syncthreads();
-
     {
-        float acc[8][2];
-        zero_acc(acc);
-        tile_gemm<2>(acc, Qs, ldk, 1, Ks, 1, ldk, d.dk, CMAX, ty, tx);
+        float A[4][4];
+        zero_acc(A);
+        mm<1, false>(A, t, Qs, ldk, Ks, ldk, d.dk, CMAX);
 #pragma unroll
-        for (int r = 0; r < 8; ++r)
-#pragma unroll
-            for (int cb = 0; cb < 2; ++cb) {
-                int i = ty + 8 * r, j = tx + 32 * cb;
-                As[i * lda + j] = (j <= i) ? acc[r][cb] : 0.f;
-            }
+        for (int a = 0; a < 4; ++a) {
+            const int i = t.row(a), j = t.col(0);
+            stf4(As, i * lda + j, make_float4(j <= i ? A[a][0] : 0.f, j + 1 <= i ? A[a][1] : 0.f, j + 2 <= i ? A[a][2] : 0.f, j + 3 <= i ? A[a][3] : 0.f));
+        }
     }
     __syncthreads();
-    float acc[8][4];
-    zero_acc(acc);
-    tile_gemm<4>(acc, As, lda, 1, Vs, ldv, 1, cn, d.dv, ty, tx);
-    tile_gemm<4>(acc, Qs, ldk, 1, Ss, ldv, 1, d.dk, d.dv, ty, tx);
+    auto emit = [&](const auto &acc) {
 #pragma unroll
-    for (int r = 0; r < 8; ++r) {
-        int i = ty + 8 * r;
-        if (i >= cn) continue;
-        size_t row = tok_row(d, b, t0 + i, h);
+        for (int a = 0; a < 4; ++a) {
+            const int i = t.row(a);
+            if (i >= cn) continue;
+            const size_t row = tok_row(d, b, t0 + i, h) * d.dv;
 #pragma unroll
-        for (int cb = 0; cb < 4; ++cb) {
-            int j = tx + 32 * cb;
-            if (j < d.dv) stf(o, row * d.dv + j, acc[r][cb]);
+            for (int blk = 0; blk < (int)(sizeof(acc[0]) / 16); ++blk)
+                if (t.col(blk) < d.dv) stf4(o, row + t.col(blk), make_float4(acc[a][4 * blk], acc[a][4 * blk + 1], acc[a][4 * blk + 2], acc[a][4 * blk + 3]));
         }
+    };
+    if (d.dv <= 64) {
+        float acc[4][4];
+        zero_acc(acc);
+        mm<1, true>(acc, t, As, lda, Vs, ldv, cn4, d.dv);
+        mm<1, true>(acc, t, Qs, ldk, Ss, ldv, d.dk, d.dv);
+        emit(acc);
+    } else {
+        float acc[4][8];
+        zero_acc(acc);
+        mm<2, true>(acc, t, As, lda, Vs, ldv, cn4, d.dv);
+        mm<2, true>(acc, t, Qs, ldk, Ss, ldv, d.dk, d.dv);
+        emit(acc);
     }
 }
 
@@ -535,7 +579,9 @@ k_dstate_scan(Dims d, const TIO *__restrict__ q, const TIO *__restrict__ k, cons
 //   dA = tril(dO V^T) ; dZ = diag(exp(b_last)) dS_next
 //   dqh = dA kh + dO S^T ; dkh = dA^T qh + V dZ^T ; dV = A^T dO + kh dZ
 //   db = qh*dqh - kh*dkh (+ rowsum(dS_next*S_next) on the last row) ; dlog_decay = suffix sum of db
-template <typename TIO>
+// The three matrices dA, dA^T, A^T take turns in one buffer (heads of 128 leave room for one), kept in registers meanwhile.
+// NB: 64-column blocks of the wider of the two head widths.
+template <typename TIO, int NB>
 __global__ void __launch_bounds__(256)
 k_grads_lin(Dims d, const TIO *__restrict__ q, const TIO *__restrict__ k, const TIO *__restrict__ v,
             const TIO *__restrict__ dO, const float *__restrict__ Gq, const float *__restrict__ Gk,
@@ -544,19 +590,21 @@ k_grads_lin(Dims d, const TIO *__restrict__ q, const TIO *__restrict__ k, const 
             TIO *__restrict__ dv, float *__restrict__ dlog_decay, float *__restrict__ dGq,
             float *__restrict__ dGk) {
     extern __shared__ float sm[];
-    int n = blockIdx.x, bh = blockIdx.y, b = bh / d.H, h = bh % d.H;
-    int t0 = n * d.C, cn = min(d.C, d.T - t0);
-    int ldk = d.dk + 1, ldv = d.dv + 1, lda = CMAX + 1;
+    const int n = blockIdx.x, bh = blockIdx.y, b = bh / d.H, h = bh % d.H;
+    const int t0 = n * d.C, cn = min(d.C, d.T - t0), cn4 = (cn + 3) & ~3;
+    const int ldk = pad4(d.dk), ldv = pad4(d.dv);
+    constexpr int lda = pad4(CMAX);
     float *Qs = sm;
     float *Ks = Qs + CMAX * ldk;
     float *Vs = Ks + CMAX * ldk;
     float *dOs = Vs + CMAX * ldv;
-    float *As = dOs + CMAX * ldv;
-    float *dAs = As + CMAX * lda;
-    float *Ss = dAs + CMAX * lda;             // [dk][ldv]: S, then dZ
+    float *Ms = dOs + CMAX * ldv;             // dA, then dA^T, then A^T
+    float *Ss = Ms + CMAX * lda;              // [dk][ldv]: S, then dZ
     float *Rs = Ss + d.dk * ldv;              // [dk]
+    float *red = Rs + d.dk;                   // [2][4][CMAX] a token's gate sums, by quarter of the columns
     const int ty = threadIdx.x >> 5, tx = threadIdx.x & 31;
-    size_t row_last = tok_row(d, b, t0 + cn - 1, h);
+    const Tile t;
+    const size_t row_last = tok_row(d, b, t0 + cn - 1, h);
 
     load_qk_hat(d, q, k, Gq, Gk, bcum, b, h, t0, cn, Qs, Ks, ldk);
     auto vrow = [&](int i) { return tok_row(d, b, t0 + i, h) * d.dv; };
@@ -565,61 +613,74 @@ k_grads_lin(Dims d, const TIO *__restrict__ q, const TIO *__restrict__ k, const 
     const float *Sg = states + state_off(d, bh, n, d.NT + 1);
     fill_rows(Ss, ldv, Sg, d.dk, d.dk, d.dv, [&](int i) { return (size_t)i * d.dv; });
     __syncthreads();
-    {
-        float a1[8][2], a2[8][2];
-        zero_acc(a1);
-        zero_acc(a2);
-        tile_gemm<2>(a1, Qs, ldk, 1, Ks, 1, ldk, d.dk, CMAX, ty, tx);
-        tile_gemm<2>(a2, dOs, ldv, 1, Vs, 1, ldv, d.dv, CMAX, ty, tx);
+    float A[4][4], dA[4][4];
+    zero_acc(A);
+    zero_acc(dA);
+    mm<1, false>(A, t, Qs, ldk, Ks, ldk, d.dk, CMAX);
+    mm<1, false>(dA, t, dOs, ldv, Vs, ldv, d.dv, CMAX);
 #pragma unroll
-        for (int r = 0; r < 8; ++r)
+    for (int a = 0; a < 4; ++a)
 #pragma unroll
-            for (int cb = 0; cb < 2; ++cb) {
-                int i = ty + 8 * r, j = tx + 32 * cb;
-                As[i * lda + j] = (j <= i) ? a1[r][cb] : 0.f;
-                dAs[i * lda + j] = (j <= i) ? a2[r][cb] : 0.f;
-            }
-    }
+        for (int c = 0; c < 4; ++c)
+            if (t.col(0) + c > t.row(a)) A[a][c] = dA[a][c] = 0.f;
+#pragma unroll
+    for (int a = 0; a < 4; ++a) stf4(Ms, t.row(a) * lda + t.col(0), make_float4(dA[a][0], dA[a][1], dA[a][2], dA[a][3]));
+    auto transposed = [&](const float (&m)[4][4]) {
+#pragma unroll
+        for (int a = 0; a < 4; ++a)
+#pragma unroll
+            for (int c = 0; c < 4; ++c) Ms[(t.col(0) + c) * lda + t.row(a)] = m[a][c];
+    };
+    // a token's sum over this thread's columns -> its quarter's slot (four lanes share a row)
+    auto row_sum = [&](float s, int which, int i) {
+        s += __shfl_xor_sync(FULL, s, 1);
+        s += __shfl_xor_sync(FULL, s, 2);
+        if ((tx & 3) == 0) red[(4 * which + (ty >> 1)) * CMAX + i] = s;
+    };
     __syncthreads();
-    float db[8][4];
+    float db[4][4 * NB];
     {   // dqh and the query-side outputs
-        float acc[8][4];
+        float acc[4][4 * NB];
         zero_acc(acc);
-        tile_gemm<4>(acc, dAs, lda, 1, Ks, ldk, 1, cn, d.dk, ty, tx);
-        tile_gemm<4>(acc, dOs, ldv, 1, Ss, 1, ldv, d.dv, d.dk, ty, tx);
+        mm<NB, true>(acc, t, Ms, lda, Ks, ldk, cn4, d.dk);
+        mm<NB, false>(acc, t, dOs, ldv, Ss, ldv, d.dv, d.dk);
 #pragma unroll
-        for (int r = 0; r < 8; ++r) {
-            int i = ty + 8 * r;
+        for (int a = 0; a < 4; ++a) {
+            const int i = t.row(a);
+            const size_t row = i < cn ? tok_row(d, b, t0 + i, h) : 0;
+            const float gq = i < cn ? Gq[row] : 0.f;
             float gsum = 0.f;
-            size_t row = i < cn ? tok_row(d, b, t0 + i, h) : 0;
-            float gq = i < cn ? Gq[row] : 0.f;
 #pragma unroll
-            for (int cb = 0; cb < 4; ++cb) {
-                int c = tx + 32 * cb;
-                db[r][cb] = 0.f;
-                if (i < cn && c < d.dk) {
-                    db[r][cb] = Qs[i * ldk + c] * acc[r][cb];
-                    float dqt = acc[r][cb] * expf(bcum_at(d, bcum, row, c));
-                    gsum = fmaf(d.scale * ldf(q, row * d.dk + c), dqt, gsum);
-                    stf(dq, row * d.dk + c, d.scale * gq * dqt);
-                }
+            for (int blk = 0; blk < NB; ++blk) {
+                const int c = t.col(blk);
+                float *dbv = &db[a][4 * blk], *y = &acc[a][4 * blk];
+#pragma unroll
+                for (int e = 0; e < 4; ++e) dbv[e] = 0.f;
+                if (i >= cn || c >= d.dk) continue;
+                const float4 qh = *reinterpret_cast<const float4 *>(Qs + i * ldk + c), bc = bcum_at4(d, bcum, row, c), qv = ldf4(q, row * d.dk + c);
+                dbv[0] = qh.x * y[0]; dbv[1] = qh.y * y[1]; dbv[2] = qh.z * y[2]; dbv[3] = qh.w * y[3];
+                const float4 g = make_float4(y[0] * expf(bc.x), y[1] * expf(bc.y), y[2] * expf(bc.z), y[3] * expf(bc.w));
+                gsum = fmaf(d.scale * qv.x, g.x, fmaf(d.scale * qv.y, g.y, fmaf(d.scale * qv.z, g.z, fmaf(d.scale * qv.w, g.w, gsum))));
+                const float f = d.scale * gq;
+                stf4(dq, row * d.dk + c, make_float4(f * g.x, f * g.y, f * g.z, f * g.w));
             }
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) gsum += __shfl_xor_sync(FULL, gsum, o);
-            if (tx == 0 && i < cn) dGq[row] = gsum;
+            row_sum(gsum, 0, i);
         }
     }
     __syncthreads();
+    transposed(dA);
     {   // Ss <- dZ = diag(exp(b_last)) dS_next ; Rs <- rowsum(dS_next * S_next)
         const float *dSg = dstates + state_off(d, bh, n, d.NT);
         const float *Sn = states + state_off(d, bh, n + 1, d.NT + 1);
+#pragma unroll 4
         for (int r0 = ty; r0 < d.dk; r0 += 8) {
-            float e = expf(bcum_at(d, bcum, row_last, r0));
+            const float e = expf(bcum_at(d, bcum, row_last, r0));
             float part = 0.f;
-            for (int j = tx; j < d.dv; j += 32) {
-                float g = dSg[(size_t)r0 * d.dv + j];
-                part = fmaf(g, Sn[(size_t)r0 * d.dv + j], part);
-                Ss[r0 * ldv + j] = e * g;
+            const int j = 4 * tx;
+            if (j < d.dv) {
+                const float4 g = ldf4(dSg, (size_t)r0 * d.dv + j), s = ldf4(Sn, (size_t)r0 * d.dv + j);
+                part = fmaf(g.x, s.x, fmaf(g.y, s.y, fmaf(g.z, s.z, g.w * s.w)));
+                stf4(Ss, r0 * ldv + j, make_float4(e * g.x, e * g.y, e * g.z, e * g.w));
             }
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(FULL, part, o);
@@ -628,65 +689,84 @@ k_grads_lin(Dims d, const TIO *__restrict__ q, const TIO *__restrict__ k, const 
     }
     __syncthreads();
     {   // dkh and the key-side outputs
-        float acc[8][4];
+        float acc[4][4 * NB];
         zero_acc(acc);
-        tile_gemm<4>(acc, dAs, 1, lda, Qs, ldk, 1, cn, d.dk, ty, tx);
-        tile_gemm<4>(acc, Vs, ldv, 1, Ss, 1, ldv, d.dv, d.dk, ty, tx);
+        mm<NB, true>(acc, t, Ms, lda, Qs, ldk, cn4, d.dk);
+        mm<NB, false>(acc, t, Vs, ldv, Ss, ldv, d.dv, d.dk);
 #pragma unroll
-        for (int r = 0; r < 8; ++r) {
-            int i = ty + 8 * r;
+        for (int a = 0; a < 4; ++a) {
+            const int i = t.row(a);
+            const size_t row = i < cn ? tok_row(d, b, t0 + i, h) : 0;
+            const float gk = i < cn ? Gk[row] : 0.f;
             float gsum = 0.f;
-            size_t row = i < cn ? tok_row(d, b, t0 + i, h) : 0;
-            float gk = i < cn ? Gk[row] : 0.f;
 #pragma unroll
-            for (int cb = 0; cb < 4; ++cb) {
-                int c = tx + 32 * cb;
-                if (i < cn && c < d.dk) {
-                    db[r][cb] -= Ks[i * ldk + c] * acc[r][cb];
-                    float dkt = acc[r][cb] * expf(-bcum_at(d, bcum, row, c));
-                    gsum = fmaf(ldf(k, row * d.dk + c), dkt, gsum);
-                    stf(dk, row * d.dk + c, gk * dkt);
-                }
+            for (int blk = 0; blk < NB; ++blk) {
+                const int c = t.col(blk);
+                if (i >= cn || c >= d.dk) continue;
+                float *dbv = &db[a][4 * blk], *y = &acc[a][4 * blk];
+                const float4 kh = *reinterpret_cast<const float4 *>(Ks + i * ldk + c), bc = bcum_at4(d, bcum, row, c), kv = ldf4(k, row * d.dk + c);
+                dbv[0] -= kh.x * y[0]; dbv[1] -= kh.y * y[1]; dbv[2] -= kh.z * y[2]; dbv[3] -= kh.w * y[3];
+                const float4 g = make_float4(y[0] * expf(-bc.x), y[1] * expf(-bc.y), y[2] * expf(-bc.z), y[3] * expf(-bc.w));
+                gsum = fmaf(kv.x, g.x, fmaf(kv.y, g.y, fmaf(kv.z, g.z, fmaf(kv.w, g.w, gsum))));
+                stf4(dk, row * d.dk + c, make_float4(gk * g.x, gk * g.y, gk * g.z, gk * g.w));
             }
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) gsum += __shfl_xor_sync(FULL, gsum, o);
-            if (tx == 0 && i < cn) dGk[row] = gsum;
+            row_sum(gsum, 1, i);
         }
     }
+    __syncthreads();
+    transposed(A);
+    if (threadIdx.x < 2 * CMAX) {     // the gates' gradients: a token's four quarters
+        const int which = threadIdx.x / CMAX, i = threadIdx.x % CMAX;
+        const float *r = red + 4 * which * CMAX + i;
+        if (i < cn) (which ? dGk : dGq)[tok_row(d, b, t0 + i, h)] = (r[0] + r[CMAX]) + (r[2 * CMAX] + r[3 * CMAX]);
+    }
+    __syncthreads();
     {   // dV = A^T dO + kh dZ
-        float acc[8][4];
+        float acc[4][4 * NB];
         zero_acc(acc);
-        tile_gemm<4>(acc, As, 1, lda, dOs, ldv, 1, cn, d.dv, ty, tx);
-        tile_gemm<4>(acc, Ks, ldk, 1, Ss, ldv, 1, d.dk, d.dv, ty, tx);
+        mm<NB, true>(acc, t, Ms, lda, dOs, ldv, cn4, d.dv);
+        mm<NB, true>(acc, t, Ks, ldk, Ss, ldv, d.dk, d.dv);
 #pragma unroll
-        for (int r = 0; r < 8; ++r) {
-            int i = ty + 8 * r;
+        for (int a = 0; a < 4; ++a) {
+            const int i = t.row(a);
             if (i >= cn) continue;
-            size_t row = tok_row(d, b, t0 + i, h);
+            const size_t row = tok_row(d, b, t0 + i, h) * d.dv;
 #pragma unroll
-            for (int cb = 0; cb < 4; ++cb) {
-                int j = tx + 32 * cb;
-                if (j < d.dv) stf(dv, row * d.dv + j, acc[r][cb]);
-            }
+            for (int blk = 0; blk < NB; ++blk)
+                if (t.col(blk) < d.dv) stf4(dv, row + t.col(blk), make_float4(acc[a][4 * blk], acc[a][4 * blk + 1], acc[a][4 * blk + 2], acc[a][4 * blk + 3]));
         }
     }
     if (d.variant != SLA_GLA || !dlog_decay) return;
-    __syncthreads();            // every thread is done with Vs
-    float *dbs = Vs;            // reuse as [CMAX][ldk] (ldk <= ldv is not needed: Vs..dOs are contiguous)
+    // db over Qs, whose last reader was the key side; warp w the suffix sums of tokens 8w .. 8w+7, the warps' totals over Vs
+    float *dbs = Qs, *tot = Vs;
 #pragma unroll
-    for (int r = 0; r < 8; ++r)
+    for (int a = 0; a < 4; ++a)
 #pragma unroll
-        for (int cb = 0; cb < 4; ++cb) {
-            int i = ty + 8 * r, c = tx + 32 * cb;
-            if (c < d.dk) dbs[i * ldk + c] = db[r][cb];
-        }
+        for (int blk = 0; blk < NB; ++blk)
+            if (t.col(blk) < d.dk)
+                stf4(dbs, t.row(a) * ldk + t.col(blk), make_float4(db[a][4 * blk], db[a][4 * blk + 1], db[a][4 * blk + 2], db[a][4 * blk + 3]));
     __syncthreads();
-    for (int c = threadIdx.x; c < d.dk; c += blockDim.x) {
-        float run = Rs[c];
-        for (int i = cn - 1; i >= 0; --i) {
-            run += dbs[i * ldk + c];
-            dlog_decay[tok_row(d, b, t0 + i, h) * d.dk + c] = run;
+    const int c = 4 * tx;
+    float4 x[8], run = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (c < d.dk) {
+#pragma unroll
+        for (int i = 7; i >= 0; --i) {
+            x[i] = *reinterpret_cast<const float4 *>(dbs + (8 * ty + i) * ldk + c);
+            run.x += x[i].x; run.y += x[i].y; run.z += x[i].z; run.w += x[i].w;
         }
+        stf4(tot, ty * ldk + c, run);
+    }
+    __syncthreads();
+    if (c >= d.dk) return;
+    run = *reinterpret_cast<const float4 *>(Rs + c);
+    for (int g = 7; g > ty; --g) {
+        const float4 y = *reinterpret_cast<const float4 *>(tot + g * ldk + c);
+        run.x += y.x; run.y += y.y; run.z += y.z; run.w += y.w;
+    }
+#pragma unroll
+    for (int i = 7; i >= 0; --i) {
+        run.x += x[i].x; run.y += x[i].y; run.z += x[i].z; run.w += x[i].w;
+        if (8 * ty + i < cn) stf4(dlog_decay, tok_row(d, b, t0 + 8 * ty + i, h) * d.dk + c, run);
     }
 }
 
@@ -698,24 +778,24 @@ size_t smem_prepare(const Dims &d) {
 size_t smem_scan(const Dims &d) {
     return sizeof(float) * (2 * CMAX * (d.dk + 1) + CMAX * VS + d.dk * VS + CMAX);
 }
-size_t smem_outer(const Dims &d) { return sizeof(float) * CMAX * (65 + d.dv + 1); }
+size_t smem_outer(const Dims &d) { return sizeof(float) * CMAX * (pad4(64) + pad4(d.dv)); }
 size_t smem_output(const Dims &d) {
-    return sizeof(float) * (2 * CMAX * (d.dk + 1) + CMAX * (d.dv + 1) + CMAX * (CMAX + 1) + d.dk * (d.dv + 1));
+    return sizeof(float) * (2 * CMAX * pad4(d.dk) + CMAX * pad4(d.dv) + CMAX * pad4(CMAX) + d.dk * pad4(d.dv));
 }
 size_t smem_dscan(const Dims &d) {
     return sizeof(float) * (3 * CMAX * (d.dk + 1) + 2 * CMAX * VS + CMAX * (CMAX + 1) + d.dk * VS);
 }
 size_t smem_grads_lin(const Dims &d) {
-    return sizeof(float) * (2 * CMAX * (d.dk + 1) + 2 * CMAX * (d.dv + 1) + 2 * CMAX * (CMAX + 1) +
-                            d.dk * (d.dv + 1) + d.dk);
+    return sizeof(float) * (2 * CMAX * pad4(d.dk) + 2 * CMAX * pad4(d.dv) + CMAX * pad4(CMAX) + d.dk * pad4(d.dv) + d.dk + 8 * CMAX);
 }
 
 template <int HP>
-void launch_gate_fwd(const float *lq, const float *lk, float *Gq, float *Gk, long n_tok, int H,
-                     cudaStream_t st) {
-    long threads = n_tok * HP;
-    dim3 grid((unsigned)((threads + 255) / 256), 2);
-    k_gate_fwd<HP><<<grid, 256, 0, st>>>(lq, lk, Gq, Gk, n_tok, H);
+void launch_gates_decay(const Dims &d, const Workspace &w, const FwdArgs &a, cudaStream_t st) {
+    const long chunks = (long)d.B * d.H * d.NT;
+    const int gate_blocks = (int)(((long)d.B * d.T * HP + 255) / 256);
+    const long decay_blocks = d.variant == SLA_GLA ? chunks : (chunks + 7) / 8;
+    k_gates_decay<HP><<<(unsigned)(gate_blocks + decay_blocks), 256, 0, st>>>(d, a.lq, a.lk, a.ws + w.Gq, a.ws + w.Gk, a.log_decay, a.ws + w.bcum,
+                                                                              gate_blocks, a.status);
 }
 template <int HP>
 void launch_gate_bwd(const float *Gq, const float *Gk, const float *dGq, const float *dGk, float *dlq,
@@ -730,24 +810,20 @@ int forward_t(const Dims &d, const Workspace &w, const FwdArgs &a, bool write_o,
     float *ws = a.ws;
     float *Gq = ws + w.Gq, *Gk = ws + w.Gk, *bcum = ws + w.bcum, *states = ws + w.states;
     float *Wws = ws + w.W, *U0ws = ws + w.U0, *Uws = ws + w.U;
-    long n_tok = (long)d.B * d.T;
     int launches = 0;
     int hp = 1;
     while (hp < d.H) hp <<= 1;
     switch (hp) {
-        case 1: launch_gate_fwd<1>(a.lq, a.lk, Gq, Gk, n_tok, d.H, st); break;
-        case 2: launch_gate_fwd<2>(a.lq, a.lk, Gq, Gk, n_tok, d.H, st); break;
-        case 4: launch_gate_fwd<4>(a.lq, a.lk, Gq, Gk, n_tok, d.H, st); break;
-        case 8: launch_gate_fwd<8>(a.lq, a.lk, Gq, Gk, n_tok, d.H, st); break;
-        case 16: launch_gate_fwd<16>(a.lq, a.lk, Gq, Gk, n_tok, d.H, st); break;
-        default: launch_gate_fwd<32>(a.lq, a.lk, Gq, Gk, n_tok, d.H, st); break;
+        case 1: launch_gates_decay<1>(d, w, a, st); break;
+        case 2: launch_gates_decay<2>(d, w, a, st); break;
+        case 4: launch_gates_decay<4>(d, w, a, st); break;
+        case 8: launch_gates_decay<8>(d, w, a, st); break;
+        case 16: launch_gates_decay<16>(d, w, a, st); break;
+        default: launch_gates_decay<32>(d, w, a, st); break;
     }
-    tr.mark("gate_fwd");
+    tr.mark("gates_decay");
     ++launches;
-    dim3 tiles(d.NT, d.B * d.H);
-    k_cumdecay<<<tiles, d.variant == SLA_GLA ? 128 : 32, 0, st>>>(d, a.log_decay, bcum, a.status);
-    tr.mark("cumdecay");
-    ++launches;
+    const dim3 tiles(d.NT, d.B * d.H);
     const TIO *q = (const TIO *)a.q, *k = (const TIO *)a.k, *v = (const TIO *)a.v;
     if (d.variant == SLA_GDN) {
         k_gdn_prepare<TIO><<<tiles, 256, smem_prepare(d), st>>>(d, k, v, a.beta, Gk, bcum, Wws, U0ws);
@@ -795,9 +871,8 @@ int backward_lin_t(const Dims &d, const Workspace &w, const BwdArgs &a, cudaStre
         tr.mark("chunk_outer");
         ++launches;
     }
-    k_grads_lin<TIO><<<tiles, 256, smem_grads_lin(d), st>>>(d, q, k, v, dO, Gq, Gk, bcum, states, dstates,
-                                                            (TIO *)a.dq, (TIO *)a.dk, (TIO *)a.dv,
-                                                            a.dlog_decay, dGq, dGk);
+    (d.dk <= 64 && d.dv <= 64 ? k_grads_lin<TIO, 1> : k_grads_lin<TIO, 2>)<<<tiles, 256, smem_grads_lin(d), st>>>(
+        d, q, k, v, dO, Gq, Gk, bcum, states, dstates, (TIO *)a.dq, (TIO *)a.dk, (TIO *)a.dv, a.dlog_decay, dGq, dGk);
     tr.mark("grads_lin");
     ++launches;
     return cudaGetLastError() == cudaSuccess ? launches : -1;
@@ -813,7 +888,7 @@ template <typename TIO> bool configure_t() {
     ok &= set_smem(k_chunk_outer<TIO, false>, smem_outer(d)) && set_smem(k_chunk_outer<TIO, true>, smem_outer(d)) &&
           set_smem(k_chunk_outer<TIO, true, true>, smem_outer(d));
     ok &= set_smem(k_dstate_scan<TIO>, smem_dscan(d));
-    ok &= set_smem(k_grads_lin<TIO>, smem_grads_lin(d));
+    ok &= set_smem(k_grads_lin<TIO, 1>, smem_grads_lin(d)) && set_smem(k_grads_lin<TIO, 2>, smem_grads_lin(d));
     return ok;
 }
 
@@ -828,11 +903,13 @@ int generic_forward(const Dims &d, const Workspace &w, const FwdArgs &a, bool wr
     return d.io_bf16 ? forward_t<__nv_bfloat16>(d, w, a, write_o, st, tr) : forward_t<float>(d, w, a, write_o, st, tr);
 }
 
-int generic_backward(const Dims &d, const Workspace &w, const BwdArgs &a, cudaStream_t st, Tracer &tr) {
-    // recompute gates, cumulative decays and the per-chunk states (no output store)
-    FwdArgs f{a.q, a.k, a.v, a.log_decay, a.beta, a.lq, a.lk, a.h0, nullptr, nullptr, a.ws, a.status};
-    int n1 = generic_forward(d, w, f, false, st, tr);
-    if (n1 < 0) return -1;
+int generic_backward(const Dims &d, const Workspace &w, const BwdArgs &a, bool have_states, cudaStream_t st, Tracer &tr) {
+    int n1 = 0;
+    if (!have_states) {     // recompute gates, cumulative decays and the per-chunk states (no output store)
+        FwdArgs f{a.q, a.k, a.v, a.log_decay, a.beta, a.lq, a.lk, a.h0, nullptr, nullptr, a.ws, a.status};
+        n1 = generic_forward(d, w, f, false, st, tr);
+        if (n1 < 0) return -1;
+    }
     int n2;
     if (d.variant == SLA_GDN) {
         float *ws = a.ws;

@@ -66,6 +66,88 @@ __device__ __forceinline__ void tile_gemm(float (&acc)[8][NB], const float *A, i
     else tile_gemm_blocks<NB, NB>(acc, A, sa_i, sa_k, Bm, sb_k, sb_j, K, N, ty, tx);
 }
 
+// ------------------------------------------------------------------------------------------
+// The same products from 4 x 4 register tiles and 16-byte shared-memory reads, for the Softmax-RetNet / -GLA kernels: 8 reads for 64
+// multiply-adds where tile_gemm issues 40, whole 16-byte pieces into shared memory and out to global memory.  Both are bound by
+// the shared-memory pipe (a 16-byte read takes it four cycles: 4,100 for a 64 x 64 x 64 product, 5,100 for tile_gemm).  2 x 1000 tokens x 4 heads of
+// 64: k_grads_lin 63 -> 41 us, k_output 18 -> 16.  256 threads: thread (tr, tc)
+// owns rows tr + 16 a and columns 64 blk + 4 tc + b (a, b < 4) of a 64 x N tile, acc[a][4 blk + b].  Operands are stored with
+// leading dimensions pad4(width): 16-byte rows, and eight neighbouring rows start in different groups of four banks.
+__host__ __device__ constexpr int pad4(int width) { return width + 4; }
+struct Tile {
+    int tr, tc;
+    __device__ __forceinline__ Tile() {
+        const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+        tr = (lane >> 2) + 8 * (w & 1);
+        tc = (lane & 3) + 4 * (w >> 1);
+    }
+    __device__ __forceinline__ int row(int a) const { return tr + 16 * a; }
+    __device__ __forceinline__ int col(int blk) const { return 64 * blk + 4 * tc; }
+};
+// acc += A[i][k] B: A has its rows along k.  BT: B[k][j], else B[j][k].  K a multiple of four (rows past the last token are zero).
+template <int NB, bool BT>
+__device__ __forceinline__ void mm(float (&acc)[4][4 * NB], const Tile &t, const float *A, int lda, const float *B, int ldb, int K, int N) {
+#pragma unroll 2
+    for (int k = 0; k < K; k += 4) {
+        float4 a[4];
+#pragma unroll
+        for (int x = 0; x < 4; ++x) a[x] = *reinterpret_cast<const float4 *>(A + t.row(x) * lda + k);
+#pragma unroll
+        for (int blk = 0; blk < NB; ++blk) {
+            if (t.col(blk) >= N) continue;
+            float4 b[4];
+#pragma unroll
+            for (int y = 0; y < 4; ++y)
+                b[y] = *reinterpret_cast<const float4 *>(BT ? B + (k + y) * ldb + t.col(blk) : B + (t.col(blk) + y) * ldb + k);
+#pragma unroll
+            for (int x = 0; x < 4; ++x)
+#pragma unroll
+                for (int y = 0; y < 4; ++y) {
+                    float &c = acc[x][4 * blk + y];
+                    if (BT) {
+                        const float *b0 = reinterpret_cast<const float *>(&b[0]), *b1 = reinterpret_cast<const float *>(&b[1]),
+                                    *b2 = reinterpret_cast<const float *>(&b[2]), *b3 = reinterpret_cast<const float *>(&b[3]);
+                        c = fmaf(a[x].x, b0[y], c); c = fmaf(a[x].y, b1[y], c); c = fmaf(a[x].z, b2[y], c); c = fmaf(a[x].w, b3[y], c);
+                    } else {
+                        c = fmaf(a[x].x, b[y].x, c); c = fmaf(a[x].y, b[y].y, c); c = fmaf(a[x].z, b[y].z, c); c = fmaf(a[x].w, b[y].w, c);
+                    }
+                }
+        }
+    }
+}
+// acc += X^T Y over the tokens: X[k][i], Y[k][j]; thread (tr, tc) owns rows 4 tr + a instead.
+template <int NB>
+__device__ __forceinline__ void mm_outer(float (&acc)[4][4 * NB], const Tile &t, const float *X, int ldx, const float *Y, int ldy, int K, int M, int N) {
+    if (4 * t.tr >= M) return;
+#pragma unroll 4
+    for (int k = 0; k < K; ++k) {
+        const float4 x4 = *reinterpret_cast<const float4 *>(X + k * ldx + 4 * t.tr);
+        const float x[4] = {x4.x, x4.y, x4.z, x4.w};
+#pragma unroll
+        for (int blk = 0; blk < NB; ++blk) {
+            if (t.col(blk) >= N) continue;
+            const float4 y4 = *reinterpret_cast<const float4 *>(Y + k * ldy + t.col(blk));
+#pragma unroll
+            for (int a = 0; a < 4; ++a) {
+                acc[a][4 * blk] = fmaf(x[a], y4.x, acc[a][4 * blk]);         acc[a][4 * blk + 1] = fmaf(x[a], y4.y, acc[a][4 * blk + 1]);
+                acc[a][4 * blk + 2] = fmaf(x[a], y4.z, acc[a][4 * blk + 2]); acc[a][4 * blk + 3] = fmaf(x[a], y4.w, acc[a][4 * blk + 3]);
+            }
+        }
+    }
+}
+template <int NC> __device__ __forceinline__ void zero_acc(float (&acc)[4][NC]) {
+#pragma unroll
+    for (int a = 0; a < 4; ++a)
+#pragma unroll
+        for (int c = 0; c < NC; ++c) acc[a][c] = 0.f;
+}
+// four neighbouring results of a tile in the I/O dtype
+__device__ __forceinline__ void stf4(float *p, size_t i, float4 v) { *reinterpret_cast<float4 *>(p + i) = v; }
+__device__ __forceinline__ void stf4(__nv_bfloat16 *p, size_t i, float4 v) {
+    const __nv_bfloat162 lo = __floats2bfloat162_rn(v.x, v.y), hi = __floats2bfloat162_rn(v.z, v.w);
+    *reinterpret_cast<uint2 *>(p + i) = make_uint2(*reinterpret_cast<const uint32_t *>(&lo), *reinterpret_cast<const uint32_t *>(&hi));
+}
+
 template <int NB> __device__ __forceinline__ void zero_acc(float (&acc)[8][NB]) {
 #pragma unroll
     for (int r = 0; r < 8; ++r)
