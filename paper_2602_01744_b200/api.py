@@ -111,7 +111,28 @@ def lib():
                      "sla_plan_kernel_timing_get", "sla_forward", "sla_backward", "sla_decode_step"):
             getattr(L, name).restype = ctypes.c_int
         _lib = L
+        _load_fast(L)
     return _lib
+
+
+# The decode calls' native marshalling (native/fastcall.cpp) and the addresses of the two entry points, or None: the same checks and the same
+# call as below in one C function, for plain contiguous CUDA tensors.  It answers None to anything else.
+_fast = None
+
+
+def _load_fast(L):
+    global _fast
+    try:
+        from . import build as _build
+        _build.build_fast()
+    except Exception:                           # no compiler here: an existing build is still fine
+        pass
+    try:
+        from . import _sla_fast
+    except ImportError:
+        return
+    addr = lambda f: ctypes.cast(f, ctypes.c_void_p).value
+    _fast = (_sla_fast.decode, addr(L.sla_decode_step), addr(L.sla_decode_steps))
 
 
 def _check(call: str, status: int):
@@ -146,6 +167,7 @@ class Plan:
         self.forward_workspace_bytes, self.backward_workspace_bytes = f.value, b.value
         self.io_torch = torch.bfloat16 if self.desc.io_dtype == SLA_BF16 else torch.float32
         self.heads, self.width_v = self.desc.H, self.desc.d_v
+        self._bf16 = int(self.desc.io_dtype == SLA_BF16)
         self._slots = B * (-(-T // chunk) + 1)                 # chunks and one more, over the sequences
 
     def close(self):
@@ -277,6 +299,13 @@ def sla_backward(plan: Plan, q, k, v, log_decay, gq_logits, gk_logits, dO, beta=
 def sla_decode_step(plan: Plan, q_t, k_t, v_t, log_decay_t, gq_logits_t, gk_logits_t, state, beta_t=None,
                     o_t=None):
     """One recurrent step on `state` ([Bdec,H,d_k,d_v] fp32, updated in place).  Returns o_t."""
+    if _fast is not None:
+        r = _fast[0](_fast[1], plan.handle.value or 0, plan.heads, plan.width_v, plan._bf16, 0, q_t, k_t, v_t, log_decay_t, gq_logits_t,
+                     gk_logits_t, state, beta_t, o_t)
+        if r is not None:
+            if r[0]:
+                _check("sla_decode_step", r[0])
+            return r[1]
     Bdec = q_t.shape[0]
     if o_t is None:
         o_t = torch.empty((Bdec, plan.heads, plan.width_v), dtype=plan.io_torch, device=q_t.device)
@@ -291,6 +320,13 @@ def sla_decode_step(plan: Plan, q_t, k_t, v_t, log_decay_t, gq_logits_t, gk_logi
 def sla_decode_steps(plan: Plan, q, k, v, log_decay, gq_logits, gk_logits, state, beta=None, o=None):
     """n consecutive recurrent steps per sequence on `state` ([Bdec,H,d_k,d_v] fp32, updated in place): q, k
     [Bdec,n,H,d_k], v [Bdec,n,H,d_v].  Returns o [Bdec,n,H,d_v]."""
+    if _fast is not None:
+        r = _fast[0](_fast[2], plan.handle.value or 0, plan.heads, plan.width_v, plan._bf16, 1, q, k, v, log_decay, gq_logits, gk_logits,
+                     state, beta, o)
+        if r is not None:
+            if r[0]:
+                _check("sla_decode_steps", r[0])
+            return r[1]
     d = plan.desc
     Bdec, n = q.shape[0], q.shape[1]
     if o is None:
