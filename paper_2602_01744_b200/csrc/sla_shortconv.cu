@@ -212,6 +212,33 @@ k_shortconv_fwd_blocks(ConvDims cd, int B, const TIO *__restrict__ x, const floa
     }
 }
 
+// Units of `per` neighbouring tokens of one sequence, for kernels in which a group of threads walks one.
+struct Units {
+    int per, per_seq;                                   // tokens of a unit, units of a sequence
+    long total;
+    __device__ __forceinline__ void at(long unit, int T, int &b, int &t0, int &t1) const {
+        b = (int)(unit / per_seq);
+        t0 = (int)(unit - (long)b * per_seq) * per;
+        t1 = min(T, t0 + per);
+    }
+};
+constexpr int AHEAD = 4;                                // tokens fetched ahead
+// four channels of a bf16 row
+struct Four {
+    static __device__ __forceinline__ void widen(const uint2 v, float (&x)[4]) {
+        const float2 a = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&v.x));
+        const float2 b = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&v.y));
+        x[0] = a.x; x[1] = a.y; x[2] = b.x; x[3] = b.y;
+    }
+    static __device__ __forceinline__ void store(__nv_bfloat16 *p, const float (&x)[4]) {
+        const __nv_bfloat162 lo = __floats2bfloat162_rn(x[0], x[1]), hi = __floats2bfloat162_rn(x[2], x[3]);
+        *reinterpret_cast<uint2 *>(p) = make_uint2(*reinterpret_cast<const uint32_t *>(&lo), *reinterpret_cast<const uint32_t *>(&hi));
+    }
+};
+__device__ __forceinline__ uint2 fetch4(const __nv_bfloat16 *row0, int t, int lo, int hi, int C, bool live) {
+    return live && t >= lo && t < hi ? __ldg(reinterpret_cast<const uint2 *>(row0 + (size_t)t * C)) : make_uint2(0u, 0u);
+}
+
 // Reverse pass.  partial: [CTAs][H*d][KMAX] per-CTA sums of the tap gradients.
 template <typename TIO, bool NORM, bool SHFL>
 __global__ void __launch_bounds__(256, 2)
@@ -326,111 +353,120 @@ k_shortconv_bwd(ConvDims cd, const TIO *__restrict__ x, const float *__restrict_
     }
 }
 
-// Reverse pass without state carried from block to block (bf16, heads that are a power-of-two run of lanes): blocks of
-// TB tokens are dealt round robin to the CTAs; a thread owns FOUR channels and fetches, packed and all in flight together,
-// the TB + 6 rows of x and the TB + 3 rows of dout its block needs (dx of a token needs dy of the three tokens after it,
-// each of which needs the three rows of x before it; the overlap with the neighbouring blocks comes from L2).  It then
-// walks the block backwards with the window in registers: every row is widened once and serves y, dx and the tap
-// gradients.  Head sums by shuffles, no shared memory, no barrier.  Tap gradients are summed per thread over its blocks
-// and written per CTA.
+// Reverse pass of bf16 heads that are a power-of-two run of lanes (four channels a thread).  The sequences are cut into as many units of
+// neighbouring tokens as the GPU holds groups of 256 threads, two groups a CTA and one CTA per SM, and a group walks its unit backwards - dx of
+// a token needs dy of the three tokens after it, so a walk starts three tokens past its unit - with the windows over x and dy in
+// registers and the rows of four tokens fetched ahead; every row of x and dout is fetched and widened once and serves y, dx
+// and the tap gradients.  Head sums by shuffles.  Tap gradients are summed per thread over its units, the two groups' sums added, and
+// written per CTA.  Bound by instruction issue (sigmoid, its derivative, three 4-tap sums and the norm terms an element).  In blocks of eight tokens,
+// 14 rows of x and 11 of dout fetched and 11 tokens recomputed for eight written, as many CTAs as the workspace has slots: 2 x 2048 tokens
+// x 2048 channels 30 us, 24 now (the layer step with three of them 490 -> 472).
+constexpr int BWD_GROUPS = 2;
 template <bool NORM>
-__global__ void __launch_bounds__(256, 2)
-k_shortconv_bwd_blocks(ConvDims cd, int B, const __nv_bfloat16 *__restrict__ x, const float *__restrict__ w,
-                       const __nv_bfloat16 *__restrict__ dout, __nv_bfloat16 *__restrict__ dx, float *__restrict__ partial) {
-    constexpr int N = 4, TB = 8;
-    const int C = cd.H * cd.d, vpr = cd.d / N, tid = threadIdx.x;
-    const int hb = blockIdx.z * cd.hpc, nh = min(cd.hpc, cd.H - hb);
-    const bool live = tid < nh * vpr;
-    const int gv = hb * vpr + tid;
+__global__ void __launch_bounds__(256 * BWD_GROUPS, 1)
+k_shortconv_bwd_walk(ConvDims cd, Units un, const __nv_bfloat16 *__restrict__ x, const float *__restrict__ w,
+                     const __nv_bfloat16 *__restrict__ dout, __nv_bfloat16 *__restrict__ dx, float *__restrict__ partial) {
+    constexpr int N = 4;
+    using F = Four;
+    __shared__ float4 sums[BWD_GROUPS - 1][N][256];
+    const int C = cd.H * cd.d, vpr = cd.d / N, group = threadIdx.x >> 8, tid = threadIdx.x & 255, gv = blockIdx.y * 256 + tid;
+    const bool live = gv < C / N;
     float wt[KMAX][N], acc[KMAX][N];
     load_taps<N>(w, gv * N, cd.K, live, wt);
 #pragma unroll
     for (int j = 0; j < KMAX; ++j)
 #pragma unroll
         for (int e = 0; e < N; ++e) acc[j][e] = 0.f;
-    auto widen = [](const uint2 v, float (&f)[N]) {
-        const float2 a = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&v.x));
-        const float2 b = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&v.y));
-        f[0] = a.x; f[1] = a.y; f[2] = b.x; f[3] = b.y;
-    };
-    const int nblk = (cd.T + TB - 1) / TB;
-    for (long item = blockIdx.x; item < (long)B * nblk; item += gridDim.x) {
-        const int b = (int)(item / nblk), t = (int)(item % nblk) * TB;
+    for (long unit = (long)blockIdx.x * BWD_GROUPS + group; unit < un.total; unit += (long)gridDim.x * BWD_GROUPS) {
+        int b, t0, t1;
+        un.at(unit, cd.T, b, t0, t1);
+        const int ue = min(cd.T, t1 + KMAX - 1) - 1;            // last token whose dy this unit needs
         const size_t rowoff = ((size_t)b * cd.T) * C + (size_t)gv * N;
         const __nv_bfloat16 *xr = x + rowoff, *gr = dout + rowoff;
-        uint2 rx[TB + 6], rg[TB + 3];                   // x rows t-3 .. t+TB+2, dout rows t .. t+TB+2 (zero outside the sequence)
+        uint2 nx[AHEAD], ng[AHEAD];                             // x of tokens u-3, u-4, ..; dout of tokens u, u-1, ..
 #pragma unroll
-        for (int s = 0; s < TB + 6; ++s) {
-            const int tt = t - 3 + s;
-            rx[s] = (live && tt >= 0 && tt < cd.T) ? __ldg(reinterpret_cast<const uint2 *>(xr + (size_t)tt * C)) : make_uint2(0u, 0u);
-        }
-#pragma unroll
-        for (int s = 0; s < TB + 3; ++s) {
-            const int tt = t + s;
-            rg[s] = (live && tt < cd.T) ? __ldg(reinterpret_cast<const uint2 *>(gr + (size_t)tt * C)) : make_uint2(0u, 0u);
+        for (int s = 0; s < AHEAD; ++s) {
+            nx[s] = fetch4(xr, ue - 3 - s, 0, cd.T, C, live);
+            ng[s] = fetch4(gr, ue - s, t0, cd.T, C, live);
         }
         float x1[N], x2[N], x3[N], dy1[N], dy2[N], dy3[N];      // x of tokens u-2, u-1, u; dy of tokens u+1, u+2, u+3
-        widen(rx[TB + 3], x1);
-        widen(rx[TB + 4], x2);
-        widen(rx[TB + 5], x3);
+        F::widen(fetch4(xr, ue - 2, 0, cd.T, C, live), x1);
+        F::widen(fetch4(xr, ue - 1, 0, cd.T, C, live), x2);
+        F::widen(fetch4(xr, ue, 0, cd.T, C, live), x3);
 #pragma unroll
         for (int e = 0; e < N; ++e) dy1[e] = dy2[e] = dy3[e] = 0.f;
+        for (int top = ue; top >= t0; top -= AHEAD) {
+            uint2 cx[AHEAD], cg[AHEAD];
 #pragma unroll
-        for (int s = TB + 2; s >= 0; --s) {             // token u = t + s; past the sequence end dout = 0 makes dy = 0
-            float x0[N], g[N], z[N], gs[N], dy[N], ss = 0.f, dot = 0.f;
-            widen(rx[s], x0);                           // x of token u-3
-            widen(rg[s], g);
-#pragma unroll
-            for (int e = 0; e < N; ++e) {
-                const float y = fmaf(wt[0][e], x0[e], fmaf(wt[1][e], x1[e], fmaf(wt[2][e], x2[e], wt[3][e] * x3[e])));
-                const float sg = __fdividef(1.f, 1.f + __expf(-y));
-                z[e] = y * sg;
-                gs[e] = sg * (1.f + y * (1.f - sg));            // d silu / dy
-                ss = fmaf(z[e], z[e], ss);
-                dot = fmaf(z[e], g[e], dot);
-            }
-            float fa = 1.f, fb = 0.f;
-            if (NORM) {                                 // out = z / r:  dz = dout / r - z (z . dout) / r^3
-                for (int o = vpr >> 1; o > 0; o >>= 1) {
-                    ss += __shfl_xor_sync(0xffffffffu, ss, o);
-                    dot += __shfl_xor_sync(0xffffffffu, dot, o);
-                }
-                const float ri = rsqrtf(ss + cd.eps);
-                fa = ri;
-                fb = dot * ri * ri * ri;
+            for (int s = 0; s < AHEAD; ++s) {
+                cx[s] = nx[s];
+                cg[s] = ng[s];
+                nx[s] = fetch4(xr, top - AHEAD - 3 - s, max(0, t0 - 3), cd.T, C, live);
+                ng[s] = fetch4(gr, top - AHEAD - s, t0, cd.T, C, live);
             }
 #pragma unroll
-            for (int e = 0; e < N; ++e) dy[e] = (g[e] * fa - z[e] * fb) * gs[e];
-            if (s < TB) {                               // this block's own tokens: dx out, tap gradients in
-                __nv_bfloat162 lo = __floats2bfloat162_rn(
-                    fmaf(wt[3][0], dy[0], fmaf(wt[2][0], dy1[0], fmaf(wt[1][0], dy2[0], wt[0][0] * dy3[0]))),
-                    fmaf(wt[3][1], dy[1], fmaf(wt[2][1], dy1[1], fmaf(wt[1][1], dy2[1], wt[0][1] * dy3[1]))));
-                __nv_bfloat162 hi = __floats2bfloat162_rn(
-                    fmaf(wt[3][2], dy[2], fmaf(wt[2][2], dy1[2], fmaf(wt[1][2], dy2[2], wt[0][2] * dy3[2]))),
-                    fmaf(wt[3][3], dy[3], fmaf(wt[2][3], dy1[3], fmaf(wt[1][3], dy2[3], wt[0][3] * dy3[3]))));
-                if (live && t + s < cd.T)
-                    *reinterpret_cast<uint2 *>(dx + rowoff + (size_t)(t + s) * C) =
-                        make_uint2(*reinterpret_cast<uint32_t *>(&lo), *reinterpret_cast<uint32_t *>(&hi));
+            for (int s = 0; s < AHEAD; ++s) {                   // token u; in front of the unit (dout read as zero) nothing leaves
+                const int u = top - s;
+                float x0[N], g[N], z[N], gs[N], dy[N], ss = 0.f, dot = 0.f;
+                F::widen(cx[s], x0);
+                F::widen(cg[s], g);
 #pragma unroll
                 for (int e = 0; e < N; ++e) {
-                    acc[0][e] = fmaf(dy[e], x0[e], acc[0][e]);
-                    acc[1][e] = fmaf(dy[e], x1[e], acc[1][e]);
-                    acc[2][e] = fmaf(dy[e], x2[e], acc[2][e]);
-                    acc[3][e] = fmaf(dy[e], x3[e], acc[3][e]);
+                    const float y = fmaf(wt[0][e], x0[e], fmaf(wt[1][e], x1[e], fmaf(wt[2][e], x2[e], wt[3][e] * x3[e])));
+                    const float sg = __fdividef(1.f, 1.f + __expf(-y));
+                    z[e] = y * sg;
+                    gs[e] = sg * (1.f + y * (1.f - sg));            // d silu / dy
+                    ss = fmaf(z[e], z[e], ss);
+                    dot = fmaf(z[e], g[e], dot);
                 }
-            }
+                float fa = 1.f, fb = 0.f;
+                if (NORM) {                                     // out = z / r:  dz = dout / r - z (z . dout) / r^3
+                    for (int o = vpr >> 1; o > 0; o >>= 1) {
+                        ss += __shfl_xor_sync(0xffffffffu, ss, o);
+                        dot += __shfl_xor_sync(0xffffffffu, dot, o);
+                    }
+                    const float ri = rsqrtf(ss + cd.eps);
+                    fa = ri;
+                    fb = dot * ri * ri * ri;
+                }
 #pragma unroll
-            for (int e = 0; e < N; ++e) {
-                dy3[e] = dy2[e]; dy2[e] = dy1[e]; dy1[e] = dy[e];
-                x3[e] = x2[e]; x2[e] = x1[e]; x1[e] = x0[e];
+                for (int e = 0; e < N; ++e) dy[e] = (g[e] * fa - z[e] * fb) * gs[e];
+                if (u < t1 && u >= t0) {                        // the unit's own tokens: dx out, tap gradients in
+                    float d[N];
+#pragma unroll
+                    for (int e = 0; e < N; ++e) {
+                        d[e] = fmaf(wt[3][e], dy[e], fmaf(wt[2][e], dy1[e], fmaf(wt[1][e], dy2[e], wt[0][e] * dy3[e])));
+                        acc[0][e] = fmaf(dy[e], x0[e], acc[0][e]);
+                        acc[1][e] = fmaf(dy[e], x1[e], acc[1][e]);
+                        acc[2][e] = fmaf(dy[e], x2[e], acc[2][e]);
+                        acc[3][e] = fmaf(dy[e], x3[e], acc[3][e]);
+                    }
+                    if (live) F::store(dx + rowoff + (size_t)u * C, d);
+                }
+#pragma unroll
+                for (int e = 0; e < N; ++e) {
+                    dy3[e] = dy2[e]; dy2[e] = dy1[e]; dy1[e] = dy[e];
+                    x3[e] = x2[e]; x2[e] = x1[e]; x1[e] = x0[e];
+                }
             }
         }
     }
-    if (live) {
-        float *dst = partial + ((size_t)blockIdx.x * C + (size_t)gv * N) * KMAX;
+    if (group > 0) {
 #pragma unroll
-        for (int e = 0; e < N; ++e)
-            *reinterpret_cast<float4 *>(dst + e * KMAX) = make_float4(acc[0][e], acc[1][e], acc[2][e], acc[3][e]);
+        for (int e = 0; e < N; ++e) sums[group - 1][e][tid] = make_float4(acc[0][e], acc[1][e], acc[2][e], acc[3][e]);
+    }
+    __syncthreads();
+    if (group > 0 || !live) return;
+    float *dst = partial + ((size_t)blockIdx.x * C + (size_t)gv * N) * KMAX;
+#pragma unroll
+    for (int e = 0; e < N; ++e) {
+        float4 v = make_float4(acc[0][e], acc[1][e], acc[2][e], acc[3][e]);
+#pragma unroll
+        for (int o = 0; o < BWD_GROUPS - 1; ++o) {
+            const float4 y = sums[o][e][tid];
+            v.x += y.x; v.y += y.y; v.z += y.z; v.w += y.w;
+        }
+        *reinterpret_cast<float4 *>(dst + e * KMAX) = v;
     }
 }
 
@@ -461,9 +497,21 @@ __global__ void __launch_bounds__(32 * DW_WARPS) k_shortconv_dw(int n_cta, int C
     for (int t = 0; t < K; ++t) dw[(size_t)c * K + t] = r[KMAX - K + t];
 }
 
-int tokens_per_cta(const Dims &d) {       // about four CTAs per SM, slices of at least 32 tokens
+int conv_sms() {
     int dev = 0, sms = 148;
     if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    return sms;
+}
+// Units of at least eight tokens (three more are read in front of each), about `groups` of them, cut alike from every sequence
+Units conv_units(const Dims &d, long groups) {
+    const long per_seq = std::max<long>(1, std::min<long>(groups / d.B, (d.T + 7) / 8));
+    Units un{(int)((d.T + per_seq - 1) / per_seq), 0, 0};
+    un.per_seq = (d.T + un.per - 1) / un.per;
+    un.total = (long)un.per_seq * d.B;
+    return un;
+}
+int tokens_per_cta(const Dims &d) {       // about four CTAs per SM, slices of at least 32 tokens
+    const int sms = conv_sms();
     const long total = (long)d.B * d.T, want = 4L * sms;
     long per = (total + want - 1) / want;
     if (per < 32) per = 32;           // (the reverse pass recomputes three tokens beyond its slice)
@@ -527,16 +575,14 @@ int shortconv_backward(const Dims &d, int width, int K, bool normalize, float ep
     const bool shfl = vpr <= 32 && (vpr & (vpr - 1)) == 0;
     const int C = d.H * width;
     const int vpr4 = width / 4;
-    if (d.io_bf16 && vpr4 <= 32 && (vpr4 & (vpr4 - 1)) == 0) {
-        int dev = 0, sms = 148;
-        if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        const int hpc4 = std::max(1, std::min(d.H, 256 / vpr4)), threads4 = (hpc4 * vpr4 + 31) / 32 * 32;
-        ConvDims cd4{d.T, d.H, width, K, cd.per, hpc4, eps};
-        // (no more CTAs than the workspace has partial-sum slots for)
-        const long slots = (long)grid.x * grid.y;
-        dim3 g((unsigned)std::min<long>(slots, 2L * sms), 1, (d.H + hpc4 - 1) / hpc4);
-        if (normalize) k_shortconv_bwd_blocks<true><<<g, threads4, 0, st>>>(cd4, d.B, (const __nv_bfloat16 *)x, w, (const __nv_bfloat16 *)dout, (__nv_bfloat16 *)dx, ws);
-        else k_shortconv_bwd_blocks<false><<<g, threads4, 0, st>>>(cd4, d.B, (const __nv_bfloat16 *)x, w, (const __nv_bfloat16 *)dout, (__nv_bfloat16 *)dx, ws);
+    if (d.io_bf16 && (vpr4 & (vpr4 - 1)) == 0) {
+        const int slabs = (d.H * vpr4 + 255) / 256;
+        // one CTA per SM (its 512 threads keep 128 registers each), and no more than the workspace has partial-sum slots for
+        const long ctas = std::min<long>((long)grid.x * grid.y, std::max(1, conv_sms() / slabs));
+        const Units un = conv_units(d, ctas * BWD_GROUPS);
+        const dim3 g((unsigned)std::min<long>(ctas, (un.total + BWD_GROUPS - 1) / BWD_GROUPS), slabs);
+        if (normalize) k_shortconv_bwd_walk<true><<<g, 256 * BWD_GROUPS, 0, st>>>(cd, un, (const __nv_bfloat16 *)x, w, (const __nv_bfloat16 *)dout, (__nv_bfloat16 *)dx, ws);
+        else k_shortconv_bwd_walk<false><<<g, 256 * BWD_GROUPS, 0, st>>>(cd, un, (const __nv_bfloat16 *)x, w, (const __nv_bfloat16 *)dout, (__nv_bfloat16 *)dx, ws);
         tr.mark("shortconv_bwd");
         k_shortconv_dw<<<(C + 31) / 32, 32 * DW_WARPS, 0, st>>>((int)g.x, C, K, ws, dw);
         tr.mark("shortconv_dw");
@@ -546,8 +592,7 @@ int shortconv_backward(const Dims &d, int width, int K, bool normalize, float ep
     k_shortconv_bwd<TIO, NORM, SH><<<grid, threads, smem, st>>>(cd, (const TIO *)x, w, (const TIO *)dout, (TIO *)dx, ws)
     if (d.io_bf16) {
         if (!normalize) SLA_LAUNCH_BWD(__nv_bfloat16, false, true);
-        else if (shfl) SLA_LAUNCH_BWD(__nv_bfloat16, true, true);
-        else SLA_LAUNCH_BWD(__nv_bfloat16, true, false);
+        else SLA_LAUNCH_BWD(__nv_bfloat16, true, false);           // (heads that are a run of lanes took the walk above)
     } else {
         if (!normalize) SLA_LAUNCH_BWD(float, false, true);
         else if (shfl) SLA_LAUNCH_BWD(float, true, true);
