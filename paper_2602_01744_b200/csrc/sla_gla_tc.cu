@@ -18,6 +18,9 @@
 // The state never leaves the SM: fp32 in TMEM (Eq. 12's S), bf16 copy in shared memory as MMA operand.
 #include "sla_gla_tc.cuh"
 
+#include <algorithm>
+#include <cmath>
+
 namespace sla {
 namespace {
 
@@ -35,13 +38,13 @@ constexpr uint32_t OFF_A = OFF_S + STATE_BF16;                  // masked A, [64
 constexpr uint32_t OFF_OST = OFF_A + HALF_BF16;                 // bf16 output tile staged for the TMA store
 constexpr uint32_t OFF_TOT = OFF_OST + TILE_BF16;               // prologue scratch
 constexpr uint32_t OFF_EB = OFF_TOT + TOT_BYTES;                // [4][128] 2^{b_last} of four chunks
-constexpr uint32_t OFF_GATE = OFF_EB + 4 * D * 4;               // [4][2][64]: scale*Gq, Gk of four chunks
+constexpr uint32_t OFF_GATE = OFF_EB + 4 * D * 4;               // [4][2][64]: scale*Gq, Gk of four chunks (a pair's, twice as many: in an unused block of the state operand)
 constexpr uint32_t OFF_BAR = OFF_GATE + 4 * 2 * C * 4;          // mbarriers, see Bar
 constexpr uint32_t OFF_TMEM = OFF_BAR + 40 * 8;                 // TMEM base address, then the abort flag
 constexpr uint32_t SMEM_BYTES = OFF_TMEM + 16 + 1024;           // + slack to align the base to 1024 B
 static_assert(SMEM_BYTES <= 232448, "shared memory budget");
 
-constexpr uint32_t COL_A = 0, COL_O = 64, COL_S = 320, TMEM_COLS = 512;   // O: two buffers of 128 columns
+constexpr uint32_t TMEM_COLS = 512;                                       // A 64 (a pair: 128), O two buffers of 128, S 128 columns
 constexpr int W_PRO = 8, W_MMA = 16, W_GATE = 17, W_TMA = 21;      // first warp of each role
 constexpr int NTHREADS = 2 * NCOMPUTE + 32 + NGATE + 32;
 
@@ -76,7 +79,9 @@ struct FwdParams {
 // The prologue of chunk n+1.. runs beside the mask / rescale / store work of chunk n, so the shared-memory,
 // special-function and FMA phases of the two groups overlap instead of following one another.
 // SCALAR: Softmax-RetNet, whose gate warps fold the constant decay into the gates and whose prologue only scales rows.
-template <bool SCALAR>
+// PAIR: two 64-wide heads a CTA (p.H, p.dk, p.dv: the single heads'; the tensor maps and blockIdx count pairs; one segment only).  Its A
+// takes 128 columns of tensor memory, its second masked A tile an unused block of the state operand.
+template <bool SCALAR, bool PAIR>
 __global__ void __launch_bounds__(NTHREADS, 1)
 k_gla_fwd_tc(const __grid_constant__ CUtensorMap gm_q, const __grid_constant__ CUtensorMap gm_k,
              const __grid_constant__ CUtensorMap gm_v, const __grid_constant__ CUtensorMap gm_g,
@@ -87,8 +92,12 @@ k_gla_fwd_tc(const __grid_constant__ CUtensorMap gm_q, const __grid_constant__ C
     uint8_t *sm = smem_raw + (base - raw);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     // a sequence may be cut into p.P segments of p.L chunks, one CTA each, every segment starting from its own state
-    const int bh = blockIdx.x / p.P, seg = blockIdx.x % p.P, h = bh % p.H;
-    int b = bh / p.H;
+    constexpr int HPC = PAIR ? 2 : 1;                       // heads per CTA
+    constexpr uint32_t COL_A = 0, COL_O = PAIR ? 128 : 64, COL_S = PAIR ? 384 : 320;
+    const int hg = p.H / HPC;
+    const int cta = blockIdx.x / p.P, seg = blockIdx.x % p.P, h = cta % hg;      // h: head, or pair of heads, as the tensor maps count them
+    int b = cta / hg;
+    const int bh = b * p.H + h * HPC;                       // the (first) head among all (sequence, head)
     // A packed batch: this CTA's sequence has its own length, chunk count, first token, state slots and tensor maps
     // (based at its first token, so token coordinates stay relative and the batch coordinate is 0).
     size_t tokb = (size_t)b * p.T, slot = (size_t)bh * (p.NT + 1);
@@ -99,8 +108,8 @@ k_gla_fwd_tc(const __grid_constant__ CUtensorMap gm_q, const __grid_constant__ C
         vm = p.vmaps + (size_t)b * Varlen::MAPS_PER_SEQ;
         p.T = si.T; p.NT = si.NT; p.L = si.NT;
         tokb = (size_t)si.t0;
-        slot = (size_t)si.slot0 * p.H + (size_t)h * (si.NT + 1);
-        sbh = (size_t)si.id * p.H + h;                      // (the table is ordered longest first, the state tensors as the caller gave them)
+        slot = (size_t)si.slot0 * p.H + (size_t)h * HPC * (si.NT + 1);
+        sbh = (size_t)si.id * p.H + h * HPC;                      // (the table is ordered longest first, the state tensors as the caller gave them)
         b = 0;
     }
     const CUtensorMap &tm_q = vm ? vm[0] : gm_q, &tm_k = vm ? vm[1] : gm_k, &tm_v = vm ? vm[2] : gm_v,
@@ -109,7 +118,7 @@ k_gla_fwd_tc(const __grid_constant__ CUtensorMap gm_q, const __grid_constant__ C
     auto bar = [&](int i) { return base + OFF_BAR + 8u * i; };
     float *tot = reinterpret_cast<float *>(sm + OFF_TOT);
     float *eblast = reinterpret_cast<float *>(sm + OFF_EB);
-    float *gate_s = reinterpret_cast<float *>(sm + OFF_GATE);
+    float *gate_s = reinterpret_cast<float *>(sm + (PAIR ? OFF_S + PAIR_FREE1 : OFF_GATE));
     // Every wait is bounded.  The first thread whose wait expires raises the CTA's abort flag; from then on nobody
     // waits any more, the control lane stops issuing and drains what is in flight, and the kernel reports the failure.
     volatile int *abort_flag = reinterpret_cast<volatile int *>(sm + OFF_TMEM + 8);
@@ -148,6 +157,7 @@ k_gla_fwd_tc(const __grid_constant__ CUtensorMap gm_q, const __grid_constant__ C
             constexpr uint32_t ID_A = idesc_bf16(64, 64, 0, 0);      // qh (K-major) x kh (K-major)
             constexpr uint32_t ID_O = idesc_bf16(64, 128, 0, 1);     // qh x S, A x V (B operand MN-major)
             constexpr uint32_t ID_Z = idesc_bf16(128, 128, 1, 1);    // kh^T (MN-major) x V (MN-major)
+            constexpr uint32_t ID_64 = idesc_bf16(64, 64, 0, 0), ID_64M = idesc_bf16(64, 64, 0, 1);
             auto issue_a = [&](int n) {                              // A_n = qh kh^T, one chunk ahead of the recurrence
                 const uint32_t sQ = base + OFF_QK + (n % 3) * QK_BYTES, sK = sQ + TILE_BF16;
                 wait(OPR + n % 3, (n / 3) & 1);                      // qh, kh of chunk n are in place
@@ -156,8 +166,9 @@ k_gla_fwd_tc(const __grid_constant__ CUtensorMap gm_q, const __grid_constant__ C
                 tc_fence_after();
                 if (leader)
 #pragma unroll
-                for (int kk = 0; kk < 8; ++kk)
-                    tc_mma_bf16(tmem + COL_A, (desc_kmajor(sQ) + kstep_kmajor(kk, HALF_BF16)), (desc_kmajor(sK) + kstep_kmajor(kk, HALF_BF16)), ID_A, kk > 0);
+                for (int kk = 0; kk < 8; ++kk)                       // (a pair: head kk / 4's half of the tiles, columns of its own)
+                    tc_mma_bf16(tmem + COL_A + (PAIR ? 64 * (kk >> 2) : 0), (desc_kmajor(sQ) + kstep_kmajor(kk, HALF_BF16)),
+                                (desc_kmajor(sK) + kstep_kmajor(kk, HALF_BF16)), PAIR ? ID_64 : ID_A, PAIR ? (kk & 3) > 0 : kk > 0);
                 if (leader) tc_commit(bar(BAR_A));
             };
             issue_a(0);
@@ -178,8 +189,13 @@ k_gla_fwd_tc(const __grid_constant__ CUtensorMap gm_q, const __grid_constant__ C
                     tc_mma_bf16(tmem + COL_S, (desc_mnmajor(sK, HALF_BF16) + kstep_mnmajor(kk)), (desc_mnmajor(sV, HALF_BF16) + kstep_mnmajor(kk)), ID_Z, 1);
                 if (leader)
 #pragma unroll
-                for (int kk = 0; kk < 8; ++kk)
-                    tc_mma_bf16(tO, (desc_kmajor(sQ) + kstep_kmajor(kk, HALF_BF16)), (desc_mnmajor(base + OFF_S, STATE_HALF) + kstep_mnmajor(kk)), ID_O, kk > 0);
+                for (int kk = 0; kk < 8; ++kk) {
+                    if (PAIR)      // head kk / 4: its half of qh, its block of S, its half of O
+                        tc_mma_bf16(tO + 64 * (kk >> 2), (desc_kmajor(sQ) + kstep_kmajor(kk, HALF_BF16)),
+                                    (desc_mnmajor(base + OFF_S + pair_block(kk >> 2), STATE_HALF) + kstep_mnmajor(kk & 3)), ID_64M, (kk & 3) > 0);
+                    else
+                        tc_mma_bf16(tO, (desc_kmajor(sQ) + kstep_kmajor(kk, HALF_BF16)), (desc_mnmajor(base + OFF_S, STATE_HALF) + kstep_mnmajor(kk)), ID_O, kk > 0);
+                }
                 if (leader) tc_commit(bar(BAR_Z));
                 if (leader) tc_commit(bar(QKFREE + n % 3));        // (same event, own barrier: the TMA lane may look at it much later)
                 // beside the rescale: A of the next chunk, then A V of this one
@@ -189,8 +205,15 @@ k_gla_fwd_tc(const __grid_constant__ CUtensorMap gm_q, const __grid_constant__ C
                 tc_fence_after();
                 if (leader)
 #pragma unroll
-                for (int kk = 0; kk < 4; ++kk)         // O += A V
-                    tc_mma_bf16(tO, (desc_kmajor(base + OFF_A) + kstep_kmajor(kk, 0)), (desc_mnmajor(sV, HALF_BF16) + kstep_mnmajor(kk)), ID_O, 1);
+                for (int kk = 0; kk < 4; ++kk) {       // O += A V
+                    if (PAIR) {
+                        tc_mma_bf16(tO, (desc_kmajor(base + OFF_A) + kstep_kmajor(kk, 0)), (desc_mnmajor(sV, HALF_BF16) + kstep_mnmajor(kk)), ID_64M, 1);
+                        tc_mma_bf16(tO + 64, (desc_kmajor(base + OFF_S + PAIR_FREE0) + kstep_kmajor(kk, 0)),
+                                    (desc_mnmajor(sV + HALF_BF16, HALF_BF16) + kstep_mnmajor(kk)), ID_64M, 1);
+                    } else {
+                        tc_mma_bf16(tO, (desc_kmajor(base + OFF_A) + kstep_kmajor(kk, 0)), (desc_mnmajor(sV, HALF_BF16) + kstep_mnmajor(kk)), ID_O, 1);
+                    }
+                }
                 if (leader) tc_commit(bar(BAR_O + (n & 1)));
             }
             // let the tensor core finish before TMEM goes away (after an abort some of its work may still be queued)
@@ -231,7 +254,12 @@ k_gla_fwd_tc(const __grid_constant__ CUtensorMap gm_q, const __grid_constant__ C
                     progress = true;
                 }
                 if (nsv <= NT && ready(SREADY, nsv & 1)) {                       // S_nsv stands in shared memory
-                    bulk_store(img0 + (size_t)nsv * STATE_BF16, base + OFF_S, STATE_BF16);
+                    if (PAIR) {
+                        bulk_store(img0 + (size_t)nsv * PAIR_STATE, base + OFF_S + pair_block(0), STATE_BLOCK);
+                        bulk_store(img0 + (size_t)nsv * PAIR_STATE + STATE_BLOCK, base + OFF_S + pair_block(1), STATE_BLOCK);
+                    } else {
+                        bulk_store(img0 + (size_t)nsv * STATE_BF16, base + OFF_S, STATE_BF16);
+                    }
                     bulk_commit();
                     bulk_wait_read0();
                     mbar_arrive(bar(SSAVED));
@@ -263,16 +291,16 @@ k_gla_fwd_tc(const __grid_constant__ CUtensorMap gm_q, const __grid_constant__ C
         // ---------------- gates: softmax over the heads, up to four chunks ahead ----------------
         const int g = tid - 32 * W_GATE, t = g & (C - 1);
         const float *l = g < C ? p.lq : p.lk;
-        const float mult = g < C ? p.scale : 1.f;
-        const float lg = SCALAR ? (g < C ? LOG2E : -LOG2E) * p.log_gamma[h] : 0.f;
+        const float mult = g < C ? p.scale : 1.f, sign = g < C ? LOG2E : -LOG2E;
+        const float lg = SCALAR ? sign * p.log_gamma[HPC * h] : 0.f, lg2 = SCALAR && PAIR ? sign * p.log_gamma[2 * h + 1] : 0.f;
         for (int n = 0; n < NT; ++n) {
             if (n >= 4) wait_relaxed(GFREE + (n & 3), ((n >> 2) - 1) & 1);
             if (failed) break;
             const int cn = min(C, p.T - (n0 + n) * C);
             const float *lc = l + (tokb + (size_t)(n0 + n) * C) * p.H;
-            float *dst = gate_s + (n & 3) * 2 * C + (g < C ? 0 : C);
-            if (SCALAR) chunk_gate_by(lc, p.H, cn, h, DecayFactor{mult, lg}, dst, t);
-            else chunk_gate(lc, p.H, cn, h, mult, dst, t);
+            float *dst = gate_s + (n & 3) * HPC * 2 * C + (g < C ? 0 : C), *dst2 = dst + 2 * C;
+            if (SCALAR) chunk_gate_by<64, HPC>(lc, p.H, cn, HPC * h, DecayFactor{mult, lg}, dst, t, DecayFactor{mult, lg2}, dst2);
+            else chunk_gate_by<64, HPC>(lc, p.H, cn, HPC * h, ConstFactor{mult}, dst, t, ConstFactor{mult}, dst2);
             __syncwarp();
             if (lane == 0) mbar_arrive(bar(GREADY + (n & 3)));
         }
@@ -284,22 +312,23 @@ k_gla_fwd_tc(const __grid_constant__ CUtensorMap gm_q, const __grid_constant__ C
             tma_load_4d(base + OFF_G, &tm_g, 0, h, (n0 + n) * C, b, bar(FULL_G));
         };
         if (ptid == 0 && !SCALAR) load_g(0);
-        if (ptid == 0 && SCALAR) check_scalar_range(p.log_gamma[h], p.T, p.status);
+        if (ptid < HPC && SCALAR) check_scalar_range(p.log_gamma[HPC * h + ptid], p.T, p.status);
         for (int n = 0; n < NT; ++n) {
             wait(GREADY + (n & 3), (n >> 2) & 1);
             if (!SCALAR) wait(FULL_G, n & 1);
             wait(FULL_QK + n % 3, (n / 3) & 1);
             if (failed) break;
             uint8_t *qk = sm + OFF_QK + (n % 3) * QK_BYTES;
-            const float *g = gate_s + (n & 3) * 2 * C;
+            const float *g = gate_s + (n & 3) * HPC * 2 * C;
+            constexpr int GH = PAIR ? 2 * C : 0;
             // eblast has four slots: these warps are never more than three chunks ahead of the rescale that reads one
             if (SCALAR) {
-                scale_rows(qk, g, ptid);
-                scale_rows(qk + TILE_BF16, g + C, ptid);
+                scale_rows(qk, g, ptid, GH);
+                scale_rows(qk + TILE_BF16, g + C, ptid, GH);
             } else {
                 chunk_prologue<true, false>(qk, qk + TILE_BF16, reinterpret_cast<const float *>(sm + OFF_G), tot, g, g + C,
                                             eblast + (n & 3) * D, nullptr, p.status, ptid, 2,
-                                            [&]() { if (ptid == 0 && n + 1 < NT) load_g(n + 1); });
+                                            [&]() { if (ptid == 0 && n + 1 < NT) load_g(n + 1); }, GH);
             }
             fence_proxy_async();
             mbar_arrive(bar(OPR + n % 3));
@@ -310,13 +339,14 @@ k_gla_fwd_tc(const __grid_constant__ CUtensorMap gm_q, const __grid_constant__ C
         const uint32_t lane_base = (uint32_t)(32 * (warp & 3)) << 16;   // this warp's TMEM lane quarter
         const int colhalf = warp >> 2;                                   // which 64 state / output columns
         const int row = 32 * (warp & 3) + lane;
-        const float lg = SCALAR ? LOG2E * p.log_gamma[h] : 0.f;
+        const float lg = SCALAR ? LOG2E * p.log_gamma[HPC * h + (PAIR ? row >> 6 : 0)] : 0.f;
+        const bool holds = !PAIR || pair_diagonal(warp & 3, colhalf);    // (a pair's threads off the diagonal blocks have no state)
 
         {   // initial state: fp32 into TMEM, bf16 copy into shared memory (row = key dimension).  A segment that is not the
             // first starts from S <- diag(gam_s) S + fin_s taken over the segments s before it (a short scan over their
             // summaries, elementwise, done here rather than in a launch of its own).
-            const float *src = state_row(p.h0, sbh, row, colhalf, p.dk, p.dv);
-            if (p.P > 1) grid_dependency_wait();
+            const float *src = PAIR ? pair_state_row(p.h0, sbh, row, colhalf) : state_row(p.h0, sbh, row, colhalf, p.dk, p.dv);
+            if (!PAIR && p.P > 1) grid_dependency_wait();
 #pragma unroll
             for (int part = 0; part < 2; ++part) {
                 float v[32];
@@ -333,6 +363,7 @@ k_gla_fwd_tc(const __grid_constant__ CUtensorMap gm_q, const __grid_constant__ C
                     }
                 }
                 tmem_st32(tmem + lane_base + COL_S + 64 * colhalf + 32 * part, v);
+                if (!holds) continue;
 #pragma unroll
                 for (int c = 0; c < 4; ++c) {
                     uint4 w;
@@ -374,8 +405,10 @@ k_gla_fwd_tc(const __grid_constant__ CUtensorMap gm_q, const __grid_constant__ C
             wait(BAR_A, m & 1);
             tc_fence_after();
             const int i0 = 16 * (warp & 3) + (lane >> 2);
-            float v[16];
-            tmem_ld_frag4(tmem + lane_base + COL_A + 32 * colhalf, v);
+            constexpr int NB = PAIR ? 8 : 4;           // blocks of eight columns a warp takes: half of A, or all of one head's
+            float v[4 * NB];
+            if constexpr (PAIR) tmem_ld_frag8(tmem + lane_base + COL_A + 64 * colhalf, v);
+            else tmem_ld_frag4(tmem + lane_base + COL_A + 32 * colhalf, v);
             tmem_wait_ld();
             tc_fence_before();
             warp_arrive(bar(ATAKEN), lane);
@@ -383,10 +416,12 @@ k_gla_fwd_tc(const __grid_constant__ CUtensorMap gm_q, const __grid_constant__ C
                 wait(BAR_O + ((m - 1) & 1), ((m - 1) >> 1) & 1);
                 tc_fence_after();
             }
+            uint8_t *tile = sm + (PAIR && colhalf ? OFF_S + PAIR_FREE0 : OFF_A);
+            const int j0 = PAIR ? 0 : 32 * colhalf;
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const int j = 32 * colhalf + 8 * i + 2 * (lane & 3);
-                uint8_t *dst = sm + OFF_A + frag_off(warp & 3, lane, 32 * colhalf, i);
+            for (int i = 0; i < NB; ++i) {
+                const int j = j0 + 8 * i + 2 * (lane & 3);
+                uint8_t *dst = tile + frag_off(warp & 3, lane, j0, i);
                 *reinterpret_cast<uint32_t *>(dst) = pack_bf16(j <= i0 ? v[4 * i] : 0.f, j + 1 <= i0 ? v[4 * i + 1] : 0.f);
                 *reinterpret_cast<uint32_t *>(dst + 1024) = pack_bf16(j <= i0 + 8 ? v[4 * i + 2] : 0.f, j + 1 <= i0 + 8 ? v[4 * i + 3] : 0.f);
             }
@@ -402,7 +437,7 @@ k_gla_fwd_tc(const __grid_constant__ CUtensorMap gm_q, const __grid_constant__ C
             wait(BAR_Z, par);
             tc_fence_after();
             if (p.simg) wait(SSAVED, par);             // the image store of S_n has read the operand copy
-            {
+            if (holds) {
                 const float e = SCALAR ? ex2f(lg * (float)min(C, p.T - (n0 + n) * C)) : eblast[(n & 3) * D + row];
 #pragma unroll
                 for (int part = 0; part < 2; ++part) {
@@ -432,7 +467,19 @@ k_gla_fwd_tc(const __grid_constant__ CUtensorMap gm_q, const __grid_constant__ C
             stage_o(n);                                // ... and this chunk's output
         }
 
-        if (p.ht && seg == p.P - 1) {   // final state, fp32 (each thread reads back what it wrote in the last rescale)
+        if (PAIR && p.ht) {
+            float *dst = pair_state_row(p.ht, sbh, row, colhalf);
+            if (holds)
+#pragma unroll
+                for (int part = 0; part < 2; ++part) {
+                    float v[32];
+                    tmem_ld32(tmem + lane_base + COL_S + 64 * colhalf + 32 * part, v);
+                    tmem_wait_ld();
+#pragma unroll
+                    for (int j = 0; j < 32; j += 4) *reinterpret_cast<float4 *>(dst + 32 * part + j) = make_float4(v[j], v[j + 1], v[j + 2], v[j + 3]);
+                }
+        }
+        if (!PAIR && p.ht && seg == p.P - 1) {   // final state, fp32 (each thread reads back what it wrote in the last rescale)
             // through shared memory (every product of the CTA has been read out, the q, k buffers are free), so that a warp writes
             // whole rows (4 x 2048 tokens x 8 heads: 46.4 -> 43.6 us a call)
             const uint32_t R = OFF_QK + row * (D * 4);
@@ -494,8 +541,31 @@ bool gla_tc_supported(const Dims &d) {
 int gla_tc_configure() {
     if (!encode_fn()) return -1;
     constexpr cudaFuncAttribute A = cudaFuncAttributeMaxDynamicSharedMemorySize;
-    return cudaFuncSetAttribute(k_gla_fwd_tc<false>, A, (int)SMEM_BYTES) == cudaSuccess &&
-                   cudaFuncSetAttribute(k_gla_fwd_tc<true>, A, (int)SMEM_BYTES) == cudaSuccess ? 0 : -1;
+    return cudaFuncSetAttribute(k_gla_fwd_tc<false, false>, A, (int)SMEM_BYTES) == cudaSuccess &&
+                   cudaFuncSetAttribute(k_gla_fwd_tc<true, false>, A, (int)SMEM_BYTES) == cudaSuccess &&
+                   cudaFuncSetAttribute(k_gla_fwd_tc<false, true>, A, (int)SMEM_BYTES) == cudaSuccess &&
+                   cudaFuncSetAttribute(k_gla_fwd_tc<true, true>, A, (int)SMEM_BYTES) == cudaSuccess ? 0 : -1;
+}
+
+// A pair's chunk takes 1.04 to 1.13 times as long as one head's (8 x 4096 tokens x 32 heads, forward and step: Softmax-GLA 381 and 1167 us one head
+// a CTA, 198 and 620 in pairs, half the CTAs; Softmax-RetNet 346 and 863, 196 and 481), so pairs gain where single heads do not all
+// run at once.  Where one long sequence of a packed batch is what a call lasts they would lose: a sequence of 4000 tokens beside 17 of 256, 32 heads,
+// step 567 us single, 585 in pairs.  Both are estimated in chunk times: the longest sequence, or what an SM gets where there are more
+// CTAs than SMs (equal sequences: whole waves of them).
+bool gla_tc_pairs(const Dims &d, const Varlen *vl) {
+    if (d.dk != 64 || d.dv != 64 || d.H % 2) return false;
+    constexpr double PAIR_CHUNK = 1.1;
+    const double sms = sm_count();
+    auto lasts = [&](long heads) {
+        if (!(vl && vl->n_seq)) return std::ceil(d.B * heads / sms) * d.NT;
+        long chunks = 0, longest = 0;
+        for (const SeqInfo &s : vl->seqs) {
+            chunks += s.NT;
+            longest = std::max<long>(longest, s.NT);
+        }
+        return std::max<double>(longest, chunks * heads / sms);
+    };
+    return PAIR_CHUNK * lasts(d.H / 2) < lasts(d.H);
 }
 
 // The backward runs the gradient sweep twice when it is cut into segments (once for the state gradients that leave
@@ -522,30 +592,32 @@ bool gla_tc_forward_can_save(const Dims &d, const Varlen *vl) {
 int gla_tc_forward(const Dims &d, const FwdArgs &a, uint8_t *simg, int *status, cudaStream_t st, Tracer &tr) {
     CUtensorMap mq, mk, mv, mg, mo;
     const bool retnet = d.variant == SLA_RETNET;
-    auto *const kernel = retnet ? k_gla_fwd_tc<true> : k_gla_fwd_tc<false>;
+    const bool pair = gla_tc_pairs(d, a.vl);
+    auto *const kernel = retnet ? (pair ? k_gla_fwd_tc<true, true> : k_gla_fwd_tc<true, false>) : pair ? k_gla_fwd_tc<false, true> : k_gla_fwd_tc<false, false>;
+    const int H = pair ? d.H / 2 : d.H, dk = pair ? 128 : d.dk, dv = pair ? 128 : d.dv;       // the heads as the tensor maps count them
     if (a.vl && a.vl->n_seq) {          // packed batch: one CTA per (sequence, head), per-sequence tensor maps
         const void *key[] = {a.q, a.k, a.v, a.log_decay, a.o};
         const CUtensorMap *vm = varlen_maps(*a.vl, 0, key, 5, st, [&](const SeqInfo &si, CUtensorMap *m) {
-            const size_t tok = (size_t)si.t0 * d.H;      // (q, k are d_k wide, v, o and their gradients d_v)
+            const size_t tok = (size_t)si.t0 * H;        // (q, k are d_k wide, v, o and their gradients d_v)
             const __nv_bfloat16 *q = (const __nv_bfloat16 *)a.q, *k = (const __nv_bfloat16 *)a.k, *v = (const __nv_bfloat16 *)a.v;
-            if (!make_tile_map(m + 0, q + tok * d.dk, 1, si.T, d.H, d.dk) || !make_tile_map(m + 1, k + tok * d.dk, 1, si.T, d.H, d.dk) ||
-                !make_tile_map(m + 2, v + tok * d.dv, 1, si.T, d.H, d.dv) || !make_tile_map(m + 4, (__nv_bfloat16 *)a.o + tok * d.dv, 1, si.T, d.H, d.dv))
+            if (!make_tile_map(m + 0, q + tok * dk, 1, si.T, H, dk) || !make_tile_map(m + 1, k + tok * dk, 1, si.T, H, dk) ||
+                !make_tile_map(m + 2, v + tok * dv, 1, si.T, H, dv) || !make_tile_map(m + 4, (__nv_bfloat16 *)a.o + tok * dv, 1, si.T, H, dv))
                 return false;
             if (retnet) { m[3] = m[0]; return true; }
-            return make_map(m + 3, a.log_decay + tok * d.dk, 1, si.T, d.H, d.dk, true, 128);
+            return make_map(m + 3, a.log_decay + tok * dk, 1, si.T, H, dk, true, 128);
         });
-        if (!vm || !make_tile_map(&mq, a.q, d.B, d.T, d.H, d.dk)) return -1;
+        if (!vm || !make_tile_map(&mq, a.q, d.B, d.T, H, dk)) return -1;
         FwdParams p{a.lq, a.lk, a.h0, nullptr, nullptr, (__nv_bfloat16 *)a.o, a.ht, simg, status, d.T, d.H, d.NT, 1, d.NT, d.scale,
                     retnet ? a.log_decay : nullptr, a.vl->d_seqs, vm, d.dk, d.dv};
-        kernel<<<a.vl->n_seq * d.H, NTHREADS, SMEM_BYTES, st>>>(mq, mq, mq, mq, mq, p);
+        kernel<<<a.vl->n_seq * H, NTHREADS, SMEM_BYTES, st>>>(mq, mq, mq, mq, mq, p);
         tr.mark("gla_fwd_tc");
         return cudaGetLastError() == cudaSuccess ? 1 : -1;
     }
-    if (!make_tile_map(&mq, a.q, d.B, d.T, d.H, d.dk) || !make_tile_map(&mk, a.k, d.B, d.T, d.H, d.dk) ||
-        !make_tile_map(&mv, a.v, d.B, d.T, d.H, d.dv) || !make_tile_map(&mo, a.o, d.B, d.T, d.H, d.dv))
+    if (!make_tile_map(&mq, a.q, d.B, d.T, H, dk) || !make_tile_map(&mk, a.k, d.B, d.T, H, dk) ||
+        !make_tile_map(&mv, a.v, d.B, d.T, H, dv) || !make_tile_map(&mo, a.o, d.B, d.T, H, dv))
         return -1;
     if (retnet) mg = mq;   // (never used: the decay is generated in the kernel)
-    else if (!make_map(&mg, a.log_decay, d.B, d.T, d.H, d.dk, true, 128)) return -1;
+    else if (!make_map(&mg, a.log_decay, d.B, d.T, H, dk, true, 128)) return -1;
     int P, L, launches = 1;
     choose_segments(d, P, L);
     float *fin = nullptr, *gam = nullptr;
@@ -567,7 +639,7 @@ int gla_tc_forward(const Dims &d, const FwdArgs &a, uint8_t *simg, int *status, 
     early.id = cudaLaunchAttributeProgrammaticStreamSerialization;
     early.val.programmaticStreamSerializationAllowed = 1;
     cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3((unsigned)(d.B * d.H * P));
+    cfg.gridDim = dim3((unsigned)(d.B * H * P));
     cfg.blockDim = dim3(NTHREADS);
     cfg.dynamicSmemBytes = SMEM_BYTES;
     cfg.stream = st;

@@ -118,6 +118,24 @@ __device__ __forceinline__ void load_state32(const float *src, float (&v)[32]) {
     }
 }
 
+// Pairs of 64-wide heads (d_k = d_v = 64, an even number of heads): the heads 2p, 2p+1 of a token lie side by side in memory, so the
+// tensors read as H/2 heads of 128, and the kernels' PAIR form runs both heads of a pair in one CTA - loads, stores and everything
+// done an element at a time as for a 128-wide head, with no padding - while products and gates are taken a head at a time.
+// The 128 x 128 state is block-diagonal: head x owns rows and columns 64 x .. 64 x + 63.  The off-diagonal blocks of the fp32
+// accumulators collect sums that nothing reads; in shared memory the two blocks' places hold other tiles (PAIR_FREE).
+constexpr uint32_t STATE_BLOCK = 64 * 128;                      // 8 KiB: one head's 64 x 64 block of a state operand
+__host__ __device__ constexpr uint32_t pair_block(int x) { return x * (STATE_HALF + STATE_BLOCK); }     // head x's block
+constexpr uint32_t PAIR_FREE0 = STATE_BLOCK, PAIR_FREE1 = STATE_HALF;                                   // the two blocks between them
+constexpr uint32_t PAIR_STATE = 2 * STATE_BLOCK;                // a pair's state image in memory: the two blocks one after the other
+// Does this warp (TMEM lane quarter `quarter`, column half `half`) hold part of a diagonal block?
+__device__ __forceinline__ bool pair_diagonal(int quarter, int half) { return (quarter >> 1) == half; }
+// Row `row` of the pair's state as the thread that owns it and column half `half` sees it in a [.., H, 64, 64] tensor; nullptr off the
+// diagonal.  sbh: (sequence, head) index of the pair's first head.
+template <typename T>
+__device__ __forceinline__ T *pair_state_row(T *t, size_t sbh, int row, int half) {
+    return (t && (row >> 6) == half) ? t + ((sbh + half) * 64 + (row & 63)) * 64 : nullptr;
+}
+
 // Where the 16 bytes (row, columns 4 c4 .. 4 c4 + 3) of a segment's fp32 summary lie, in floats: rows next to one another, because the
 // kernels that write and read it have a row of the state in each thread and a warp then moves 512 bytes at a time (in rows of 512 bytes
 // a warp touched 32 lines an access: 4 x 2048 tokens x 8 heads 52.0 us a call, 45.5 now).
@@ -177,13 +195,16 @@ constexpr uint32_t TOT_BYTES = 8 * D * 4;
 // bytes of each of eight rows at once, which without the swizzle all sit in the same banks
 __device__ __forceinline__ uint32_t e2_off(uint32_t row, uint32_t chunk) { return row * (D * 4) + ((chunk ^ ((row & 3) << 1)) << 4); }
 struct NoHook { __device__ __forceinline__ void operator()() const {} };
+// gate_half: distance between the gates of columns 0..63 and those of columns 64..127 (a pair of heads; 0: one head).
 template <bool WITH_Q, bool WITH_E, class Hook = NoHook>
 __device__ __forceinline__ void chunk_prologue(uint8_t *q_tile, uint8_t *k_tile, const float *gs, float *tot,
                                                const float *gq_s, const float *gk_s, float *eblast,
                                                uint8_t *e2_tile, int *status, int tid, int bar_id = 1,
-                                               Hook tile_read = Hook()) {
+                                               Hook tile_read = Hook(), int gate_half = 0) {
     using namespace ptx;
     const int rg = tid >> 5, cj = tid & 31;
+    gq_s += (cj >> 4) * gate_half;
+    gk_s += (cj >> 4) * gate_half;
     float4 gl[8];                               // this thread's log-decay rows: read once, kept for the second pass
     {
         float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -262,14 +283,14 @@ __device__ __forceinline__ void chunk_prologue(uint8_t *q_tile, uint8_t *k_tile,
 // which the gate warps have already multiplied into its gates (DecayFactor): f_i = scale*Gq_i 2^{b_i} or Gk_i 2^{-b_i}, so a tile
 // becomes qh or kh by scaling its rows - no log-decay tile, no scan, no exponential an element.  256 threads, a thread every
 // fourth 16-byte chunk of one row (the rows of a pair start in opposite halves of a swizzled line: no bank is asked twice).
-__device__ __forceinline__ void scale_rows(uint8_t *tile, const float *f, int tid) {
+__device__ __forceinline__ void scale_rows(uint8_t *tile, const float *f, int tid, int gate_half = 0) {
     using namespace ptx;
     const int r = tid >> 2;
-    const float g = f[r];
     uint8_t *at = tile + swz(r, (tid & 3) + 4 * (r & 1));
 #pragma unroll
     for (int hf = 0; hf < 2; ++hf, at += HALF_BF16) {
         uint8_t *other = reinterpret_cast<uint8_t *>(reinterpret_cast<uintptr_t>(at) ^ 64);      // the chunk four further (tiles are 1 KiB aligned)
+        const float g = f[hf * gate_half + r];
         uint4 v[2] = {*reinterpret_cast<const uint4 *>(at), *reinterpret_cast<const uint4 *>(other)};
 #pragma unroll
         for (int x = 0; x < 2; ++x) {
@@ -330,17 +351,18 @@ __device__ __forceinline__ void gate_fetch(const float *__restrict__ L, int cn, 
 }
 // What a gate is multiplied with on its way out: a constant, or (a constant decay per head) also 2^{lg (token + 1)}.
 struct ConstFactor {
-    float mult;
+    float mult = 0.f;
     __device__ __forceinline__ float operator()(int) const { return mult; }
 };
 struct DecayFactor {
-    float mult, lg;
+    float mult = 0.f, lg = 0.f;
     __device__ __forceinline__ float operator()(int token) const { return mult * ex2f(lg * (float)(token + 1)); }
 };
 // finish: softmax over the H/4 lanes of every token, dst[token] = mult(token) * G[token][h].  Stage by stage over all of the
 // thread's float4s, so that the shuffles and exponentials of different tokens overlap.
-template <int LPT, int NTH, class Mult>
-__device__ __forceinline__ void gate_finish(float4 (&x)[LPT * 64 / NTH], int cn, int h, Mult mult, float *dst, int t) {
+// HPC = 2: of head h + 1, too (h even: the two lie in one float4), dst2[token] = mult2(token) * G[token][h + 1].
+template <int LPT, int NTH, int HPC = 1, class Mult>
+__device__ __forceinline__ void gate_finish(float4 (&x)[LPT * 64 / NTH], int cn, int h, Mult mult, float *dst, int t, Mult mult2 = Mult(), float *dst2 = nullptr) {
     constexpr int NF = LPT * 64 / NTH;
     float m[NF], sum[NF];
 #pragma unroll
@@ -368,24 +390,28 @@ __device__ __forceinline__ void gate_finish(float4 (&x)[LPT * 64 / NTH], int cn,
             const int token = (i * NTH + t) / LPT;
             const float eh = j == 0 ? x[i].x : j == 1 ? x[i].y : j == 2 ? x[i].z : x[i].w;
             dst[token] = token < cn ? mult(token) * __fdividef(eh, sum[i]) : 0.f;
+            if (HPC == 2) dst2[token] = token < cn ? mult2(token) * __fdividef(j == 0 ? x[i].y : x[i].w, sum[i]) : 0.f;
         }
     }
 }
-template <int LPT, int NTH, class Mult>
-__device__ __forceinline__ void chunk_gate_vec(const float *__restrict__ L, int cn, int h, Mult mult, float *dst, int t) {
+template <int LPT, int NTH, int HPC, class Mult>
+__device__ __forceinline__ void chunk_gate_vec(const float *__restrict__ L, int cn, int h, Mult mult, float *dst, int t, Mult mult2, float *dst2) {
     float4 x[LPT * 64 / NTH];
     gate_fetch<LPT, NTH>(L, cn, t, x);
-    gate_finish<LPT, NTH, Mult>(x, cn, h, mult, dst, t);
+    gate_finish<LPT, NTH, HPC>(x, cn, h, mult, dst, t, mult2, dst2);
 }
 // NTH = 64 (threads t = 0..63, two whole warps) or 32 (one warp) serve one gate of one chunk.
-template <int NTH = 64, class Mult>
-__device__ __forceinline__ void chunk_gate_by(const float *L, int H, int cn, int h, Mult mult, float *dst, int t) {
-    if (H == 16) chunk_gate_vec<4, NTH>(L, cn, h, mult, dst, t);
-    else if (H == 8) chunk_gate_vec<2, NTH>(L, cn, h, mult, dst, t);
-    else if (H == 4) chunk_gate_vec<1, NTH>(L, cn, h, mult, dst, t);
-    else if (H == 32) chunk_gate_vec<8, NTH>(L, cn, h, mult, dst, t);
+template <int NTH = 64, int HPC = 1, class Mult>
+__device__ __forceinline__ void chunk_gate_by(const float *L, int H, int cn, int h, Mult mult, float *dst, int t, Mult mult2 = Mult(), float *dst2 = nullptr) {
+    if (H == 16) chunk_gate_vec<4, NTH, HPC>(L, cn, h, mult, dst, t, mult2, dst2);
+    else if (H == 8) chunk_gate_vec<2, NTH, HPC>(L, cn, h, mult, dst, t, mult2, dst2);
+    else if (H == 4) chunk_gate_vec<1, NTH, HPC>(L, cn, h, mult, dst, t, mult2, dst2);
+    else if (H == 32) chunk_gate_vec<8, NTH, HPC>(L, cn, h, mult, dst, t, mult2, dst2);
     else {
-        for (int i = t; i < C; i += NTH) dst[i] = i < cn ? mult(i) * token_gate_any(L + (size_t)i * H, H, h) : 0.f;
+        for (int i = t; i < C; i += NTH) {
+            dst[i] = i < cn ? mult(i) * token_gate_any(L + (size_t)i * H, H, h) : 0.f;
+            if (HPC == 2) dst2[i] = i < cn ? mult2(i) * token_gate_any(L + (size_t)i * H, H, h + 1) : 0.f;
+        }
     }
 }
 template <int NTH = 64>
@@ -409,7 +435,7 @@ struct BwdParams {
 };
 // maps: q, k, v, dO, dq, dk, dv
 int retnet_tc_bwd_configure();
-void retnet_tc_bwd_launch(const CUtensorMap (&maps)[7], const BwdParams &p, int ctas, cudaStream_t st);
+void retnet_tc_bwd_launch(const CUtensorMap (&maps)[7], const BwdParams &p, bool pair, int ctas, cudaStream_t st);
 
 }  // namespace tc
 }  // namespace sla

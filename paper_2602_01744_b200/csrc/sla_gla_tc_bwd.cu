@@ -47,8 +47,8 @@ constexpr uint32_t OFF_V = OFF_K + 3 * TILE_BF16;           // [2] v tiles
 constexpr uint32_t OFF_IMG = OFF_V + 2 * TILE_BF16;         // bf16 state image staged for the bulk store
 constexpr uint32_t OFF_TOT = OFF_IMG + STATE_BF16;          // prologue scratch
 constexpr uint32_t OFF_EB = OFF_TOT + TOT_BYTES;            // [2][128] 2^{b_last}
-constexpr uint32_t OFF_GATE = OFF_EB + 2 * D * 4;           // [4][64] Gk of four chunks
-constexpr uint32_t OFF_BAR = OFF_GATE + 4 * C * 4;
+constexpr uint32_t OFF_GATE = OFF_EB + 2 * D * 4;           // [4][heads][64] Gk of four chunks
+constexpr uint32_t OFF_BAR = OFF_GATE + 2 * 4 * C * 4;
 constexpr uint32_t OFF_TMEM = OFF_BAR + 32 * 8;             // TMEM base address, then the abort flag
 constexpr uint32_t SMEM_BYTES = OFF_TMEM + 16 + 1024;
 constexpr uint32_t TMEM_COLS = 128;
@@ -91,8 +91,8 @@ __device__ __forceinline__ void store_state_part(uint8_t *img, int row, int colh
 // Summary mode (simg == nullptr) serves the segmented forward of long sequences: every CTA runs one segment of a
 // sequence from a zero state and leaves only where it ended and the segment's total decay; a scan over the segments
 // then gives every segment its true starting state.
-// SCALAR: Softmax-RetNet (its constant decay comes in with the gates; the prologue only scales rows).
-template <bool SCALAR>
+// SCALAR: Softmax-RetNet (its constant decay comes in with the gates; the prologue only scales rows).  PAIR: two 64-wide heads a CTA.
+template <bool SCALAR, bool PAIR>
 __global__ void __launch_bounds__(st1::NTHREADS, 1)
 k_gla_states_tc(const __grid_constant__ CUtensorMap gm_k, const __grid_constant__ CUtensorMap gm_v,
                 const __grid_constant__ CUtensorMap gm_g, StatesParams p) {
@@ -102,9 +102,12 @@ k_gla_states_tc(const __grid_constant__ CUtensorMap gm_k, const __grid_constant_
     const uint32_t base = (raw + 1023u) & ~1023u;
     uint8_t *sm = smem_raw + (base - raw);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int bh = blockIdx.x / p.PS, seg = blockIdx.x % p.PS, h = bh % p.H;
+    constexpr int HPC = PAIR ? 2 : 1;                       // heads per CTA
+    const int hg = p.H / HPC;
+    const int cta = blockIdx.x / p.PS, seg = blockIdx.x % p.PS, h = cta % hg;
+    int b = cta / hg;
+    const int bh = b * p.H + h * HPC;
     const size_t sum_i = (size_t)bh * p.P + seg;            // summary slot of this segment
-    int b = bh / p.H;
     size_t tokb = (size_t)b * p.T, slot = (size_t)bh * (p.NT + 1);
     size_t sbh = (size_t)bh;                                // (sequence, head) index into h0 / ht / dht / dh0
     const CUtensorMap *vm = nullptr;
@@ -113,8 +116,8 @@ k_gla_states_tc(const __grid_constant__ CUtensorMap gm_k, const __grid_constant_
         vm = p.vmaps + (size_t)b * Varlen::MAPS_PER_SEQ;
         p.T = si.T; p.NT = si.NT; p.L = si.NT;
         tokb = (size_t)si.t0;
-        slot = (size_t)si.slot0 * p.H + (size_t)h * (si.NT + 1);
-        sbh = (size_t)si.id * p.H + h;                      // (the table is ordered longest first, the state tensors as the caller gave them)
+        slot = (size_t)si.slot0 * p.H + (size_t)h * HPC * (si.NT + 1);
+        sbh = (size_t)si.id * p.H + h * HPC;                      // (the table is ordered longest first, the state tensors as the caller gave them)
         b = 0;
     }
     const CUtensorMap &tm_k = vm ? vm[0] : gm_k, &tm_v = vm ? vm[1] : gm_v, &tm_g = vm ? vm[2] : gm_g;
@@ -215,7 +218,12 @@ k_gla_states_tc(const __grid_constant__ CUtensorMap gm_k, const __grid_constant_
                 if (!images) continue;
                 wait_relaxed(STAGED, n & 1);           // image of S_{n+1} is staged
                 if (failed) break;
-                bulk_store(img0 + (size_t)(n + 1) * STATE_BF16, base + OFF_IMG, STATE_BF16);
+                if (PAIR) {
+                    bulk_store(img0 + (size_t)(n + 1) * PAIR_STATE, base + OFF_IMG + pair_block(0), STATE_BLOCK);
+                    bulk_store(img0 + (size_t)(n + 1) * PAIR_STATE + STATE_BLOCK, base + OFF_IMG + pair_block(1), STATE_BLOCK);
+                } else {
+                    bulk_store(img0 + (size_t)(n + 1) * STATE_BF16, base + OFF_IMG, STATE_BF16);
+                }
                 bulk_commit();
                 bulk_wait_read0();
                 mbar_arrive(bar(STFREE));
@@ -229,14 +237,15 @@ k_gla_states_tc(const __grid_constant__ CUtensorMap gm_k, const __grid_constant_
     } else if (warp >= 9) {
         // ---------------- gates (Gk only), up to four chunks ahead ----------------
         const int t = tid - (NCOMPUTE + 32);
-        const float lg = SCALAR ? -LOG2E * p.log_gamma[h] : 0.f;
+        const float lg = SCALAR ? -LOG2E * p.log_gamma[HPC * h] : 0.f, lg2 = SCALAR && PAIR ? -LOG2E * p.log_gamma[2 * h + 1] : 0.f;
         for (int n = 0; n < NT; ++n) {
             if (n >= 4) wait_relaxed(GFREE + (n & 3), ((n >> 2) - 1) & 1);
             if (failed) break;
             const int cn = min(C, p.T - (n0 + n) * C);
             const float *lc = p.lk + (tokb + (size_t)(n0 + n) * C) * p.H;
-            if (SCALAR) chunk_gate_by(lc, p.H, cn, h, DecayFactor{1.f, lg}, gate_s + (n & 3) * C, t);
-            else chunk_gate(lc, p.H, cn, h, 1.f, gate_s + (n & 3) * C, t);
+            float *dst = gate_s + (n & 3) * HPC * C, *dst2 = dst + C;
+            if (SCALAR) chunk_gate_by<64, HPC>(lc, p.H, cn, HPC * h, DecayFactor{1.f, lg}, dst, t, DecayFactor{1.f, lg2}, dst2);
+            else chunk_gate_by<64, HPC>(lc, p.H, cn, HPC * h, ConstFactor{1.f}, dst, t, ConstFactor{1.f}, dst2);
             __syncwarp();
             if (lane == 0) mbar_arrive(bar(GREADY + (n & 3)));
         }
@@ -245,30 +254,34 @@ k_gla_states_tc(const __grid_constant__ CUtensorMap gm_k, const __grid_constant_
         const uint32_t lane_base = (uint32_t)(32 * (warp & 3)) << 16;
         const int colhalf = warp >> 2;
         const int row = 32 * (warp & 3) + lane;
-        {   // S_0: fp32 into TMEM, bf16 image into slot 0
-            const float *src = images ? state_row(p.h0, sbh, row, colhalf, p.dk, p.dv) : nullptr;
+        const bool holds = !PAIR || pair_diagonal(warp & 3, colhalf);
+        {   // S_0: fp32 into TMEM, bf16 image into slot 0 (a pair's image: its two blocks one after the other)
+            const float *src = !images ? nullptr : PAIR ? pair_state_row(p.h0, sbh, row, colhalf) : state_row(p.h0, sbh, row, colhalf, p.dk, p.dv);
 #pragma unroll
             for (int part = 0; part < 2; ++part) {
                 float v[32];
                 load_state32(src ? src + 32 * part : nullptr, v);
                 tmem_st32(tmem + lane_base + 64 * colhalf + 32 * part, v);
-                if (images) store_state_part(img0, row, colhalf, part, v);
+                if (PAIR && holds) store_state_part(img0 + colhalf * STATE_BLOCK, row & 63, 0, part, v);
+                else if (!PAIR && images) store_state_part(img0, row, colhalf, part, v);
             }
             tmem_wait_st();
         }
         tc_fence_before();
         mbar_arrive(bar(SREADY));
 
-        const float lg = SCALAR ? LOG2E * p.log_gamma[h] : 0.f;
-        if (SCALAR && tid == 0) check_scalar_range(p.log_gamma[h], p.T, p.status);
+        const float lg = SCALAR ? LOG2E * p.log_gamma[HPC * h + (PAIR ? row >> 6 : 0)] : 0.f;
+        if (SCALAR && tid < HPC) check_scalar_range(p.log_gamma[HPC * h + tid], p.T, p.status);
+        constexpr int GH = PAIR ? C : 0;
         auto prologue = [&](int n) {
             wait(GREADY + (n & 3), (n >> 2) & 1);
             if (!SCALAR) wait(FULL_G + (n & 1), (n >> 1) & 1);
             wait(FULL_K + n % 3, (n / 3) & 1);
             uint8_t *kt = sm + OFF_K + (n % 3) * TILE_BF16;
-            if (SCALAR) scale_rows(kt, gate_s + (n & 3) * C, tid);
-            else chunk_prologue<false, false>(nullptr, kt, reinterpret_cast<const float *>(sm + OFF_G + (n & 1) * TILE_G), tot, nullptr,
-                                              gate_s + (n & 3) * C, eblast + (n & 1) * D, nullptr, p.status, tid);
+            const float *gk = gate_s + (n & 3) * HPC * C;
+            if (SCALAR) scale_rows(kt, gk, tid, GH);
+            else chunk_prologue<false, false>(nullptr, kt, reinterpret_cast<const float *>(sm + OFF_G + (n & 1) * TILE_G), tot, gk,
+                                              gk, eblast + (n & 1) * D, nullptr, p.status, tid, 1, NoHook(), GH);
             fence_proxy_async();
             mbar_arrive(bar(OPR + n % 3));
             mbar_arrive(bar(GFREE + (n & 3)));
@@ -279,7 +292,7 @@ k_gla_states_tc(const __grid_constant__ CUtensorMap gm_k, const __grid_constant_
             if (n + 1 < NT) prologue(n + 1);         // overlaps the MMA of chunk n
             wait(BAR_Z, n & 1);
             tc_fence_after();
-            {   // S_{n+1} = diag(2^{b_last}) (S_n + kh^T V): fp32 back into TMEM, bf16 image staged for slot n+1
+            if (holds) {   // S_{n+1} = diag(2^{b_last}) (S_n + kh^T V): fp32 back into TMEM, bf16 image staged for slot n+1
                 const float e = SCALAR ? ex2f(lg * (float)min(C, p.T - (n0 + n) * C)) : eblast[(n & 1) * D + row];
                 gam *= e;
                 float v0[32], v1[32];
@@ -332,13 +345,13 @@ constexpr uint32_t OFF_A = OFF_DZ + STATE_BF16;         // masked A, [64 rows][1
 constexpr uint32_t OFF_DA = OFF_A + HALF_BF16;          // masked dA; afterwards A|dA hold the dv tile staged for the store
 constexpr uint32_t OFF_TOT = OFF_DA + HALF_BF16;        // prologue scratch
 constexpr uint32_t OFF_EB = OFF_TOT + TOT_BYTES;        // [128] 2^{b_last}
-constexpr uint32_t OFF_GATE = OFF_EB + D * 4;           // [4][2][64]: scale*Gq, Gk of four chunks
-constexpr uint32_t OFF_R = OFF_GATE + 4 * 2 * C * 4;    // [2 buffers][2 column halves][128] rowsum(dS*S) partials
+constexpr uint32_t OFF_GATE = OFF_EB + D * 4;           // [4][heads][2][64]: scale*Gq, Gk of four chunks
+constexpr uint32_t OFF_R = OFF_GATE + 4 * 2 * 2 * C * 4;    // [2 buffers][2 column halves][128] rowsum(dS*S) partials
 constexpr uint32_t OFF_RED = OFF_R + 4 * D * 4;            // [2][2 column halves][64] gate partial sums
 constexpr uint32_t OFF_BAR = OFF_RED + 2 * 2 * C * 4;
 constexpr uint32_t OFF_TMEM = OFF_BAR + 32 * 8;         // TMEM base address, then the abort flag
 constexpr uint32_t SMEM_BYTES = OFF_TMEM + 16 + 1024;
-constexpr uint32_t COL_DS = 0, COL_A = 128, COL_DA = 192, COL_DV = 128 /* once A and dA are read */, COL_DQ = 256, COL_DK = 384, TMEM_COLS = 512;
+constexpr uint32_t TMEM_COLS = 512;
 constexpr int NTHREADS = NCOMPUTE + 32 + NGATE + 32;    // warps 0..7 compute, 8 MMA issue, 9..12 gates, 13 TMA
 enum Bar { FULL_G = 0, FULL_QK, FULL_V, FULL_DO, FULL_S, OPR, GREADY /*[4]*/, GFREE = GREADY + 4 /*[4]*/, ZREADY = GFREE + 4,
            AREADY, OUT1, OUT2, SNFREE, INIT_DONE, DVREAD, DGFREE, BAR_A, BAR_M1, BAR_M2, DOFREE, INIT_FULL, DRAIN, BAR_DS, NBAR };
@@ -352,6 +365,9 @@ static_assert(NBAR <= 32, "barrier slots");
 // masked tiles after the mask.  kh dZ waits for the mask too: dV takes over the columns of A and dA, which AREADY says have been
 // read (and DVREAD that the next chunk's dA may come there); it is issued before the masked products, after whose commit dk is
 // written over kh.  All four gradient tensors leave through staged TMA stores (rows past T are clipped by the tensor map).
+// PAIR (two 64-wide heads a CTA): A, dA take 64 columns a head, dkh takes over dA's as dV does A's, so dkh's first product waits for the mask,
+// too; the second head's masked tiles lie in the unused blocks of the state image's buffer.
+template <bool PAIR>
 __global__ void __launch_bounds__(st2::NTHREADS, 1)
 k_gla_bwd_tc(const __grid_constant__ CUtensorMap gm_q, const __grid_constant__ CUtensorMap gm_k,
              const __grid_constant__ CUtensorMap gm_v, const __grid_constant__ CUtensorMap gm_do,
@@ -364,8 +380,12 @@ k_gla_bwd_tc(const __grid_constant__ CUtensorMap gm_q, const __grid_constant__ C
     const uint32_t base = (raw + 1023u) & ~1023u;
     uint8_t *sm = smem_raw + (base - raw);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int bh = blockIdx.x, h = bh % p.H;
-    int b = bh / p.H;
+    constexpr int HPC = PAIR ? 2 : 1;                       // heads per CTA
+    constexpr uint32_t COL_DS = 0, COL_A = 128, COL_DA = PAIR ? 256 : 192, COL_DV = 128 /* once A and dA are read */, COL_DQ = PAIR ? 384 : 256,
+                       COL_DK = PAIR ? 256 /* once dA is read */ : 384;
+    const int hg = p.H / HPC, h = blockIdx.x % hg;          // h: head, or pair of heads, as the tensor maps count them
+    int b = blockIdx.x / hg;
+    const int bh = b * p.H + h * HPC;
     size_t tokb = (size_t)b * p.T, slot = (size_t)bh * (p.NT + 1);
     size_t sbh = (size_t)bh;                                // (sequence, head) index into h0 / ht / dht / dh0
     const CUtensorMap *vm = nullptr;
@@ -374,8 +394,8 @@ k_gla_bwd_tc(const __grid_constant__ CUtensorMap gm_q, const __grid_constant__ C
         vm = p.vmaps + (size_t)b * Varlen::MAPS_PER_SEQ;
         p.T = si.T; p.NT = si.NT;
         tokb = (size_t)si.t0;
-        slot = (size_t)si.slot0 * p.H + (size_t)h * (si.NT + 1);
-        sbh = (size_t)si.id * p.H + h;                      // (the table is ordered longest first, the state tensors as the caller gave them)
+        slot = (size_t)si.slot0 * p.H + (size_t)h * HPC * (si.NT + 1);
+        sbh = (size_t)si.id * p.H + h * HPC;                      // (the table is ordered longest first, the state tensors as the caller gave them)
         b = 0;
     }
     const CUtensorMap &tm_q = vm ? vm[0] : gm_q, &tm_k = vm ? vm[1] : gm_k, &tm_v = vm ? vm[2] : gm_v,
@@ -434,6 +454,7 @@ k_gla_bwd_tc(const __grid_constant__ CUtensorMap gm_q, const __grid_constant__ C
             constexpr uint32_t ID_A = idesc_bf16(64, 64, 0, 0);
             constexpr uint32_t ID_KK = idesc_bf16(64, 128, 0, 0), ID_KM = idesc_bf16(64, 128, 0, 1),
                                ID_MM = idesc_bf16(64, 128, 1, 1), ID_S = idesc_bf16(128, 128, 1, 1);
+            constexpr uint32_t ID_KM64 = idesc_bf16(64, 64, 0, 1), ID_MM64 = idesc_bf16(64, 64, 1, 1);
             const uint64_t kS = desc_kmajor(base + OFF_S), kDZ = desc_kmajor(base + OFF_DZ),
                            mDZ = desc_mnmajor(base + OFF_DZ, STATE_HALF), mA = desc_mnmajor(base + OFF_A, HALF_BF16),
                            kDA = desc_kmajor(base + OFF_DA), mDA = desc_mnmajor(base + OFF_DA, HALF_BF16);
@@ -447,21 +468,27 @@ k_gla_bwd_tc(const __grid_constant__ CUtensorMap gm_q, const __grid_constant__ C
                 // dA = dO V^T and S_n dO^T need no prologue: they are issued while the compute warps still scale q and k
                 wait(FULL_V, par);
                 wait(FULL_DO, par);
-                if (k > 0) wait(DVREAD, (k - 1) & 1);  // dV of the previous chunk, in the columns of A and dA, has been read out
+                if (k > 0) wait(DVREAD, (k - 1) & 1);  // dV of the previous chunk, in the columns of A and dA, has been read out (a pair's dkh before)
                 if (failed) break;
                 tc_fence_after();
                 if (leader)
 #pragma unroll
-                for (int kk = 0; kk < 8; ++kk)         // dA = dO V^T
-                    tc_mma_bf16(tmem + COL_DA, kDO + kstep_kmajor(kk, HALF_BF16), kV + kstep_kmajor(kk, HALF_BF16), ID_A, kk > 0);
+                for (int kk = 0; kk < 8; ++kk)         // dA = dO V^T (a pair: head kk / 4)
+                    tc_mma_bf16(tmem + COL_DA + (PAIR ? 64 * (kk >> 2) : 0), kDO + kstep_kmajor(kk, HALF_BF16), kV + kstep_kmajor(kk, HALF_BF16), ID_A,
+                                PAIR ? (kk & 3) > 0 : kk > 0);
                 bool sdo_done = false;
                 auto issue_sdo = [&]() {               // dqh = dO S_n^T ...
                     if (k > 0) wait(OUT1, (k - 1) & 1);    // dqh, dkh of the previous chunk have been read out (long ago)
                     tc_fence_after();
                     if (leader)
 #pragma unroll
-                    for (int kk = 0; kk < 8; ++kk)
-                        tc_mma_bf16(tmem + COL_DQ, kDO + kstep_kmajor(kk, HALF_BF16), kS + kstep_kmajor(kk, STATE_HALF), ID_KK, kk > 0);
+                    for (int kk = 0; kk < 8; ++kk) {
+                        if (PAIR)
+                            tc_mma_bf16(tmem + COL_DQ + 64 * (kk >> 2), kDO + kstep_kmajor(kk, HALF_BF16),
+                                        desc_kmajor(base + OFF_S + pair_block(kk >> 2)) + kstep_kmajor(kk & 3, 0), ID_A, (kk & 3) > 0);
+                        else
+                            tc_mma_bf16(tmem + COL_DQ, kDO + kstep_kmajor(kk, HALF_BF16), kS + kstep_kmajor(kk, STATE_HALF), ID_KK, kk > 0);
+                    }
                     sdo_done = true;
                 };
                 {   // whichever comes first: S_n landed, or the prologue done
@@ -477,7 +504,8 @@ k_gla_bwd_tc(const __grid_constant__ CUtensorMap gm_q, const __grid_constant__ C
                 if (leader)
 #pragma unroll
                 for (int kk = 0; kk < 8; ++kk)         // A = qh kh^T
-                    tc_mma_bf16(tmem + COL_A, kQ + kstep_kmajor(kk, HALF_BF16), kK + kstep_kmajor(kk, HALF_BF16), ID_A, kk > 0);
+                    tc_mma_bf16(tmem + COL_A + (PAIR ? 64 * (kk >> 2) : 0), kQ + kstep_kmajor(kk, HALF_BF16), kK + kstep_kmajor(kk, HALF_BF16), ID_A,
+                                PAIR ? (kk & 3) > 0 : kk > 0);
                 if (leader) tc_commit(bar(BAR_A));
                 if (!sdo_done) {
                     wait(FULL_S, par);
@@ -491,7 +519,7 @@ k_gla_bwd_tc(const __grid_constant__ CUtensorMap gm_q, const __grid_constant__ C
                 if (leader)
 #pragma unroll
                 for (int kk = 0; kk < 8; ++kk) {       // two independent accumulation chains, interleaved
-                    tc_mma_bf16(tmem + COL_DK, kV + kstep_kmajor(kk, HALF_BF16), kDZ + kstep_kmajor(kk, STATE_HALF), ID_KK, kk > 0);   // dkh = V dZ^T ...
+                    if (!PAIR) tc_mma_bf16(tmem + COL_DK, kV + kstep_kmajor(kk, HALF_BF16), kDZ + kstep_kmajor(kk, STATE_HALF), ID_KK, kk > 0);   // dkh = V dZ^T ...
                     if (kk < 4) tc_mma_bf16(tmem + COL_DS, mQ + kstep_mnmajor(kk), mDO + kstep_mnmajor(kk), ID_S, 1);                // dS_n = dZ + qh^T dO
                 }
                 if (leader) tc_commit(bar(BAR_DS));                // dS_n is complete (and S_n dO^T has read S_n)
@@ -500,19 +528,43 @@ k_gla_bwd_tc(const __grid_constant__ CUtensorMap gm_q, const __grid_constant__ C
                 tc_fence_after();
                 if (leader)
 #pragma unroll
-                for (int kk = 0; kk < 8; ++kk)         // dV = kh dZ ... (A and dA have been read; before M1, after which dk goes over kh)
-                    tc_mma_bf16(tmem + COL_DV, kK + kstep_kmajor(kk, HALF_BF16), mDZ + kstep_mnmajor(kk), ID_KM, kk > 0);
+                for (int kk = 0; kk < 8; ++kk) {       // dV = kh dZ ... (A and dA have been read; before M1, after which dk goes over kh)
+                    if (PAIR) {                        // (head kk / 4; and dkh = V dZ^T)
+                        const uint32_t dz = base + OFF_DZ + pair_block(kk >> 2);
+                        tc_mma_bf16(tmem + COL_DV + 64 * (kk >> 2), kK + kstep_kmajor(kk, HALF_BF16), desc_mnmajor(dz, STATE_HALF) + kstep_mnmajor(kk & 3), ID_KM64, (kk & 3) > 0);
+                        tc_mma_bf16(tmem + COL_DK + 64 * (kk >> 2), kV + kstep_kmajor(kk, HALF_BF16), desc_kmajor(dz) + kstep_kmajor(kk & 3, 0), ID_A, (kk & 3) > 0);
+                    } else {
+                        tc_mma_bf16(tmem + COL_DV, kK + kstep_kmajor(kk, HALF_BF16), mDZ + kstep_mnmajor(kk), ID_KM, kk > 0);
+                    }
+                }
+                // ... + dA kh  and  ... + dA^T qh, interleaved; a pair: head x's tiles and its half of kh, qh
+                auto head = [&](int x, uint32_t sDA, int kk) {
+                    tc_mma_bf16(tmem + COL_DQ + 64 * x, desc_kmajor(sDA) + kstep_kmajor(kk, 0), desc_mnmajor(sK + x * HALF_BF16, HALF_BF16) + kstep_mnmajor(kk), ID_KM64, 1);
+                    tc_mma_bf16(tmem + COL_DK + 64 * x, desc_mnmajor(sDA, HALF_BF16) + kstep_mnmajor(kk), desc_mnmajor(sQ + x * HALF_BF16, HALF_BF16) + kstep_mnmajor(kk), ID_MM64, 1);
+                };
                 if (leader)
 #pragma unroll
-                for (int kk = 0; kk < 4; ++kk) {       // ... + dA kh  and  ... + dA^T qh, interleaved
-                    tc_mma_bf16(tmem + COL_DQ, kDA + kstep_kmajor(kk, 0), mK + kstep_mnmajor(kk), ID_KM, 1);
-                    tc_mma_bf16(tmem + COL_DK, mDA + kstep_mnmajor(kk), mQ + kstep_mnmajor(kk), ID_MM, 1);
+                for (int kk = 0; kk < 4; ++kk) {
+                    if (PAIR) {
+                        head(0, base + OFF_DA, kk);
+                        head(1, base + OFF_S + PAIR_FREE1, kk);
+                    } else {
+                        tc_mma_bf16(tmem + COL_DQ, kDA + kstep_kmajor(kk, 0), mK + kstep_mnmajor(kk), ID_KM, 1);
+                        tc_mma_bf16(tmem + COL_DK, mDA + kstep_mnmajor(kk), mQ + kstep_mnmajor(kk), ID_MM, 1);
+                    }
                 }
                 if (leader) tc_commit(bar(BAR_M1));
                 if (leader)
 #pragma unroll
-                for (int kk = 0; kk < 4; ++kk)         // ... + A^T dO
-                    tc_mma_bf16(tmem + COL_DV, mA + kstep_mnmajor(kk), mDO + kstep_mnmajor(kk), ID_MM, 1);
+                for (int kk = 0; kk < 4; ++kk) {       // ... + A^T dO
+                    if (PAIR) {
+                        tc_mma_bf16(tmem + COL_DV, mA + kstep_mnmajor(kk), mDO + kstep_mnmajor(kk), ID_MM64, 1);
+                        tc_mma_bf16(tmem + COL_DV + 64, desc_mnmajor(base + OFF_S + PAIR_FREE0, HALF_BF16) + kstep_mnmajor(kk),
+                                    desc_mnmajor(sDO + HALF_BF16, HALF_BF16) + kstep_mnmajor(kk), ID_MM64, 1);
+                    } else {
+                        tc_mma_bf16(tmem + COL_DV, mA + kstep_mnmajor(kk), mDO + kstep_mnmajor(kk), ID_MM, 1);
+                    }
+                }
                 if (leader) tc_commit(bar(BAR_M2));
                 if (leader) tc_commit(bar(DOFREE));                // (same event, for the TMA lane)
             }
@@ -540,14 +592,18 @@ k_gla_bwd_tc(const __grid_constant__ CUtensorMap gm_q, const __grid_constant__ C
                 mbar_expect_tx(bar(FULL_DO), TILE_BF16);
                 tma_load_5d(dst + TILE_BF16, &tm_do, 0, n * C, 0, h, b, bar(FULL_DO));
             };
-            auto load_s = [&](int n) {
-                mbar_expect_tx(bar(FULL_S), STATE_BF16);
-                bulk_load(base + OFF_S, img0 + (size_t)n * STATE_BF16, STATE_BF16, bar(FULL_S));
+            constexpr uint32_t IMAGE = PAIR ? PAIR_STATE : STATE_BF16;
+            auto load_image = [&](int n, uint32_t full) {
+                mbar_expect_tx(full, IMAGE);
+                if (PAIR) {
+                    bulk_load(base + OFF_S + pair_block(0), img0 + (size_t)n * IMAGE, STATE_BLOCK, full);
+                    bulk_load(base + OFF_S + pair_block(1), img0 + (size_t)n * IMAGE + STATE_BLOCK, STATE_BLOCK, full);
+                } else {
+                    bulk_load(base + OFF_S, img0 + (size_t)n * IMAGE, IMAGE, full);
+                }
             };
-            if (p.dht) {                               // S_NT, for rowsum(dht * S_NT)
-                mbar_expect_tx(bar(INIT_FULL), STATE_BF16);
-                bulk_load(base + OFF_S, img0 + (size_t)NT * STATE_BF16, STATE_BF16, bar(INIT_FULL));
-            }
+            auto load_s = [&](int n) { load_image(n, bar(FULL_S)); };
+            if (p.dht) load_image(NT, bar(INIT_FULL));  // S_NT, for rowsum(dht * S_NT)
             load_g(NT - 1);
             load_qk(NT - 1, 0);
             load_vdo(NT - 1, 0);
@@ -563,7 +619,7 @@ k_gla_bwd_tc(const __grid_constant__ CUtensorMap gm_q, const __grid_constant__ C
                     tma_prefetch_l2_5d(&tm_k, 0, (n - 1) * C, 0, h, b);
                     tma_prefetch_l2_5d(&tm_v, 0, (n - 1) * C, 0, h, b);
                     tma_prefetch_l2_5d(&tm_do, 0, (n - 1) * C, 0, h, b);
-                    bulk_prefetch_l2(img0 + (size_t)(n - 1) * STATE_BF16, STATE_BF16);
+                    bulk_prefetch_l2(img0 + (size_t)(n - 1) * IMAGE, IMAGE);
                     wait(OPR, par);                    // prologue done: the log-decay buffer is free
                     if (failed) break;
                     load_g(n - 1);
@@ -607,7 +663,8 @@ k_gla_bwd_tc(const __grid_constant__ CUtensorMap gm_q, const __grid_constant__ C
             if (k >= 4) wait_relaxed(GFREE + (k & 3), ((k >> 2) - 1) & 1);
             if (failed) break;
             const int cn = min(C, p.T - n * C);
-            chunk_gate(l + (tokb + (size_t)n * C) * p.H, p.H, cn, h, mult, gate_s + (k & 3) * 2 * C + (g < C ? 0 : C), t);
+            float *dst = gate_s + (k & 3) * HPC * 2 * C + (g < C ? 0 : C);
+            chunk_gate_by<64, HPC>(l + (tokb + (size_t)n * C) * p.H, p.H, cn, HPC * h, ConstFactor{mult}, dst, t, ConstFactor{mult}, dst + 2 * C);
             __syncwarp();
             if (lane == 0) mbar_arrive(bar(GREADY + (k & 3)));
         }
@@ -617,6 +674,8 @@ k_gla_bwd_tc(const __grid_constant__ CUtensorMap gm_q, const __grid_constant__ C
         const int wh = warp >> 2;                       // column half, of the state and of the gradient tiles
         const int row = 32 * (warp & 3) + lane;         // state row of this thread (its TMEM lane)
         const int qr = warp & 3, tr = 16 * qr + (lane >> 2);       // gradient tiles: tokens tr, tr + 8
+
+        const bool holds = !PAIR || pair_diagonal(warp & 3, wh);     // (a pair's threads off the diagonal blocks have no state)
 
         // rowsum(dS * S) over this thread's 64 columns, with dS in registers part by part
         auto rowdot_part = [&](const float (&v)[32], int part) {
@@ -638,13 +697,13 @@ k_gla_bwd_tc(const __grid_constant__ CUtensorMap gm_q, const __grid_constant__ C
         {   // dS_NT = dht (or zero) into TMEM; R_{NT-1} = rowsum(dht * S_NT)
             float rpart = 0.f;
             if (p.dht) wait(INIT_FULL, 0);
-            const float *src = state_row(p.dht, sbh, row, wh, p.dk, p.dv);
+            const float *src = PAIR ? pair_state_row(p.dht, sbh, row, wh) : state_row(p.dht, sbh, row, wh, p.dk, p.dv);
 #pragma unroll
             for (int part = 0; part < 2; ++part) {
                 float v[32];
                 load_state32(src ? src + 32 * part : nullptr, v);
                 tmem_st32(tmem + lane_base + COL_DS + 64 * wh + 32 * part, v);
-                if (p.dht) rpart += rowdot_part(v, part);
+                if (p.dht && holds) rpart += rowdot_part(v, part);
             }
             tmem_wait_st();
             Rs[((NT - 1) & 1) * 2 * D + wh * D + row] = rpart;
@@ -660,9 +719,9 @@ k_gla_bwd_tc(const __grid_constant__ CUtensorMap gm_q, const __grid_constant__ C
             wait(FULL_G, par);
             wait(FULL_QK, par);
             {
-                const float *g = gate_s + (k & 3) * 2 * C;
+                const float *g = gate_s + (k & 3) * HPC * 2 * C;
                 chunk_prologue<true, true>(qk, qk + TILE_BF16, reinterpret_cast<const float *>(sm + OFF_G), tot, g, g + C,
-                                           eblast, sm + OFF_E2, p.status, tid);
+                                           eblast, sm + OFF_E2, p.status, tid, 1, NoHook(), PAIR ? 2 * C : 0);
             }
             fence_proxy_async();
             warp_arrive(bar(OPR), lane);
@@ -670,7 +729,7 @@ k_gla_bwd_tc(const __grid_constant__ CUtensorMap gm_q, const __grid_constant__ C
 
             // ---- dZ = diag(2^{b_last}) dS_{n+1}: fp32 back into TMEM (dS_n accumulates on it), bf16 operand copy ----
             if (k > 0) wait(DGFREE, (k - 1) & 1);       // the staged tiles of the previous chunk have left dZ and A|dA
-            {
+            if (holds) {
                 float bl = 0.f;                         // b_last of key dimension `row` from the prologue's 8-row sums
 #pragma unroll
                 for (int g8 = 0; g8 < 8; ++g8) bl += tot[g8 * D + row];
@@ -696,9 +755,11 @@ k_gla_bwd_tc(const __grid_constant__ CUtensorMap gm_q, const __grid_constant__ C
             wait(BAR_A, par);
             tc_fence_after();
             {
-                uint8_t *dst = sm + (wh ? OFF_DA : OFF_A);
+#pragma unroll
+              for (int x = 0; x < HPC; ++x) {
+                uint8_t *dst = sm + (x == 0 ? (wh ? OFF_DA : OFF_A) : OFF_S + (wh ? PAIR_FREE1 : PAIR_FREE0));
                 float v[32];
-                tmem_ld_frag8(tmem + lane_base + (wh ? COL_DA : COL_A), v);
+                tmem_ld_frag8(tmem + lane_base + (wh ? COL_DA : COL_A) + 64 * x, v);
                 tmem_wait_ld();
 #pragma unroll
                 for (int i = 0; i < 8; ++i) {
@@ -707,6 +768,7 @@ k_gla_bwd_tc(const __grid_constant__ CUtensorMap gm_q, const __grid_constant__ C
                     *reinterpret_cast<uint32_t *>(dst + off) = pack_bf16(j <= tr ? v[4 * i] : 0.f, j + 1 <= tr ? v[4 * i + 1] : 0.f);
                     *reinterpret_cast<uint32_t *>(dst + off + 1024) = pack_bf16(j <= tr + 8 ? v[4 * i + 2] : 0.f, j + 1 <= tr + 8 ? v[4 * i + 3] : 0.f);
                 }
+              }
             }
             fence_proxy_async();
             tc_fence_before();
@@ -715,12 +777,14 @@ k_gla_bwd_tc(const __grid_constant__ CUtensorMap gm_q, const __grid_constant__ C
             // ---- R_{n-1} = rowsum(dS_n * S_n), while the tensor core works on the products with the masked tiles ----
             wait(BAR_DS, par);
             tc_fence_after();
-            {
+            if (holds) {
                 float v0[32], v1[32];
                 tmem_ld32(tmem + lane_base + COL_DS + 64 * wh, v0);
                 tmem_ld32(tmem + lane_base + COL_DS + 64 * wh + 32, v1);
                 tmem_wait_ld();
                 Rs[((n & 1) ^ 1) * 2 * D + wh * D + row] = rowdot_part(v0, 0) + rowdot_part(v1, 1);
+            } else {
+                Rs[((n & 1) ^ 1) * 2 * D + wh * D + row] = 0.f;
             }
             warp_arrive(bar(SNFREE), lane);                   // S_n is no longer needed: the next image may land
 
@@ -820,7 +884,14 @@ k_gla_bwd_tc(const __grid_constant__ CUtensorMap gm_q, const __grid_constant__ C
                     *reinterpret_cast<float4 *>(dgt + (8 * warp + ii) * D + 4 * lane) =
                         make_float4(sfx[ii].x + offs.x, sfx[ii].y + offs.y, sfx[ii].z + offs.z, sfx[ii].w + offs.w);
             }
-            if (tid < C) {   // Gq*dGq and Gk*dGk of token tid: sum over the two column halves
+            if (PAIR && tid < 2 * C) {   // Gq*dGq and Gk*dGk of token tid % 64: a head's sums are one column half's
+                const int x = tid / C, i = tid % C;
+                if (i < min(C, p.T - t0)) {
+                    p.pq[(tokb + t0 + i) * p.H + 2 * h + x] = red[x * C + i];
+                    p.pk[(tokb + t0 + i) * p.H + 2 * h + x] = red[(2 + x) * C + i];
+                }
+            }
+            if (!PAIR && tid < C) {   // Gq*dGq and Gk*dGk of token tid: sum over the two column halves
                 const int cn = min(C, p.T - t0);
                 if (tid < cn) {
                     const float sq = red[tid] + red[C + tid], sk = red[2 * C + tid] + red[3 * C + tid];
@@ -834,7 +905,7 @@ k_gla_bwd_tc(const __grid_constant__ CUtensorMap gm_q, const __grid_constant__ C
         }
 
         if (p.dh0) {   // dS_0, fp32 (the last chunk's MMAs were waited for above)
-            float *dst = state_row(p.dh0, sbh, row, wh, p.dk, p.dv);
+            float *dst = PAIR ? pair_state_row(p.dh0, sbh, row, wh) : state_row(p.dh0, sbh, row, wh, p.dk, p.dv);
 #pragma unroll
             for (int part = 0; part < 2; ++part) {
                 float v[32];
@@ -917,10 +988,13 @@ __global__ void k_fold_segment_dstates(int H, int P, int dk, int dv, const float
 }  // namespace
 
 int gla_tc_bwd_configure() {
-    if (cudaFuncSetAttribute(k_gla_states_tc<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)st1::SMEM_BYTES) != cudaSuccess ||
-        cudaFuncSetAttribute(k_gla_states_tc<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)st1::SMEM_BYTES) != cudaSuccess)
-        return -1;
-    if (cudaFuncSetAttribute(k_gla_bwd_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)st2::SMEM_BYTES) != cudaSuccess)
+    constexpr cudaFuncAttribute A = cudaFuncAttributeMaxDynamicSharedMemorySize;
+    if (cudaFuncSetAttribute(k_gla_states_tc<false, false>, A, (int)st1::SMEM_BYTES) != cudaSuccess ||
+        cudaFuncSetAttribute(k_gla_states_tc<true, false>, A, (int)st1::SMEM_BYTES) != cudaSuccess ||
+        cudaFuncSetAttribute(k_gla_states_tc<false, true>, A, (int)st1::SMEM_BYTES) != cudaSuccess ||
+        cudaFuncSetAttribute(k_gla_states_tc<true, true>, A, (int)st1::SMEM_BYTES) != cudaSuccess ||
+        cudaFuncSetAttribute(k_gla_bwd_tc<false>, A, (int)st2::SMEM_BYTES) != cudaSuccess ||
+        cudaFuncSetAttribute(k_gla_bwd_tc<true>, A, (int)st2::SMEM_BYTES) != cudaSuccess)
         return -1;
     return retnet_tc_bwd_configure();
 }
@@ -960,7 +1034,7 @@ int gla_tc_segment_summaries(const Dims &d, const FwdArgs &a, int P, int L, int 
     else if (!make_map(&mg, a.log_decay, d.B, d.T, d.H, d.dk, true, 128)) return -1;
     StatesParams sp{a.lq, a.lk, nullptr, nullptr, fin, gam, status, d.T, d.H, d.NT, P, L, PS, retnet ? a.log_decay : nullptr,
                     nullptr, nullptr, d.dk, d.dv};
-    (retnet ? k_gla_states_tc<true> : k_gla_states_tc<false>)<<<d.B * d.H * PS, st1::NTHREADS, st1::SMEM_BYTES, st>>>(mk, mv, mg, sp);
+    (retnet ? k_gla_states_tc<true, false> : k_gla_states_tc<false, false>)<<<d.B * d.H * PS, st1::NTHREADS, st1::SMEM_BYTES, st>>>(mk, mv, mg, sp);
     tr.mark("gla_segment_states_tc");
     return cudaGetLastError() == cudaSuccess ? 1 : -1;
 }
@@ -969,24 +1043,26 @@ uint8_t *gla_tc_state_images(float *ws) { return reinterpret_cast<uint8_t *>(ws)
 
 int gla_tc_backward(const Dims &d, const BwdArgs &a, bool have_states, int *status, cudaStream_t st, Tracer &tr) {
     CUtensorMap mq, mk, mv, mdo, mg, mdq, mdk, mdv, mdg;
+    Varlen *vl = (a.vl && a.vl->n_seq) ? a.vl : nullptr;
+    const bool pair = gla_tc_pairs(d, vl);
+    const int H = pair ? d.H / 2 : d.H, dk = pair ? 128 : d.dk, dv = pair ? 128 : d.dv;       // the heads as the tensor maps count them
     const bool retnet = d.variant == SLA_RETNET;      // constant decay: no log-decay tensor to read, no gradient for it
-    if (!make_tile_map(&mq, a.q, d.B, d.T, d.H, d.dk) || !make_tile_map(&mk, a.k, d.B, d.T, d.H, d.dk) ||
-        !make_tile_map(&mv, a.v, d.B, d.T, d.H, d.dv) || !make_tile_map(&mdo, a.dO, d.B, d.T, d.H, d.dv) ||
-        !make_tile_map(&mdq, a.dq, d.B, d.T, d.H, d.dk) || !make_tile_map(&mdk, a.dk, d.B, d.T, d.H, d.dk) ||
-        !make_tile_map(&mdv, a.dv, d.B, d.T, d.H, d.dv))
+    if (!make_tile_map(&mq, a.q, d.B, d.T, H, dk) || !make_tile_map(&mk, a.k, d.B, d.T, H, dk) ||
+        !make_tile_map(&mv, a.v, d.B, d.T, H, dv) || !make_tile_map(&mdo, a.dO, d.B, d.T, H, dv) ||
+        !make_tile_map(&mdq, a.dq, d.B, d.T, H, dk) || !make_tile_map(&mdk, a.dk, d.B, d.T, H, dk) ||
+        !make_tile_map(&mdv, a.dv, d.B, d.T, H, dv))
         return -1;
     if (retnet) { mg = mq; mdg = mdq; }               // (never used)
-    else if (!make_map(&mg, a.log_decay, d.B, d.T, d.H, d.dk, true, 128) ||
-             !make_map(&mdg, a.dlog_decay, d.B, d.T, d.H, d.dk, true, 128))
+    else if (!make_map(&mg, a.log_decay, d.B, d.T, H, dk, true, 128) ||
+             !make_map(&mdg, a.dlog_decay, d.B, d.T, H, dk, true, 128))
         return -1;
     // workspace: state images, then the two [B,T,H] gate products
-    Varlen *vl = (a.vl && a.vl->n_seq) ? a.vl : nullptr;
     const size_t bth = (size_t)d.B * d.T * d.H;
     const size_t img_floats = state_slots(d, vl) * (STATE_BF16 / 4);
     uint8_t *simg = reinterpret_cast<uint8_t *>(a.ws);
     float *pq = a.ws + img_floats;
     float *pk = pq + ((bth + 63) & ~(size_t)63);
-    const int ctas = vl ? vl->n_seq * d.H : d.B * d.H;
+    const int ctas = vl ? vl->n_seq * H : d.B * H;
     const SeqInfo *dseqs = vl ? vl->d_seqs : nullptr;
     const __nv_bfloat16 *q = (const __nv_bfloat16 *)a.q, *k = (const __nv_bfloat16 *)a.k, *v = (const __nv_bfloat16 *)a.v,
                         *dO = (const __nv_bfloat16 *)a.dO;
@@ -996,38 +1072,40 @@ int gla_tc_backward(const Dims &d, const BwdArgs &a, bool have_states, int *stat
         if (vl) {
             const void *key[] = {a.k, a.v, a.log_decay};
             vm = varlen_maps(*vl, 1, key, 3, st, [&](const SeqInfo &si, CUtensorMap *m) {
-                const size_t tok = (size_t)si.t0 * d.H;      // (q, k are d_k wide, v, o and their gradients d_v)
-                if (!make_tile_map(m + 0, k + tok * d.dk, 1, si.T, d.H, d.dk) || !make_tile_map(m + 1, v + tok * d.dv, 1, si.T, d.H, d.dv)) return false;
+                const size_t tok = (size_t)si.t0 * H;      // (q, k are d_k wide, v, o and their gradients d_v)
+                if (!make_tile_map(m + 0, k + tok * dk, 1, si.T, H, dk) || !make_tile_map(m + 1, v + tok * dv, 1, si.T, H, dv)) return false;
                 if (retnet) { m[2] = m[0]; return true; }
-                return make_map(m + 2, a.log_decay + tok * d.dk, 1, si.T, d.H, d.dk, true, 128);
+                return make_map(m + 2, a.log_decay + tok * dk, 1, si.T, H, dk, true, 128);
             });
             if (!vm) return -1;
         }
         StatesParams sp{a.lq, a.lk, a.h0, simg, nullptr, nullptr, status, d.T, d.H, d.NT, 1, d.NT, 1, retnet ? a.log_decay : nullptr,
                         dseqs, vm, d.dk, d.dv};
-        (retnet ? k_gla_states_tc<true> : k_gla_states_tc<false>)<<<ctas, st1::NTHREADS, st1::SMEM_BYTES, st>>>(mk, mv, mg, sp);
+        auto *const kernel = retnet ? (pair ? k_gla_states_tc<true, true> : k_gla_states_tc<true, false>)
+                                    : pair ? k_gla_states_tc<false, true> : k_gla_states_tc<false, false>;
+        kernel<<<ctas, st1::NTHREADS, st1::SMEM_BYTES, st>>>(mk, mv, mg, sp);
         tr.mark("gla_states_tc");
     }
     const CUtensorMap *vm = nullptr;
     if (vl) {
         const void *key[] = {a.q, a.k, a.v, a.dO, a.log_decay, a.dq, a.dk, a.dv, a.dlog_decay};
         vm = varlen_maps(*vl, 2, key, 9, st, [&](const SeqInfo &si, CUtensorMap *m) {
-            const size_t tok = (size_t)si.t0 * d.H;      // (q, k are d_k wide, v, o and their gradients d_v)
-            if (!make_tile_map(m + 0, q + tok * d.dk, 1, si.T, d.H, d.dk) || !make_tile_map(m + 1, k + tok * d.dk, 1, si.T, d.H, d.dk) ||
-                !make_tile_map(m + 2, v + tok * d.dv, 1, si.T, d.H, d.dv) || !make_tile_map(m + 3, dO + tok * d.dv, 1, si.T, d.H, d.dv) ||
-                !make_tile_map(m + 5, (__nv_bfloat16 *)a.dq + tok * d.dk, 1, si.T, d.H, d.dk) ||
-                !make_tile_map(m + 6, (__nv_bfloat16 *)a.dk + tok * d.dk, 1, si.T, d.H, d.dk) ||
-                !make_tile_map(m + 7, (__nv_bfloat16 *)a.dv + tok * d.dv, 1, si.T, d.H, d.dv))
+            const size_t tok = (size_t)si.t0 * H;      // (q, k are d_k wide, v, o and their gradients d_v)
+            if (!make_tile_map(m + 0, q + tok * dk, 1, si.T, H, dk) || !make_tile_map(m + 1, k + tok * dk, 1, si.T, H, dk) ||
+                !make_tile_map(m + 2, v + tok * dv, 1, si.T, H, dv) || !make_tile_map(m + 3, dO + tok * dv, 1, si.T, H, dv) ||
+                !make_tile_map(m + 5, (__nv_bfloat16 *)a.dq + tok * dk, 1, si.T, H, dk) ||
+                !make_tile_map(m + 6, (__nv_bfloat16 *)a.dk + tok * dk, 1, si.T, H, dk) ||
+                !make_tile_map(m + 7, (__nv_bfloat16 *)a.dv + tok * dv, 1, si.T, H, dv))
                 return false;
             if (retnet) { m[4] = m[0]; m[8] = m[5]; return true; }
-            return make_map(m + 4, a.log_decay + tok * d.dk, 1, si.T, d.H, d.dk, true, 128) &&
-                   make_map(m + 8, a.dlog_decay + tok * d.dk, 1, si.T, d.H, d.dk, true, 128);
+            return make_map(m + 4, a.log_decay + tok * dk, 1, si.T, H, dk, true, 128) &&
+                   make_map(m + 8, a.dlog_decay + tok * dk, 1, si.T, H, dk, true, 128);
         });
         if (!vm) return -1;
     }
     BwdParams bp{a.lq, a.lk, a.dht, simg, pq, pk, a.dh0, status, d.T, d.H, d.NT, d.scale, retnet ? a.log_decay : nullptr, dseqs, vm, d.dk, d.dv};
-    if (retnet) retnet_tc_bwd_launch({mq, mk, mv, mdo, mdq, mdk, mdv}, bp, ctas, st);
-    else k_gla_bwd_tc<<<ctas, st2::NTHREADS, st2::SMEM_BYTES, st>>>(mq, mk, mv, mdo, mg, mdq, mdk, mdv, mdg, bp);
+    if (retnet) retnet_tc_bwd_launch({mq, mk, mv, mdo, mdq, mdk, mdv}, bp, pair, ctas, st);
+    else (pair ? k_gla_bwd_tc<true> : k_gla_bwd_tc<false>)<<<ctas, st2::NTHREADS, st2::SMEM_BYTES, st>>>(mq, mk, mv, mdo, mg, mdq, mdk, mdv, mdg, bp);
     tr.mark("gla_bwd_tc");
     if (gate_bwd_prod(a.lq, a.lk, pq, pk, a.dlq, a.dlk, (long)d.B * d.T, d.H, st) < 0) return -1;
     tr.mark("gate_bwd");

@@ -140,6 +140,8 @@ int gdn_configure();
 // ---- tensor-core (tcgen05 / TMEM / TMA) Softmax-GLA kernels: sla_gla_tc.cu ----
 bool gla_tc_supported(const Dims &d);
 int gla_tc_configure();
+// Do the kernels of this call take two 64-wide heads a CTA?  (All of them or none: the state images differ.)
+bool gla_tc_pairs(const Dims &d, const Varlen *vl);
 // With `simg` not null (and gla_tc_forward_can_save) the forward also leaves the bf16 image of the state before every
 // chunk there, in the layout the gradient sweep reads: the backward pass of the same inputs then needs no state sweep.
 bool gla_tc_forward_can_save(const Dims &d, const Varlen *vl = nullptr);

@@ -25,18 +25,20 @@ constexpr uint32_t OFF_S = 2 * STAGE;                   // bf16 S_n image
 constexpr uint32_t OFF_DZ = OFF_S + STATE_BF16;         // bf16 dZ operand
 constexpr uint32_t OFF_A = OFF_DZ + STATE_BF16;         // masked A, [64 rows][128 B]
 constexpr uint32_t OFF_DA = OFF_A + HALF_BF16;          // masked dA; afterwards A|dA hold the dv tile staged for the store
-constexpr uint32_t OFF_GATE = OFF_DA + HALF_BF16;       // [4][2][64]: f, c of four chunks
-constexpr uint32_t OFF_RED = OFF_GATE + 4 * 2 * C * 4;  // [2][2 column halves][64] gate partial sums
+constexpr uint32_t OFF_GATE = OFF_DA + HALF_BF16;       // [4][heads][2][64]: f, c of four chunks
+constexpr uint32_t OFF_RED = OFF_GATE + 4 * 2 * 2 * C * 4;  // [2][2 column halves][64] gate partial sums
 constexpr uint32_t OFF_BAR = OFF_RED + 2 * 2 * C * 4;
 constexpr uint32_t OFF_TMEM = OFF_BAR + 32 * 8;         // TMEM base address, then the abort flag
 constexpr uint32_t SMEM_BYTES = OFF_TMEM + 16 + 1024;
-constexpr uint32_t COL_DS = 0, COL_A = 128, COL_DA = 192, COL_DV = 128 /* once A and dA are read */, COL_DQ = 256, COL_DK = 384, TMEM_COLS = 512;
+constexpr uint32_t TMEM_COLS = 512;
 constexpr int NTHREADS = NCOMPUTE + 32 + NGATE + 32;    // warps 0..7 compute, 8 MMA issue, 9..12 gates, 13 TMA
 enum Bar { FULL_QK = 0 /*[2]*/, FULL_VO = 2 /*[2]*/, FULL_S = 4, OPR, GREADY = 6 /*[4]*/, GFREE = 10 /*[4]*/, ZREADY = 14, AREADY, OUT1, OUT2,
            DVREAD, DVFREE, BAR_A, BAR_M1, BAR_M2, ALLREAD, SFREE, DRAIN, NBAR };
 static_assert(SMEM_BYTES <= 232448, "shared memory budget");
 static_assert(NBAR <= 32, "barrier slots");
 
+// PAIR: two 64-wide heads a CTA, as in k_gla_bwd_tc.
+template <bool PAIR>
 __global__ void __launch_bounds__(NTHREADS, 1)
 k_retnet_bwd_tc(const __grid_constant__ CUtensorMap gm_q, const __grid_constant__ CUtensorMap gm_k, const __grid_constant__ CUtensorMap gm_v,
                 const __grid_constant__ CUtensorMap gm_do, const __grid_constant__ CUtensorMap gm_dq, const __grid_constant__ CUtensorMap gm_dk,
@@ -46,8 +48,12 @@ k_retnet_bwd_tc(const __grid_constant__ CUtensorMap gm_q, const __grid_constant_
     const uint32_t base = (raw + 1023u) & ~1023u;
     uint8_t *sm = smem_raw + (base - raw);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int bh = blockIdx.x, h = bh % p.H;
-    int b = bh / p.H;
+    constexpr int HPC = PAIR ? 2 : 1;                       // heads per CTA
+    constexpr uint32_t COL_DS = 0, COL_A = 128, COL_DA = PAIR ? 256 : 192, COL_DV = 128 /* once A and dA are read */, COL_DQ = PAIR ? 384 : 256,
+                       COL_DK = PAIR ? 256 /* once dA is read */ : 384;
+    const int hg = p.H / HPC, h = blockIdx.x % hg;          // h: head, or pair of heads, as the tensor maps count them
+    int b = blockIdx.x / hg;
+    const int bh = b * p.H + h * HPC;
     size_t tokb = (size_t)b * p.T, slot = (size_t)bh * (p.NT + 1);
     size_t sbh = (size_t)bh;                                // (sequence, head) index into dht / dh0
     const CUtensorMap *vm = nullptr;
@@ -56,8 +62,8 @@ k_retnet_bwd_tc(const __grid_constant__ CUtensorMap gm_q, const __grid_constant_
         vm = p.vmaps + (size_t)b * Varlen::MAPS_PER_SEQ;
         p.T = si.T; p.NT = si.NT;
         tokb = (size_t)si.t0;
-        slot = (size_t)si.slot0 * p.H + (size_t)h * (si.NT + 1);
-        sbh = (size_t)si.id * p.H + h;                      // (the table is ordered longest first, the state tensors as the caller gave them)
+        slot = (size_t)si.slot0 * p.H + (size_t)h * HPC * (si.NT + 1);
+        sbh = (size_t)si.id * p.H + h * HPC;                      // (the table is ordered longest first, the state tensors as the caller gave them)
         b = 0;
     }
     const CUtensorMap &tm_q = vm ? vm[0] : gm_q, &tm_k = vm ? vm[1] : gm_k, &tm_v = vm ? vm[2] : gm_v, &tm_do = vm ? vm[3] : gm_do,
@@ -88,7 +94,7 @@ k_retnet_bwd_tc(const __grid_constant__ CUtensorMap gm_q, const __grid_constant_
         tma_prefetch_desc(&tm_dq);
         tma_prefetch_desc(&tm_dk);
         tma_prefetch_desc(&tm_dv);
-        check_scalar_range(p.log_gamma[h], p.T, p.status);
+        for (int x = 0; x < HPC; ++x) check_scalar_range(p.log_gamma[HPC * h + x], p.T, p.status);
     }
     if (warp == 0) tmem_alloc(base + OFF_TMEM, TMEM_COLS);
     tc_fence_before();
@@ -97,7 +103,6 @@ k_retnet_bwd_tc(const __grid_constant__ CUtensorMap gm_q, const __grid_constant_
     const uint32_t tmem = *reinterpret_cast<volatile uint32_t *>(sm + OFF_TMEM);
     const uint8_t *img0 = p.simg + slot * STATE_BF16;
     const int NT = p.NT;
-    const float lg = LOG2E * p.log_gamma[h];
     // chunks are visited in the order n = NT-1 ... 0; k = NT-1-n is the visit number that drives every buffer and parity
 
     if (warp == 8) {
@@ -110,6 +115,7 @@ k_retnet_bwd_tc(const __grid_constant__ CUtensorMap gm_q, const __grid_constant_
         constexpr uint32_t ID_A = idesc_bf16(64, 64, 0, 0);
         constexpr uint32_t ID_KK = idesc_bf16(64, 128, 0, 0), ID_KM = idesc_bf16(64, 128, 0, 1),
                            ID_MM = idesc_bf16(64, 128, 1, 1), ID_S = idesc_bf16(128, 128, 1, 1);
+        constexpr uint32_t ID_KM64 = idesc_bf16(64, 64, 0, 1), ID_MM64 = idesc_bf16(64, 64, 1, 1);
         const uint64_t kS = desc_kmajor(base + OFF_S), kDZ = desc_kmajor(base + OFF_DZ),
                        mDZ = desc_mnmajor(base + OFF_DZ, STATE_HALF), mA = desc_mnmajor(base + OFF_A, HALF_BF16),
                        kDA = desc_kmajor(base + OFF_DA), mDA = desc_mnmajor(base + OFF_DA, HALF_BF16);
@@ -126,8 +132,9 @@ k_retnet_bwd_tc(const __grid_constant__ CUtensorMap gm_q, const __grid_constant_
             if (leader) {
 #pragma unroll
                 for (int kk = 0; kk < 8; ++kk) {       // A = qh kh^T,  dA = dO V^T
-                    tc_mma_bf16(tmem + COL_A, kQ + kstep_kmajor(kk, HALF_BF16), kK + kstep_kmajor(kk, HALF_BF16), ID_A, kk > 0);
-                    tc_mma_bf16(tmem + COL_DA, kDO + kstep_kmajor(kk, HALF_BF16), kV + kstep_kmajor(kk, HALF_BF16), ID_A, kk > 0);
+                    const uint32_t hc = PAIR ? 64 * (kk >> 2) : 0, acc = PAIR ? (kk & 3) > 0 : kk > 0;      // (a pair: head kk / 4)
+                    tc_mma_bf16(tmem + COL_A + hc, kQ + kstep_kmajor(kk, HALF_BF16), kK + kstep_kmajor(kk, HALF_BF16), ID_A, acc);
+                    tc_mma_bf16(tmem + COL_DA + hc, kDO + kstep_kmajor(kk, HALF_BF16), kV + kstep_kmajor(kk, HALF_BF16), ID_A, acc);
                 }
                 tc_commit(bar(BAR_A));
             }
@@ -137,8 +144,13 @@ k_retnet_bwd_tc(const __grid_constant__ CUtensorMap gm_q, const __grid_constant_
             tc_fence_after();
             if (leader) {
 #pragma unroll
-                for (int kk = 0; kk < 8; ++kk)         // dqh = dO S_n^T ...
-                    tc_mma_bf16(tmem + COL_DQ, kDO + kstep_kmajor(kk, HALF_BF16), kS + kstep_kmajor(kk, STATE_HALF), ID_KK, kk > 0);
+                for (int kk = 0; kk < 8; ++kk) {       // dqh = dO S_n^T ...
+                    if (PAIR)
+                        tc_mma_bf16(tmem + COL_DQ + 64 * (kk >> 2), kDO + kstep_kmajor(kk, HALF_BF16),
+                                    desc_kmajor(base + OFF_S + pair_block(kk >> 2)) + kstep_kmajor(kk & 3, 0), ID_A, (kk & 3) > 0);
+                    else
+                        tc_mma_bf16(tmem + COL_DQ, kDO + kstep_kmajor(kk, HALF_BF16), kS + kstep_kmajor(kk, STATE_HALF), ID_KK, kk > 0);
+                }
                 tc_commit(bar(SFREE));                 // (for the TMA lane: the next image may land)
             }
             wait(ZREADY, par);                         // dZ: fp32 in TMEM, bf16 in shared memory
@@ -147,7 +159,7 @@ k_retnet_bwd_tc(const __grid_constant__ CUtensorMap gm_q, const __grid_constant_
             if (leader) {
 #pragma unroll
                 for (int kk = 0; kk < 8; ++kk) {       // two independent accumulation chains, interleaved
-                    tc_mma_bf16(tmem + COL_DK, kV + kstep_kmajor(kk, HALF_BF16), kDZ + kstep_kmajor(kk, STATE_HALF), ID_KK, kk > 0);   // dkh = V dZ^T ...
+                    if (!PAIR) tc_mma_bf16(tmem + COL_DK, kV + kstep_kmajor(kk, HALF_BF16), kDZ + kstep_kmajor(kk, STATE_HALF), ID_KK, kk > 0);   // dkh = V dZ^T ...
                     if (kk < 4) tc_mma_bf16(tmem + COL_DS, mQ + kstep_mnmajor(kk), mDO + kstep_mnmajor(kk), ID_S, 1);                // dS_n = dZ + qh^T dO
                 }
             }
@@ -156,17 +168,41 @@ k_retnet_bwd_tc(const __grid_constant__ CUtensorMap gm_q, const __grid_constant_
             tc_fence_after();
             if (leader) {
 #pragma unroll
-                for (int kk = 0; kk < 8; ++kk)         // dV = kh dZ ... (A and dA have been read; before M1, after which dk goes over kh)
-                    tc_mma_bf16(tmem + COL_DV, kK + kstep_kmajor(kk, HALF_BF16), mDZ + kstep_mnmajor(kk), ID_KM, kk > 0);
+                for (int kk = 0; kk < 8; ++kk) {       // dV = kh dZ ... (A and dA have been read; before M1, after which dk goes over kh)
+                    if (PAIR) {                        // (head kk / 4; and dkh = V dZ^T)
+                        const uint32_t dz = base + OFF_DZ + pair_block(kk >> 2);
+                        tc_mma_bf16(tmem + COL_DV + 64 * (kk >> 2), kK + kstep_kmajor(kk, HALF_BF16), desc_mnmajor(dz, STATE_HALF) + kstep_mnmajor(kk & 3), ID_KM64, (kk & 3) > 0);
+                        tc_mma_bf16(tmem + COL_DK + 64 * (kk >> 2), kV + kstep_kmajor(kk, HALF_BF16), desc_kmajor(dz) + kstep_kmajor(kk & 3, 0), ID_A, (kk & 3) > 0);
+                    } else {
+                        tc_mma_bf16(tmem + COL_DV, kK + kstep_kmajor(kk, HALF_BF16), mDZ + kstep_mnmajor(kk), ID_KM, kk > 0);
+                    }
+                }
+                // ... + dA kh  and  ... + dA^T qh, interleaved; a pair: head x's tile and its half of kh, qh
+                auto head = [&](int x, uint32_t sDA, int kk) {
+                    tc_mma_bf16(tmem + COL_DQ + 64 * x, desc_kmajor(sDA) + kstep_kmajor(kk, 0), desc_mnmajor(st + T_K + x * HALF_BF16, HALF_BF16) + kstep_mnmajor(kk), ID_KM64, 1);
+                    tc_mma_bf16(tmem + COL_DK + 64 * x, desc_mnmajor(sDA, HALF_BF16) + kstep_mnmajor(kk), desc_mnmajor(st + T_Q + x * HALF_BF16, HALF_BF16) + kstep_mnmajor(kk), ID_MM64, 1);
+                };
 #pragma unroll
-                for (int kk = 0; kk < 4; ++kk) {       // ... + dA kh  and  ... + dA^T qh, interleaved
-                    tc_mma_bf16(tmem + COL_DQ, kDA + kstep_kmajor(kk, 0), mK + kstep_mnmajor(kk), ID_KM, 1);
-                    tc_mma_bf16(tmem + COL_DK, mDA + kstep_mnmajor(kk), mQ + kstep_mnmajor(kk), ID_MM, 1);
+                for (int kk = 0; kk < 4; ++kk) {
+                    if (PAIR) {
+                        head(0, base + OFF_DA, kk);
+                        head(1, base + OFF_S + PAIR_FREE1, kk);
+                    } else {
+                        tc_mma_bf16(tmem + COL_DQ, kDA + kstep_kmajor(kk, 0), mK + kstep_mnmajor(kk), ID_KM, 1);
+                        tc_mma_bf16(tmem + COL_DK, mDA + kstep_mnmajor(kk), mQ + kstep_mnmajor(kk), ID_MM, 1);
+                    }
                 }
                 tc_commit(bar(BAR_M1));
 #pragma unroll
-                for (int kk = 0; kk < 4; ++kk)         // ... + A^T dO
-                    tc_mma_bf16(tmem + COL_DV, mA + kstep_mnmajor(kk), mDO + kstep_mnmajor(kk), ID_MM, 1);
+                for (int kk = 0; kk < 4; ++kk) {       // ... + A^T dO
+                    if (PAIR) {
+                        tc_mma_bf16(tmem + COL_DV, mA + kstep_mnmajor(kk), mDO + kstep_mnmajor(kk), ID_MM64, 1);
+                        tc_mma_bf16(tmem + COL_DV + 64, desc_mnmajor(base + OFF_S + PAIR_FREE0, HALF_BF16) + kstep_mnmajor(kk),
+                                    desc_mnmajor(st + T_DO + HALF_BF16, HALF_BF16) + kstep_mnmajor(kk), ID_MM64, 1);
+                    } else {
+                        tc_mma_bf16(tmem + COL_DV, mA + kstep_mnmajor(kk), mDO + kstep_mnmajor(kk), ID_MM, 1);
+                    }
+                }
                 tc_commit(bar(BAR_M2));
                 tc_commit(bar(ALLREAD));               // (same event, for the TMA lane)
             }
@@ -186,9 +222,15 @@ k_retnet_bwd_tc(const __grid_constant__ CUtensorMap gm_q, const __grid_constant_
                 tma_load_5d(dst + T_V, &tm_v, 0, n * C, 0, h, b, vo);
                 tma_load_5d(dst + T_DO, &tm_do, 0, n * C, 0, h, b, vo);
             };
+            constexpr uint32_t IMAGE = PAIR ? PAIR_STATE : STATE_BF16;
             auto load_s = [&](int n) {
-                mbar_expect_tx(bar(FULL_S), STATE_BF16);
-                bulk_load(base + OFF_S, img0 + (size_t)n * STATE_BF16, STATE_BF16, bar(FULL_S));
+                mbar_expect_tx(bar(FULL_S), IMAGE);
+                if (PAIR) {
+                    bulk_load(base + OFF_S + pair_block(0), img0 + (size_t)n * IMAGE, STATE_BLOCK, bar(FULL_S));
+                    bulk_load(base + OFF_S + pair_block(1), img0 + (size_t)n * IMAGE + STATE_BLOCK, STATE_BLOCK, bar(FULL_S));
+                } else {
+                    bulk_load(base + OFF_S, img0 + (size_t)n * IMAGE, IMAGE, bar(FULL_S));
+                }
             };
             load_tiles(0);
             load_s(NT - 1);
@@ -201,7 +243,7 @@ k_retnet_bwd_tc(const __grid_constant__ CUtensorMap gm_q, const __grid_constant_
                     tma_prefetch_l2_5d(&tm_k, 0, (n - 2) * C, 0, h, b);
                     tma_prefetch_l2_5d(&tm_v, 0, (n - 2) * C, 0, h, b);
                     tma_prefetch_l2_5d(&tm_do, 0, (n - 2) * C, 0, h, b);
-                    bulk_prefetch_l2(img0 + (size_t)(n - 2) * STATE_BF16, STATE_BF16);
+                    bulk_prefetch_l2(img0 + (size_t)(n - 2) * IMAGE, IMAGE);
                 }
                 if (n > 0) {
                     wait(SFREE, par);                  // S_n has been read
@@ -234,13 +276,15 @@ k_retnet_bwd_tc(const __grid_constant__ CUtensorMap gm_q, const __grid_constant_
         // ---------------- gates with the tokens' decay, up to four chunks ahead ----------------
         const int g = tid - (NCOMPUTE + 32), t = g & (C - 1);
         const float *l = g < C ? p.lq : p.lk;
-        const DecayFactor f{g < C ? p.scale : 1.f, g < C ? lg : -lg};
+        const float mult = g < C ? p.scale : 1.f, sign = g < C ? LOG2E : -LOG2E;
+        const DecayFactor f{mult, sign * p.log_gamma[HPC * h]}, f2{mult, PAIR ? sign * p.log_gamma[2 * h + 1] : 0.f};
         for (int k = 0; k < NT; ++k) {
             const int n = NT - 1 - k;
             if (k >= 4) wait_relaxed(GFREE + (k & 3), ((k >> 2) - 1) & 1);
             if (failed) break;
             const int cn = min(C, p.T - n * C);
-            chunk_gate_by(l + (tokb + (size_t)n * C) * p.H, p.H, cn, h, f, gate_s + (k & 3) * 2 * C + (g < C ? 0 : C), t);
+            float *dst = gate_s + (k & 3) * HPC * 2 * C + (g < C ? 0 : C);
+            chunk_gate_by<64, HPC>(l + (tokb + (size_t)n * C) * p.H, p.H, cn, HPC * h, f, dst, t, f2, dst + 2 * C);
             __syncwarp();
             if (lane == 0) mbar_arrive(bar(GREADY + (k & 3)));
         }
@@ -250,18 +294,20 @@ k_retnet_bwd_tc(const __grid_constant__ CUtensorMap gm_q, const __grid_constant_
         const int wh = warp >> 2;                       // column half, of the state and of the gradient tiles
         const int row = 32 * (warp & 3) + lane;         // state row of this thread (its TMEM lane)
         const int qr = warp & 3, tr = 16 * qr + (lane >> 2);       // gradient tiles: tokens tr, tr + 8
+        const bool holds = !PAIR || pair_diagonal(warp & 3, wh);   // (a pair's threads off the diagonal blocks have no state)
+        const float lg = LOG2E * p.log_gamma[HPC * h + (PAIR ? row >> 6 : 0)];
         auto prologue = [&](int k) {
             wait(GREADY + (k & 3), (k >> 2) & 1);
             wait(FULL_QK + (k & 1), (k >> 1) & 1);
             uint8_t *qk = sm + (k & 1) * STAGE;
-            const float *g = gate_s + (k & 3) * 2 * C;
-            scale_rows(qk + T_Q, g, tid);
-            scale_rows(qk + T_K, g + C, tid);
+            const float *g = gate_s + (k & 3) * HPC * 2 * C;
+            scale_rows(qk + T_Q, g, tid, PAIR ? 2 * C : 0);
+            scale_rows(qk + T_K, g + C, tid, PAIR ? 2 * C : 0);
             fence_proxy_async();
             warp_arrive(bar(OPR), lane);
         };
         {   // dS_NT = dht (or zero) into TMEM
-            const float *src = state_row(p.dht, sbh, row, wh, p.dk, p.dv);
+            const float *src = PAIR ? pair_state_row(p.dht, sbh, row, wh) : state_row(p.dht, sbh, row, wh, p.dk, p.dv);
 #pragma unroll
             for (int part = 0; part < 2; ++part) {
                 float v[32];
@@ -275,11 +321,11 @@ k_retnet_bwd_tc(const __grid_constant__ CUtensorMap gm_q, const __grid_constant_
             const int n = NT - 1 - k, t0 = n * C, cn = min(C, p.T - t0);
             const uint32_t par = k & 1;
             uint8_t *qk = sm + (k & 1) * STAGE;
-            const float *gate = gate_s + (k & 3) * 2 * C;
+            const float *gate = gate_s + ((k & 3) * HPC + (PAIR ? wh : 0)) * 2 * C;       // (of the head whose columns this warp reads out)
 
             // ---- dZ = e^{b_last} dS_{n+1}: fp32 back into TMEM (dS_n accumulates on it), bf16 operand copy (every product of the
             // previous chunk is complete, see BAR_M2 below) ----
-            {
+            if (holds) {
                 const float e = ex2f(lg * (float)cn);
                 float v0[32], v1[32];
                 const uint32_t ta = tmem + lane_base + COL_DS + 64 * wh;
@@ -310,17 +356,20 @@ k_retnet_bwd_tc(const __grid_constant__ CUtensorMap gm_q, const __grid_constant_
             wait(BAR_A, par);
             tc_fence_after();
             {
-                uint8_t *dst = sm + (wh ? OFF_DA : OFF_A);
-                float v[32];
-                tmem_ld_frag8(tmem + lane_base + (wh ? COL_DA : COL_A), v);
-                tmem_wait_ld();
-                if (k > 0) wait(DVFREE, (k - 1) & 1);   // the staged dv of the previous chunk has left A|dA
 #pragma unroll
-                for (int i = 0; i < 8; ++i) {
-                    const int j = 8 * i + 2 * (lane & 3);
-                    const uint32_t off = frag_off(qr, lane, 0, i);
-                    *reinterpret_cast<uint32_t *>(dst + off) = pack_bf16(j <= tr ? v[4 * i] : 0.f, j + 1 <= tr ? v[4 * i + 1] : 0.f);
-                    *reinterpret_cast<uint32_t *>(dst + off + 1024) = pack_bf16(j <= tr + 8 ? v[4 * i + 2] : 0.f, j + 1 <= tr + 8 ? v[4 * i + 3] : 0.f);
+                for (int x = 0; x < HPC; ++x) {
+                    uint8_t *dst = sm + (x == 0 ? (wh ? OFF_DA : OFF_A) : OFF_S + (wh ? PAIR_FREE1 : PAIR_FREE0));
+                    float v[32];
+                    tmem_ld_frag8(tmem + lane_base + (wh ? COL_DA : COL_A) + 64 * x, v);
+                    tmem_wait_ld();
+                    if (x == 0 && k > 0) wait(DVFREE, (k - 1) & 1);   // the staged dv of the previous chunk has left A|dA
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) {
+                        const int j = 8 * i + 2 * (lane & 3);
+                        const uint32_t off = frag_off(qr, lane, 0, i);
+                        *reinterpret_cast<uint32_t *>(dst + off) = pack_bf16(j <= tr ? v[4 * i] : 0.f, j + 1 <= tr ? v[4 * i + 1] : 0.f);
+                        *reinterpret_cast<uint32_t *>(dst + off + 1024) = pack_bf16(j <= tr + 8 ? v[4 * i + 2] : 0.f, j + 1 <= tr + 8 ? v[4 * i + 3] : 0.f);
+                    }
                 }
             }
             fence_proxy_async();
@@ -398,14 +447,21 @@ k_retnet_bwd_tc(const __grid_constant__ CUtensorMap gm_q, const __grid_constant_
             fence_proxy_async();
             warp_arrive(bar(OUT2), lane);
             named_bar_sync(1, NCOMPUTE);                // red is complete
-            if (tid < cn) {   // Gq*dGq and Gk*dGk of token tid: sum over the two column halves
+            if (PAIR && tid < 2 * C) {        // Gq*dGq and Gk*dGk of token tid % 64: a head's sums are one column half's
+                const int x = tid / C, i = tid % C;
+                if (i < cn) {
+                    p.pq[(tokb + t0 + i) * p.H + 2 * h + x] = red[x * C + i];
+                    p.pk[(tokb + t0 + i) * p.H + 2 * h + x] = red[(2 + x) * C + i];
+                }
+            }
+            if (!PAIR && tid < cn) {          // ... of token tid: sum over the two column halves
                 p.pq[(tokb + t0 + tid) * p.H + h] = red[tid] + red[C + tid];
                 p.pk[(tokb + t0 + tid) * p.H + h] = red[2 * C + tid] + red[3 * C + tid];
             }
         }
 
         if (p.dh0) {   // dS_0, fp32 (the last chunk's MMAs were waited for above)
-            float *dst = state_row(p.dh0, sbh, row, wh, p.dk, p.dv);
+            float *dst = PAIR ? pair_state_row(p.dh0, sbh, row, wh) : state_row(p.dh0, sbh, row, wh, p.dk, p.dv);
 #pragma unroll
             for (int part = 0; part < 2; ++part) {
                 float v[32];
@@ -428,11 +484,13 @@ k_retnet_bwd_tc(const __grid_constant__ CUtensorMap gm_q, const __grid_constant_
 namespace tc {
 
 int retnet_tc_bwd_configure() {
-    return cudaFuncSetAttribute(k_retnet_bwd_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_BYTES) == cudaSuccess ? 0 : -1;
+    constexpr cudaFuncAttribute A = cudaFuncAttributeMaxDynamicSharedMemorySize;
+    return cudaFuncSetAttribute(k_retnet_bwd_tc<false>, A, (int)SMEM_BYTES) == cudaSuccess &&
+                   cudaFuncSetAttribute(k_retnet_bwd_tc<true>, A, (int)SMEM_BYTES) == cudaSuccess ? 0 : -1;
 }
 
-void retnet_tc_bwd_launch(const CUtensorMap (&m)[7], const BwdParams &p, int ctas, cudaStream_t st) {
-    k_retnet_bwd_tc<<<ctas, NTHREADS, SMEM_BYTES, st>>>(m[0], m[1], m[2], m[3], m[4], m[5], m[6], p);
+void retnet_tc_bwd_launch(const CUtensorMap (&m)[7], const BwdParams &p, bool pair, int ctas, cudaStream_t st) {
+    (pair ? k_retnet_bwd_tc<true> : k_retnet_bwd_tc<false>)<<<ctas, NTHREADS, SMEM_BYTES, st>>>(m[0], m[1], m[2], m[3], m[4], m[5], m[6], p);
 }
 
 }  // namespace tc

@@ -48,8 +48,9 @@ def test_pairs_match_the_oracle(base, B, T, H):
 
 @pytest.mark.parametrize("base", ["C2", "R2"])
 def test_packed_pairs_match_sequences_run_alone(base):
-    """Twelve sequences of 16 heads (192 single heads: paired) against each sequence as a call of its own (16 heads: single)."""
-    lens = [1, 63, 64, 65, 300, 130, 2, 128, 129, 17, 190, 64]
+    """Thirty-six sequences of 16 heads (more chunks an SM than the longest sequence has: paired) against each sequence as a call of its
+    own (16 heads: single)."""
+    lens = [1, 63, 64, 65, 300, 130, 2, 128, 129, 17, 190, 64] * 3
     H, cu = 16, [0]
     for n in lens:
         cu.append(cu[-1] + n)
