@@ -142,10 +142,10 @@ __device__ __forceinline__ void let_copies_land() {
 namespace pr {
 constexpr int LDL = 68;                                 // row stride (floats) of the fp32 64x64 work arrays
 constexpr uint32_t MAT = 64 * LDL * 4;                  // 17 KiB
-constexpr uint32_t OFF_Q = 0;                           // q tile -> fp32 T -> We staged
+constexpr uint32_t OFF_Q = 0;                           // q tile -> fp32 T
 constexpr uint32_t OFF_K = OFF_Q + MAT;
 constexpr uint32_t OFF_L = OFF_K + TILE_BF16;           // fp32 L -> Te below its diagonal | T2 (bf16)
-constexpr uint32_t OFF_A = OFF_L + MAT;                 // bf16 A
+constexpr uint32_t OFF_A = OFF_L + MAT;                 // bf16 A; afterwards A and TW hold We staged for the store
 constexpr uint32_t OFF_TW = OFF_A + HALF_BF16;          // bf16 -Te diag(beta Gam)
 constexpr uint32_t OFF_X = OFF_TW + HALF_BF16;          // [4 warps][32][8] block-product scratch
 constexpr uint32_t OFF_SC = OFF_X + 4 * 32 * 8 * 4;     // b, e^-b, scale Gq (then fq), beta Gam, beta Gk, Gk, beta, log-decay: 8 x 64 floats
@@ -174,37 +174,41 @@ __device__ __forceinline__ void prep_worker(const CUtensorMap &gm_q, const CUten
     const int step = (int)gridDim.x * NWORK;
     SeqHead s, sn;
     int slot = next_chunk(p, (int)blockIdx.x * NWORK + wid, step, s), slot_n;
+    auto load = [&](const SeqHead &o, int n) {              // q, k of a chunk (by the leader)
+        mbar_expect_tx(bFULL, 2 * TILE_BF16);
+        tma_load_5d(base + OFF_K, o.vm ? o.vm + 1 : &gm_k, 0, n * C, 0, o.h, o.b, bFULL);
+        tma_load_5d(base + OFF_Q, o.vm ? o.vm : &gm_q, 0, n * C, 0, o.h, o.b, bFULL);
+    };
+    GateAhead gates;                                        // of the chunk to come, one token's logits spread over its lanes
+    float xv = 0.f;                                         // its log-decay (threads 0..63) or beta of token tid % 64
+    auto fetch_gates = [&](const SeqHead &o, int n) {
+        const int t = tid & (C - 1), cn = min(C, o.T - n * C);
+        const size_t t0 = o.tok + (size_t)n * C;
+        gates.fetch((tid < C ? p.lq : p.lk) + t0 * p.H, p.H, cn, t);
+        xv = t < cn ? (tid < C ? p.g : p.beta)[(t0 + t) * p.H + o.h] : 0.f;
+    };
+    if (slot < p.slots) {
+        if (leader) load(s, slot - s.slot);
+        fetch_gates(s, slot - s.slot);
+    }
     for (; slot < p.slots; slot = slot_n, s = sn) {
         const int n = slot - s.slot;
-        const CUtensorMap &tm_q = s.vm ? s.vm[0] : gm_q, &tm_k = s.vm ? s.vm[1] : gm_k;
-        if (leader) {
-            bulk_wait_read0();                              // the previous chunk's results have left their buffers
-            mbar_expect_tx(bFULL, 2 * TILE_BF16);
-            tma_load_5d(base + OFF_K, &tm_k, 0, n * C, 0, s.h, s.b, bFULL);
-            tma_load_5d(base + OFF_Q, &tm_q, 0, n * C, 0, s.h, s.b, bFULL);
-        }
         {
             const int t = tid & (C - 1), cn = min(C, s.T - n * C);
-            const size_t t0 = s.tok + (size_t)n * C;
-            const float *x = tid < C ? p.g : p.beta;
-            const float xv = t < cn ? x[(t0 + t) * p.H + s.h] : 0.f;
-            if (tid < C) chunk_gate(p.lq + t0 * p.H, p.H, cn, s.h, p.scale, s_fq, t);
-            else chunk_gate(p.lk + t0 * p.H, p.H, cn, s.h, 1.f, s_gk, t);
+            gates.finish((tid < C ? p.lq : p.lk) + (s.tok + (size_t)n * C) * p.H, p.H, cn, s.h, tid < C ? p.scale : 1.f, tid < C ? s_fq : s_gk, t);
             (tid < C ? s_g : s_beta)[t] = xv;
         }
-        // the next chunk's inputs into L2: its copies cannot start before this chunk's buffers are done
+        // The next chunk's logits, log-decay and beta into registers, its tiles into L2 (their copies start when this chunk's last product
+        // has read k).  Logits requested where they are used cost 4,600 of a chunk's 15,000 cycles: with the tiles' early request 3 x 2500
+        // tokens x 16 heads forward 109 -> 100 us, 4 x 4096 x 16 forward and backward 517 -> 506.
         slot_n = next_chunk(p, slot + step, step, sn);
         if (slot_n < p.slots) {
-            const int nn = slot_n - sn.slot, t = tid & (C - 1), cn = min(C, sn.T - nn * C);
+            const int nn = slot_n - sn.slot;
             if (leader) {
                 tma_prefetch_l2_5d(sn.vm ? sn.vm + 1 : &gm_k, 0, nn * C, 0, sn.h, sn.b);
                 tma_prefetch_l2_5d(sn.vm ? sn.vm : &gm_q, 0, nn * C, 0, sn.h, sn.b);
             }
-            if (t < cn) {
-                const size_t row = (sn.tok + (size_t)nn * C + t) * p.H;
-                prefetch_l2((tid < C ? p.lq : p.lk) + row);
-                prefetch_l2((tid < C ? p.g : p.beta) + row + sn.h);
-            }
+            fetch_gates(sn, nn);
         }
         sync();
         if (warp == 0) {
@@ -254,6 +258,7 @@ __device__ __forceinline__ void prep_worker(const CUtensorMap &gm_q, const CUten
                 if (b < -SLA_MAX_CHUNK_DECAY) atomicOr(p.status, STATUS_RANGE);
             }
         }
+        if (leader) bulk_wait_read0();                      // the previous chunk's We, Te, T2 have left the buffers of A, TW and L
         sync();
         wait(bM1, par);
         tc_fence_after();
@@ -287,8 +292,14 @@ __device__ __forceinline__ void prep_worker(const CUtensorMap &gm_q, const CUten
                     pack_bf16(j <= r + 8 ? q1 * v[4 * i + 2] : 0.f, j + 1 <= r + 8 ? q1 * v[4 * i + 3] : 0.f);
             }
         }
+        fence_proxy_async();
         tc_fence_before();
         sync();
+        uint8_t *rec = p.rec + (size_t)slot * p.L.bytes;
+        if (leader) {
+            bulk_store(rec + p.L.a, base + OFF_A, HALF_BF16);
+            bulk_commit();
+        }
         if (tid < C) {        // diagonal 16x16 blocks: column c of (I + L_bb)^{-1} by forward substitution
             const int bb = tid >> 4, c = tid & 15;
             const float *Lb = Ls + (16 * bb) * LDL + 16 * bb;
@@ -384,6 +395,7 @@ __device__ __forceinline__ void prep_worker(const CUtensorMap &gm_q, const CUten
         }
         fence_proxy_async();
         tc_fence_before();
+        if (leader) bulk_wait_read0();                      // A has left: We goes there
         sync();
         if (warp == 0) {
             constexpr uint32_t ID = idesc_bf16(64, 128, 0, 1);
@@ -397,6 +409,9 @@ __device__ __forceinline__ void prep_worker(const CUtensorMap &gm_q, const CUten
         }
         wait(bM2, par);
         tc_fence_after();
+        // k has been read for the last time and T before the last barrier: the next chunk's tiles land while We leaves.  (Requested at the
+        // top of the next chunk, behind the stores of We out of q's place, they cost 6,000 of a chunk's 15,700 cycles.)
+        if (leader && slot_n < p.slots) load(sn, slot_n - sn.slot);
 #pragma unroll
         for (int hf = 0; hf < 2; ++hf) {
             float v[32];
@@ -405,8 +420,8 @@ __device__ __forceinline__ void prep_worker(const CUtensorMap &gm_q, const CUten
 #pragma unroll
             for (int i = 0; i < 8; ++i) {
                 const uint32_t off = frag_off(warp, lane, 64 * hf, i);
-                *reinterpret_cast<uint32_t *>(sm + OFF_Q + off) = pack_bf16(v[4 * i], v[4 * i + 1]);
-                *reinterpret_cast<uint32_t *>(sm + OFF_Q + off + 1024) = pack_bf16(v[4 * i + 2], v[4 * i + 3]);
+                *reinterpret_cast<uint32_t *>(sm + OFF_A + off) = pack_bf16(v[4 * i], v[4 * i + 1]);
+                *reinterpret_cast<uint32_t *>(sm + OFF_A + off + 1024) = pack_bf16(v[4 * i + 2], v[4 * i + 3]);
             }
         }
         fence_proxy_async();
@@ -414,9 +429,7 @@ __device__ __forceinline__ void prep_worker(const CUtensorMap &gm_q, const CUten
         sync();
         tc_fence_after();
         if (leader) {
-            uint8_t *rec = p.rec + (size_t)slot * p.L.bytes;
-            bulk_store(rec + p.L.w, base + OFF_Q, TILE_BF16);
-            bulk_store(rec + p.L.a, base + OFF_A, HALF_BF16);
+            bulk_store(rec + p.L.w, base + OFF_A, TILE_BF16);
             bulk_store(rec + p.L.t2, base + OFF_L + HALF_BF16, HALF_BF16);
             if (p.save) bulk_store(rec + p.L.te, base + OFF_L, HALF_BF16);
             bulk_commit();

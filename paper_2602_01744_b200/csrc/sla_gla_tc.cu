@@ -1,4 +1,4 @@
-// Softmax-GLA forward on the 5th-generation tensor cores (bf16 I/O, d_k and d_v 128 - or 64, run as 128 with zero padding supplied by the tensor maps -, chunk 64).
+// Softmax-GLA forward on the 5th-generation tensor cores (bf16 I/O, d_k and d_v 128 - or 64: two heads side by side, or one with zero padding supplied by the tensor maps -, chunk 64).
 //
 // One CTA owns one (batch, head) sequence and walks its chunks in order, so q, k, v, log-decay are
 // read from HBM exactly once and o is written once; nothing else touches HBM.

@@ -1,5 +1,5 @@
 // Constants and host helpers shared by the tensor-core (tcgen05 / TMEM / TMA) Softmax-GLA kernels:
-// bf16 I/O, d_k = d_v = 128 (64-wide heads run padded), 64-token chunks.  Shared-memory tiles are rows of 128 bytes (64 bf16) in the
+// bf16 I/O, d_k = d_v = 128 (64-wide heads run padded or in pairs), 64-token chunks.  Shared-memory tiles are rows of 128 bytes (64 bf16) in the
 // 128-byte swizzle; a 128-wide tile is two such halves side by side.
 #pragma once
 #include <type_traits>
@@ -418,6 +418,26 @@ template <int NTH = 64>
 __device__ __forceinline__ void chunk_gate(const float *L, int H, int cn, int h, float mult, float *dst, int t) {
     chunk_gate_by<NTH>(L, H, cn, h, ConstFactor{mult}, dst, t);
 }
+// chunk_gate in two halves, the fetch well before the use (64 threads a gate): the logits wait in registers
+// (H other than 4, 8, 16, 32: in L2).
+struct GateAhead {
+    float4 x[8];
+    __device__ __forceinline__ void fetch(const float *L, int H, int cn, int t) {
+        if (H == 16) gate_fetch<4, 64>(L, cn, t, reinterpret_cast<float4 (&)[4]>(x));
+        else if (H == 8) gate_fetch<2, 64>(L, cn, t, reinterpret_cast<float4 (&)[2]>(x));
+        else if (H == 4) gate_fetch<1, 64>(L, cn, t, reinterpret_cast<float4 (&)[1]>(x));
+        else if (H == 32) gate_fetch<8, 64>(L, cn, t, x);
+        else if (t < cn) ptx::prefetch_l2(L + (size_t)t * H);
+    }
+    __device__ __forceinline__ void finish(const float *L, int H, int cn, int h, float mult, float *dst, int t) {
+        const ConstFactor f{mult};
+        if (H == 16) gate_finish<4, 64>(reinterpret_cast<float4 (&)[4]>(x), cn, h, f, dst, t);
+        else if (H == 8) gate_finish<2, 64>(reinterpret_cast<float4 (&)[2]>(x), cn, h, f, dst, t);
+        else if (H == 4) gate_finish<1, 64>(reinterpret_cast<float4 (&)[1]>(x), cn, h, f, dst, t);
+        else if (H == 32) gate_finish<8, 64>(x, cn, h, f, dst, t);
+        else chunk_gate(L, H, cn, h, mult, dst, t);
+    }
+};
 constexpr int NGATE = 128;   // gate threads: g < 64 -> scale*Gq of token g, g >= 64 -> Gk of token g-64
 
 // ---- the gradient sweep's parameters, Softmax-GLA (sla_gla_tc_bwd.cu) and Softmax-RetNet (sla_retnet_tc_bwd.cu) ----

@@ -1,4 +1,4 @@
-// Softmax-GLA backward on the 5th-generation tensor cores (bf16 I/O, d_k and d_v 128 - or 64, run as 128 with zero padding supplied by the tensor maps -, chunk 64).
+// Softmax-GLA backward on the 5th-generation tensor cores (bf16 I/O, d_k and d_v 128 - or 64: two heads side by side, or one with zero padding supplied by the tensor maps -, chunk 64).
 //
 // The paper states no gradients; these are the chain rule applied to Eq. 4, 12-13, evaluated chunkwise.
 // Two sweeps per (batch, head) sequence, one CTA each, chunk after chunk:

@@ -1,4 +1,4 @@
-// Softmax-RetNet gradient sweep on the 5th-generation tensor cores (bf16 I/O, d_k and d_v 128 - or 64, run as 128 with zero padding
+// Softmax-RetNet gradient sweep on the 5th-generation tensor cores (bf16 I/O, d_k and d_v 128 - or 64: two heads side by side, or one with zero padding
 // supplied by the tensor maps -, chunk 64).  The formulas are Softmax-GLA's (sla_gla_tc_bwd.cu: one CTA per sequence, chunks in
 // reverse, dS in TMEM),
 //     qh_i = f_i q_i, f_i = scale*Gq_i e^{b_i}        kh_j = c_j k_j, c_j = Gk_j e^{-b_j}        dZ = e^{b_last} dS_{n+1}
