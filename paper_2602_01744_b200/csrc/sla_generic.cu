@@ -299,6 +299,7 @@ k_chunk_outer(Dims d, const TIO *__restrict__ x, const TIO *__restrict__ y, cons
     float *Xs = sm;                          // [CMAX][ldx]
     float *Ys = Xs + CMAX * ldx;             // [CMAX][ldv]
     const size_t row_last = tok_row(d, b, t0 + cn - 1, h);
+    copy_rows(Ys, ldv, y, cn, cn, d.dv, tok_row(d, b, t0, h) * d.dv, (size_t)d.H * d.dv);
     struct In { float4 x, b, bl; float g; };
     const int w4 = nr >> 2;
     fill<2>(cn * w4,
@@ -317,7 +318,7 @@ k_chunk_outer(Dims d, const TIO *__restrict__ x, const TIO *__restrict__ y, cons
             const float4 e = GRAD ? v.b : make_float4(v.bl.x - v.b.x, v.bl.y - v.b.y, v.bl.z - v.b.z, v.bl.w - v.b.w);
             stf4(Xs, i * ldx + 4 * (idx - i * w4), make_float4(v.g * v.x.x * expf(e.x), v.g * v.x.y * expf(e.y), v.g * v.x.z * expf(e.z), v.g * v.x.w * expf(e.w)));
         });
-    fill_rows(Ys, ldv, y, cn, cn, d.dv, [&](int i) { return tok_row(d, b, t0 + i, h) * d.dv; });
+    copies_wait();
     __syncthreads();
     const Tile t;
     auto emit = [&](const auto &acc) {
@@ -405,12 +406,12 @@ k_output(Dims d, const TIO *__restrict__ q, const TIO *__restrict__ k, const TIO
     const bool gdn = d.variant == SLA_GDN;
     const Tile t;
 
+    const size_t v0 = tok_row(d, b, t0, h) * d.dv, vs = (size_t)d.H * d.dv;
+    if (gdn) copy_rows(Vs, ldv, Uws, CMAX, cn, d.dv, v0, vs);
+    else copy_rows(Vs, ldv, v, CMAX, cn, d.dv, v0, vs);
+    copy_rows(Ss, ldv, states + state_off(d, bh, n, d.NT + 1), d.dk, d.dk, d.dv, 0, d.dv);
     load_qk_hat(d, q, k, Gq, Gk, bcum, b, h, t0, cn, Qs, Ks, ldk);
-    auto vrow = [&](int i) { return tok_row(d, b, t0 + i, h) * d.dv; };
-    if (gdn) fill_rows(Vs, ldv, Uws, CMAX, cn, d.dv, vrow);
-    else fill_rows(Vs, ldv, v, CMAX, cn, d.dv, vrow);
-    const float *Sg = states + state_off(d, bh, n, d.NT + 1);
-    fill_rows(Ss, ldv, Sg, d.dk, d.dk, d.dv, [&](int i) { return (size_t)i * d.dv; });
+    copies_wait();
     __syncthreads();
     {
         float A[4][4];
@@ -606,12 +607,12 @@ k_grads_lin(Dims d, const TIO *__restrict__ q, const TIO *__restrict__ k, const 
     const Tile t;
     const size_t row_last = tok_row(d, b, t0 + cn - 1, h);
 
-    load_qk_hat(d, q, k, Gq, Gk, bcum, b, h, t0, cn, Qs, Ks, ldk);
-    auto vrow = [&](int i) { return tok_row(d, b, t0 + i, h) * d.dv; };
-    fill_rows(Vs, ldv, v, CMAX, cn, d.dv, vrow);
-    fill_rows(dOs, ldv, dO, CMAX, cn, d.dv, vrow);
-    const float *Sg = states + state_off(d, bh, n, d.NT + 1);
-    fill_rows(Ss, ldv, Sg, d.dk, d.dk, d.dv, [&](int i) { return (size_t)i * d.dv; });
+    const size_t v0 = tok_row(d, b, t0, h) * d.dv, vs = (size_t)d.H * d.dv;
+    copy_rows(Vs, ldv, v, CMAX, cn, d.dv, v0, vs);
+    copy_rows(dOs, ldv, dO, CMAX, cn, d.dv, v0, vs);
+    copy_rows(Ss, ldv, states + state_off(d, bh, n, d.NT + 1), d.dk, d.dk, d.dv, 0, d.dv);
+    load_qk_hat<4>(d, q, k, Gq, Gk, bcum, b, h, t0, cn, Qs, Ks, ldk);
+    copies_wait();
     __syncthreads();
     float A[4][4], dA[4][4];
     zero_acc(A);
