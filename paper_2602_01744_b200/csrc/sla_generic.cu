@@ -450,6 +450,66 @@ k_output(Dims d, const TIO *__restrict__ q, const TIO *__restrict__ k, const TIO
     }
 }
 
+// The same for heads of at most 64 x 64, 512 threads in two groups of 256: the masked product beside qh S, then A V with the contraction
+// halved; the groups' sums meet in shared memory, two row groups each.
+template <typename TIO>
+__global__ void __launch_bounds__(512)
+k_output_narrow(Dims d, const TIO *__restrict__ q, const TIO *__restrict__ k, const TIO *__restrict__ v,
+                const float *__restrict__ Gq, const float *__restrict__ Gk, const float *__restrict__ bcum,
+                const float *__restrict__ states, const float *__restrict__ Uws, TIO *__restrict__ o) {
+    extern __shared__ float sm[];
+    const int n = blockIdx.x, bh = blockIdx.y, b = bh / d.H, h = bh % d.H;
+    const int t0 = n * d.C, cn = min(d.C, d.T - t0), cn4 = (cn + 3) & ~3;
+    const int ldk = pad4(d.dk), ldv = pad4(d.dv);
+    constexpr int lda = pad4(CMAX);
+    float *Qs = sm;
+    float *Ks = Qs + CMAX * ldk;
+    float *Vs = Ks + CMAX * ldk;
+    float *As = Vs + CMAX * ldv;
+    float *Ss = As + CMAX * lda;             // [dk][ldv]
+    float *Xs = Ss + d.dk * ldv;             // [64][lda]: what a group hands the other
+    const int grp = threadIdx.x >> 8;
+    const Tile t(threadIdx.x & 255);
+
+    const size_t v0 = tok_row(d, b, t0, h) * d.dv, vs = (size_t)d.H * d.dv;
+    if (d.variant == SLA_GDN) copy_rows(Vs, ldv, Uws, CMAX, cn, d.dv, v0, vs);
+    else copy_rows(Vs, ldv, v, CMAX, cn, d.dv, v0, vs);
+    copy_rows(Ss, ldv, states + state_off(d, bh, n, d.NT + 1), d.dk, d.dk, d.dv, 0, d.dv);
+    load_qk_hat(d, q, k, Gq, Gk, bcum, b, h, t0, cn, Qs, Ks, ldk);
+    copies_wait();
+    __syncthreads();
+    float acc[4][4];
+    zero_acc(acc);
+    if (grp == 0) {
+        float A[4][4];
+        zero_acc(A);
+        mm_tril(A, t, Qs, ldk, Ks, ldk, d.dk);
+#pragma unroll
+        for (int a = 0; a < 4; ++a) stf4(As, t.row(a) * lda + t.col(0), make_float4(A[a][0], A[a][1], A[a][2], A[a][3]));
+    } else {
+        mm<1, true>(acc, t, Qs, ldk, Ss, ldv, d.dk, d.dv);
+    }
+    __syncthreads();
+    if (grp == 0) {                          // tokens 0 .. 31 of v
+        mm<1, true, 0>(acc, t, As, lda, Vs, ldv, min(cn4, 16), d.dv);
+        if (cn4 > 16) mm<1, true, 1>(acc, t, As + 16, lda, Vs + 16 * ldv, ldv, min(cn4 - 16, 16), d.dv);
+    } else {
+        if (cn4 > 32) mm<1, true, 2>(acc, t, As + 32, lda, Vs + 32 * ldv, ldv, min(cn4 - 32, 16), d.dv);
+        if (cn4 > 48) mm<1, true, 3>(acc, t, As + 48, lda, Vs + 48 * ldv, ldv, cn4 - 48, d.dv);
+    }
+#pragma unroll
+    for (int a = 0; a < 4; ++a)
+        if ((a >> 1) != grp) stf4(Xs, t.row(a) * lda + t.col(0), make_float4(acc[a][0], acc[a][1], acc[a][2], acc[a][3]));
+    __syncthreads();
+#pragma unroll
+    for (int a = 0; a < 4; ++a) {
+        const int i = t.row(a);
+        if ((a >> 1) != grp || i >= cn || t.col(0) >= d.dv) continue;
+        const float4 x = *reinterpret_cast<const float4 *>(Xs + i * lda + t.col(0));
+        stf4(o, tok_row(d, b, t0 + i, h) * d.dv + t.col(0), make_float4(acc[a][0] + x.x, acc[a][1] + x.y, acc[a][2] + x.z, acc[a][3] + x.w));
+    }
+}
+
 // ------------------------------------------------------------------------------------------
 // backward for GDN, state-gradient pass (reverse chunk order).  grid (dv/VS, B*H), 256 threads on a [dk x VS] slice of dS.
 // Stores dS entering each chunk from the right (slot n = gradient w.r.t. the state after chunk n) and
@@ -771,6 +831,186 @@ k_grads_lin(Dims d, const TIO *__restrict__ q, const TIO *__restrict__ k, const 
     }
 }
 
+// The same for heads of at most 64 x 64: everything has room at once, so 512 threads in two groups of 256 take a product of every result
+// each - A beside dA; then dA kh, dA^T qh, A^T dO (triangular: their blocks of zeros are left out) beside dO S^T, V dZ^T, kh dZ -
+// without a barrier in between, and finish two row groups each after one exchange.  k_grads_lin's one group runs through eight phases with
+// eight warps on an SM; what bounds both is the shared-memory pipe and, with so few warps, its latency.  2 x 1000 tokens x 4 heads of 64 (128 chunks): 37 ->
+// 28 us, k_output 15 -> 12.  (The blocks of zeros left out in k_output and k_grads_lin, too: 4 x 2048 tokens x 8 heads of 32 slower by 6 to 10 %, 8 x 2048 x 16
+// of 64 forward 424 -> 409 us, backward 974 -> 1008.)
+template <typename TIO>
+__global__ void __launch_bounds__(512)
+k_grads_narrow(Dims d, const TIO *__restrict__ q, const TIO *__restrict__ k, const TIO *__restrict__ v,
+               const TIO *__restrict__ dO, const float *__restrict__ Gq, const float *__restrict__ Gk,
+               const float *__restrict__ bcum, const float *__restrict__ states,
+               const float *__restrict__ dstates, TIO *__restrict__ dq, TIO *__restrict__ dk,
+               TIO *__restrict__ dv, float *__restrict__ dlog_decay, float *__restrict__ dGq,
+               float *__restrict__ dGk) {
+    extern __shared__ float sm[];
+    const int n = blockIdx.x, bh = blockIdx.y, b = bh / d.H, h = bh % d.H;
+    const int t0 = n * d.C, cn = min(d.C, d.T - t0), cn4 = (cn + 3) & ~3;
+    const int ldk = pad4(d.dk), ldv = pad4(d.dv);
+    constexpr int lda = pad4(CMAX);
+    float *Qs = sm;
+    float *Ks = Qs + CMAX * ldk;
+    float *Vs = Ks + CMAX * ldk;
+    float *dOs = Vs + CMAX * ldv;
+    float *Ss = dOs + CMAX * ldv;             // [dk][ldv]
+    float *Zs = Ss + d.dk * ldv;              // [dk][ldv]: dZ
+    float *Ms = Zs + d.dk * ldv;              // [3][64][lda]: dA, dA^T, A^T; then the exchange of dqh, dkh, dV
+    float *Rs = Ms + 3 * CMAX * lda;          // [dk]
+    float *red = Rs + d.dk;                   // [2][4][CMAX] a token's gate sums, by quarter of the columns
+    const int grp = threadIdx.x >> 8, warp = threadIdx.x >> 5, tx = threadIdx.x & 31;
+    const Tile t(threadIdx.x & 255);
+    const size_t row_last = tok_row(d, b, t0 + cn - 1, h);
+    const bool decay_grad = d.variant == SLA_GLA && dlog_decay;
+
+    const size_t v0 = tok_row(d, b, t0, h) * d.dv, vs = (size_t)d.H * d.dv;
+    copy_rows(Vs, ldv, v, CMAX, cn, d.dv, v0, vs);
+    copy_rows(dOs, ldv, dO, CMAX, cn, d.dv, v0, vs);
+    copy_rows(Ss, ldv, states + state_off(d, bh, n, d.NT + 1), d.dk, d.dk, d.dv, 0, d.dv);
+    load_qk_hat(d, q, k, Gq, Gk, bcum, b, h, t0, cn, Qs, Ks, ldk);
+    {   // Zs <- dZ = diag(exp(b_last)) dS_next ; Rs <- rowsum(dS_next * S_next); half a warp a row
+        const float *dSg = dstates + state_off(d, bh, n, d.NT);
+        const float *Sn = states + state_off(d, bh, n + 1, d.NT + 1);
+        const int j = 4 * (tx & 15);
+#pragma unroll
+        for (int x = 0; x < 2; ++x) {
+            const int r0 = 32 * x + 2 * warp + (tx >> 4);
+            float part = 0.f;
+            if (r0 < d.dk && j < d.dv) {
+                const float e = expf(bcum_at(d, bcum, row_last, r0));
+                const float4 g = ldf4(dSg, (size_t)r0 * d.dv + j);
+                if (decay_grad) {
+                    const float4 y = ldf4(Sn, (size_t)r0 * d.dv + j);
+                    part = fmaf(g.x, y.x, fmaf(g.y, y.y, fmaf(g.z, y.z, g.w * y.w)));
+                }
+                stf4(Zs, r0 * ldv + j, make_float4(e * g.x, e * g.y, e * g.z, e * g.w));
+            }
+            if (decay_grad) {
+#pragma unroll
+                for (int o = 8; o > 0; o >>= 1) part += __shfl_xor_sync(FULL, part, o);
+                if ((tx & 15) == 0 && r0 < d.dk) Rs[r0] = part;
+            }
+        }
+    }
+    copies_wait();
+    __syncthreads();
+    {
+        float A[4][4];                        // A; the second group: dA
+        zero_acc(A);
+        if (grp == 0) mm_tril(A, t, Qs, ldk, Ks, ldk, d.dk);
+        else mm_tril(A, t, dOs, ldv, Vs, ldv, d.dv);
+        float *Mt = Ms + (grp == 0 ? 2 : 1) * CMAX * lda;
+#pragma unroll
+        for (int a = 0; a < 4; ++a) {
+            if (grp) stf4(Ms, t.row(a) * lda + t.col(0), make_float4(A[a][0], A[a][1], A[a][2], A[a][3]));
+#pragma unroll
+            for (int c = 0; c < 4; ++c) Mt[(t.col(0) + c) * lda + t.row(a)] = A[a][c];
+        }
+    }
+    __syncthreads();
+    float acc[3][4][4];                       // this group's half of dqh, dkh, dV
+#pragma unroll
+    for (int x = 0; x < 3; ++x) zero_acc(acc[x]);
+    if (grp == 0) {
+        mm_lower(acc[0], t, Ms, lda, Ks, ldk, cn4, d.dk);
+        mm_upper(acc[1], t, Ms + CMAX * lda, lda, Qs, ldk, cn4, d.dk);
+        mm_upper(acc[2], t, Ms + 2 * CMAX * lda, lda, dOs, ldv, cn4, d.dv);
+    } else {
+        mm<1, false>(acc[0], t, dOs, ldv, Ss, ldv, d.dv, d.dk);
+        mm<1, false>(acc[1], t, Vs, ldv, Zs, ldv, d.dv, d.dk);
+        mm<1, true>(acc[2], t, Ks, ldk, Zs, ldv, d.dk, d.dv);
+    }
+    const int c = t.col(0);
+    struct Raw { float4 q, k, b; float gq, gk; } in[2];      // of the two rows this thread finishes, on their way during the exchange
+#pragma unroll
+    for (int x = 0; x < 2; ++x) {
+        const int i = t.row(0) + 16 * (2 * grp + x);
+        if (i < cn && c < d.dk) {
+            const size_t row = tok_row(d, b, t0 + i, h);
+            in[x].q = ldf4(q, row * d.dk + c);
+            in[x].k = ldf4(k, row * d.dk + c);
+            in[x].b = bcum_at4(d, bcum, row, c);
+            in[x].gq = Gq[row];
+            in[x].gk = Gk[row];
+        }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int x = 0; x < 3; ++x)
+#pragma unroll
+        for (int a = 0; a < 4; ++a)
+            if ((a >> 1) != grp) stf4(Ms, (x * CMAX + t.row(a)) * lda + c, make_float4(acc[x][a][0], acc[x][a][1], acc[x][a][2], acc[x][a][3]));
+    __syncthreads();
+#pragma unroll
+    for (int x = 0; x < 2; ++x) {
+        const int i = t.row(0) + 16 * (2 * grp + x);
+        auto sum = [&](int m) {
+            const float4 y = *reinterpret_cast<const float4 *>(Ms + (m * CMAX + i) * lda + c);
+            const float (&lo)[4] = acc[m][x], (&hi)[4] = acc[m][2 + x];
+            return make_float4((grp ? hi[0] : lo[0]) + y.x, (grp ? hi[1] : lo[1]) + y.y, (grp ? hi[2] : lo[2]) + y.z, (grp ? hi[3] : lo[3]) + y.w);
+        };
+        float sq = 0.f, sk = 0.f;
+        float4 db = make_float4(0.f, 0.f, 0.f, 0.f);
+        const size_t row = i < cn ? tok_row(d, b, t0 + i, h) : 0;
+        if (i < cn && c < d.dk) {
+            const Raw &r = in[x];
+            const float4 yq = sum(0), yk = sum(1);
+            const float4 qh = *reinterpret_cast<const float4 *>(Qs + i * ldk + c), kh = *reinterpret_cast<const float4 *>(Ks + i * ldk + c);
+            db = make_float4(qh.x * yq.x - kh.x * yk.x, qh.y * yq.y - kh.y * yk.y, qh.z * yq.z - kh.z * yk.z, qh.w * yq.w - kh.w * yk.w);
+            const float4 g = make_float4(yq.x * expf(r.b.x), yq.y * expf(r.b.y), yq.z * expf(r.b.z), yq.w * expf(r.b.w));
+            sq = fmaf(d.scale * r.q.x, g.x, fmaf(d.scale * r.q.y, g.y, fmaf(d.scale * r.q.z, g.z, d.scale * r.q.w * g.w)));
+            const float f = d.scale * r.gq;
+            stf4(dq, row * d.dk + c, make_float4(f * g.x, f * g.y, f * g.z, f * g.w));
+            const float4 u = make_float4(yk.x * expf(-r.b.x), yk.y * expf(-r.b.y), yk.z * expf(-r.b.z), yk.w * expf(-r.b.w));
+            sk = fmaf(r.k.x, u.x, fmaf(r.k.y, u.y, fmaf(r.k.z, u.z, r.k.w * u.w)));
+            stf4(dk, row * d.dk + c, make_float4(r.gk * u.x, r.gk * u.y, r.gk * u.z, r.gk * u.w));
+        }
+        if (i < cn && c < d.dv) stf4(dv, row * d.dv + c, sum(2));
+        if (decay_grad && c < d.dk) stf4(Qs, i * ldk + c, db);          // its own elements: nobody else reads them here
+        // a token's sums over this thread's columns -> its quarter's slots (four lanes share a row)
+        sq += __shfl_xor_sync(FULL, sq, 1);
+        sk += __shfl_xor_sync(FULL, sk, 1);
+        sq += __shfl_xor_sync(FULL, sq, 2);
+        sk += __shfl_xor_sync(FULL, sk, 2);
+        if ((tx & 3) == 0) {
+            red[(t.tc >> 2) * CMAX + i] = sq;
+            red[(4 + (t.tc >> 2)) * CMAX + i] = sk;
+        }
+    }
+    __syncthreads();
+    if (threadIdx.x < 2 * CMAX) {     // the gates' gradients: a token's four quarters
+        const int which = threadIdx.x / CMAX, i = threadIdx.x % CMAX;
+        const float *r = red + 4 * which * CMAX + i;
+        if (i < cn) (which ? dGk : dGq)[tok_row(d, b, t0 + i, h)] = (r[0] + r[CMAX]) + (r[2 * CMAX] + r[3 * CMAX]);
+    }
+    if (!decay_grad) return;
+    // warp w the suffix sums of tokens 4w .. 4w+3, the warps' totals over Vs
+    float *tot = Vs;
+    const int e = 4 * tx;
+    float4 x[4], run = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (e < d.dk) {
+#pragma unroll
+        for (int i = 3; i >= 0; --i) {
+            x[i] = *reinterpret_cast<const float4 *>(Qs + (4 * warp + i) * ldk + e);
+            run.x += x[i].x; run.y += x[i].y; run.z += x[i].z; run.w += x[i].w;
+        }
+        stf4(tot, warp * ldk + e, run);
+    }
+    __syncthreads();
+    if (e >= d.dk) return;
+    run = *reinterpret_cast<const float4 *>(Rs + e);
+    for (int g = 15; g > warp; --g) {
+        const float4 y = *reinterpret_cast<const float4 *>(tot + g * ldk + e);
+        run.x += y.x; run.y += y.y; run.z += y.z; run.w += y.w;
+    }
+#pragma unroll
+    for (int i = 3; i >= 0; --i) {
+        run.x += x[i].x; run.y += x[i].y; run.z += x[i].z; run.w += x[i].w;
+        if (4 * warp + i < cn) stf4(dlog_decay, tok_row(d, b, t0 + 4 * warp + i, h) * d.dk + e, run);
+    }
+}
+
 // ------------------------------------------------------------------------------------------
 // host side
 size_t smem_prepare(const Dims &d) {
@@ -782,6 +1022,19 @@ size_t smem_scan(const Dims &d) {
 size_t smem_outer(const Dims &d) { return sizeof(float) * CMAX * (pad4(64) + pad4(d.dv)); }
 size_t smem_output(const Dims &d) {
     return sizeof(float) * (2 * CMAX * pad4(d.dk) + CMAX * pad4(d.dv) + CMAX * pad4(CMAX) + d.dk * pad4(d.dv));
+}
+size_t smem_output_narrow(const Dims &d) { return smem_output(d) + sizeof(float) * CMAX * pad4(CMAX); }
+size_t smem_grads_narrow(const Dims &d) {
+    return sizeof(float) * (2 * CMAX * pad4(d.dk) + 2 * CMAX * pad4(d.dv) + 3 * CMAX * pad4(CMAX) + 2 * d.dk * pad4(d.dv) + d.dk + 8 * CMAX);
+}
+// Heads of at most 64 x 64 on few chunks: no SM gets a second CTA (B x H x chunks, forward and backward, us: 2 x 4 x 16 34.7 and 73.4 -> 33.6 and 67;
+// 4 x 8 x 16 72 and 160 -> 76 and 166, where two CTAs of the general kernels hide one another's phases).
+bool narrow(const Dims &d) {
+    static const int sms = [] {
+        int dev = 0, n = 0;
+        return cudaGetDevice(&dev) == cudaSuccess && cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && n > 0 ? n : 148;
+    }();
+    return d.dk <= 64 && d.dv <= 64 && (long)d.NT * d.B * d.H <= sms;
 }
 size_t smem_dscan(const Dims &d) {
     return sizeof(float) * (3 * CMAX * (d.dk + 1) + 2 * CMAX * VS + CMAX * (CMAX + 1) + d.dk * VS);
@@ -844,7 +1097,8 @@ int forward_t(const Dims &d, const Workspace &w, const FwdArgs &a, bool write_o,
         launches += 2;
     }
     if (write_o) {
-        k_output<TIO><<<tiles, 256, smem_output(d), st>>>(d, q, k, v, Gq, Gk, bcum, states, Uws, (TIO *)a.o);
+        if (narrow(d)) k_output_narrow<TIO><<<tiles, 512, smem_output_narrow(d), st>>>(d, q, k, v, Gq, Gk, bcum, states, Uws, (TIO *)a.o);
+        else k_output<TIO><<<tiles, 256, smem_output(d), st>>>(d, q, k, v, Gq, Gk, bcum, states, Uws, (TIO *)a.o);
         tr.mark("output");
         ++launches;
     }
@@ -872,7 +1126,7 @@ int backward_lin_t(const Dims &d, const Workspace &w, const BwdArgs &a, cudaStre
         tr.mark("chunk_outer");
         ++launches;
     }
-    (d.dk <= 64 && d.dv <= 64 ? k_grads_lin<TIO, 1> : k_grads_lin<TIO, 2>)<<<tiles, 256, smem_grads_lin(d), st>>>(
+    (narrow(d) ? k_grads_narrow<TIO> : d.dk <= 64 && d.dv <= 64 ? k_grads_lin<TIO, 1> : k_grads_lin<TIO, 2>)<<<tiles, narrow(d) ? 512 : 256, narrow(d) ? smem_grads_narrow(d) : smem_grads_lin(d), st>>>(
         d, q, k, v, dO, Gq, Gk, bcum, states, dstates, (TIO *)a.dq, (TIO *)a.dk, (TIO *)a.dv, a.dlog_decay, dGq, dGk);
     tr.mark("grads_lin");
     ++launches;
@@ -890,6 +1144,8 @@ template <typename TIO> bool configure_t() {
           set_smem(k_chunk_outer<TIO, true, true>, smem_outer(d));
     ok &= set_smem(k_dstate_scan<TIO>, smem_dscan(d));
     ok &= set_smem(k_grads_lin<TIO, 1>, smem_grads_lin(d)) && set_smem(k_grads_lin<TIO, 2>, smem_grads_lin(d));
+    d.dk = d.dv = 64;
+    ok &= set_smem(k_output_narrow<TIO>, smem_output_narrow(d)) && set_smem(k_grads_narrow<TIO>, smem_grads_narrow(d));
     return ok;
 }
 

@@ -76,8 +76,8 @@ __device__ __forceinline__ void tile_gemm(float (&acc)[8][NB], const float *A, i
 __host__ __device__ constexpr int pad4(int width) { return width + 4; }
 struct Tile {
     int tr, tc;
-    __device__ __forceinline__ Tile() {
-        const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    __device__ __forceinline__ explicit Tile(int tid = threadIdx.x) {
+        const int w = tid >> 5, lane = tid & 31;
         tr = (lane >> 2) + 8 * (w & 1);
         tc = (lane & 3) + 4 * (w >> 1);
     }
@@ -85,13 +85,14 @@ struct Tile {
     __device__ __forceinline__ int col(int blk) const { return 64 * blk + 4 * tc; }
 };
 // acc += A[i][k] B: A has its rows along k.  BT: B[k][j], else B[j][k].  K a multiple of four (rows past the last token are zero).
-template <int NB, bool BT>
+// Only the row groups a = A0 .. A1 - 1 (rows 16 A0 .. 16 A1 - 1) where A is triangular, see mm_lower, mm_upper.
+template <int NB, bool BT, int A0 = 0, int A1 = 4>
 __device__ __forceinline__ void mm(float (&acc)[4][4 * NB], const Tile &t, const float *A, int lda, const float *B, int ldb, int K, int N) {
 #pragma unroll 2
     for (int k = 0; k < K; k += 4) {
         float4 a[4];
 #pragma unroll
-        for (int x = 0; x < 4; ++x) a[x] = *reinterpret_cast<const float4 *>(A + t.row(x) * lda + k);
+        for (int x = A0; x < A1; ++x) a[x] = *reinterpret_cast<const float4 *>(A + t.row(x) * lda + k);
 #pragma unroll
         for (int blk = 0; blk < NB; ++blk) {
             if (t.col(blk) >= N) continue;
@@ -100,7 +101,7 @@ __device__ __forceinline__ void mm(float (&acc)[4][4 * NB], const Tile &t, const
             for (int y = 0; y < 4; ++y)
                 b[y] = *reinterpret_cast<const float4 *>(BT ? B + (k + y) * ldb + t.col(blk) : B + (t.col(blk) + y) * ldb + k);
 #pragma unroll
-            for (int x = 0; x < 4; ++x)
+            for (int x = A0; x < A1; ++x)
 #pragma unroll
                 for (int y = 0; y < 4; ++y) {
                     float &c = acc[x][4 * blk + y];
@@ -114,6 +115,33 @@ __device__ __forceinline__ void mm(float (&acc)[4][4 * NB], const Tile &t, const
                 }
         }
     }
+}
+// acc += A B with A lower (upper) triangular [64][64], K of its columns and of B's rows: the 16 x 16 blocks of zeros are left out.
+template <int S = 0>
+__device__ __forceinline__ void mm_lower(float (&acc)[4][4], const Tile &t, const float *A, int lda, const float *B, int ldb, int K, int N) {
+    if (K <= 16 * S) return;
+    mm<1, true, S, 4>(acc, t, A + 16 * S, lda, B + 16 * S * ldb, ldb, min(K - 16 * S, 16), N);
+    if constexpr (S < 3) mm_lower<S + 1>(acc, t, A, lda, B, ldb, K, N);
+}
+template <int S = 0>
+__device__ __forceinline__ void mm_upper(float (&acc)[4][4], const Tile &t, const float *A, int lda, const float *B, int ldb, int K, int N) {
+    if (K <= 16 * S) return;
+    mm<1, true, 0, S + 1>(acc, t, A + 16 * S, lda, B + 16 * S * ldb, ldb, min(K - 16 * S, 16), N);
+    if constexpr (S < 3) mm_upper<S + 1>(acc, t, A, lda, B, ldb, K, N);
+}
+// acc = tril(X Y^T), 64 x 64: a warp's 16 columns meet the row groups from its own on
+__device__ __forceinline__ void mm_tril(float (&acc)[4][4], const Tile &t, const float *X, int ldx, const float *Y, int ldy, int K) {
+    switch (t.tc >> 2) {
+        case 0: mm<1, false, 0>(acc, t, X, ldx, Y, ldy, K, CMAX); break;
+        case 1: mm<1, false, 1>(acc, t, X, ldx, Y, ldy, K, CMAX); break;
+        case 2: mm<1, false, 2>(acc, t, X, ldx, Y, ldy, K, CMAX); break;
+        default: mm<1, false, 3>(acc, t, X, ldx, Y, ldy, K, CMAX);
+    }
+#pragma unroll
+    for (int a = 0; a < 4; ++a)
+#pragma unroll
+        for (int c = 0; c < 4; ++c)
+            if (t.col(0) + c > t.row(a)) acc[a][c] = 0.f;
 }
 // acc += X^T Y over the tokens: X[k][i], Y[k][j]; thread (tr, tc) owns rows 4 tr + a instead.
 template <int NB>
