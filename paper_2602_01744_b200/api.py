@@ -168,6 +168,7 @@ class Plan:
         self.io_torch = torch.bfloat16 if self.desc.io_dtype == SLA_BF16 else torch.float32
         self.heads, self.width_v = self.desc.H, self.desc.d_v
         self._bf16 = int(self.desc.io_dtype == SLA_BF16)
+        self._packed = False
         self._slots = B * (-(-T // chunk) + 1)                 # chunks and one more, over the sequences
 
     def close(self):
@@ -192,6 +193,7 @@ class Plan:
         _check("sla_plan_workspace_bytes", lib().sla_plan_workspace_bytes(self.handle, ctypes.byref(f), ctypes.byref(b)))
         self.forward_workspace_bytes, self.backward_workspace_bytes = f.value, b.value
         self.n_seq = n
+        self._packed = n > 0
         lens = [b - a for a, b in zip(cu, cu[1:])] or [self.desc.T] * self.desc.B
         self._slots = sum(-(-t // self.desc.chunk) + 1 for t in lens)
 
@@ -227,17 +229,18 @@ class Plan:
 
     def scratch(self, backward, device):
         """The workspace of a call that brings none.  Where memory is too short for the fast Softmax-GatedDeltaNet kernels' (130 or 34 KiB a
-        chunk and head), the least that sla_plan_workspace_bytes documents: 56 KiB and the gate sums, or nothing."""
+        chunk and head), or for a packed Softmax-GLA or -RetNet batch with its long sequences cut, the least that
+        sla_plan_workspace_bytes documents: 56 or 32 KiB and the gate sums, or nothing."""
         try:
             return self.workspace(backward, device)
         except torch.OutOfMemoryError:
             d = self.desc
-            if (d.variant != SLA_GDN or d.io_dtype != SLA_BF16 or d.flags & SLA_FLAG_FORCE_GENERIC or d.chunk != 64
+            if ((d.variant != SLA_GDN and not self._packed) or d.io_dtype != SLA_BF16 or d.flags & SLA_FLAG_FORCE_GENERIC or d.chunk != 64
                     or not {d.d_k, d.d_v} <= {64, 128}):
                 raise
             n = 0
             if backward or d.flags & SLA_FLAG_SAVE_FOR_BACKWARD:
-                n = self._slots * d.H * (56 << 10) + 2 * ((d.B * d.T * d.H * 4 + 255) // 256 * 256)
+                n = self._slots * d.H * ((56 if d.variant == SLA_GDN else 32) << 10) + 2 * ((d.B * d.T * d.H * 4 + 255) // 256 * 256)
             if n >= (self.backward_workspace_bytes if backward else self.forward_workspace_bytes):
                 raise
             return torch.empty(max(n, 16), dtype=torch.uint8, device=device)

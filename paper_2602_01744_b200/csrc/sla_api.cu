@@ -74,10 +74,15 @@ static void plan_workspace_sizes(sla_plan *p) {
     const bool generic = p->flags & SLA_FLAG_FORCE_GENERIC;
     p->fwd_bytes = p->ws.fwd_floats * sizeof(float);
     p->bwd_bytes = p->ws.bwd_floats * sizeof(float);
+    size_t cut_fwd = 0, cut_bwd = 0;                 // a packed batch with cut sequences: what is asked for; with less it runs uncut
     if (sla::gla_tc_supported(d) && !generic) {
         p->fwd_bytes = sla::gla_tc_forward_workspace_bytes(d, &p->varlen);
         p->bwd_bytes = (!p->varlen.n_seq && p->segs.n_seq) ? sla::gla_tc_backward_segmented_workspace_bytes(d, p->segs)
                                                            : sla::gla_tc_backward_workspace_bytes(d, &p->varlen);
+        if (p->cut.n_seq) {
+            cut_bwd = sla::gla_tc_backward_workspace_bytes(d, &p->cut);
+            cut_fwd = (p->flags & SLA_FLAG_SAVE_FOR_BACKWARD) ? cut_bwd : p->cut.fwd ? sla::gla_tc_forward_workspace_bytes(d, &p->cut) : 0;
+        }
     }
     if (sla::gdn_tc_supported(d) && !generic) {
         p->fwd_bytes = sla::gdn_tc_forward_workspace_bytes(d, &p->varlen);
@@ -87,6 +92,10 @@ static void plan_workspace_sizes(sla_plan *p) {
         p->fwd_bytes = p->bwd_bytes;     // the forward writes into the backward pass's workspace layout
     p->fwd_least = p->fwd_bytes;
     p->bwd_least = p->bwd_bytes;
+    if (cut_bwd) {
+        p->fwd_bytes = cut_fwd;
+        p->bwd_bytes = cut_bwd;
+    }
     if (sla::gdn_tc_supported(d) && !generic) {      // its one-CTA kernels keep smaller records, and none in a forward pass alone
         p->bwd_least = sla::gdn_tc_one_cta_workspace_bytes(d, &p->varlen);
         p->fwd_least = (p->flags & SLA_FLAG_SAVE_FOR_BACKWARD) ? p->bwd_least : 0;
@@ -95,6 +104,7 @@ static void plan_workspace_sizes(sla_plan *p) {
 
 static void varlen_release(sla::Varlen &v) {
     if (v.d_seqs) cudaFree(v.d_seqs);
+    if (v.d_cut) cudaFree(v.d_cut);
     for (auto &g : v.reg) {
         if (g.dev) cudaFree(g.dev);
         if (g.host) cudaFreeHost(g.host);
@@ -109,6 +119,9 @@ static bool varlen_to_device(sla::Varlen &v) {
     const int n_seq = v.n_seq;
     bool ok = cudaMalloc((void **)&v.d_seqs, sizeof(sla::SeqInfo) * n_seq) == cudaSuccess &&
               cudaMemcpy(v.d_seqs, v.seqs.data(), sizeof(sla::SeqInfo) * n_seq, cudaMemcpyHostToDevice) == cudaSuccess;
+    if (!v.cut.empty())
+        ok = ok && cudaMalloc((void **)&v.d_cut, sizeof(int) * v.cut.size()) == cudaSuccess &&
+             cudaMemcpy(v.d_cut, v.cut.data(), sizeof(int) * v.cut.size(), cudaMemcpyHostToDevice) == cudaSuccess;
     const size_t mb = (size_t)n_seq * sla::Varlen::MAPS_PER_SEQ * sizeof(CUtensorMap);
     for (auto &g : v.reg)
         ok = ok && cudaMalloc((void **)&g.dev, mb) == cudaSuccess && cudaMallocHost((void **)&g.host, mb) == cudaSuccess &&
@@ -198,6 +211,7 @@ sla_status sla_plan_destroy(sla_plan *plan) {
     if (!plan) return SLA_OK;
     if (plan->d_status) cudaFree(plan->d_status);
     varlen_release(plan->varlen);
+    varlen_release(plan->cut);
     varlen_release(plan->segs);
     plan->tracer.destroy();
     delete plan;
@@ -209,6 +223,7 @@ sla_status sla_plan_set_sequences(sla_plan *plan, const int32_t *cu_seqlens, int
     const sla::Dims &d = plan->dims;
     plan->saved.valid = false;
     varlen_release(plan->varlen);
+    varlen_release(plan->cut);
     if (n_seq == 0) {
         plan_workspace_sizes(plan);
         return SLA_OK;
@@ -232,8 +247,10 @@ sla_status sla_plan_set_sequences(sla_plan *plan, const int32_t *cu_seqlens, int
     }
     v.slots = slots;
     v.n_seq = n_seq;
-    if (!varlen_to_device(v)) {
+    if (sla::gla_tc_supported(d)) sla::gla_tc_cut_sequences(d, v, plan->cut);
+    if (!varlen_to_device(v) || (plan->cut.n_seq && !varlen_to_device(plan->cut))) {
         varlen_release(v);
+        varlen_release(plan->cut);
         plan_workspace_sizes(plan);
         return sla::cuda_error();
     }
@@ -333,6 +350,11 @@ sla_status sla_forward(sla_plan *plan, const void *q, const void *k, const void 
     // given the backward pass's: scratch of the forward's own size may be gone, and its place taken, by the time of the backward.
     const bool kept = (plan->flags & SLA_FLAG_SAVE_FOR_BACKWARD) && !on_tensor_cores(*plan) && workspace_bytes >= plan->bwd_bytes;
     bool chunked = !generic && sla::gdn_tc_supported(d) && sla::gdn_tc_chunked(d, &plan->varlen, save, workspace_bytes);
+    if (!generic && sla::gla_tc_supported(d)) {
+        // (the state a sequence starts from and its final one in one buffer: a cut sequence's last segment may be done before its first begins)
+        if (plan->cut.fwd && workspace_bytes >= plan->fwd_bytes && !(ht && ht == h0)) a.vl = &plan->cut;
+        chunked = sla::gla_tc_pairs(d, a.vl);
+    }
     plan->saved.valid = false;
     int n = (!generic && sla::gla_tc_supported(d))
                 ? sla::gla_tc_forward(d, a, save ? sla::gla_tc_state_images(a.ws) : nullptr, plan->d_status,
@@ -391,13 +413,17 @@ sla_status sla_backward(sla_plan *plan, const void *q, const void *k, const void
     // the states (GLA) or per-chunk records (GDN) are taken from the workspace only if the last sla_forward of this plan
     // left them there for exactly these inputs, on this stream; anything else recomputes them
     bool chunked = !generic && sla::gdn_tc_supported(d) && sla::gdn_tc_chunked(d, &plan->varlen, true, workspace_bytes);
+    if (!generic && sla::gla_tc_supported(d)) {
+        if (plan->cut.n_seq && workspace_bytes >= plan->bwd_bytes && !(dh0 && dh0 == dht)) a.vl = &plan->cut;
+        chunked = sla::gla_tc_pairs(d, a.vl);
+    }
     sla_plan::Saved &sv = plan->saved;
     const bool have = sv.valid && sv.chunked == chunked && sv.ws == workspace && sv.q == q && sv.k == k && sv.v == v && sv.log_decay == log_decay &&
                       sv.beta == beta && sv.lq == gq_logits && sv.lk == gk_logits && sv.h0 == h0 && sv.stream == cuda_stream;
     // a backward pass that recomputes writes its own states into `workspace`: whatever an earlier forward left there
     // (for other inputs) is gone, and must not be taken for valid by a later call
     if (!have && sv.ws == workspace) sv.valid = false;
-    const bool chunked_records = have && chunked;
+    const bool chunked_records = have && chunked && sla::gdn_tc_supported(d);
     int n = (!generic && sla::gla_tc_supported(d) && !a.vl && plan->segs.n_seq)
                 ? sla::gla_tc_backward_segmented(d, a, plan->segs, plan->d_status, (cudaStream_t)cuda_stream, plan->tracer)
             : (!generic && sla::gla_tc_supported(d))

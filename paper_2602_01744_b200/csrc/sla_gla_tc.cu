@@ -68,6 +68,7 @@ struct FwdParams {
     const SeqInfo *seqs;            // packed variable-length batch: per-sequence table and tensor maps (q, k, v, g, o), else nullptr
     const CUtensorMap *vmaps;
     int dk, dv;             // head widths, each 128 or 64 (the upper half of a 128-wide tile is then zero padding)
+    const float *edge = nullptr;    // packed batch with cut sequences: the states segments with a left neighbour start from, by id
 };
 
 // One CTA per (batch, head) sequence, five roles that only meet on mbarriers:
@@ -100,16 +101,15 @@ k_gla_fwd_tc(const __grid_constant__ CUtensorMap gm_q, const __grid_constant__ C
     const int bh = b * p.H + h * HPC;                       // the (first) head among all (sequence, head)
     // A packed batch: this CTA's sequence has its own length, chunk count, first token, state slots and tensor maps
     // (based at its first token, so token coordinates stay relative and the batch coordinate is 0).
-    size_t tokb = (size_t)b * p.T, slot = (size_t)bh * (p.NT + 1);
-    size_t sbh = (size_t)bh;                                // (sequence, head) index into h0 / ht / dht / dh0
+    // The roles that need more of its entry read it where they use it: kept from here on it costs registers (4 x 2048 tokens x 8 heads, which
+    // has no table, 43.4 -> 45.0 us a call).
+    size_t tokb = (size_t)b * p.T;
     const CUtensorMap *vm = nullptr;
     if (p.seqs) {
-        const SeqInfo si = p.seqs[b];
+        const SeqInfo &si = p.seqs[b];
         vm = p.vmaps + (size_t)b * Varlen::MAPS_PER_SEQ;
         p.T = si.T; p.NT = si.NT; p.L = si.NT;
         tokb = (size_t)si.t0;
-        slot = (size_t)si.slot0 * p.H + (size_t)h * HPC * (si.NT + 1);
-        sbh = (size_t)si.id * p.H + h * HPC;                      // (the table is ordered longest first, the state tensors as the caller gave them)
         b = 0;
     }
     const CUtensorMap &tm_q = vm ? vm[0] : gm_q, &tm_k = vm ? vm[1] : gm_k, &tm_v = vm ? vm[2] : gm_v,
@@ -234,16 +234,24 @@ k_gla_fwd_tc(const __grid_constant__ CUtensorMap gm_q, const __grid_constant__ C
                 mbar_expect_tx(bf, TILE_BF16);
                 tma_load_5d(dst, &tm_v, 0, (n0 + n) * C, 0, h, b, bf);
             };
+            int last_img = NT;
+            size_t slot = (size_t)bh * (p.NT + 1), img_n0 = 0;
+            if (p.seqs) {
+                const SeqInfo &si = p.seqs[cta / hg];
+                slot = (size_t)si.slot0 * p.H + (size_t)h * HPC * (si.img_NT + 1);
+                img_n0 = si.img_n0;
+                if (si.ht_id < 0) last_img = NT - 1;        // (its right neighbour leaves the image between them)
+            }
             // save mode: S_m (the bf16 operand copy, as it stands in shared memory) -> image slot m, for the backward pass
-            uint8_t *img0 = p.simg ? p.simg + slot * STATE_BF16 : nullptr;
+            uint8_t *img0 = p.simg ? p.simg + slot * STATE_BF16 + img_n0 * (PAIR ? PAIR_STATE : STATE_BF16) : nullptr;
             for (int n = 0; n < 3 && n < NT; ++n) load_qk(n);
             for (int n = 0; n < 2 && n < NT; ++n) load_v(n);
             // From here on the lane serves whichever buffer falls free or fills first (no fixed order: the prologue warps
             // run ahead of the tensor core by a varying distance).  Next chunk to load / store per stream:
-            int nqk = 3, nv = 2, nst = 0, nsv = img0 ? 0 : NT + 1;
+            int nqk = 3, nv = 2, nst = 0, nsv = img0 ? 0 : last_img + 1;
             auto ready = [&](int i, uint32_t parity) { return mbar_test_wait(bar(i), parity) != 0; };
             uint64_t t_idle = globaltimer_ns();
-            for (uint32_t it = 0; !failed && (nst < NT || nsv <= NT); ++it) {
+            for (uint32_t it = 0; !failed && (nst < NT || nsv <= last_img); ++it) {
                 bool progress = false;
                 if (nqk < NT && ready(QKFREE + nqk % 3, ((nqk - 3) / 3) & 1)) { // A, qh S and kh^T V of chunk nqk-3 have read it
                     load_qk(nqk++);
@@ -253,7 +261,7 @@ k_gla_fwd_tc(const __grid_constant__ CUtensorMap gm_q, const __grid_constant__ C
                     load_v(nv++);
                     progress = true;
                 }
-                if (nsv <= NT && ready(SREADY, nsv & 1)) {                       // S_nsv stands in shared memory
+                if (nsv <= last_img && ready(SREADY, nsv & 1)) {                       // S_nsv stands in shared memory
                     if (PAIR) {
                         bulk_store(img0 + (size_t)nsv * PAIR_STATE, base + OFF_S + pair_block(0), STATE_BLOCK);
                         bulk_store(img0 + (size_t)nsv * PAIR_STATE + STATE_BLOCK, base + OFF_S + pair_block(1), STATE_BLOCK);
@@ -345,7 +353,14 @@ k_gla_fwd_tc(const __grid_constant__ CUtensorMap gm_q, const __grid_constant__ C
         {   // initial state: fp32 into TMEM, bf16 copy into shared memory (row = key dimension).  A segment that is not the
             // first starts from S <- diag(gam_s) S + fin_s taken over the segments s before it (a short scan over their
             // summaries, elementwise, done here rather than in a launch of its own).
-            const float *src = PAIR ? pair_state_row(p.h0, sbh, row, colhalf) : state_row(p.h0, sbh, row, colhalf, p.dk, p.dv);
+            size_t sbh = (size_t)bh;                        // (the table is ordered longest first, the state tensors as the caller gave them)
+            const float *h0 = p.h0;
+            if (p.seqs) {
+                const SeqInfo &si = p.seqs[cta / hg];
+                if (si.dh0_id < 0) h0 = p.edge;
+                sbh = (size_t)(si.dh0_id < 0 ? si.id : si.dh0_id) * p.H + h * HPC;
+            }
+            const float *src = PAIR ? pair_state_row(h0, sbh, row, colhalf) : state_row(h0, sbh, row, colhalf, p.dk, p.dv);
             if (!PAIR && p.P > 1) grid_dependency_wait();
 #pragma unroll
             for (int part = 0; part < 2; ++part) {
@@ -467,8 +482,15 @@ k_gla_fwd_tc(const __grid_constant__ CUtensorMap gm_q, const __grid_constant__ C
             stage_o(n);                                // ... and this chunk's output
         }
 
-        if (PAIR && p.ht) {
-            float *dst = pair_state_row(p.ht, sbh, row, colhalf);
+        size_t hbh = (size_t)bh;
+        bool leaves = p.ht && seg == p.P - 1;               // a final state
+        if (p.seqs && leaves) {
+            const int id = p.seqs[cta / hg].ht_id;
+            leaves = id >= 0;
+            hbh = (size_t)max(id, 0) * p.H + h * HPC;
+        }
+        if (PAIR && leaves) {
+            float *dst = pair_state_row(p.ht, hbh, row, colhalf);
             if (holds)
 #pragma unroll
                 for (int part = 0; part < 2; ++part) {
@@ -479,7 +501,7 @@ k_gla_fwd_tc(const __grid_constant__ CUtensorMap gm_q, const __grid_constant__ C
                     for (int j = 0; j < 32; j += 4) *reinterpret_cast<float4 *>(dst + 32 * part + j) = make_float4(v[j], v[j + 1], v[j + 2], v[j + 3]);
                 }
         }
-        if (!PAIR && p.ht && seg == p.P - 1) {   // final state, fp32 (each thread reads back what it wrote in the last rescale)
+        if (!PAIR && leaves) {   // final state, fp32 (each thread reads back what it wrote in the last rescale)
             // through shared memory (every product of the CTA has been read out, the q, k buffers are free), so that a warp writes
             // whole rows (4 x 2048 tokens x 8 heads: 46.4 -> 43.6 us a call)
             const uint32_t R = OFF_QK + row * (D * 4);
@@ -494,7 +516,7 @@ k_gla_fwd_tc(const __grid_constant__ CUtensorMap gm_q, const __grid_constant__ C
                         make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
             }
             named_bar_sync(1, NCOMPUTE);
-            float *dst = p.ht + sbh * p.dk * p.dv + 4 * lane;
+            float *dst = p.ht + hbh * p.dk * p.dv + 4 * lane;
             if (4 * lane < p.dv)
                 for (int r = warp; r < p.dk; r += NCOMPUTE / 32)
                     *reinterpret_cast<float4 *>(dst + (size_t)r * p.dv) = *reinterpret_cast<const float4 *>(sm + OFF_QK + r * (D * 4) + ((lane ^ (r & 31)) << 4));
@@ -552,10 +574,11 @@ int gla_tc_configure() {
 // run at once.  Where one long sequence of a packed batch is what a call lasts they would lose: a sequence of 4000 tokens beside 17 of 256, 32 heads,
 // step 567 us single, 585 in pairs.  Both are estimated in chunk times: the longest sequence, or what an SM gets where there are more
 // CTAs than SMs (equal sequences: whole waves of them).
+constexpr double PAIR_CHUNK = 1.1;
 bool gla_tc_pairs(const Dims &d, const Varlen *vl) {
     if (d.dk != 64 || d.dv != 64 || d.H % 2) return false;
-    constexpr double PAIR_CHUNK = 1.1;
     const double sms = sm_count();
+    if (vl && vl->n_of && !vl->fwd) vl = vl->whole;         // (the form in which the forward pass leaves the state images)
     auto lasts = [&](long heads) {
         if (!(vl && vl->n_seq)) return std::ceil(d.B * heads / sms) * d.NT;
         long chunks = 0, longest = 0;
@@ -568,6 +591,64 @@ bool gla_tc_pairs(const Dims &d, const Varlen *vl) {
     return PAIR_CHUNK * lasts(d.H / 2) < lasts(d.H);
 }
 
+// A packed batch lasts as long as its longest sequence's chain of chunks, or what an SM gets.  Cut into segments the chain gets shorter, for a
+// pass over the cut sequences' k, v and decay beside the forward pass (the state every segment starts from) and one over q, dO and decay beside
+// the backward pass, each with a fold over its results.  Estimated in chunk times of the pass (2.1 us forward, 6.6 backward, one CTA an SM): an SM that gets
+// work all the time takes 1.2 times as long a chunk as a chain by itself, a chunk of the first pass 0.8 of a forward one, of the second 0.33 of a backward
+// one, launches and first loads 7 and 4, a segment's states 2.5 and 0.8 in what all SMs together move.  Against measured calls (T x heads of 128, longest
+// sequence; forward, and backward with gates: before -> cut, us): 8192 x 8, 4880 tokens 161 -> 56, 449 -> 100; 4096 x 16, 1695 64.5 -> 60.3, 173 -> 108;
+// 32768 x 16, 11120 372 -> 303, 1013 -> 635; 16384 x 16, 3167 119 -> 136 (not taken), 323 -> 269.  Segments have at least 8 chunks.
+void gla_tc_cut_sequences(const Dims &d, Varlen &vl, Varlen &cut) {
+    const double sms = sm_count(), size = d.dk * d.dv / (double)(D * D);
+    long longest = 0;
+    for (const SeqInfo &s : vl.seqs) longest = std::max<long>(longest, s.NT);
+    if (longest < 16) return;
+    const int whole_hpc = gla_tc_pairs(d, &vl) ? 2 : 1;
+    auto lasts = [&](long L, int hpc, double pass, double fixed, double edge) {     // sequences longer than L in equal segments, hpc heads a CTA
+        double chunks = 0, cut_chunks = 0, top = 0, cut_top = 0, segs = 0;
+        const double heads = (double)d.H / hpc;
+        for (const SeqInfo &s : vl.seqs) {
+            const long n = (s.NT + L - 1) / L, len = (s.NT + n - 1) / n;
+            chunks += s.NT;
+            top = std::max<double>(top, len);
+            if (n > 1) { cut_chunks += s.NT; cut_top = std::max<double>(cut_top, len); segs += n; }
+        }
+        const double all = std::max(top, 1.2 * chunks * heads / sms), chunk = hpc == 2 ? PAIR_CHUNK : 1;
+        return segs > 0 ? chunk * (all + pass * std::max(cut_top, 1.2 * cut_chunks * heads / sms)) + fixed + edge * size * segs * d.H / sms : chunk * all;
+    };
+    const double whole = lasts(longest, whole_hpc, 0, 0, 0);
+    double best = 0.95 * whole;
+    long best_L = 0;
+    for (int hpc = whole_hpc; hpc <= (d.dk == 64 && d.dv == 64 && d.H % 2 == 0 ? 2 : 1); ++hpc)
+        for (long P = 2; P <= 64 && (longest + P - 1) / P >= 8; ++P) {
+            const long L = (longest + P - 1) / P;
+            const bool fwd = lasts(L, hpc, 0.8, 7, 2.5) < whole;
+            const double t = lasts(L, hpc, 0.33, 4, 0.8);
+            if (t < best && (fwd || hpc == whole_hpc)) { best = t; best_L = L; cut.fwd = fwd; }     // (a whole forward pass decides on the pairs)
+        }
+    if (!best_L) return;
+    cut.whole = &vl;
+    std::vector<SeqInfo> by_id(vl.seqs);
+    std::sort(by_id.begin(), by_id.end(), [](const SeqInfo &a, const SeqInfo &b) { return a.id < b.id; });
+    for (const SeqInfo &s : by_id) {
+        cut.cut.push_back((int)cut.seqs.size());
+        const int n = (int)((s.NT + best_L - 1) / best_L), len = (s.NT + n - 1) / n;
+        for (int t0 = 0; t0 < s.T; t0 += len * C) {
+            const int T = std::min(len * C, s.T - t0), id = (int)cut.seqs.size();
+            cut.seqs.push_back({s.t0 + t0, T, (T + C - 1) / C, s.slot0, id, t0 + T == s.T ? s.id : -1, t0 == 0 ? s.id : -1, s.NT, t0 / C});
+        }
+    }
+    cut.cut.push_back((int)cut.seqs.size());
+    std::stable_sort(cut.seqs.begin(), cut.seqs.end(), [](const SeqInfo &a, const SeqInfo &b) { return a.NT > b.NT; });
+    cut.slots = vl.slots;
+    cut.n_of = (int)by_id.size();
+    cut.n_seq = (int)cut.seqs.size();
+    for (int i = 0; i < cut.n_seq; ++i)
+        if (cut.seqs[i].ht_id < 0) { cut.cut.push_back(i); ++cut.n_left; }
+    for (int i = 0; i < cut.n_seq; ++i)
+        if (cut.seqs[i].dh0_id < 0) { cut.cut.push_back(i); ++cut.n_right; }
+}
+
 // The backward runs the gradient sweep twice when it is cut into segments (once for the state gradients that leave
 // each segment, once for the results), so cutting pays only from three segments per sequence on.
 void gla_tc_backward_choose_segments(const Dims &d, int &P, int &L) {
@@ -576,14 +657,15 @@ void gla_tc_backward_choose_segments(const Dims &d, int &P, int &L) {
 }
 
 size_t gla_tc_forward_workspace_bytes(const Dims &d, const Varlen *vl) {
+    if (vl && vl->n_seq) return vl->n_of ? gla_tc_cut_floats(d, *vl) * sizeof(float) : 0;
     int P, L;
     choose_segments(d, P, L);
-    if (P == 1 || (vl && vl->n_seq)) return 0;
+    if (P == 1) return 0;
     return (size_t)d.B * d.H * P * (D * D + D) * sizeof(float);
 }
 
 bool gla_tc_forward_can_save(const Dims &d, const Varlen *vl) {
-    if (vl && vl->n_seq) return true;     // (a packed batch always runs one CTA per sequence)
+    if (vl && vl->n_seq) return true;     // (its images are those of whole sequences, cut or not)
     int P, L;
     choose_segments(d, P, L);
     return P == 1;
@@ -607,11 +689,13 @@ int gla_tc_forward(const Dims &d, const FwdArgs &a, uint8_t *simg, int *status, 
             return make_map(m + 3, a.log_decay + tok * dk, 1, si.T, H, dk, true, 128);
         });
         if (!vm || !make_tile_map(&mq, a.q, d.B, d.T, H, dk)) return -1;
+        const float *edge = nullptr;
+        if (a.vl->n_of && !(edge = gla_tc_cut_starts(d, a, a.ws + (simg ? gla_tc_images_floats(d, a.vl) : 0), status, st, tr))) return -1;
         FwdParams p{a.lq, a.lk, a.h0, nullptr, nullptr, (__nv_bfloat16 *)a.o, a.ht, simg, status, d.T, d.H, d.NT, 1, d.NT, d.scale,
-                    retnet ? a.log_decay : nullptr, a.vl->d_seqs, vm, d.dk, d.dv};
+                    retnet ? a.log_decay : nullptr, a.vl->d_seqs, vm, d.dk, d.dv, edge};
         kernel<<<a.vl->n_seq * H, NTHREADS, SMEM_BYTES, st>>>(mq, mq, mq, mq, mq, p);
         tr.mark("gla_fwd_tc");
-        return cudaGetLastError() == cudaSuccess ? 1 : -1;
+        return cudaGetLastError() == cudaSuccess ? (a.vl->n_of ? 3 : 1) : -1;
     }
     if (!make_tile_map(&mq, a.q, d.B, d.T, H, dk) || !make_tile_map(&mk, a.k, d.B, d.T, H, dk) ||
         !make_tile_map(&mv, a.v, d.B, d.T, H, dv) || !make_tile_map(&mo, a.o, d.B, d.T, H, dv))

@@ -195,8 +195,9 @@ constexpr uint32_t TOT_BYTES = 8 * D * 4;
 // bytes of each of eight rows at once, which without the swizzle all sit in the same banks
 __device__ __forceinline__ uint32_t e2_off(uint32_t row, uint32_t chunk) { return row * (D * 4) + ((chunk ^ ((row & 3) << 1)) << 4); }
 struct NoHook { __device__ __forceinline__ void operator()() const {} };
+// POS: k_i * gk_i * 2^{+b_i} instead (the reverse summaries, whose tile is q).
 // gate_half: distance between the gates of columns 0..63 and those of columns 64..127 (a pair of heads; 0: one head).
-template <bool WITH_Q, bool WITH_E, class Hook = NoHook>
+template <bool WITH_Q, bool WITH_E, class Hook = NoHook, bool POS = false>
 __device__ __forceinline__ void chunk_prologue(uint8_t *q_tile, uint8_t *k_tile, const float *gs, float *tot,
                                                const float *gq_s, const float *gk_s, float *eblast,
                                                uint8_t *e2_tile, int *status, int tid, int bar_id = 1,
@@ -254,7 +255,7 @@ __device__ __forceinline__ void chunk_prologue(uint8_t *q_tile, uint8_t *k_tile,
         uint32_t *e2w = reinterpret_cast<uint32_t *>(&e2v);
 #pragma unroll
         for (int e = 0; e < 2; ++e) {
-            const float i0 = gk * ex2f(-bsum[2 * e]), i1 = gk * ex2f(-bsum[2 * e + 1]);
+            const float i0 = gk * ex2f(POS ? bsum[2 * e] : -bsum[2 * e]), i1 = gk * ex2f(POS ? bsum[2 * e + 1] : -bsum[2 * e + 1]);
             const float2 kf = unpack_bf16(kw[e]);
             kw[e] = pack_bf16(kf.x * i0, kf.y * i1);
             if (WITH_Q) {
@@ -452,6 +453,7 @@ struct BwdParams {
     const SeqInfo *seqs;            // packed variable-length batch: per-sequence table and tensor maps (the nine below), else nullptr
     const CUtensorMap *vmaps;       // q, k, v, dO, log-decay, dq, dk, dv, dlog_decay (Softmax-RetNet: neither of the decay's)
     int dk, dv;             // head widths, each 128 or 64 (the upper half of a 128-wide tile is then zero padding)
+    const float *edge = nullptr;    // packed batch with cut sequences: the state gradients that enter segments with a right neighbour, by id
 };
 // maps: q, k, v, dO, dq, dk, dv
 int retnet_tc_bwd_configure();

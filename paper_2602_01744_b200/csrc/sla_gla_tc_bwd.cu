@@ -71,6 +71,9 @@ struct StatesParams {
     const SeqInfo *seqs;    // packed variable-length batch: per-sequence table and tensor maps (k, v, g), else nullptr
     const CUtensorMap *vmaps;
     int dk, dv;             // head widths, each 128 or 64 (the upper half of a 128-wide tile is then zero padding)
+    const int *pick = nullptr;  // summary mode on a table: the places of the segments to run (fin [n][H][dk][dv], gam [n][H][dk] by id)
+    float scale = 1.f;          // REV
+    const float *edge = nullptr;    // image mode on a table with cut sequences: see FwdParams
 };
 
 // thread (row, colhalf) holds 32 consecutive state values of its row: bf16 them into the operand image
@@ -92,7 +95,9 @@ __device__ __forceinline__ void store_state_part(uint8_t *img, int row, int colh
 // sequence from a zero state and leaves only where it ended and the segment's total decay; a scan over the segments
 // then gives every segment its true starting state.
 // SCALAR: Softmax-RetNet (its constant decay comes in with the gates; the prologue only scales rows).  PAIR: two 64-wide heads a CTA.
-template <bool SCALAR, bool PAIR>
+// REV (summary mode): the state gradient a segment alone sends out of its left edge, and the segment's decay.  dS_n = diag(2^{b_last}) dS_{n+1} +
+// qh^T dO is the same walk from the last chunk to the first, with q, dO in the places of k, v and the decay before the sum.
+template <bool SCALAR, bool PAIR, bool REV = false>
 __global__ void __launch_bounds__(st1::NTHREADS, 1)
 k_gla_states_tc(const __grid_constant__ CUtensorMap gm_k, const __grid_constant__ CUtensorMap gm_v,
                 const __grid_constant__ CUtensorMap gm_g, StatesParams p) {
@@ -105,24 +110,30 @@ k_gla_states_tc(const __grid_constant__ CUtensorMap gm_k, const __grid_constant_
     constexpr int HPC = PAIR ? 2 : 1;                       // heads per CTA
     const int hg = p.H / HPC;
     const int cta = blockIdx.x / p.PS, seg = blockIdx.x % p.PS, h = cta % hg;
-    int b = cta / hg;
+    int b = p.pick ? p.pick[cta / hg] : cta / hg;
     const int bh = b * p.H + h * HPC;
     const size_t sum_i = (size_t)bh * p.P + seg;            // summary slot of this segment
     size_t tokb = (size_t)b * p.T, slot = (size_t)bh * (p.NT + 1);
-    size_t sbh = (size_t)bh;                                // (sequence, head) index into h0 / ht / dht / dh0
+    size_t sbh = (size_t)bh;                                // (sequence, head) index into h0
+    const SeqInfo *const entry = p.seqs ? p.seqs + b : nullptr;
+    int img_n0 = 0;
     const CUtensorMap *vm = nullptr;
     if (p.seqs) {                                           // packed batch: see k_gla_fwd_tc
         const SeqInfo si = p.seqs[b];
         vm = p.vmaps + (size_t)b * Varlen::MAPS_PER_SEQ;
         p.T = si.T; p.NT = si.NT; p.L = si.NT;
         tokb = (size_t)si.t0;
-        slot = (size_t)si.slot0 * p.H + (size_t)h * HPC * (si.NT + 1);
-        sbh = (size_t)si.id * p.H + h * HPC;                      // (the table is ordered longest first, the state tensors as the caller gave them)
+        slot = (size_t)si.slot0 * p.H + (size_t)h * HPC * (si.img_NT + 1);
+        img_n0 = si.img_n0;
+        if (si.dh0_id < 0) p.h0 = p.edge;
+        sbh = (size_t)(si.dh0_id < 0 ? si.id : si.dh0_id) * p.H + h * HPC;      // (the table is ordered longest first, the state tensors as the caller gave them)
         b = 0;
     }
-    const CUtensorMap &tm_k = vm ? vm[0] : gm_k, &tm_v = vm ? vm[1] : gm_v, &tm_g = vm ? vm[2] : gm_g;
+    // (REV: q, dO and the decay among the gradient sweep's maps)
+    const CUtensorMap &tm_k = vm ? vm[0] : gm_k, &tm_v = vm ? vm[REV ? 3 : 1] : gm_v, &tm_g = vm ? vm[REV ? 4 : 2] : gm_g;
     const int n0 = seg * p.L, NT = min(p.L, p.NT - n0);     // this CTA's chunks: n0 .. n0+NT-1
-    const bool images = p.simg != nullptr;
+    const bool images = !REV && p.simg != nullptr;
+    auto chunk_of = [&](int n) { return n0 + (REV ? NT - 1 - n : n); };     // the n-th chunk of the walk
     auto bar = [&](int i) { return base + OFF_BAR + 8u * i; };
     float *tot = reinterpret_cast<float *>(sm + OFF_TOT);
     float *eblast = reinterpret_cast<float *>(sm + OFF_EB);
@@ -152,7 +163,7 @@ k_gla_states_tc(const __grid_constant__ CUtensorMap gm_k, const __grid_constant_
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *reinterpret_cast<volatile uint32_t *>(sm + OFF_TMEM);
-    uint8_t *img0 = p.simg + slot * STATE_BF16;                       // (image mode: one segment, NT = p.NT)
+    uint8_t *img0 = p.simg + slot * STATE_BF16 + (size_t)img_n0 * (PAIR ? PAIR_STATE : STATE_BF16);                       // (image mode: one segment, NT = p.NT)
     grid_launch_dependents();                               // the segmented forward's second pass: see gla_tc_forward
 
     if (warp == 8) {
@@ -184,17 +195,17 @@ k_gla_states_tc(const __grid_constant__ CUtensorMap gm_k, const __grid_constant_
         if (lane == 0) {
             auto load_g = [&](int n) {
                 mbar_expect_tx(bar(FULL_G + (n & 1)), TILE_G);
-                tma_load_4d(base + OFF_G + (n & 1) * TILE_G, &tm_g, 0, h, (n0 + n) * C, b, bar(FULL_G + (n & 1)));
+                tma_load_4d(base + OFF_G + (n & 1) * TILE_G, &tm_g, 0, h, chunk_of(n) * C, b, bar(FULL_G + (n & 1)));
             };
             auto load_k = [&](int n) {
                 const uint32_t bf = bar(FULL_K + n % 3);
                 mbar_expect_tx(bf, TILE_BF16);
-                tma_load_5d(base + OFF_K + (n % 3) * TILE_BF16, &tm_k, 0, (n0 + n) * C, 0, h, b, bf);
+                tma_load_5d(base + OFF_K + (n % 3) * TILE_BF16, &tm_k, 0, chunk_of(n) * C, 0, h, b, bf);
             };
             auto load_v = [&](int n) {
                 const uint32_t bf = bar(FULL_V + (n & 1));
                 mbar_expect_tx(bf, TILE_BF16);
-                tma_load_5d(base + OFF_V + (n & 1) * TILE_BF16, &tm_v, 0, (n0 + n) * C, 0, h, b, bf);
+                tma_load_5d(base + OFF_V + (n & 1) * TILE_BF16, &tm_v, 0, chunk_of(n) * C, 0, h, b, bf);
             };
             for (int n = 0; n < 2 && n < NT && !SCALAR; ++n) load_g(n);
             for (int n = 0; n < 3 && n < NT; ++n) load_k(n);
@@ -218,7 +229,8 @@ k_gla_states_tc(const __grid_constant__ CUtensorMap gm_k, const __grid_constant_
                 if (!images) continue;
                 wait_relaxed(STAGED, n & 1);           // image of S_{n+1} is staged
                 if (failed) break;
-                if (PAIR) {
+                if (n + 1 == NT && entry && entry->ht_id < 0) {         // its right neighbour leaves the image between them
+                } else if (PAIR) {
                     bulk_store(img0 + (size_t)(n + 1) * PAIR_STATE, base + OFF_IMG + pair_block(0), STATE_BLOCK);
                     bulk_store(img0 + (size_t)(n + 1) * PAIR_STATE + STATE_BLOCK, base + OFF_IMG + pair_block(1), STATE_BLOCK);
                 } else {
@@ -235,17 +247,18 @@ k_gla_states_tc(const __grid_constant__ CUtensorMap gm_k, const __grid_constant_
             }
         }
     } else if (warp >= 9) {
-        // ---------------- gates (Gk only), up to four chunks ahead ----------------
+        // ---------------- gates (Gk only; REV: Gq only), up to four chunks ahead ----------------
         const int t = tid - (NCOMPUTE + 32);
-        const float lg = SCALAR ? -LOG2E * p.log_gamma[HPC * h] : 0.f, lg2 = SCALAR && PAIR ? -LOG2E * p.log_gamma[2 * h + 1] : 0.f;
+        constexpr float SIGN = REV ? LOG2E : -LOG2E;
+        const float lg = SCALAR ? SIGN * p.log_gamma[HPC * h] : 0.f, lg2 = SCALAR && PAIR ? SIGN * p.log_gamma[2 * h + 1] : 0.f, mult = REV ? p.scale : 1.f;
         for (int n = 0; n < NT; ++n) {
             if (n >= 4) wait_relaxed(GFREE + (n & 3), ((n >> 2) - 1) & 1);
             if (failed) break;
-            const int cn = min(C, p.T - (n0 + n) * C);
-            const float *lc = p.lk + (tokb + (size_t)(n0 + n) * C) * p.H;
+            const int cn = min(C, p.T - chunk_of(n) * C);
+            const float *lc = (REV ? p.lq : p.lk) + (tokb + (size_t)chunk_of(n) * C) * p.H;
             float *dst = gate_s + (n & 3) * HPC * C, *dst2 = dst + C;
-            if (SCALAR) chunk_gate_by<64, HPC>(lc, p.H, cn, HPC * h, DecayFactor{1.f, lg}, dst, t, DecayFactor{1.f, lg2}, dst2);
-            else chunk_gate_by<64, HPC>(lc, p.H, cn, HPC * h, ConstFactor{1.f}, dst, t, ConstFactor{1.f}, dst2);
+            if (SCALAR) chunk_gate_by<64, HPC>(lc, p.H, cn, HPC * h, DecayFactor{mult, lg}, dst, t, DecayFactor{mult, lg2}, dst2);
+            else chunk_gate_by<64, HPC>(lc, p.H, cn, HPC * h, ConstFactor{mult}, dst, t, ConstFactor{mult}, dst2);
             __syncwarp();
             if (lane == 0) mbar_arrive(bar(GREADY + (n & 3)));
         }
@@ -262,8 +275,9 @@ k_gla_states_tc(const __grid_constant__ CUtensorMap gm_k, const __grid_constant_
                 float v[32];
                 load_state32(src ? src + 32 * part : nullptr, v);
                 tmem_st32(tmem + lane_base + 64 * colhalf + 32 * part, v);
+                if (!images) continue;
                 if (PAIR && holds) store_state_part(img0 + colhalf * STATE_BLOCK, row & 63, 0, part, v);
-                else if (!PAIR && images) store_state_part(img0, row, colhalf, part, v);
+                else if (!PAIR) store_state_part(img0, row, colhalf, part, v);
             }
             tmem_wait_st();
         }
@@ -280,20 +294,26 @@ k_gla_states_tc(const __grid_constant__ CUtensorMap gm_k, const __grid_constant_
             uint8_t *kt = sm + OFF_K + (n % 3) * TILE_BF16;
             const float *gk = gate_s + (n & 3) * HPC * C;
             if (SCALAR) scale_rows(kt, gk, tid, GH);
-            else chunk_prologue<false, false>(nullptr, kt, reinterpret_cast<const float *>(sm + OFF_G + (n & 1) * TILE_G), tot, gk,
+            else chunk_prologue<false, false, NoHook, REV>(nullptr, kt, reinterpret_cast<const float *>(sm + OFF_G + (n & 1) * TILE_G), tot, gk,
                                               gk, eblast + (n & 1) * D, nullptr, p.status, tid, 1, NoHook(), GH);
             fence_proxy_async();
             mbar_arrive(bar(OPR + n % 3));
             mbar_arrive(bar(GFREE + (n & 3)));
         };
         prologue(0);
+        auto decay_of = [&](int n) { return SCALAR ? ex2f(lg * (float)min(C, p.T - chunk_of(n) * C)) : eblast[(n & 1) * D + row]; };
         float gam = 1.f;                               // product of the chunks' 2^{b_last} for key dimension `row`
+        if (REV) {
+            if (!SCALAR) named_bar_sync(1, NCOMPUTE);
+            gam = decay_of(0);
+        }
         for (int n = 0; n < NT; ++n) {
             if (n + 1 < NT) prologue(n + 1);         // overlaps the MMA of chunk n
+            if (REV && !SCALAR && n + 1 < NT) named_bar_sync(1, NCOMPUTE);      // (its decay is used at once)
             wait(BAR_Z, n & 1);
             tc_fence_after();
             if (holds) {   // S_{n+1} = diag(2^{b_last}) (S_n + kh^T V): fp32 back into TMEM, bf16 image staged for slot n+1
-                const float e = SCALAR ? ex2f(lg * (float)min(C, p.T - (n0 + n) * C)) : eblast[(n & 1) * D + row];
+                const float e = !REV ? decay_of(n) : n + 1 < NT ? decay_of(n + 1) : 1.f;
                 gam *= e;
                 float v0[32], v1[32];
                 const uint32_t ta = tmem + lane_base + 64 * colhalf;
@@ -308,7 +328,19 @@ k_gla_states_tc(const __grid_constant__ CUtensorMap gm_k, const __grid_constant_
                     if (n > 0) wait(STFREE, (n - 1) & 1);  // the previous image has left the staging buffer
                     store_state_part(sm + OFF_IMG, row, colhalf, 0, v0);
                     store_state_part(sm + OFF_IMG, row, colhalf, 1, v1);
-                } else if (n == NT - 1) {              // summary mode: where the segment ended, fp32
+                } else if (n == NT - 1 && p.pick) {    // summary mode: where the segment ended, fp32
+                    const size_t own = (size_t)entry->id * p.H + h * HPC;
+                    float *dst = PAIR ? pair_state_row(p.fin, own, row, colhalf) : state_row(p.fin, own, row, colhalf, p.dk, p.dv);
+                    if (dst) {
+#pragma unroll
+                        for (int j = 0; j < 32; j += 4) {
+                            *reinterpret_cast<float4 *>(dst + j) = make_float4(v0[j], v0[j + 1], v0[j + 2], v0[j + 3]);
+                            *reinterpret_cast<float4 *>(dst + 32 + j) = make_float4(v1[j], v1[j + 1], v1[j + 2], v1[j + 3]);
+                        }
+                    }
+                    if (PAIR) p.gam[(own + colhalf) * 64 + (row & 63)] = gam;
+                    else if (colhalf == 0 && row < p.dk) p.gam[own * p.dk + row] = gam;
+                } else if (n == NT - 1) {
                     float *dst = p.fin + sum_i * D * D + fin_off(row, 16 * colhalf);
 #pragma unroll
                     for (int j = 0; j < 8; ++j) {
@@ -387,15 +419,20 @@ k_gla_bwd_tc(const __grid_constant__ CUtensorMap gm_q, const __grid_constant__ C
     int b = blockIdx.x / hg;
     const int bh = b * p.H + h * HPC;
     size_t tokb = (size_t)b * p.T, slot = (size_t)bh * (p.NT + 1);
-    size_t sbh = (size_t)bh;                                // (sequence, head) index into h0 / ht / dht / dh0
+    size_t sbh = (size_t)bh, hbh = sbh;                     // (sequence, head) index into dht, into dh0
+    int img_n0 = 0;
     const CUtensorMap *vm = nullptr;
     if (p.seqs) {                                           // packed batch: see k_gla_fwd_tc
         const SeqInfo si = p.seqs[b];
         vm = p.vmaps + (size_t)b * Varlen::MAPS_PER_SEQ;
         p.T = si.T; p.NT = si.NT;
         tokb = (size_t)si.t0;
-        slot = (size_t)si.slot0 * p.H + (size_t)h * HPC * (si.NT + 1);
-        sbh = (size_t)si.id * p.H + h * HPC;                      // (the table is ordered longest first, the state tensors as the caller gave them)
+        slot = (size_t)si.slot0 * p.H + (size_t)h * HPC * (si.img_NT + 1);
+        img_n0 = si.img_n0;
+        hbh = (size_t)max(si.dh0_id, 0) * p.H + h * HPC;
+        if (si.dh0_id < 0) p.dh0 = nullptr;
+        if (si.ht_id < 0) p.dht = p.edge;
+        sbh = (size_t)(si.ht_id < 0 ? si.id : si.ht_id) * p.H + h * HPC;        // (the table is ordered longest first, the state tensors as the caller gave them)
         b = 0;
     }
     const CUtensorMap &tm_q = vm ? vm[0] : gm_q, &tm_k = vm ? vm[1] : gm_k, &tm_v = vm ? vm[2] : gm_v,
@@ -439,7 +476,7 @@ k_gla_bwd_tc(const __grid_constant__ CUtensorMap gm_q, const __grid_constant__ C
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *reinterpret_cast<volatile uint32_t *>(sm + OFF_TMEM);
-    const uint8_t *img0 = p.simg + slot * STATE_BF16;
+    const uint8_t *img0 = p.simg + slot * STATE_BF16 + (size_t)img_n0 * (PAIR ? PAIR_STATE : STATE_BF16);
     const int NT = p.NT;
     // chunks are visited in the order n = NT-1 ... 0; k = NT-1-n is the visit number that drives every barrier parity
 
@@ -905,7 +942,7 @@ k_gla_bwd_tc(const __grid_constant__ CUtensorMap gm_q, const __grid_constant__ C
         }
 
         if (p.dh0) {   // dS_0, fp32 (the last chunk's MMAs were waited for above)
-            float *dst = PAIR ? pair_state_row(p.dh0, sbh, row, wh) : state_row(p.dh0, sbh, row, wh, p.dk, p.dv);
+            float *dst = PAIR ? pair_state_row(p.dh0, hbh, row, wh) : state_row(p.dh0, hbh, row, wh, p.dk, p.dv);
 #pragma unroll
             for (int part = 0; part < 2; ++part) {
                 float v[32];
@@ -985,6 +1022,25 @@ __global__ void k_fold_segment_dstates(int H, int P, int dk, int dv, const float
     }
 }
 
+// The same for a packed batch whose long sequences are cut (states [id][H][dk][dv], decays [id][H][dk]; sequence s is the segments first[s] ..
+// first[s + 1] - 1; what enters the first of them is the caller's): four neighbouring elements a thread.  RIGHT: state gradients, from the right.
+template <bool RIGHT>
+__global__ void __launch_bounds__(256)
+k_fold_cut(int H, int dk, int dv, const int *__restrict__ first, const float *__restrict__ edge, const float *__restrict__ sent,
+           const float *__restrict__ gam, float *__restrict__ st) {
+    const int s = blockIdx.x / H, h = blockIdx.x % H, e = 4 * (blockIdx.y * 256 + threadIdx.x), row = e / dv, sz = dk * dv;
+    const int i0 = first[s], n = first[s + 1] - i0;
+    if (e >= sz || n == 1) return;
+    float4 v = edge ? *reinterpret_cast<const float4 *>(edge + (size_t)blockIdx.x * sz + e) : make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int x = 0; x + 1 < n; ++x) {
+        const size_t at = (size_t)(i0 + (RIGHT ? n - 1 - x : x)) * H + h, to = RIGHT ? at - H : at + H;
+        const float4 y = *reinterpret_cast<const float4 *>(sent + at * sz + e);
+        const float g = gam[at * dk + row];
+        v = make_float4(fmaf(g, v.x, y.x), fmaf(g, v.y, y.y), fmaf(g, v.z, y.z), fmaf(g, v.w, y.w));
+        *reinterpret_cast<float4 *>(st + to * sz + e) = v;
+    }
+}
+
 }  // namespace
 
 int gla_tc_bwd_configure() {
@@ -993,6 +1049,10 @@ int gla_tc_bwd_configure() {
         cudaFuncSetAttribute(k_gla_states_tc<true, false>, A, (int)st1::SMEM_BYTES) != cudaSuccess ||
         cudaFuncSetAttribute(k_gla_states_tc<false, true>, A, (int)st1::SMEM_BYTES) != cudaSuccess ||
         cudaFuncSetAttribute(k_gla_states_tc<true, true>, A, (int)st1::SMEM_BYTES) != cudaSuccess ||
+        cudaFuncSetAttribute(k_gla_states_tc<false, false, true>, A, (int)st1::SMEM_BYTES) != cudaSuccess ||
+        cudaFuncSetAttribute(k_gla_states_tc<true, false, true>, A, (int)st1::SMEM_BYTES) != cudaSuccess ||
+        cudaFuncSetAttribute(k_gla_states_tc<false, true, true>, A, (int)st1::SMEM_BYTES) != cudaSuccess ||
+        cudaFuncSetAttribute(k_gla_states_tc<true, true, true>, A, (int)st1::SMEM_BYTES) != cudaSuccess ||
         cudaFuncSetAttribute(k_gla_bwd_tc<false>, A, (int)st2::SMEM_BYTES) != cudaSuccess ||
         cudaFuncSetAttribute(k_gla_bwd_tc<true>, A, (int)st2::SMEM_BYTES) != cudaSuccess)
         return -1;
@@ -1020,9 +1080,58 @@ static size_t state_slots(const Dims &d, const Varlen *vl) {
     return (vl && vl->n_seq) ? (size_t)vl->slots * d.H : (size_t)d.B * d.H * (d.NT + 1);
 }
 
-size_t gla_tc_backward_workspace_bytes(const Dims &d, const Varlen *vl) {
+// state images, then the two [B,T,H] gate products
+size_t gla_tc_images_floats(const Dims &d, const Varlen *vl) {
     const size_t bth = (size_t)d.B * d.T * d.H;
-    return state_slots(d, vl) * STATE_BF16 + 2 * ((bth + 63) & ~(size_t)63) * sizeof(float);
+    return state_slots(d, vl) * (STATE_BF16 / 4) + 2 * ((bth + 63) & ~(size_t)63);
+}
+size_t gla_tc_backward_workspace_bytes(const Dims &d, const Varlen *vl) {
+    return (gla_tc_images_floats(d, vl) + (vl && vl->n_of ? gla_tc_cut_floats(d, *vl) : 0)) * sizeof(float);
+}
+
+// Scratch of a packed batch with cut sequences: what the segments send on, the states at their edges, their decays (both directions in turn).
+size_t gla_tc_cut_floats(const Dims &d, const Varlen &cut) { return (size_t)cut.n_seq * d.H * d.dk * (2 * d.dv + 1); }
+
+namespace {
+struct CutScratch { float *sent, *st, *gam; };
+CutScratch cut_scratch(const Dims &d, const Varlen &cut, float *scratch) {
+    const size_t sz = (size_t)cut.n_seq * d.H * d.dk * d.dv;
+    return {scratch, scratch + sz, scratch + 2 * sz};
+}
+template <bool RIGHT>
+void fold_cut(const Dims &d, const Varlen &cut, const CutScratch &c, const float *edge, cudaStream_t st) {
+    k_fold_cut<RIGHT><<<dim3(cut.n_of * d.H, (d.dk * d.dv + 1023) / 1024), 256, 0, st>>>(d.H, d.dk, d.dv, cut.d_cut, edge, c.sent, c.gam, c.st);
+}
+// k, v, log-decay of every sequence of a table
+const CUtensorMap *states_maps(Varlen &vl, bool retnet, const void *k, const void *v, const float *g, int H, int dk, int dv, cudaStream_t st) {
+    const void *key[] = {k, v, g};
+    return varlen_maps(vl, 1, key, 3, st, [&](const SeqInfo &si, CUtensorMap *m) {
+        const size_t tok = (size_t)si.t0 * H;      // (q, k are d_k wide, v, o and their gradients d_v)
+        if (!make_tile_map(m + 0, (const __nv_bfloat16 *)k + tok * dk, 1, si.T, H, dk) ||
+            !make_tile_map(m + 1, (const __nv_bfloat16 *)v + tok * dv, 1, si.T, H, dv)) return false;
+        if (retnet) { m[2] = m[0]; return true; }
+        return make_map(m + 2, g + tok * dk, 1, si.T, H, dk, true, 128);
+    });
+}
+}  // namespace
+
+const float *gla_tc_cut_starts(const Dims &d, const FwdArgs &a, float *scratch, int *status, cudaStream_t st, Tracer &tr) {
+    const Varlen &cut = *a.vl;
+    const bool retnet = d.variant == SLA_RETNET, pair = gla_tc_pairs(d, a.vl);
+    const int H = pair ? d.H / 2 : d.H, dk = pair ? 128 : d.dk, dv = pair ? 128 : d.dv;
+    const CutScratch c = cut_scratch(d, cut, scratch);
+    const CUtensorMap *vm = states_maps(*a.vl, retnet, a.k, a.v, a.log_decay, H, dk, dv, st);
+    CUtensorMap mk;
+    if (!vm || !make_tile_map(&mk, a.k, d.B, d.T, H, dk)) return nullptr;
+    StatesParams sp{a.lq, a.lk, nullptr, nullptr, c.sent, c.gam, status, d.T, d.H, d.NT, 1, d.NT, 1, retnet ? a.log_decay : nullptr,
+                    cut.d_seqs, vm, d.dk, d.dv, cut.d_cut + cut.n_of + 1};
+    auto *const kernel = retnet ? (pair ? k_gla_states_tc<true, true> : k_gla_states_tc<true, false>)
+                                : pair ? k_gla_states_tc<false, true> : k_gla_states_tc<false, false>;
+    kernel<<<cut.n_left * H, st1::NTHREADS, st1::SMEM_BYTES, st>>>(mk, mk, mk, sp);
+    tr.mark("gla_segment_states_tc");
+    fold_cut<false>(d, cut, c, a.h0, st);
+    tr.mark("fold_segment_states");
+    return cudaGetLastError() == cudaSuccess ? c.st : nullptr;
 }
 
 int gla_tc_segment_summaries(const Dims &d, const FwdArgs &a, int P, int L, int PS, float *fin, float *gam, int *status,
@@ -1067,20 +1176,23 @@ int gla_tc_backward(const Dims &d, const BwdArgs &a, bool have_states, int *stat
     const __nv_bfloat16 *q = (const __nv_bfloat16 *)a.q, *k = (const __nv_bfloat16 *)a.k, *v = (const __nv_bfloat16 *)a.v,
                         *dO = (const __nv_bfloat16 *)a.dO;
 
-    if (!have_states) {   // (otherwise the forward pass of the same inputs has left the images in this workspace)
+    Varlen *const whole = vl;
+    const float *starts = nullptr, *ends = nullptr;
+    int launches = have_states ? 2 : 3;
+    float *scratch = a.ws + gla_tc_images_floats(d, vl);            // (a table with cut sequences)
+    if (!have_states) {   // (otherwise the forward pass of the same inputs has left the images in this workspace); in the forward pass's form
         const CUtensorMap *vm = nullptr;
-        if (vl) {
-            const void *key[] = {a.k, a.v, a.log_decay};
-            vm = varlen_maps(*vl, 1, key, 3, st, [&](const SeqInfo &si, CUtensorMap *m) {
-                const size_t tok = (size_t)si.t0 * H;      // (q, k are d_k wide, v, o and their gradients d_v)
-                if (!make_tile_map(m + 0, k + tok * dk, 1, si.T, H, dk) || !make_tile_map(m + 1, v + tok * dv, 1, si.T, H, dv)) return false;
-                if (retnet) { m[2] = m[0]; return true; }
-                return make_map(m + 2, a.log_decay + tok * dk, 1, si.T, H, dk, true, 128);
-            });
-            if (!vm) return -1;
+        Varlen *const vl = !whole ? nullptr : whole->n_of && !whole->fwd ? whole->whole : whole;
+        const SeqInfo *dseqs = vl ? vl->d_seqs : nullptr;
+        const int ctas = vl ? vl->n_seq * H : d.B * H;
+        if (vl && vl->n_of) {
+            const FwdArgs f{a.q, a.k, a.v, a.log_decay, a.beta, a.lq, a.lk, a.h0, nullptr, nullptr, a.ws, a.status, vl};
+            if (!(starts = gla_tc_cut_starts(d, f, scratch, status, st, tr))) return -1;
+            launches += 2;
         }
+        if (vl && !(vm = states_maps(*vl, retnet, a.k, a.v, a.log_decay, H, dk, dv, st))) return -1;
         StatesParams sp{a.lq, a.lk, a.h0, simg, nullptr, nullptr, status, d.T, d.H, d.NT, 1, d.NT, 1, retnet ? a.log_decay : nullptr,
-                        dseqs, vm, d.dk, d.dv};
+                        dseqs, vm, d.dk, d.dv, nullptr, 1.f, starts};
         auto *const kernel = retnet ? (pair ? k_gla_states_tc<true, true> : k_gla_states_tc<true, false>)
                                     : pair ? k_gla_states_tc<false, true> : k_gla_states_tc<false, false>;
         kernel<<<ctas, st1::NTHREADS, st1::SMEM_BYTES, st>>>(mk, mv, mg, sp);
@@ -1103,13 +1215,26 @@ int gla_tc_backward(const Dims &d, const BwdArgs &a, bool have_states, int *stat
         });
         if (!vm) return -1;
     }
-    BwdParams bp{a.lq, a.lk, a.dht, simg, pq, pk, a.dh0, status, d.T, d.H, d.NT, d.scale, retnet ? a.log_decay : nullptr, dseqs, vm, d.dk, d.dv};
+    if (vl && vl->n_of) {       // the state gradients that enter the segments from their right
+        const CutScratch c = cut_scratch(d, *vl, scratch);
+        StatesParams sp{a.lq, a.lk, nullptr, nullptr, c.sent, c.gam, status, d.T, d.H, d.NT, 1, d.NT, 1, retnet ? a.log_decay : nullptr,
+                        dseqs, vm, d.dk, d.dv, vl->d_cut + vl->n_of + 1 + vl->n_left, d.scale};
+        auto *const kernel = retnet ? (pair ? k_gla_states_tc<true, true, true> : k_gla_states_tc<true, false, true>)
+                                    : pair ? k_gla_states_tc<false, true, true> : k_gla_states_tc<false, false, true>;
+        kernel<<<vl->n_right * H, st1::NTHREADS, st1::SMEM_BYTES, st>>>(mq, mdo, mg, sp);
+        tr.mark("gla_segment_dstates_tc");
+        fold_cut<true>(d, *vl, c, a.dht, st);
+        tr.mark("fold_segment_dstates");
+        ends = c.st;
+        launches += 2;
+    }
+    BwdParams bp{a.lq, a.lk, a.dht, simg, pq, pk, a.dh0, status, d.T, d.H, d.NT, d.scale, retnet ? a.log_decay : nullptr, dseqs, vm, d.dk, d.dv, ends};
     if (retnet) retnet_tc_bwd_launch({mq, mk, mv, mdo, mdq, mdk, mdv}, bp, pair, ctas, st);
     else (pair ? k_gla_bwd_tc<true> : k_gla_bwd_tc<false>)<<<ctas, st2::NTHREADS, st2::SMEM_BYTES, st>>>(mq, mk, mv, mdo, mg, mdq, mdk, mdv, mdg, bp);
     tr.mark("gla_bwd_tc");
     if (gate_bwd_prod(a.lq, a.lk, pq, pk, a.dlq, a.dlk, (long)d.B * d.T, d.H, st) < 0) return -1;
     tr.mark("gate_bwd");
-    return cudaGetLastError() == cudaSuccess ? (have_states ? 2 : 3) : -1;
+    return cudaGetLastError() == cudaSuccess ? launches : -1;
 }
 
 
@@ -1129,10 +1254,7 @@ void gla_tc_backward_segment_table(const Dims &d, int P, int L, Varlen &segs) {
 }
 
 // floats: [images of the segments' slots | pq | pk] as gla_tc_backward lays them out, then fin, gam, h0seg, dhtseg, dsfin
-static size_t segmented_base_floats(const Dims &d, const Varlen &segs) {
-    const size_t bth = (size_t)d.B * d.T * d.H;
-    return state_slots(d, &segs) * (STATE_BF16 / 4) + 2 * ((bth + 63) & ~(size_t)63);
-}
+static size_t segmented_base_floats(const Dims &d, const Varlen &segs) { return gla_tc_images_floats(d, &segs); }
 size_t gla_tc_backward_segmented_workspace_bytes(const Dims &d, const Varlen &segs) {
     const size_t nseg = (size_t)d.B * d.H * segs.seg_P, st = (size_t)segs.n_seq * d.H * d.dk * d.dv;
     return (segmented_base_floats(d, segs) + nseg * (D * D + D) + 3 * st) * sizeof(float);

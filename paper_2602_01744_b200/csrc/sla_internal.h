@@ -35,7 +35,11 @@ struct Dims {
 // chunks cut from each sequence's own start).  Per sequence: first token, length, chunks, and the index of its first
 // state slot (the sum of chunks + 1 over the sequences before it).  The table is kept longest sequence first, so that the
 // CTAs of long sequences are dispatched first (one CTA per (sequence, head), in table order).
-struct SeqInfo { int t0, T, NT, slot0, id; };     // id: the sequence's number as the caller counts them
+// id: the sequence's number as the caller counts them.  ht_id, dh0_id: the number by which its final state and its initial one (and
+// their gradients) are the caller's; -1: a segment of a longer sequence, which takes that state from scratch, by its own id, and hands none out.
+// Its state images are those of chunks img_n0 .. img_n0 + NT of a sequence of img_NT chunks (the one that a segment belongs to; segments leave the image
+// of a cut to the right one of the two).
+struct SeqInfo { int t0, T, NT, slot0, id, ht_id = id, dh0_id = id, img_NT = NT, img_n0 = 0; };
 // Host side of a plan's sequence table.  The tensor-core kernels address a sequence through tensor maps of its own
 // (based at its first token, T = its length: loads past its end read zeros, stores are clipped there, exactly as at the
 // end of a batch row); those live in device arrays, one region per kernel kind, encoded again only when the tensors
@@ -52,6 +56,16 @@ struct Varlen {
         cudaEvent_t uploaded = nullptr;
     } reg[3];                           // 0: forward, 1: state / record sweep, 2: gradient sweep
     static constexpr int MAPS_PER_SEQ = 9;
+    // An internal table in which the long sequences of a packed batch are cut into segments (gla_tc_cut_sequences): the caller has n_of
+    // sequences, sequence s is the segments first[s] .. first[s + 1] - 1 (their ids); cut: first, then the n_left table places of segments
+    // with a right neighbour, then the n_right places of those with a left one.
+    // The state images are those of the uncut table (`whole`), so a forward pass and the backward pass that reads them may be of either form;
+    // fwd: the forward pass by itself gains, too.
+    int n_of = 0, n_left = 0, n_right = 0;
+    bool fwd = false;
+    Varlen *whole = nullptr;
+    std::vector<int> cut;
+    int *d_cut = nullptr;
     int seg_P = 0, seg_L = 0;           // > 0: an internal table that cuts each of the B batch rows into seg_P segments of seg_L chunks
 };
 
@@ -146,6 +160,13 @@ bool gla_tc_pairs(const Dims &d, const Varlen *vl);
 // chunk there, in the layout the gradient sweep reads: the backward pass of the same inputs then needs no state sweep.
 bool gla_tc_forward_can_save(const Dims &d, const Varlen *vl = nullptr);
 uint8_t *gla_tc_state_images(float *ws);   // where in the backward workspace the images sit
+// Few long sequences in a packed batch: fills `cut` (host side) where segments pay.  A call takes that table in place of the batch's own if its
+// scratch is large enough.
+void gla_tc_cut_sequences(const Dims &d, Varlen &vl, Varlen &cut);
+// The states the segments with a left neighbour start from, into scratch (returned; nullptr on failure): two launches.
+const float *gla_tc_cut_starts(const Dims &d, const FwdArgs &a, float *scratch, int *status, cudaStream_t st, Tracer &tr);
+size_t gla_tc_cut_floats(const Dims &d, const Varlen &cut);         // scratch of a call on such a table
+size_t gla_tc_images_floats(const Dims &d, const Varlen *vl);       // where it starts in the backward pass's workspace
 int gla_tc_forward(const Dims &d, const FwdArgs &a, uint8_t *simg, int *status, cudaStream_t st, Tracer &tr);
 // Backward: chunk-state sweep, gradient sweep, gate softmax backward.  Needs the first
 // B*H*(NT+1)*32 KiB + 2*B*T*H*4 bytes (rounded up) of the workspace, less than the generic path.
@@ -238,9 +259,10 @@ struct sla_plan {
         const void *ws = nullptr, *q = nullptr, *k = nullptr, *v = nullptr, *log_decay = nullptr, *beta = nullptr, *lq = nullptr,
                    *lk = nullptr, *h0 = nullptr;
         void *stream = nullptr;
-        bool chunked = false;       // Softmax-GatedDeltaNet: in which of the two forms
+        bool chunked = false;       // in which of the two forms (Softmax-GatedDeltaNet: chunk-parallel; Softmax-GLA, -RetNet: pairs of heads)
     } saved;
     sla::Varlen varlen;     // sla_plan_set_sequences: packed variable-length batch (n_seq == 0: regular batch)
+    sla::Varlen cut;        // its table with long sequences cut into segments, where that pays (tensor-core GLA / RetNet)
     sla::Varlen segs;       // tensor-core GLA / RetNet plans with few long sequences: the segments the backward runs in
     sla::Tracer tracer;
     std::vector<std::pair<const char *, std::pair<int, float>>> agg;   // name -> (launches, total ms)

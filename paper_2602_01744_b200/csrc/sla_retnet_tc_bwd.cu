@@ -55,15 +55,20 @@ k_retnet_bwd_tc(const __grid_constant__ CUtensorMap gm_q, const __grid_constant_
     int b = blockIdx.x / hg;
     const int bh = b * p.H + h * HPC;
     size_t tokb = (size_t)b * p.T, slot = (size_t)bh * (p.NT + 1);
-    size_t sbh = (size_t)bh;                                // (sequence, head) index into dht / dh0
+    size_t sbh = (size_t)bh, hbh = sbh;                     // (sequence, head) index into dht, into dh0
+    int img_n0 = 0;
     const CUtensorMap *vm = nullptr;
     if (p.seqs) {                                           // packed batch: see k_gla_fwd_tc
         const SeqInfo si = p.seqs[b];
         vm = p.vmaps + (size_t)b * Varlen::MAPS_PER_SEQ;
         p.T = si.T; p.NT = si.NT;
         tokb = (size_t)si.t0;
-        slot = (size_t)si.slot0 * p.H + (size_t)h * HPC * (si.NT + 1);
-        sbh = (size_t)si.id * p.H + h * HPC;                      // (the table is ordered longest first, the state tensors as the caller gave them)
+        slot = (size_t)si.slot0 * p.H + (size_t)h * HPC * (si.img_NT + 1);
+        img_n0 = si.img_n0;
+        hbh = (size_t)max(si.dh0_id, 0) * p.H + h * HPC;
+        if (si.dh0_id < 0) p.dh0 = nullptr;
+        if (si.ht_id < 0) p.dht = p.edge;
+        sbh = (size_t)(si.ht_id < 0 ? si.id : si.ht_id) * p.H + h * HPC;        // (the table is ordered longest first, the state tensors as the caller gave them)
         b = 0;
     }
     const CUtensorMap &tm_q = vm ? vm[0] : gm_q, &tm_k = vm ? vm[1] : gm_k, &tm_v = vm ? vm[2] : gm_v, &tm_do = vm ? vm[3] : gm_do,
@@ -101,7 +106,7 @@ k_retnet_bwd_tc(const __grid_constant__ CUtensorMap gm_q, const __grid_constant_
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *reinterpret_cast<volatile uint32_t *>(sm + OFF_TMEM);
-    const uint8_t *img0 = p.simg + slot * STATE_BF16;
+    const uint8_t *img0 = p.simg + slot * STATE_BF16 + (size_t)img_n0 * (PAIR ? PAIR_STATE : STATE_BF16);
     const int NT = p.NT;
     // chunks are visited in the order n = NT-1 ... 0; k = NT-1-n is the visit number that drives every buffer and parity
 
@@ -461,7 +466,7 @@ k_retnet_bwd_tc(const __grid_constant__ CUtensorMap gm_q, const __grid_constant_
         }
 
         if (p.dh0) {   // dS_0, fp32 (the last chunk's MMAs were waited for above)
-            float *dst = PAIR ? pair_state_row(p.dh0, sbh, row, wh) : state_row(p.dh0, sbh, row, wh, p.dk, p.dv);
+            float *dst = PAIR ? pair_state_row(p.dh0, hbh, row, wh) : state_row(p.dh0, hbh, row, wh, p.dk, p.dv);
 #pragma unroll
             for (int part = 0; part < 2; ++part) {
                 float v[32];
