@@ -75,10 +75,9 @@ typedef enum { SLA_FP32 = 0, SLA_BF16 = 1 } sla_dtype;
  * given the same workspace, the same q, k, v, log_decay, beta, logits and h0 pointers and the same
  * stream as that sla_forward uses what was left and skips its recomputation; any other call
  * recomputes, so results never depend on the flag.  Contract: between the two calls the caller
- * changes neither the workspace nor the contents of those inputs.  The fp32 CUDA-core kernels leave their
- * gates, decays and states where sla_forward was given at least the backward size (the forward size that is
- * reported stays the smaller one, and with it nothing is left).  Ignored (nothing is left, the backward
- * recomputes) where the forward cuts long sequences into segments. */
+ * changes neither the workspace nor the contents of those inputs.  Ignored (nothing is left, the
+ * backward recomputes) by the fp32 CUDA-core kernels and where the forward cuts long sequences
+ * into segments. */
 
 typedef struct {
     uint32_t struct_size;      /* sizeof(sla_desc) */

@@ -57,15 +57,12 @@ __global__ void k_selftest_bounded_wait(int *status, unsigned long long limit_ns
     if (!sla::ptx::mbar_wait_bounded(bar, 0, nullptr, limit_ns) && threadIdx.x == 0) atomicOr(status, sla::STATUS_TIMEOUT);
 }
 
-static bool on_tensor_cores(const sla_plan &p) {
-    return !(p.flags & SLA_FLAG_FORCE_GENERIC) && (sla::gla_tc_supported(p.dims) || sla::gdn_tc_supported(p.dims));
-}
-// Does sla_forward of this plan write into the backward pass's workspace layout (SLA_FLAG_SAVE_FOR_BACKWARD)?  The tensor-core
-// paths do, Softmax-GLA only where the forward runs each sequence in one piece.
+// Can sla_forward of this plan leave what sla_backward needs (SLA_FLAG_SAVE_FOR_BACKWARD)?  Only the tensor-core
+// paths do, and Softmax-GLA only where the forward runs each sequence in one piece.
 static bool forward_can_save(const sla_plan &p) {
-    if (!on_tensor_cores(p)) return false;
+    if (p.flags & SLA_FLAG_FORCE_GENERIC) return false;
     if (sla::gla_tc_supported(p.dims)) return sla::gla_tc_forward_can_save(p.dims, &p.varlen);
-    return true;
+    return sla::gdn_tc_supported(p.dims);
 }
 
 // What the kernels this plan selects need as workspace (regular batch, or the packed batch of sla_plan_set_sequences).
@@ -346,9 +343,6 @@ sla_status sla_forward(sla_plan *plan, const void *q, const void *k, const void 
     plan->tracer.start((cudaStream_t)cuda_stream);
     const bool generic = plan->flags & SLA_FLAG_FORCE_GENERIC;
     const bool save = (plan->flags & SLA_FLAG_SAVE_FOR_BACKWARD) && forward_can_save(*plan);
-    // What the fp32 CUDA-core kernels leave lies at the same place in both passes' workspaces.  It counts as kept where the forward was
-    // given the backward pass's: scratch of the forward's own size may be gone, and its place taken, by the time of the backward.
-    const bool kept = (plan->flags & SLA_FLAG_SAVE_FOR_BACKWARD) && !on_tensor_cores(*plan) && workspace_bytes >= plan->bwd_bytes;
     bool chunked = !generic && sla::gdn_tc_supported(d) && sla::gdn_tc_chunked(d, &plan->varlen, save, workspace_bytes);
     if (!generic && sla::gla_tc_supported(d)) {
         // (the state a sequence starts from and its final one in one buffer: a cut sequence's last segment may be done before its first begins)
@@ -365,7 +359,7 @@ sla_status sla_forward(sla_plan *plan, const void *q, const void *k, const void 
                 : sla::generic_forward(d, plan->ws, a, true, (cudaStream_t)cuda_stream, plan->tracer);
     if (n < 0) return sla::cuda_error();
     plan->last_launches = n;
-    if (save || kept) {
+    if (save) {
         sla_plan::Saved &sv = plan->saved;
         sv.valid = true;
         sv.ws = workspace; sv.q = q; sv.k = k; sv.v = v; sv.log_decay = log_decay; sv.beta = beta;
@@ -430,7 +424,7 @@ sla_status sla_backward(sla_plan *plan, const void *q, const void *k, const void
                 ? sla::gla_tc_backward(d, a, have, plan->d_status, (cudaStream_t)cuda_stream, plan->tracer)
             : (!generic && sla::gdn_tc_supported(d))
                 ? sla::gdn_tc_backward(d, a, have, chunked, plan->d_status, (cudaStream_t)cuda_stream, plan->tracer)
-                : sla::generic_backward(d, plan->ws, a, have, (cudaStream_t)cuda_stream, plan->tracer);
+                : sla::generic_backward(d, plan->ws, a, (cudaStream_t)cuda_stream, plan->tracer);
     if (chunked_records && !chunked) sv.valid = false;   // (the one-CTA kernels stepped in and wrote records of their own there)
     if (n == -2) return SLA_ERR_UNSUPPORTED;
     if (n < 0) return sla::cuda_error();

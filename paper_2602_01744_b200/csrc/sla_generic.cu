@@ -1160,13 +1160,11 @@ int generic_forward(const Dims &d, const Workspace &w, const FwdArgs &a, bool wr
     return d.io_bf16 ? forward_t<__nv_bfloat16>(d, w, a, write_o, st, tr) : forward_t<float>(d, w, a, write_o, st, tr);
 }
 
-int generic_backward(const Dims &d, const Workspace &w, const BwdArgs &a, bool have_states, cudaStream_t st, Tracer &tr) {
-    int n1 = 0;
-    if (!have_states) {     // recompute gates, cumulative decays and the per-chunk states (no output store)
-        FwdArgs f{a.q, a.k, a.v, a.log_decay, a.beta, a.lq, a.lk, a.h0, nullptr, nullptr, a.ws, a.status};
-        n1 = generic_forward(d, w, f, false, st, tr);
-        if (n1 < 0) return -1;
-    }
+int generic_backward(const Dims &d, const Workspace &w, const BwdArgs &a, cudaStream_t st, Tracer &tr) {
+    // recompute gates, cumulative decays and the per-chunk states (no output store)
+    FwdArgs f{a.q, a.k, a.v, a.log_decay, a.beta, a.lq, a.lk, a.h0, nullptr, nullptr, a.ws, a.status};
+    int n1 = generic_forward(d, w, f, false, st, tr);
+    if (n1 < 0) return -1;
     int n2;
     if (d.variant == SLA_GDN) {
         float *ws = a.ws;

@@ -142,8 +142,7 @@ struct Tracer {
 
 // Each returns the number of kernels launched (>0) or -1 after a CUDA launch error.
 int generic_forward(const Dims &d, const Workspace &w, const FwdArgs &a, bool write_o, cudaStream_t st, Tracer &tr);
-// have_states: the workspace holds the gates, decays and states that a forward of the same inputs left there
-int generic_backward(const Dims &d, const Workspace &w, const BwdArgs &a, bool have_states, cudaStream_t st, Tracer &tr);
+int generic_backward(const Dims &d, const Workspace &w, const BwdArgs &a, cudaStream_t st, Tracer &tr);
 // recurrent decode (sla_decode.cu): streaming kernel over column slices of the state, 64 or 128 wide
 int decode_step(const Dims &d, const DecArgs &a, int *status, cudaStream_t st, Tracer &tr);
 int decode_configure();
