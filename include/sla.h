@@ -134,6 +134,10 @@ sla_status sla_plan_poll(sla_plan *plan);
  * context stays usable. */
 sla_status sla_plan_selftest_timeout(sla_plan *plan, void *cuda_stream);
 
+/* Forgets what the last sla_forward of a SLA_FLAG_SAVE_FOR_BACKWARD plan left: the next sla_backward recomputes.  For a caller whose
+ * workspace is given up between the two passes, so that another one at the same address is not taken for it. */
+sla_status sla_plan_forget_saved(sla_plan *plan);
+
 /* Number of kernel launches the last sla_forward / sla_backward / sla_decode_step on this plan
  * enqueued (for launch accounting in benchmarks). */
 int32_t sla_plan_last_launch_count(const sla_plan *plan);

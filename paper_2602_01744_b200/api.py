@@ -27,7 +27,7 @@ EXPORTS = (
     "sla_forward_noalloc", "sla_plan_selftest_timeout", "sla_decode_steps", "sla_gate_scores_forward",
     "sla_gate_scores_backward", "sla_plan_gate_scores_workspace_bytes", "sla_shortconv_forward",
     "sla_shortconv_backward", "sla_plan_shortconv_workspace_bytes", "sla_plan_set_sequences",
-    "sla_out_proj_forward", "sla_out_proj_backward",
+    "sla_out_proj_forward", "sla_out_proj_backward", "sla_plan_forget_saved",
 )
 SLA_NOALLOC_SCRATCH_BYTES = 32 << 20
 
@@ -73,6 +73,8 @@ def lib():
         L.sla_plan_poll.argtypes = [vp]
         L.sla_plan_selftest_timeout.argtypes = [vp, vp]
         L.sla_plan_selftest_timeout.restype = ctypes.c_int
+        L.sla_plan_forget_saved.argtypes = [vp]
+        L.sla_plan_forget_saved.restype = ctypes.c_int
         L.sla_plan_last_launch_count.argtypes = [vp]
         L.sla_plan_last_launch_count.restype = i32
         L.sla_plan_set_kernel_timing.argtypes = [vp, i32]
@@ -256,11 +258,14 @@ def sla_forward(plan: Plan, q, k, v, log_decay, gq_logits, gk_logits, beta=None,
     d = plan.desc
     if o is None:
         o = torch.empty((d.B, d.T, d.H, d.d_v), dtype=plan.io_torch, device=q.device)
-    if workspace is None:
+    given_up = workspace is None                # scratch of this call goes back to the allocator on return
+    if given_up:
         workspace = plan.scratch(False, q.device)
     _check("sla_forward", lib().sla_forward(
         plan.handle, _ptr(q), _ptr(k), _ptr(v), _ptr(log_decay), _ptr(beta), _ptr(gq_logits),
         _ptr(gk_logits), _ptr(h0), _ptr(o), _ptr(ht), _ptr(workspace), workspace.numel(), _stream()))
+    if given_up and d.flags & SLA_FLAG_SAVE_FOR_BACKWARD:       # (a backward pass that is handed the same memory must not look for it there)
+        _check("sla_plan_forget_saved", lib().sla_plan_forget_saved(plan.handle))
     return o, ht
 
 

@@ -273,6 +273,12 @@ sla_status sla_plan_poll(sla_plan *plan) {
     return SLA_OK;
 }
 
+sla_status sla_plan_forget_saved(sla_plan *plan) {
+    if (!plan) return SLA_ERR_INVALID_ARG;
+    plan->saved.valid = false;
+    return SLA_OK;
+}
+
 int32_t sla_plan_last_launch_count(const sla_plan *plan) { return plan ? plan->last_launches : 0; }
 
 sla_status sla_plan_selftest_timeout(sla_plan *plan, void *cuda_stream) {
