@@ -83,7 +83,8 @@ k_gates_decay(Dims d, const float *__restrict__ lq, const float *__restrict__ lk
         const float t = __shfl_up_sync(FULL, incl, o);
         if (lane >= o) incl += t;
     }
-    if (2 * lane < cn) bcum[tok_row(d, b, t0 + 2 * lane, h)] = incl - g1;
+    const float before = __shfl_up_sync(FULL, incl, 1);        // (the first of the two not as incl - g1, which keeps only what g1 leaves of it)
+    if (2 * lane < cn) bcum[tok_row(d, b, t0 + 2 * lane, h)] = lane ? before + g0 : g0;
     if (2 * lane + 1 < cn) bcum[tok_row(d, b, t0 + 2 * lane + 1, h)] = incl;
     if (lane == 31 && incl < -SLA_MAX_CHUNK_DECAY) atomicOr(status, STATUS_RANGE);
 }
