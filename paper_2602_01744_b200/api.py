@@ -7,6 +7,9 @@ There is no fallback: if the shared library is missing or a call is refused, an 
 from __future__ import annotations
 
 import ctypes
+import importlib.machinery
+import importlib.util
+import warnings
 from pathlib import Path
 
 import torch
@@ -123,18 +126,18 @@ _fast = None
 
 
 def _load_fast(L):
+    """Without an extension built for this Python, this torch and this source, the Python path serves (a decode call costs the host 4 us more)."""
     global _fast
     try:
         from . import build as _build
-        _build.build_fast()
-    except Exception:                           # no compiler here: an existing build is still fine
-        pass
-    try:
-        from . import _sla_fast
-    except ImportError:
+        loader = importlib.machinery.ExtensionFileLoader("_sla_fast", str(_build.build_fast()))
+        module = importlib.util.module_from_spec(importlib.util.spec_from_loader("_sla_fast", loader))
+        loader.exec_module(module)
+    except Exception as e:
+        warnings.warn(f"decode calls take the Python path: their native marshalling could not be built or loaded ({e})", RuntimeWarning)
         return
     addr = lambda f: ctypes.cast(f, ctypes.c_void_p).value
-    _fast = (_sla_fast.decode, addr(L.sla_decode_step), addr(L.sla_decode_steps))
+    _fast = (module.decode, addr(L.sla_decode_step), addr(L.sla_decode_steps))
 
 
 def _check(call: str, status: int):

@@ -29,24 +29,34 @@ def build(force: bool = False, verbose: bool = False) -> Path:
     return SO
 
 
-FAST_SO = PKG / "_sla_fast.so"
 FAST_SOURCE = PKG / "native" / "fastcall.cpp"
+
+
+def fast_so() -> Path:
+    """Where the extension of this Python, this torch and this source lies.  It is compiled against torch's inline accessors, so one that was built for
+    another of the three must not be loaded: all three are in its name."""
+    import hashlib
+    import sysconfig
+    import torch
+    key = [sysconfig.get_config_var("SOABI"), torch.__version__, str(int(torch._C._GLIBCXX_USE_CXX11_ABI)), FAST_SOURCE.read_text()]
+    return PKG / f"_sla_fast.{hashlib.sha256(chr(0).join(map(str, key)).encode()).hexdigest()[:16]}.so"
 
 
 def build_fast(force: bool = False) -> Path:
     """The native argument marshalling of the decode calls (a Python extension against torch's headers)."""
-    if not force and FAST_SO.exists() and FAST_SO.stat().st_mtime >= FAST_SOURCE.stat().st_mtime:
-        return FAST_SO
+    so = fast_so()
+    if not force and so.exists():
+        return so
     import sysconfig
     import torch
     t = Path(torch.__file__).resolve().parent
-    tmp = FAST_SO.with_suffix(f".so.{os.getpid()}.tmp")
+    tmp = so.with_suffix(f".so.{os.getpid()}.tmp")
     subprocess.run(["g++", "-O2", "-std=c++20", "-fPIC", "-shared", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
                     f"-I{sysconfig.get_paths()['include']}", f"-I{t / 'include'}", f"-I{t / 'include/torch/csrc/api/include'}",
                     "-I/usr/local/cuda/include", str(FAST_SOURCE), "-o", str(tmp), f"-L{t / 'lib'}", f"-Wl,-rpath,{t / 'lib'}",
                     "-ltorch_python", "-ltorch_cpu", "-ltorch_cuda", "-lc10_cuda", "-lc10"], check=True)
-    os.replace(tmp, FAST_SO)
-    return FAST_SO
+    os.replace(tmp, so)
+    return so
 
 
 if __name__ == "__main__":
