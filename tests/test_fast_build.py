@@ -39,3 +39,28 @@ def test_without_a_current_build_the_python_path_serves_and_says_so(monkeypatch)
 def test_the_extension_loads():
     api.lib()
     assert api._fast is not None
+
+
+def test_the_library_builds_without_a_compiler_for_the_extension(monkeypatch, capsys):
+    import __graft_entry__
+
+    def no_compiler(force=False):
+        raise FileNotFoundError("g++")
+
+    monkeypatch.setattr(build, "build_fast", no_compiler)
+    __graft_entry__.build()
+    assert "g++" in capsys.readouterr().err
+
+
+def test_the_extension_takes_the_toolkit_that_builds_the_library(monkeypatch, tmp_path):
+    (tmp_path / "bin").mkdir()
+    nvcc = tmp_path / "bin" / "nvcc"
+    nvcc.write_text("")
+    nvcc.chmod(0o755)
+    seen = []
+    monkeypatch.setenv("NVCC", str(nvcc))
+    monkeypatch.setattr(build, "fast_so", lambda: tmp_path / "fast.so")
+    monkeypatch.setattr(build.subprocess, "run", lambda cmd, check: seen.extend(cmd))
+    monkeypatch.setattr(build.os, "replace", lambda a, b: None)
+    build.build_fast()
+    assert f"-I{tmp_path / 'include'}" in seen and "-I/usr/local/cuda/include" not in seen
