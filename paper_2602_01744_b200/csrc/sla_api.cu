@@ -218,10 +218,10 @@ sla_status sla_plan_destroy(sla_plan *plan) {
 sla_status sla_plan_set_sequences(sla_plan *plan, const int32_t *cu_seqlens, int32_t n_seq) {
     if (!plan || n_seq < 0 || (n_seq > 0 && !cu_seqlens)) return SLA_ERR_INVALID_ARG;
     const sla::Dims &d = plan->dims;
-    plan->saved.valid = false;
-    varlen_release(plan->varlen);
-    varlen_release(plan->cut);
     if (n_seq == 0) {
+        plan->saved.valid = false;
+        varlen_release(plan->varlen);
+        varlen_release(plan->cut);
         plan_workspace_sizes(plan);
         return SLA_OK;
     }
@@ -229,13 +229,17 @@ sla_status sla_plan_set_sequences(sla_plan *plan, const int32_t *cu_seqlens, int
     if ((plan->flags & SLA_FLAG_FORCE_GENERIC) || !(sla::gla_tc_supported(d) || sla::gdn_tc_supported(d))) return SLA_ERR_UNSUPPORTED;
     if (d.B != 1 || cu_seqlens[0] != 0 || cu_seqlens[n_seq] != d.T) return SLA_ERR_INVALID_ARG;
     if ((uint64_t)n_seq * d.H > 0x7fffffffu) return SLA_ERR_UNSUPPORTED;
+    for (int s = 0; s < n_seq; ++s)
+        if (cu_seqlens[s + 1] <= cu_seqlens[s]) return SLA_ERR_INVALID_ARG;      // (empty sequences are not allowed)
+    // nothing of the plan has changed up to here, so a refused table leaves it as it was: its tables and its sizes belong together
+    plan->saved.valid = false;
+    varlen_release(plan->varlen);
+    varlen_release(plan->cut);
     sla::Varlen &v = plan->varlen;
     long slots = 0;
     for (int s = 0; s < n_seq; ++s) {
         const int len = cu_seqlens[s + 1] - cu_seqlens[s];
-        if (len <= 0) { v.seqs.clear(); return SLA_ERR_INVALID_ARG; }      // (empty sequences are not allowed)
-        const int nt = (len + d.C - 1) / d.C;
-        v.seqs.push_back({cu_seqlens[s], len, nt, 0, s});
+        v.seqs.push_back({cu_seqlens[s], len, (len + d.C - 1) / d.C, 0, s});
     }
     std::stable_sort(v.seqs.begin(), v.seqs.end(), [](const sla::SeqInfo &a, const sla::SeqInfo &b) { return a.NT > b.NT; });
     for (auto &si : v.seqs) {
