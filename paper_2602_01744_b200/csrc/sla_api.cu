@@ -1,5 +1,6 @@
 // Host side of the C ABI: plan validation, workspace carve-up, launch order.
 #include "sla_internal.h"
+#include "sla_tables.h"
 #include "sla_ptx.cuh"
 
 #include <algorithm>
@@ -99,33 +100,6 @@ static void plan_workspace_sizes(sla_plan *p) {
     }
 }
 
-static void varlen_release(sla::Varlen &v) {
-    if (v.d_seqs) cudaFree(v.d_seqs);
-    if (v.d_cut) cudaFree(v.d_cut);
-    for (auto &g : v.reg) {
-        if (g.dev) cudaFree(g.dev);
-        if (g.host) cudaFreeHost(g.host);
-        if (g.uploaded) cudaEventDestroy(g.uploaded);
-        g = sla::Varlen::Region();
-    }
-    v = sla::Varlen();
-}
-
-// Device side of a filled sequence table: the table itself and, per kernel kind, room for the sequences' tensor maps.
-static bool varlen_to_device(sla::Varlen &v) {
-    const int n_seq = v.n_seq;
-    bool ok = cudaMalloc((void **)&v.d_seqs, sizeof(sla::SeqInfo) * n_seq) == cudaSuccess &&
-              cudaMemcpy(v.d_seqs, v.seqs.data(), sizeof(sla::SeqInfo) * n_seq, cudaMemcpyHostToDevice) == cudaSuccess;
-    if (!v.cut.empty())
-        ok = ok && cudaMalloc((void **)&v.d_cut, sizeof(int) * v.cut.size()) == cudaSuccess &&
-             cudaMemcpy(v.d_cut, v.cut.data(), sizeof(int) * v.cut.size(), cudaMemcpyHostToDevice) == cudaSuccess;
-    const size_t mb = (size_t)n_seq * sla::Varlen::MAPS_PER_SEQ * sizeof(CUtensorMap);
-    for (auto &g : v.reg)
-        ok = ok && cudaMalloc((void **)&g.dev, mb) == cudaSuccess && cudaMallocHost((void **)&g.host, mb) == cudaSuccess &&
-             cudaEventCreateWithFlags(&g.uploaded, cudaEventDisableTiming) == cudaSuccess;
-    return ok;
-}
-
 extern "C" {
 
 const char *sla_status_string(sla_status s) {
@@ -183,8 +157,7 @@ sla_status sla_plan_create(sla_plan **out, const sla_desc *desc) {
         sla::gla_tc_backward_choose_segments(d, P, L);
         if (P > 1) {
             sla::gla_tc_backward_segment_table(d, P, L, p->segs);
-            if (!varlen_to_device(p->segs)) {
-                varlen_release(p->segs);
+            if (!sla::varlen_to_device(p->segs)) {
                 delete p;
                 return sla::cuda_error();
             }
@@ -207,9 +180,9 @@ sla_status sla_plan_create(sla_plan **out, const sla_desc *desc) {
 sla_status sla_plan_destroy(sla_plan *plan) {
     if (!plan) return SLA_OK;
     if (plan->d_status) cudaFree(plan->d_status);
-    varlen_release(plan->varlen);
-    varlen_release(plan->cut);
-    varlen_release(plan->segs);
+    sla::varlen_release(plan->varlen);
+    sla::varlen_release(plan->cut);
+    sla::varlen_release(plan->segs);
     plan->tracer.destroy();
     delete plan;
     return SLA_OK;
@@ -220,8 +193,8 @@ sla_status sla_plan_set_sequences(sla_plan *plan, const int32_t *cu_seqlens, int
     const sla::Dims &d = plan->dims;
     if (n_seq == 0) {
         plan->saved.valid = false;
-        varlen_release(plan->varlen);
-        varlen_release(plan->cut);
+        sla::varlen_release(plan->varlen);
+        sla::varlen_release(plan->cut);
         plan_workspace_sizes(plan);
         return SLA_OK;
     }
@@ -231,11 +204,7 @@ sla_status sla_plan_set_sequences(sla_plan *plan, const int32_t *cu_seqlens, int
     if ((uint64_t)n_seq * d.H > 0x7fffffffu) return SLA_ERR_UNSUPPORTED;
     for (int s = 0; s < n_seq; ++s)
         if (cu_seqlens[s + 1] <= cu_seqlens[s]) return SLA_ERR_INVALID_ARG;      // (empty sequences are not allowed)
-    // nothing of the plan has changed up to here, so a refused table leaves it as it was: its tables and its sizes belong together
-    plan->saved.valid = false;
-    varlen_release(plan->varlen);
-    varlen_release(plan->cut);
-    sla::Varlen &v = plan->varlen;
+    sla::Varlen v, cut;
     long slots = 0;
     for (int s = 0; s < n_seq; ++s) {
         const int len = cu_seqlens[s + 1] - cu_seqlens[s];
@@ -248,13 +217,10 @@ sla_status sla_plan_set_sequences(sla_plan *plan, const int32_t *cu_seqlens, int
     }
     v.slots = slots;
     v.n_seq = n_seq;
-    if (sla::gla_tc_supported(d)) sla::gla_tc_cut_sequences(d, v, plan->cut);
-    if (!varlen_to_device(v) || (plan->cut.n_seq && !varlen_to_device(plan->cut))) {
-        varlen_release(v);
-        varlen_release(plan->cut);
-        plan_workspace_sizes(plan);
-        return sla::cuda_error();
-    }
+    if (sla::gla_tc_supported(d)) sla::gla_tc_cut_sequences(d, v, cut);
+    // (nothing of the plan has changed up to here: a refused table leaves it as it was, its tables and its sizes belong together)
+    if (!sla::replace_tables(plan->varlen, plan->cut, std::move(v), std::move(cut))) return sla::cuda_error();
+    plan->saved.valid = false;
     plan_workspace_sizes(plan);
     return SLA_OK;
 }

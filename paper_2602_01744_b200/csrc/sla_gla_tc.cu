@@ -598,7 +598,7 @@ bool gla_tc_pairs(const Dims &d, const Varlen *vl) {
 // one, launches and first loads 7 and 4, a segment's states 2.5 and 0.8 in what all SMs together move.  Against measured calls (T x heads of 128, longest
 // sequence; forward, and backward with gates: before -> cut, us): 8192 x 8, 4880 tokens 161 -> 56, 449 -> 100; 4096 x 16, 1695 64.5 -> 60.3, 173 -> 108;
 // 32768 x 16, 11120 372 -> 303, 1013 -> 635; 16384 x 16, 3167 119 -> 136 (not taken), 323 -> 269.  Segments have at least 8 chunks.
-void gla_tc_cut_sequences(const Dims &d, Varlen &vl, Varlen &cut) {
+void gla_tc_cut_sequences(const Dims &d, const Varlen &vl, Varlen &cut) {
     const double sms = sm_count(), size = d.dk * d.dv / (double)(D * D);
     long longest = 0;
     for (const SeqInfo &s : vl.seqs) longest = std::max<long>(longest, s.NT);
@@ -627,7 +627,6 @@ void gla_tc_cut_sequences(const Dims &d, Varlen &vl, Varlen &cut) {
             if (t < best && (fwd || hpc == whole_hpc)) { best = t; best_L = L; cut.fwd = fwd; }     // (a whole forward pass decides on the pairs)
         }
     if (!best_L) return;
-    cut.whole = &vl;
     std::vector<SeqInfo> by_id(vl.seqs);
     std::sort(by_id.begin(), by_id.end(), [](const SeqInfo &a, const SeqInfo &b) { return a.id < b.id; });
     for (const SeqInfo &s : by_id) {

@@ -161,7 +161,7 @@ bool gla_tc_forward_can_save(const Dims &d, const Varlen *vl = nullptr);
 uint8_t *gla_tc_state_images(float *ws);   // where in the backward workspace the images sit
 // Few long sequences in a packed batch: fills `cut` (host side) where segments pay.  A call takes that table in place of the batch's own if its
 // scratch is large enough.
-void gla_tc_cut_sequences(const Dims &d, Varlen &vl, Varlen &cut);
+void gla_tc_cut_sequences(const Dims &d, const Varlen &vl, Varlen &cut);
 // The states the segments with a left neighbour start from, into scratch (returned; nullptr on failure): two launches.
 const float *gla_tc_cut_starts(const Dims &d, const FwdArgs &a, float *scratch, int *status, cudaStream_t st, Tracer &tr);
 size_t gla_tc_cut_floats(const Dims &d, const Varlen &cut);         // scratch of a call on such a table
