@@ -151,7 +151,8 @@ inline const CUtensorMap *varlen_maps(Varlen &vl, int r, const void *const *key,
     for (int i = 0; i < nkey && same; ++i) same = g.key[i] == key[i];
     if (same) return g.dev;
     g.valid = false;
-    if (cudaEventSynchronize(g.uploaded) != cudaSuccess) return nullptr;      // the mirror's last upload has been read
+    if ((g.uploaded ? cudaEventSynchronize(g.uploaded)                        // the mirror's last upload has been read
+                    : cudaEventCreateWithFlags(&g.uploaded, cudaEventDisableTiming)) != cudaSuccess) return nullptr;
     for (int s = 0; s < vl.n_seq; ++s)
         if (!make(vl.seqs[s], g.host + (size_t)s * Varlen::MAPS_PER_SEQ)) return nullptr;
     const size_t bytes = (size_t)vl.n_seq * Varlen::MAPS_PER_SEQ * sizeof(CUtensorMap);

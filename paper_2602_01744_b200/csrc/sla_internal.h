@@ -48,12 +48,13 @@ struct Varlen {
     int n_seq = 0;
     long slots = 0;                     // sum over the sequences of (chunks + 1)
     std::vector<SeqInfo> seqs;
+    void *block = nullptr, *mirror = nullptr;           // device and pinned memory that the pointers below point into
     SeqInfo *d_seqs = nullptr;
     struct Region {
         CUtensorMap *dev = nullptr, *host = nullptr;    // [n_seq][MAPS_PER_SEQ]; host: pinned mirror
         const void *key[10] = {};
         bool valid = false;
-        cudaEvent_t uploaded = nullptr;
+        cudaEvent_t uploaded = nullptr;                 // made by the first upload
     } reg[3];                           // 0: forward, 1: state / record sweep, 2: gradient sweep
     static constexpr int MAPS_PER_SEQ = 9;
     // An internal table in which the long sequences of a packed batch are cut into segments (gla_tc_cut_sequences): the caller has n_of
