@@ -689,7 +689,8 @@ int gla_tc_forward(const Dims &d, const FwdArgs &a, uint8_t *simg, int *status, 
         });
         if (!vm || !make_tile_map(&mq, a.q, d.B, d.T, H, dk)) return -1;
         const float *edge = nullptr;
-        if (a.vl->n_of && !(edge = gla_tc_cut_starts(d, a, a.ws + (simg ? gla_tc_images_floats(d, a.vl) : 0), status, st, tr))) return -1;
+        // (the summaries read this region's k, v and log-decay, which stand side by side: what a backward pass uploads is no business of a captured forward's)
+        if (a.vl->n_of && !(edge = gla_tc_cut_starts(d, a, vm + 1, a.ws + (simg ? gla_tc_images_floats(d, a.vl) : 0), status, st, tr))) return -1;
         FwdParams p{a.lq, a.lk, a.h0, nullptr, nullptr, (__nv_bfloat16 *)a.o, a.ht, simg, status, d.T, d.H, d.NT, 1, d.NT, d.scale,
                     retnet ? a.log_decay : nullptr, a.vl->d_seqs, vm, d.dk, d.dv, edge};
         kernel<<<a.vl->n_seq * H, NTHREADS, SMEM_BYTES, st>>>(mq, mq, mq, mq, mq, p);

@@ -1115,14 +1115,13 @@ const CUtensorMap *states_maps(Varlen &vl, bool retnet, const void *k, const voi
 }
 }  // namespace
 
-const float *gla_tc_cut_starts(const Dims &d, const FwdArgs &a, float *scratch, int *status, cudaStream_t st, Tracer &tr) {
+const float *gla_tc_cut_starts(const Dims &d, const FwdArgs &a, const CUtensorMap *vm, float *scratch, int *status, cudaStream_t st, Tracer &tr) {
     const Varlen &cut = *a.vl;
     const bool retnet = d.variant == SLA_RETNET, pair = gla_tc_pairs(d, a.vl);
-    const int H = pair ? d.H / 2 : d.H, dk = pair ? 128 : d.dk, dv = pair ? 128 : d.dv;
+    const int H = pair ? d.H / 2 : d.H, dk = pair ? 128 : d.dk;
     const CutScratch c = cut_scratch(d, cut, scratch);
-    const CUtensorMap *vm = states_maps(*a.vl, retnet, a.k, a.v, a.log_decay, H, dk, dv, st);
     CUtensorMap mk;
-    if (!vm || !make_tile_map(&mk, a.k, d.B, d.T, H, dk)) return nullptr;
+    if (!make_tile_map(&mk, a.k, d.B, d.T, H, dk)) return nullptr;
     StatesParams sp{a.lq, a.lk, nullptr, nullptr, c.sent, c.gam, status, d.T, d.H, d.NT, 1, d.NT, 1, retnet ? a.log_decay : nullptr,
                     cut.d_seqs, vm, d.dk, d.dv, cut.d_cut + cut.n_of + 1};
     auto *const kernel = retnet ? (pair ? k_gla_states_tc<true, true> : k_gla_states_tc<true, false>)
@@ -1185,12 +1184,12 @@ int gla_tc_backward(const Dims &d, const BwdArgs &a, bool have_states, int *stat
         Varlen *const vl = !whole ? nullptr : whole->n_of && !whole->fwd ? whole->whole : whole;
         const SeqInfo *dseqs = vl ? vl->d_seqs : nullptr;
         const int ctas = vl ? vl->n_seq * H : d.B * H;
+        if (vl && !(vm = states_maps(*vl, retnet, a.k, a.v, a.log_decay, H, dk, dv, st))) return -1;
         if (vl && vl->n_of) {
             const FwdArgs f{a.q, a.k, a.v, a.log_decay, a.beta, a.lq, a.lk, a.h0, nullptr, nullptr, a.ws, a.status, vl};
-            if (!(starts = gla_tc_cut_starts(d, f, scratch, status, st, tr))) return -1;
+            if (!(starts = gla_tc_cut_starts(d, f, vm, scratch, status, st, tr))) return -1;
             launches += 2;
         }
-        if (vl && !(vm = states_maps(*vl, retnet, a.k, a.v, a.log_decay, H, dk, dv, st))) return -1;
         StatesParams sp{a.lq, a.lk, a.h0, simg, nullptr, nullptr, status, d.T, d.H, d.NT, 1, d.NT, 1, retnet ? a.log_decay : nullptr,
                         dseqs, vm, d.dk, d.dv, nullptr, 1.f, starts};
         auto *const kernel = retnet ? (pair ? k_gla_states_tc<true, true> : k_gla_states_tc<true, false>)

@@ -163,8 +163,9 @@ uint8_t *gla_tc_state_images(float *ws);   // where in the backward workspace th
 // Few long sequences in a packed batch: fills `cut` (host side) where segments pay.  A call takes that table in place of the batch's own if its
 // scratch is large enough.
 void gla_tc_cut_sequences(const Dims &d, const Varlen &vl, Varlen &cut);
-// The states the segments with a left neighbour start from, into scratch (returned; nullptr on failure): two launches.
-const float *gla_tc_cut_starts(const Dims &d, const FwdArgs &a, float *scratch, int *status, cudaStream_t st, Tracer &tr);
+// The states the segments with a left neighbour start from, into scratch (returned; nullptr on failure): two launches.  vm: the table's tensor maps of
+// k, v and log-decay, MAPS_PER_SEQ apart.
+const float *gla_tc_cut_starts(const Dims &d, const FwdArgs &a, const CUtensorMap *vm, float *scratch, int *status, cudaStream_t st, Tracer &tr);
 size_t gla_tc_cut_floats(const Dims &d, const Varlen &cut);         // scratch of a call on such a table
 size_t gla_tc_images_floats(const Dims &d, const Varlen *vl);       // where it starts in the backward pass's workspace
 int gla_tc_forward(const Dims &d, const FwdArgs &a, uint8_t *simg, int *status, cudaStream_t st, Tracer &tr);
