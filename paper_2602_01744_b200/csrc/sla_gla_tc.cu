@@ -135,7 +135,7 @@ k_gla_fwd_tc(const __grid_constant__ CUtensorMap gm_q, const __grid_constant__ C
         for (int i = 0; i < NBAR; ++i) {
             const bool all = (i >= OPR && i < GREADY) || (i >= GFREE && i < SREADY);                          // every prologue thread
             const bool warps = (i >= SREADY && i <= AREADY) || i == OSTAGED || i == ATAKEN || i == OFREE2;     // one arrival per warp
-            mbar_init(bar(i), all ? NCOMPUTE : warps ? NCOMPUTE / 32 : (i >= GREADY && i < GFREE) ? NGATE / 32 : 1);
+            mbar_init(bar(i), all ? NCOMPUTE : warps ? NCOMPUTE / 32 : (i >= GREADY && i < GFREE) ? NGATE / 32 : i == FULL_G ? 1 + NCOMPUTE / 32 : 1);
         }
         fence_mbar_init();
         tma_prefetch_desc(&tm_q);
@@ -319,7 +319,10 @@ k_gla_fwd_tc(const __grid_constant__ CUtensorMap gm_q, const __grid_constant__ C
             mbar_expect_tx(bar(FULL_G), TILE_G);
             tma_load_4d(base + OFF_G, &tm_g, 0, h, (n0 + n) * C, b, bar(FULL_G));
         };
+        // A chunk's decay counts as there when its tile is and every warp has read what the chunk before left in tot: there is one tot, and a
+        // warp goes on to write it with no other wait in between.
         if (ptid == 0 && !SCALAR) load_g(0);
+        if (!SCALAR) warp_arrive(bar(FULL_G), lane);
         if (ptid < HPC && SCALAR) check_scalar_range(p.log_gamma[HPC * h + ptid], p.T, p.status);
         for (int n = 0; n < NT; ++n) {
             wait(GREADY + (n & 3), (n >> 2) & 1);
@@ -336,7 +339,8 @@ k_gla_fwd_tc(const __grid_constant__ CUtensorMap gm_q, const __grid_constant__ C
             } else {
                 chunk_prologue<true, false>(qk, qk + TILE_BF16, reinterpret_cast<const float *>(sm + OFF_G), tot, g, g + C,
                                             eblast + (n & 3) * D, nullptr, p.status, ptid, 2,
-                                            [&]() { if (ptid == 0 && n + 1 < NT) load_g(n + 1); }, GH);
+                                            [&]() { if (ptid == 0 && n + 1 < NT) load_g(n + 1); }, GH,
+                                            [&]() { warp_arrive(bar(FULL_G), lane); });
             }
             fence_proxy_async();
             mbar_arrive(bar(OPR + n % 3));

@@ -198,11 +198,12 @@ __device__ __forceinline__ uint32_t e2_off(uint32_t row, uint32_t chunk) { retur
 struct NoHook { __device__ __forceinline__ void operator()() const {} };
 // POS: k_i * gk_i * 2^{+b_i} instead (the reverse summaries, whose tile is q).
 // gate_half: distance between the gates of columns 0..63 and those of columns 64..127 (a pair of heads; 0: one head).
-template <bool WITH_Q, bool WITH_E, class Hook = NoHook, bool POS = false>
+// tot_read: called when this thread has read tot, for a caller with neither two of them nor a barrier of its own between two prologues.
+template <bool WITH_Q, bool WITH_E, class Hook = NoHook, bool POS = false, class TotRead = NoHook>
 __device__ __forceinline__ void chunk_prologue(uint8_t *q_tile, uint8_t *k_tile, const float *gs, float *tot,
                                                const float *gq_s, const float *gk_s, float *eblast,
                                                uint8_t *e2_tile, int *status, int tid, int bar_id = 1,
-                                               Hook tile_read = Hook(), int gate_half = 0) {
+                                               Hook tile_read = Hook(), int gate_half = 0, TotRead tot_read = TotRead()) {
     using namespace ptx;
     const int rg = tid >> 5, cj = tid & 31;
     gq_s += (cj >> 4) * gate_half;
@@ -225,6 +226,7 @@ __device__ __forceinline__ void chunk_prologue(uint8_t *q_tile, uint8_t *k_tile,
         const float4 a = g < rg ? *reinterpret_cast<const float4 *>(tot + g * D + 4 * cj) : make_float4(0.f, 0.f, 0.f, 0.f);
         bsum[0] += a.x; bsum[1] += a.y; bsum[2] += a.z; bsum[3] += a.w;
     }
+    tot_read();
 #pragma unroll
     for (int e = 0; e < 4; ++e) bsum[e] *= LOG2E;
     // columns 4cj..4cj+3 = 8 bytes of a bf16 row: half cj>>4, 16-byte chunk (cj&15)>>1, upper or lower 8 bytes

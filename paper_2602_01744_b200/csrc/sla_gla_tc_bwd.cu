@@ -45,8 +45,8 @@ constexpr uint32_t OFF_G = 0;                               // [2] fp32 log-deca
 constexpr uint32_t OFF_K = OFF_G + 2 * TILE_G;              // [3] k tiles (kh after the prologue)
 constexpr uint32_t OFF_V = OFF_K + 3 * TILE_BF16;           // [2] v tiles
 constexpr uint32_t OFF_IMG = OFF_V + 2 * TILE_BF16;         // bf16 state image staged for the bulk store
-constexpr uint32_t OFF_TOT = OFF_IMG + STATE_BF16;          // prologue scratch
-constexpr uint32_t OFF_EB = OFF_TOT + TOT_BYTES;            // [2][128] 2^{b_last}
+constexpr uint32_t OFF_TOT = OFF_IMG + STATE_BF16;          // [2] prologue scratch: a warp may still be reading one chunk's when another writes the next's
+constexpr uint32_t OFF_EB = OFF_TOT + 2 * TOT_BYTES;        // [2][128] 2^{b_last}
 constexpr uint32_t OFF_GATE = OFF_EB + 2 * D * 4;           // [4][heads][64] Gk of four chunks
 constexpr uint32_t OFF_BAR = OFF_GATE + 2 * 4 * C * 4;
 constexpr uint32_t OFF_TMEM = OFF_BAR + 32 * 8;             // TMEM base address, then the abort flag
@@ -294,8 +294,8 @@ k_gla_states_tc(const __grid_constant__ CUtensorMap gm_k, const __grid_constant_
             uint8_t *kt = sm + OFF_K + (n % 3) * TILE_BF16;
             const float *gk = gate_s + (n & 3) * HPC * C;
             if (SCALAR) scale_rows(kt, gk, tid, GH);
-            else chunk_prologue<false, false, NoHook, REV>(nullptr, kt, reinterpret_cast<const float *>(sm + OFF_G + (n & 1) * TILE_G), tot, gk,
-                                              gk, eblast + (n & 1) * D, nullptr, p.status, tid, 1, NoHook(), GH);
+            else chunk_prologue<false, false, NoHook, REV>(nullptr, kt, reinterpret_cast<const float *>(sm + OFF_G + (n & 1) * TILE_G),
+                                              tot + (n & 1) * (TOT_BYTES / 4), gk, gk, eblast + (n & 1) * D, nullptr, p.status, tid, 1, NoHook(), GH);
             fence_proxy_async();
             mbar_arrive(bar(OPR + n % 3));
             mbar_arrive(bar(GFREE + (n & 3)));
