@@ -18,6 +18,12 @@ using StepFn = int (*)(void *plan, int32_t Bdec, const void *q, const void *k, c
 using StepsFn = int (*)(void *plan, int32_t Bdec, int32_t n_tokens, const void *q, const void *k, const void *v, const float *log_decay,
                         const float *beta, const float *lq, const float *lk, float *state, void *o, void *stream);
 
+// The interpreter's lock is given up for as long as this lives (and is back before an exception reaches a handler).
+struct Unlocked {
+    PyThreadState *state = PyEval_SaveThread();
+    ~Unlocked() { PyEval_RestoreThread(state); }
+};
+
 // Is obj None, or exactly a torch.Tensor (no subclass) on a CUDA device and contiguous?  Then its data goes to *p.
 bool pointer(PyObject *obj, void **p) {
     *p = nullptr;
@@ -56,23 +62,33 @@ PyObject *decode(PyObject *, PyObject *const *a, Py_ssize_t n) {
         const int32_t B = (int32_t)q.size(0);
         void *stream = (void *)c10::cuda::getCurrentCUDAStream(c10::cuda::current_device()).stream();
         int status;
-        Py_BEGIN_ALLOW_THREADS              // (a launch waits where the stream's queue is full)
-        if (several)
-            status = reinterpret_cast<StepsFn>(fn)(plan, B, (int32_t)q.size(1), p[0], p[1], p[2], (const float *)p[3], (const float *)p[7],
-                                                   (const float *)p[4], (const float *)p[5], (float *)p[6], p[8], stream);
-        else
-            status = reinterpret_cast<StepFn>(fn)(plan, B, p[0], p[1], p[2], (const float *)p[3], (const float *)p[7], (const float *)p[4],
-                                                  (const float *)p[5], (float *)p[6], p[8], stream);
-        Py_END_ALLOW_THREADS
-        PyObject *res = PyTuple_New(2);
-        if (!res) return nullptr;
-        PyTuple_SET_ITEM(res, 0, PyLong_FromLong(status));
+        {
+            Unlocked unlocked;              // (a launch waits where the stream's queue is full)
+            if (several)
+                status = reinterpret_cast<StepsFn>(fn)(plan, B, (int32_t)q.size(1), p[0], p[1], p[2], (const float *)p[3], (const float *)p[7],
+                                                       (const float *)p[4], (const float *)p[5], (float *)p[6], p[8], stream);
+            else
+                status = reinterpret_cast<StepFn>(fn)(plan, B, p[0], p[1], p[2], (const float *)p[3], (const float *)p[7], (const float *)p[4],
+                                                      (const float *)p[5], (float *)p[6], p[8], stream);
+        }
         if (o == Py_None) o = THPVariable_Wrap(out);
         else Py_INCREF(o);
+        if (!o) return nullptr;
+        PyObject *code = PyLong_FromLong(status), *res = PyTuple_New(2);
+        if (!code || !res) {
+            Py_DECREF(o);
+            Py_XDECREF(code);
+            Py_XDECREF(res);
+            return nullptr;
+        }
+        PyTuple_SET_ITEM(res, 0, code);
         PyTuple_SET_ITEM(res, 1, o);
         return res;
     } catch (const std::exception &e) {
         PyErr_SetString(PyExc_RuntimeError, e.what());
+        return nullptr;
+    } catch (...) {
+        PyErr_SetString(PyExc_RuntimeError, "unknown C++ exception");
         return nullptr;
     }
 }
