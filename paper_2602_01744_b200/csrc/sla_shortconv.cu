@@ -354,22 +354,26 @@ k_shortconv_bwd(ConvDims cd, const TIO *__restrict__ x, const float *__restrict_
 }
 
 // Reverse pass of bf16 heads that are a power-of-two run of lanes (four channels a thread).  The sequences are cut into as many units of
-// neighbouring tokens as the GPU holds groups of 256 threads, two groups a CTA and one CTA per SM, and a group walks its unit backwards - dx of
+// neighbouring tokens as the GPU holds groups of threads, at one CTA of 512 per SM, and a group walks its unit backwards - dx of
 // a token needs dy of the three tokens after it, so a walk starts three tokens past its unit - with the windows over x and dy in
 // registers and the rows of four tokens fetched ahead; every row of x and dout is fetched and widened once and serves y, dx
-// and the tap gradients.  Head sums by shuffles.  Tap gradients are summed per thread over its units, the two groups' sums added, and
+// and the tap gradients.  Head sums by shuffles.  Tap gradients are summed per thread over its units, the groups' sums added, and
 // written per CTA.  Bound by instruction issue (sigmoid, its derivative, three 4-tap sums and the norm terms an element).  In blocks of eight tokens,
 // 14 rows of x and 11 of dout fetched and 11 tokens recomputed for eight written, as many CTAs as the workspace has slots: 2 x 2048 tokens
 // x 2048 channels 30 us, 24 now (the layer step with three of them 490 -> 472).
-constexpr int BWD_GROUPS = 2;
-template <bool NORM>
-__global__ void __launch_bounds__(256 * BWD_GROUPS, 1)
-k_shortconv_bwd_walk(ConvDims cd, Units un, const __nv_bfloat16 *__restrict__ x, const float *__restrict__ w,
+// A group has as many threads as there are fours of channels, up to 256 (`width`, whole warps), and a CTA as many groups as 512 threads hold:
+// of few channels most threads of a group of 256 would have nothing (1 x 50000 tokens x 256 channels: blocks 88 us, groups of 256 107, of 64 37;
+// 64 x 128 x 512: 23.7, 27.3, 19.7).
+constexpr int BWD_THREADS = 512;
+template <bool NORM, int WIDTH>     // WIDTH: 256, or 0 for any
+__global__ void __launch_bounds__(BWD_THREADS, 1)
+k_shortconv_bwd_walk(ConvDims cd, Units un, int group_width, const __nv_bfloat16 *__restrict__ x, const float *__restrict__ w,
                      const __nv_bfloat16 *__restrict__ dout, __nv_bfloat16 *__restrict__ dx, float *__restrict__ partial) {
     constexpr int N = 4;
     using F = Four;
-    __shared__ float4 sums[BWD_GROUPS - 1][N][256];
-    const int C = cd.H * cd.d, vpr = cd.d / N, group = threadIdx.x >> 8, tid = threadIdx.x & 255, gv = blockIdx.y * 256 + tid;
+    __shared__ float4 sums[N][BWD_THREADS];
+    const int C = cd.H * cd.d, vpr = cd.d / N, width = WIDTH ? WIDTH : group_width, groups = WIDTH ? BWD_THREADS / WIDTH : blockDim.x / width,
+              group = threadIdx.x / width, tid = threadIdx.x - group * width, gv = blockIdx.y * 256 + tid;
     const bool live = gv < C / N;
     float wt[KMAX][N], acc[KMAX][N];
     load_taps<N>(w, gv * N, cd.K, live, wt);
@@ -377,7 +381,7 @@ k_shortconv_bwd_walk(ConvDims cd, Units un, const __nv_bfloat16 *__restrict__ x,
     for (int j = 0; j < KMAX; ++j)
 #pragma unroll
         for (int e = 0; e < N; ++e) acc[j][e] = 0.f;
-    for (long unit = (long)blockIdx.x * BWD_GROUPS + group; unit < un.total; unit += (long)gridDim.x * BWD_GROUPS) {
+    for (long unit = (long)blockIdx.x * groups + group; unit < un.total; unit += (long)gridDim.x * groups) {
         int b, t0, t1;
         un.at(unit, cd.T, b, t0, t1);
         const int ue = min(cd.T, t1 + KMAX - 1) - 1;            // last token whose dy this unit needs
@@ -453,7 +457,7 @@ k_shortconv_bwd_walk(ConvDims cd, Units un, const __nv_bfloat16 *__restrict__ x,
     }
     if (group > 0) {
 #pragma unroll
-        for (int e = 0; e < N; ++e) sums[group - 1][e][tid] = make_float4(acc[0][e], acc[1][e], acc[2][e], acc[3][e]);
+        for (int e = 0; e < N; ++e) sums[e][threadIdx.x] = make_float4(acc[0][e], acc[1][e], acc[2][e], acc[3][e]);
     }
     __syncthreads();
     if (group > 0 || !live) return;
@@ -461,9 +465,8 @@ k_shortconv_bwd_walk(ConvDims cd, Units un, const __nv_bfloat16 *__restrict__ x,
 #pragma unroll
     for (int e = 0; e < N; ++e) {
         float4 v = make_float4(acc[0][e], acc[1][e], acc[2][e], acc[3][e]);
-#pragma unroll
-        for (int o = 0; o < BWD_GROUPS - 1; ++o) {
-            const float4 y = sums[o][e][tid];
+        for (int o = 1; o < groups; ++o) {
+            const float4 y = sums[e][o * width + tid];
             v.x += y.x; v.y += y.y; v.z += y.z; v.w += y.w;
         }
         *reinterpret_cast<float4 *>(dst + e * KMAX) = v;
@@ -579,10 +582,12 @@ int shortconv_backward(const Dims &d, int width, int K, bool normalize, float ep
         const int slabs = (d.H * vpr4 + 255) / 256;
         // one CTA per SM (its 512 threads keep 128 registers each), and no more than the workspace has partial-sum slots for
         const long ctas = std::min<long>((long)grid.x * grid.y, std::max(1, conv_sms() / slabs));
-        const Units un = conv_units(d, ctas * BWD_GROUPS);
-        const dim3 g((unsigned)std::min<long>(ctas, (un.total + BWD_GROUPS - 1) / BWD_GROUPS), slabs);
-        if (normalize) k_shortconv_bwd_walk<true><<<g, 256 * BWD_GROUPS, 0, st>>>(cd, un, (const __nv_bfloat16 *)x, w, (const __nv_bfloat16 *)dout, (__nv_bfloat16 *)dx, ws);
-        else k_shortconv_bwd_walk<false><<<g, 256 * BWD_GROUPS, 0, st>>>(cd, un, (const __nv_bfloat16 *)x, w, (const __nv_bfloat16 *)dout, (__nv_bfloat16 *)dx, ws);
+        const int width = slabs > 1 ? 256 : (d.H * vpr4 + 31) / 32 * 32, groups = BWD_THREADS / width;
+        const Units un = conv_units(d, ctas * groups);
+        const dim3 g((unsigned)std::min<long>(ctas, (un.total + groups - 1) / groups), slabs);
+        (width == 256 ? (normalize ? k_shortconv_bwd_walk<true, 256> : k_shortconv_bwd_walk<false, 256>)
+                      : normalize ? k_shortconv_bwd_walk<true, 0> : k_shortconv_bwd_walk<false, 0>)<<<g, groups * width, 0, st>>>(
+            cd, un, width, (const __nv_bfloat16 *)x, w, (const __nv_bfloat16 *)dout, (__nv_bfloat16 *)dx, ws);
         tr.mark("shortconv_bwd");
         k_shortconv_dw<<<(C + 31) / 32, 32 * DW_WARPS, 0, st>>>((int)g.x, C, K, ws, dw);
         tr.mark("shortconv_dw");

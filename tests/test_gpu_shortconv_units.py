@@ -22,3 +22,10 @@ def test_reverse_pass_at_the_edges_of_units(B, T, H, d, K, normalize):
     dx_ref, dw_ref = orc.shortconv_backward(f["x_q"], f["w_q"], f["dout"], normalize)
     assert gu.rel_l2(dx, dx_ref) <= gu.TOL["bf16"] and gu.row_err(dx, dx_ref) <= gu.ROW_TOL["bf16"]
     assert gu.rel_l2(dw, dw_ref) <= gu.TOL["bf16"]
+
+
+# groups of 32, 64, 96, 160 and 224 threads (four channels each), as many as a CTA holds, and the first shape of two slabs
+@pytest.mark.parametrize("B,T,H,d,K", [(1, 5000, 1, 64, 4), (3, 1500, 4, 64, 4), (2, 900, 3, 128, 4), (1, 1200, 10, 64, 3), (40, 33, 7, 128, 4), (1, 700, 17, 64, 4)])
+@pytest.mark.parametrize("normalize", [True, False])
+def test_groups_as_wide_as_the_channels(B, T, H, d, K, normalize):
+    test_reverse_pass_at_the_edges_of_units(B, T, H, d, K, normalize)
