@@ -17,9 +17,7 @@
 // mbarrier arrival a warp instead of 32; 8 x 4096 x 16: 188 -> 183 us, Softmax-RetNet 172 -> 165 us; 156 with its prologue by rows).
 // The state never leaves the SM: fp32 in TMEM (Eq. 12's S), bf16 copy in shared memory as MMA operand.
 #include "sla_gla_tc.cuh"
-
-#include <algorithm>
-#include <cmath>
+#include "sla_gla_route.h"
 
 namespace sla {
 namespace {
@@ -573,84 +571,8 @@ int gla_tc_configure() {
                    cudaFuncSetAttribute(k_gla_fwd_tc<true, true>, A, (int)SMEM_BYTES) == cudaSuccess ? 0 : -1;
 }
 
-// A pair's chunk takes 1.04 to 1.13 times as long as one head's (8 x 4096 tokens x 32 heads, forward and step: Softmax-GLA 381 and 1167 us one head
-// a CTA, 198 and 620 in pairs, half the CTAs; Softmax-RetNet 346 and 863, 196 and 481), so pairs gain where single heads do not all
-// run at once.  Where one long sequence of a packed batch is what a call lasts they would lose: a sequence of 4000 tokens beside 17 of 256, 32 heads,
-// step 567 us single, 585 in pairs.  Both are estimated in chunk times: the longest sequence, or what an SM gets where there are more
-// CTAs than SMs (equal sequences: whole waves of them).
-constexpr double PAIR_CHUNK = 1.1;
-bool gla_tc_pairs(const Dims &d, const Varlen *vl) {
-    if (d.dk != 64 || d.dv != 64 || d.H % 2) return false;
-    const double sms = sm_count();
-    if (vl && vl->n_of && !vl->fwd) vl = vl->whole;         // (the form in which the forward pass leaves the state images)
-    auto lasts = [&](long heads) {
-        if (!(vl && vl->n_seq)) return std::ceil(d.B * heads / sms) * d.NT;
-        long chunks = 0, longest = 0;
-        for (const SeqInfo &s : vl->seqs) {
-            chunks += s.NT;
-            longest = std::max<long>(longest, s.NT);
-        }
-        return std::max<double>(longest, chunks * heads / sms);
-    };
-    return PAIR_CHUNK * lasts(d.H / 2) < lasts(d.H);
-}
-
-// A packed batch lasts as long as its longest sequence's chain of chunks, or what an SM gets.  Cut into segments the chain gets shorter, for a
-// pass over the cut sequences' k, v and decay beside the forward pass (the state every segment starts from) and one over q, dO and decay beside
-// the backward pass, each with a fold over its results.  Estimated in chunk times of the pass (2.1 us forward, 6.6 backward, one CTA an SM): an SM that gets
-// work all the time takes 1.2 times as long a chunk as a chain by itself, a chunk of the first pass 0.8 of a forward one, of the second 0.33 of a backward
-// one, launches and first loads 7 and 4, a segment's states 2.5 and 0.8 in what all SMs together move.  Against measured calls (T x heads of 128, longest
-// sequence; forward, and backward with gates: before -> cut, us): 8192 x 8, 4880 tokens 161 -> 56, 449 -> 100; 4096 x 16, 1695 64.5 -> 60.3, 173 -> 108;
-// 32768 x 16, 11120 372 -> 303, 1013 -> 635; 16384 x 16, 3167 119 -> 136 (not taken), 323 -> 269.  Segments have at least 8 chunks.
-void gla_tc_cut_sequences(const Dims &d, const Varlen &vl, Varlen &cut) {
-    const double sms = sm_count(), size = d.dk * d.dv / (double)(D * D);
-    long longest = 0;
-    for (const SeqInfo &s : vl.seqs) longest = std::max<long>(longest, s.NT);
-    if (longest < 16) return;
-    const int whole_hpc = gla_tc_pairs(d, &vl) ? 2 : 1;
-    auto lasts = [&](long L, int hpc, double pass, double fixed, double edge) {     // sequences longer than L in equal segments, hpc heads a CTA
-        double chunks = 0, cut_chunks = 0, top = 0, cut_top = 0, segs = 0;
-        const double heads = (double)d.H / hpc;
-        for (const SeqInfo &s : vl.seqs) {
-            const long n = (s.NT + L - 1) / L, len = (s.NT + n - 1) / n;
-            chunks += s.NT;
-            top = std::max<double>(top, len);
-            if (n > 1) { cut_chunks += s.NT; cut_top = std::max<double>(cut_top, len); segs += n; }
-        }
-        const double all = std::max(top, 1.2 * chunks * heads / sms), chunk = hpc == 2 ? PAIR_CHUNK : 1;
-        return segs > 0 ? chunk * (all + pass * std::max(cut_top, 1.2 * cut_chunks * heads / sms)) + fixed + edge * size * segs * d.H / sms : chunk * all;
-    };
-    const double whole = lasts(longest, whole_hpc, 0, 0, 0);
-    double best = 0.95 * whole;
-    long best_L = 0;
-    for (int hpc = whole_hpc; hpc <= (d.dk == 64 && d.dv == 64 && d.H % 2 == 0 ? 2 : 1); ++hpc)
-        for (long P = 2; P <= 64 && (longest + P - 1) / P >= 8; ++P) {
-            const long L = (longest + P - 1) / P;
-            const bool fwd = lasts(L, hpc, 0.8, 7, 2.5) < whole;
-            const double t = lasts(L, hpc, 0.33, 4, 0.8);
-            if (t < best && (fwd || hpc == whole_hpc)) { best = t; best_L = L; cut.fwd = fwd; }     // (a whole forward pass decides on the pairs)
-        }
-    if (!best_L) return;
-    std::vector<SeqInfo> by_id(vl.seqs);
-    std::sort(by_id.begin(), by_id.end(), [](const SeqInfo &a, const SeqInfo &b) { return a.id < b.id; });
-    for (const SeqInfo &s : by_id) {
-        cut.cut.push_back((int)cut.seqs.size());
-        const int n = (int)((s.NT + best_L - 1) / best_L), len = (s.NT + n - 1) / n;
-        for (int t0 = 0; t0 < s.T; t0 += len * C) {
-            const int T = std::min(len * C, s.T - t0), id = (int)cut.seqs.size();
-            cut.seqs.push_back({s.t0 + t0, T, (T + C - 1) / C, s.slot0, id, t0 + T == s.T ? s.id : -1, t0 == 0 ? s.id : -1, s.NT, t0 / C});
-        }
-    }
-    cut.cut.push_back((int)cut.seqs.size());
-    std::stable_sort(cut.seqs.begin(), cut.seqs.end(), [](const SeqInfo &a, const SeqInfo &b) { return a.NT > b.NT; });
-    cut.slots = vl.slots;
-    cut.n_of = (int)by_id.size();
-    cut.n_seq = (int)cut.seqs.size();
-    for (int i = 0; i < cut.n_seq; ++i)
-        if (cut.seqs[i].ht_id < 0) { cut.cut.push_back(i); ++cut.n_left; }
-    for (int i = 0; i < cut.n_seq; ++i)
-        if (cut.seqs[i].dh0_id < 0) { cut.cut.push_back(i); ++cut.n_right; }
-}
+bool gla_tc_pairs(const Dims &d, const Varlen *vl) { return pairs_of_heads(d, vl, sm_count()); }
+void gla_tc_cut_sequences(const Dims &d, const Varlen &vl, Varlen &cut) { cut_sequences(d, vl, cut, sm_count()); }
 
 // The backward runs the gradient sweep twice when it is cut into segments (once for the state gradients that leave
 // each segment, once for the results), so cutting pays only from three segments per sequence on.

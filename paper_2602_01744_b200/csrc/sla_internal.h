@@ -61,9 +61,9 @@ struct Varlen {
     // sequences, sequence s is the segments first[s] .. first[s + 1] - 1 (their ids); cut: first, then the n_left table places of segments
     // with a right neighbour, then the n_right places of those with a left one.
     // The state images are those of the uncut table (`whole`), so a forward pass and the backward pass that reads them may be of either form;
-    // fwd: the forward pass by itself gains, too.
+    // fwd: the forward pass by itself gains, too; pairs: with two 64-wide heads a CTA (where fwd is not set, the uncut table decides).
     int n_of = 0, n_left = 0, n_right = 0;
-    bool fwd = false;
+    bool fwd = false, pairs = false;
     Varlen *whole = nullptr;
     std::vector<int> cut;
     int *d_cut = nullptr;
