@@ -134,10 +134,6 @@ sla_status sla_plan_create(sla_plan **out, const sla_desc *desc) {
     if (cudaGetDevice(&dev) != cudaSuccess) return sla::cuda_error();
     if (cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, dev) != cudaSuccess) return sla::cuda_error();
     if (major != 10) return SLA_ERR_ARCH;
-    if (sla::generic_configure() != 0 || sla::gdn_configure() != 0 || sla::gla_tc_configure() != 0 ||
-        sla::gla_tc_bwd_configure() != 0 || sla::gdn_tc_configure() != 0 ||
-        sla::gdn_tc_bwd_configure() != 0 || sla::decode_configure() != 0 || sla::out_proj_configure() != 0)
-        return sla::cuda_error();
 
     sla_plan *p = new (std::nothrow) sla_plan();
     if (!p) return sla::cuda_error();
@@ -148,6 +144,15 @@ sla_status sla_plan_create(sla_plan **out, const sla_desc *desc) {
     d.dk = desc->d_k; d.dv = desc->d_v; d.C = desc->chunk;
     d.NT = (desc->T + desc->chunk - 1) / desc->chunk;
     d.scale = desc->scale;
+    // the kernels that this plan's calls can launch (all of the library's: 22.5 us a plan, 20.5 so; the first of a process loads them, too)
+    const bool tensor = !(desc->flags & SLA_FLAG_FORCE_GENERIC);
+    if (sla::generic_configure(d.io_bf16) != 0 || (d.variant == SLA_GDN && sla::gdn_configure() != 0) ||
+        (tensor && sla::gla_tc_supported(d) && (sla::gla_tc_configure() != 0 || sla::gla_tc_bwd_configure() != 0)) ||
+        (tensor && sla::gdn_tc_supported(d) && (sla::gdn_tc_configure() != 0 || sla::gdn_tc_bwd_configure() != 0)) ||
+        sla::decode_configure(d.variant, d.io_bf16) != 0 || (d.io_bf16 && sla::out_proj_configure() != 0)) {
+        delete p;
+        return sla::cuda_error();
+    }
     d.coop_sms = sla::gdn_tc_supported(d) && !(desc->flags & SLA_FLAG_FORCE_GENERIC) ? sla::gdn_chunk_sms() : 0;
     p->ws = sla::plan_workspace(d);
     p->flags = desc->flags;

@@ -473,12 +473,8 @@ bool decode_configure_one(bool bf16, int variant) {
 
 }  // namespace
 
-int decode_configure() {
-    if (!tc::encode_fn()) return -1;
-    for (int variant : {SLA_RETNET, SLA_GLA, SLA_GDN})
-        for (bool bf16 : {false, true})
-            if (!decode_configure_one<64>(bf16, variant) || !decode_configure_one<128>(bf16, variant)) return -1;
-    return 0;
+int decode_configure(int variant, bool bf16) {
+    return tc::encode_fn() && decode_configure_one<64>(bf16, variant) && decode_configure_one<128>(bf16, variant) ? 0 : -1;
 }
 
 template <int CW>

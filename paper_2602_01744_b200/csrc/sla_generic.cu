@@ -1152,10 +1152,7 @@ template <typename TIO> bool configure_t() {
 
 }  // namespace
 
-int generic_configure() {
-    bool ok = configure_t<float>() && configure_t<__nv_bfloat16>();
-    return ok ? 0 : -1;
-}
+int generic_configure(bool bf16) { return (bf16 ? configure_t<__nv_bfloat16>() : configure_t<float>()) ? 0 : -1; }
 
 int generic_forward(const Dims &d, const Workspace &w, const FwdArgs &a, bool write_o, cudaStream_t st, Tracer &tr) {
     return d.io_bf16 ? forward_t<__nv_bfloat16>(d, w, a, write_o, st, tr) : forward_t<float>(d, w, a, write_o, st, tr);

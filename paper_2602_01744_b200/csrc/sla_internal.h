@@ -146,9 +146,9 @@ int generic_forward(const Dims &d, const Workspace &w, const FwdArgs &a, bool wr
 int generic_backward(const Dims &d, const Workspace &w, const BwdArgs &a, cudaStream_t st, Tracer &tr);
 // recurrent decode (sla_decode.cu): streaming kernel over column slices of the state, 64 or 128 wide
 int decode_step(const Dims &d, const DecArgs &a, int *status, cudaStream_t st, Tracer &tr);
-int decode_configure();
+int decode_configure(int variant, bool bf16);
 // Opt the kernels into the shared memory they need (once per device).
-int generic_configure();
+int generic_configure(bool bf16);
 int gdn_configure();
 
 // ---- tensor-core (tcgen05 / TMEM / TMA) Softmax-GLA kernels: sla_gla_tc.cu ----
