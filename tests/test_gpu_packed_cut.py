@@ -43,7 +43,7 @@ def test_cut_sequences_match_the_oracle_and_the_uncut_form(base, lens, H, dk, dv
     got, launches = step(ws, ws)
     assert launches == [3 if fwd else 1, 4]
     again, launches = step(ws, ws2)
-    assert launches == [3, 7] if fwd else [1, 5]                              # other workspace: recomputed, the same bits
+    assert launches == ([3, 7] if fwd else [1, 5])                             # other workspace: recomputed, the same bits
     whole, launches = step(uncut, uncut)
     assert launches == [1, 2]
     mixed, launches = step(uncut, ws)                      # what the other form left is not taken
@@ -125,3 +125,61 @@ def test_states_in_one_buffer():
     torch.cuda.synchronize()
     plan.poll()
     assert gu.rel_l2(o2, o.double().cpu().numpy()) <= 1e-2 and gu.rel_l2(state, ht.double().cpu().numpy()) <= 1e-2
+
+
+@pytest.mark.parametrize("base", ["C2", "R2"])
+def test_state_gradients_in_one_buffer(base):
+    """dh0 in dht's buffer: a segment may write its sequence's dh0 before the last one has read dht, so the backward pass runs uncut."""
+    lens, H = (64, 2561), 2
+    cu = [0, *np.cumsum(lens).tolist()]
+    cfg = small(CONFIGS[base], B=1, T=cu[-1], H=H, seed=2710)
+    x = gu.to_dev(make_inputs(cfg, with_dO=True))
+    args = (x["q"], x["k"], x["v"], x["log_decay"], x["gq_logits"], x["gk_logits"])
+    dht = torch.randn(2, H, 128, 128, generator=torch.Generator(device="cuda").manual_seed(6), device="cuda") * 0.1
+    plan = api.sla_plan_create(cfg.variant, cfg.dtype, 1, cfg.T, H, 128, 128)
+    plan.set_sequences(cu)
+    ws = plan.workspace(backward=True)
+    g = api.sla_backward(plan, *args, x["dO"], dht=dht, want_dh0=True, workspace=ws)
+    assert plan.last_launch_count == 7
+    state = dht.clone()
+    out = {n: None if t is None else torch.empty_like(t) for n, t in g.items()}
+    out["dh0"] = state
+    api.sla_backward(plan, *args, x["dO"], dht=state, workspace=ws, out=out)
+    assert plan.last_launch_count == 3
+    whole = torch.empty(sum(-(-m // 64) + 1 for m in lens) * H * (32 << 10) + 2 * -(-cfg.T * H * 4 // 256) * 256, dtype=torch.uint8, device="cuda")
+    ref = api.sla_backward(plan, *args, x["dO"], dht=dht, want_dh0=True, workspace=whole)
+    assert plan.last_launch_count == 3
+    torch.cuda.synchronize()
+    plan.poll()
+    for n, t in ref.items():
+        if t is not None:
+            assert torch.equal(t, out[n]), n
+            assert gu.rel_l2(g[n], t.double().cpu().numpy()) <= 1e-2, n
+
+
+@pytest.mark.parametrize("flags", [0, api.SLA_FLAG_SAVE_FOR_BACKWARD])
+def test_calls_without_a_workspace_run_uncut_where_memory_is_short(monkeypatch, flags):
+    lens, H = (64, 2561), 2
+    cu = [0, *np.cumsum(lens).tolist()]
+    cfg = small(CONFIGS["C2"], B=1, T=cu[-1], H=H, seed=2720)
+    x = gu.to_dev(make_inputs(cfg, with_dO=True))
+    args = (x["q"], x["k"], x["v"], x["log_decay"], x["gq_logits"], x["gk_logits"])
+    plan = api.sla_plan_create(cfg.variant, cfg.dtype, 1, cfg.T, H, 128, 128, flags=flags)
+    plan.set_sequences(cu)
+    calls = [lambda: api.sla_forward(plan, *args)[0], lambda: api.sla_backward(plan, *args, x["dO"])["dq"]]
+    cut = [(c(), plan.last_launch_count) for c in calls]
+    assert [n for _, n in cut] == [3, 7]
+    real = torch.empty
+
+    def short(*size, **kw):
+        if kw.get("dtype") == torch.uint8 and size[0] in (plan.forward_workspace_bytes, plan.backward_workspace_bytes):
+            raise torch.OutOfMemoryError("short")
+        return real(*size, **kw)
+
+    monkeypatch.setattr(torch, "empty", short)
+    uncut = [(c(), plan.last_launch_count) for c in calls]
+    assert [n for _, n in uncut] == [1, 3]
+    torch.cuda.synchronize()
+    plan.poll()
+    for (a, _), (b, _) in zip(cut, uncut):
+        assert gu.rel_l2(a, b.double().cpu().numpy()) <= 1e-2
