@@ -118,8 +118,8 @@ sla_status sla_plan_set_sequences(sla_plan *plan, const int32_t *cu_seqlens, int
  * and then runs on slower kernels: a backward pass (and a forward pass that saves) from 56 KiB per chunk and head on, a forward pass
  * alone with any workspace or none.  (Each sequence counts as one chunk more than it has; 8 bytes per token and head, each of
  * two arrays rounded up to 256 bytes, come on top of the 130 and the 56 KiB.)  A packed Softmax-GLA or -RetNet plan whose long sequences
- * are worth cutting into segments reports scratch for their states, up to 2 x 4 d_k d_v bytes per segment and head on top of what it needs uncut; it
- * accepts that, too - nothing for a forward pass that saves nothing, 32 KiB per chunk and head and the 8 bytes per token and head otherwise - and runs uncut. */
+ * are worth cutting into segments reports scratch for their states on top of what it needs uncut: 4 d_k (2 d_v + 1) bytes per head for every segment and every sequence
+ * that stays whole.  It accepts what it needs uncut, too - nothing for a forward pass that saves nothing, 32 KiB per chunk and head and the 8 bytes per token and head otherwise - and runs uncut. */
 sla_status sla_plan_workspace_bytes(const sla_plan *plan, size_t *forward_bytes, size_t *backward_bytes);
 
 /* Synchronises with nothing; copies the plan's device status word back (on the legacy default

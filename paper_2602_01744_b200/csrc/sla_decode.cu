@@ -16,9 +16,10 @@
 // (three shuffle steps) and the warps meet nobody but the operand ring: the delta rule's chain from token to token has no
 // block-wide barrier.  A lane holds 16 rows (lane group x: x, x + 8, x + 16 ..) of CW / 32 columns, as pairs of rows in packed
 // fp32 registers (two multiply-adds an instruction).  With the rows spread over the warps, three block barriers and two trips
-// through shared memory a token set the pace.  Device time of a call, before and now, 16 heads of 128, delta rule: 16 streams x 8 tokens
-// 23.9 -> 17.4 us, 64 x 8 70.3 -> 47.4, 64 x 4 41.8 -> 31.2, one stream x 8 12.3 -> 8.8; one token: 1 stream 4.5 -> 3.8, 16 streams 10.1 -> 9.0,
-// 64 streams 23.6 -> 23.3 (5.8 TB/s: HBM).
+// through shared memory a token set the pace.  Device time of a call, before and now, 16 heads of 128, states in turn (256 MiB and more), delta rule:
+// 16 streams x 8 tokens 23.8 -> 17.4 us, 64 x 8 69.8 -> 47.1, 64 x 4 41.6 -> 30.9, one stream x 8 12.2 -> 8.7; one token: 1 stream 4.5 -> 3.9, 16 streams
+// 10.4 -> 9.3, 64 streams 23.6 -> 23.4.  Softmax-GLA, one token: 4.4 -> 3.7, 10.1 -> 8.7, 64 streams 23.3 -> 23.6 (HBM: 5.7 TB/s; 20.1 -> 14.9
+// where the 64 MiB of states stay in L2).
 // A single token takes slices of 64 columns and two CTAs per SM, whose loads and stores cover one another's barriers and whose
 // smaller items fill the last wave; several tokens take 128 columns, because preparing the operands does not shrink with the slice.
 // Both add up the rows of a state in the same order, so that n tokens in one call give the bits of n calls.

@@ -1028,8 +1028,10 @@ size_t smem_output_narrow(const Dims &d) { return smem_output(d) + sizeof(float)
 size_t smem_grads_narrow(const Dims &d) {
     return sizeof(float) * (2 * CMAX * pad4(d.dk) + 2 * CMAX * pad4(d.dv) + 3 * CMAX * pad4(CMAX) + 2 * d.dk * pad4(d.dv) + d.dk + 8 * CMAX);
 }
-// Heads of at most 64 x 64 on few chunks: no SM gets a second CTA (B x H x chunks, forward and backward, us: 2 x 4 x 16 34.7 and 73.4 -> 33.6 and 67;
-// 4 x 8 x 16 72 and 160 -> 76 and 166, where two CTAs of the general kernels hide one another's phases).
+// Heads of at most 64 x 64 on few chunks: no SM gets a second CTA.  Softmax-RetNet, 4 heads x 2 sequences, forward and step, us, general -> narrow:
+// 128 chunks of 64 x 64 26.9 and 85.6 -> 24.9 and 75.9, 144 27.2 and 89.6 -> 25.4 and 78.0, of 32 x 32 20.2 and 63.7 -> 19.8 and 60.2; past one a SM two CTAs of
+// the general kernels hide one another's phases: 152 chunks 36.4 and 117.5 -> 36.9 and 117.8 (32 x 32: 23.8 and 73.5 -> 25.3 and 78.6), 256
+// 38.7 and 125.2 -> 40.0 and 126.3, 512 64.4 and 214 -> 67.6 and 222.
 bool narrow(const Dims &d) {
     static const int sms = [] {
         int dev = 0, n = 0;
