@@ -298,6 +298,8 @@ def sla_backward(plan: Plan, q, k, v, log_decay, gq_logits, gk_logits, dO, beta=
             dh0=torch.empty((getattr(plan, "n_seq", 0) or d.B, d.H, d.d_k, d.d_v), dtype=torch.float32, device=dev) if want_dh0 else None,
         )
     if workspace is None:
+        if d.flags & SLA_FLAG_SAVE_FOR_BACKWARD:                # (nor may fresh memory be taken for a workspace that a forward pass was given and that is gone)
+            _check("sla_plan_forget_saved", lib().sla_plan_forget_saved(plan.handle))
         workspace = plan.scratch(True, dev)
     _check("sla_backward", lib().sla_backward(
         plan.handle, _ptr(q), _ptr(k), _ptr(v), _ptr(log_decay), _ptr(beta), _ptr(gq_logits),
